@@ -268,3 +268,133 @@ def tolerance(case):
     if case["kind"] == "project" and case["cache"] == "e4m3":
         t["differ"] = 0.02               # codes of values that round to another bf16: ties of the fp32 sums
     return t
+
+
+# ---------------------------------------------------------------------------------------------------------------------
+# The same in 64 bits and plain torch.  Depth slots as plain tensors: [slots, B, T, Hk, d], for K and for V.
+def _read_cache(kind, cache, B, T, Hk, d, slots):
+    Tp = -(-T // 128) * 128
+    if kind == "pm":
+        x = cache.view(slots, B, Hk, Tp, 2, d).permute(4, 0, 1, 3, 2, 5)
+    elif kind == "bf16":
+        x = cache.view(slots, B, Hk, Tp // 128, 2, d // 8, 128, 8).permute(4, 0, 1, 3, 6, 2, 5, 7).reshape(2, slots, B, Tp, Hk, d)
+    else:
+        blocks = cache.view(slots, B, Hk, Tp // 128, 2, 128 * d + 512)
+        codes = blocks[..., :128 * d].contiguous().view(torch.float8_e4m3fn).float()
+        codes = codes.view(slots, B, Hk, Tp // 128, 2, d // 16, 128, 16).permute(4, 0, 1, 3, 6, 2, 5, 7)
+        row_scale = blocks[..., 128 * d:].contiguous().view(torch.float32).permute(4, 0, 1, 3, 5, 2)
+        x = (codes.double() * row_scale[..., None, None].double()).reshape(2, slots, B, Tp, Hk, d)
+    return x[0][:, :, :T], x[1][:, :, :T]
+
+
+def _as_cache(kind, Kd, Vd):
+    slots, B, T, Hk, d = Kd.shape
+    Tp = -(-T // 128) * 128
+    x = torch.zeros(2, slots, B, Tp, Hk, d, dtype=Kd.dtype, device=Kd.device)
+    x[0, :, :, :T], x[1, :, :, :T] = Kd, Vd
+    if kind == "pm":
+        return x.permute(1, 2, 4, 3, 0, 5).reshape(-1)
+    return x.view(2, slots, B, Tp // 128, 128, Hk, d // 8, 8).permute(1, 2, 5, 3, 0, 6, 4, 7).reshape(-1)
+
+
+def _attend64(Q, K, V, Kd, Vd, scale, dO=None):
+    """(O, LSE), and with dO (O, LSE, dQ, dK, dV, dKd, dVd), head by head over blocks of queries; the last query sees every key."""
+    (B, Tq, H, d), T, Hk = Q.shape, K.shape[1], K.shape[2]
+    new = lambda x: torch.zeros(x.shape, dtype=torch.float64, device=x.device)
+    O, LSE = new(Q), torch.zeros(B, H, Tq, dtype=torch.float64, device=Q.device)
+    if dO is not None:
+        dQ, dK, dV, dKd, dVd = new(Q), new(K), new(V), new(Kd), new(Vd)
+    rows = max(128, min(2048, (1 << 27) // T))
+    for b in range(B):
+        for h in range(H):
+            j = h // (H // Hk)
+            k, v = K[b, :, j].double(), V[b, :, j].double()
+            for t in range(0, Tq, rows):
+                u = min(Tq, t + rows)
+                n = u + T - Tq                                             # keys that the block's last query sees
+                q, kd, vd = Q[b, t:u, h].double(), Kd[:, b, t:u, j].double(), Vd[:, b, t:u, j].double()
+                s = (q @ k[:n].t()).mul_(scale)
+                s.masked_fill_(torch.ones(u - t, n, dtype=torch.bool, device=s.device).triu_(n - (u - t) + 1), -math.inf)
+                sd = (q * kd).sum(-1).t() * scale
+                lse = torch.logsumexp(torch.cat([torch.logsumexp(s, 1, keepdim=True), sd], 1), 1, keepdim=True)
+                p, pd = s.sub_(lse).exp_(), (sd - lse).exp()
+                o = p @ v[:n] + (pd.t()[..., None] * vd).sum(0)
+                O[b, t:u, h], LSE[b, h, t:u] = o, lse[:, 0]
+                if dO is None:
+                    continue
+                g = dO[b, t:u, h].double()
+                D = (g * o).sum(-1, keepdim=True)
+                dV[b, :n, j] += p.t() @ g
+                ds = (g @ v[:n].t()).sub_(D).mul_(p)
+                dsd = (((g * vd).sum(-1).t() - D) * pd).t()[..., None] * scale
+                dQ[b, t:u, h] = (ds @ k[:n]).mul_(scale) + (dsd * kd).sum(0)
+                dK[b, :n, j] += (ds.t() @ q).mul_(scale)
+                dKd[:, b, t:u, j] += dsd * q
+                dVd[:, b, t:u, j] += pd.t()[..., None] * g
+    return (O, LSE) if dO is None else (O, LSE, dQ, dK, dV, dKd, dVd)
+
+
+@torch.no_grad()
+def exact(case, seed):
+    s = prepare(case, seed)
+    kind, B, T, Hk, d = s["kind"], s["B"], s["T"], s["Hk"], s["d"]
+    scale = d ** -0.5
+    if kind in ("attend", "layer"):
+        l, form = s["l"], s.get("cache", "bf16")
+        if l:
+            Kd, Vd = _read_cache(form, s["depth"].detach(), B, T, Hk, d, s["l"] + (kind == "layer"))
+        else:
+            Kd = Vd = s["K"].detach()[None][:0]
+        O, LSE, dQ, dK, dV, dKd, dVd = _attend64(s["Q"].detach(), s["K"].detach(), s["V"].detach(), Kd[:l], Vd[:l], scale, s["dO"])
+        # the gradients of the largest caches would not fit the card in 64 bits and in the order of the cache
+        parts = -(-l // -(-l // 32)) if l else 0
+        grad = _as_cache("pm" if form == "pm" else "bf16", dKd, dVd) if l and dKd.numel() < 2.5e9 else None
+        if kind == "attend":
+            return [O, LSE, dQ, dK, dV] + ([grad] if l else [])
+        slot = None if form == "e4m3" else _as_cache(form, s["K"][None].double(), s["V"][None].double())
+        return [O, LSE, slot, dQ, dK, dV, *([None] * parts if grad is None else _parts(grad, l))]
+    if kind == "stack":
+        n = s["n"]
+        Ks, Vs = [], []                                                    # what the slots hold, in their order
+        for i in range(n):
+            Ks.append(s["qkv"][i][1].detach().double())
+            Vs.append(s["qkv"][i][2].detach().double())
+            if i < n - 1:
+                X, Wk, Wv = (x.detach().double() for x in s["ffn"][i])
+                Ks.append((X @ Wk.t()).view(B, T, Hk, d))
+                Vs.append((X @ Wv.t()).view(B, T, Hk, d))
+        Ks, Vs = torch.stack(Ks), torch.stack(Vs)
+        gK, gV, outs, dQs = torch.zeros_like(Ks), torch.zeros_like(Vs), [], []
+        for i in range(n):
+            O, _, dQ, dK, dV, dKd, dVd = _attend64(s["qkv"][i][0].detach(), Ks[2 * i], Vs[2 * i], Ks[:2 * i], Vs[:2 * i], scale, s["dO"][i])
+            outs.append(O)
+            dQs.append(dQ)
+            gK[:2 * i] += dKd
+            gV[:2 * i] += dVd
+            gK[2 * i] += dK
+            gV[2 * i] += dV
+        grads = [x for i in range(n) for x in (dQs[i], gK[2 * i], gV[2 * i])]
+        for i in range(n - 1):
+            X, Wk, Wv = (x.detach().double() for x in s["ffn"][i])
+            k, v, x = gK[2 * i + 1].reshape(B * T, -1), gV[2 * i + 1].reshape(B * T, -1), X.view(B * T, -1)
+            grads += [(k @ Wk + v @ Wv).view_as(X), k.t() @ x, v.t() @ x]
+        return [*outs, *grads]
+    if kind == "prefill":
+        Kd, Vd = _read_cache("bf16", s["depth"], B, s["Tq"], Hk, d, s["l"])
+        return list(_attend64(s["Q"], s["K"], s["V"], Kd, Vd, scale))
+    if kind == "decode":
+        O, LSE = [], []
+        for b in range(B):
+            n = int(s["lens"][b]) if "lens" in s else T
+            if s["form"] == "paged":
+                K, V = (s[x][s["table"][b].long()].reshape(-1, Hk, d)[None, :n] for x in ("K", "V"))
+            else:
+                K, V = s["K"][b:b + 1, :n], s["V"][b:b + 1, :n]
+            pair = s["depth"][:, b:b + 1, None]                            # [l, 1, 1, Hk, 2, d]
+            o, lse = _attend64(s["q"][b:b + 1, None], K, V, pair[..., 0, :], pair[..., 1, :], scale)
+            O.append(o[:, 0])
+            LSE.append(lse[..., 0])
+        return [torch.cat(O), torch.cat(LSE)]
+    X = s["X"].double()
+    K, V = ((X @ s[w].double().t()).view(B, T, Hk, d) for w in ("Wk", "Wv"))
+    return [K, V, _as_cache("bf16", K[None], V[None]) if s["cache"] == "bf16" else None]
