@@ -368,6 +368,20 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
     return G == 1 || l == 0 || gqa_depth_split_bwd(d, G, l);
 }
 
+// How many SMs the depth part of a fused backward gets beside the sequence part.  Measured SM time: an entry of the row
+// ring 1.7 us (2.2 us for e4m3 codes at d = 64); an iteration of the sequence part 2.9 us (d = 64: 1.9 us) and 5 us (7 us)
+// per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both parts end together; a few SMs
+// more than that cost less than a few too few, because SMs that the depth part leaves go on with the sequence part
+// (T = 8192, l = 16, d = 128, whole backward: 24 SMs 2.53 ms, 32 2.09, 36 2.04, 48 2.12, 88 2.25; x = 33), and below
+// 16 SMs the tail of the depth part shows (T = 65536, l = 24: 12 SMs 47.0 ms, 16 46.9, 40 46.7; x = 8).
+inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, bool fp8, unsigned units) {
+    const double nq = num_tiles(T);
+    const double depth = double(units) * (l + 1) * (fp8 && d == 64 ? 2.2 : 1.7);
+    const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.45 * (nq + 1) : 7.0 + 0.95 * (nq + 1));
+    const double x = 148.0 * depth / (depth + seq);
+    return std::min(units, unsigned(std::min(148.0, std::max(16.0, std::ceil(1.06 * x + 1.0)))));
+}
+
 template <int D>
 int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     const int B = a.B, T = a.T, H = a.H, Hk = a.Hk, G = a.H / a.Hk;
@@ -381,7 +395,9 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     int dev = 0;
     if (!cuda_ok(cudaGetDevice(&dev))) return MODA_ERR_CUDA;
     if (configured_dev != dev) {
-        if (!set_smem_limit(moda_bwd_fused_kernel<D>, L::kDynamic)) return MODA_ERR_CUDA;
+        if (!set_smem_limit(moda_bwd_fused_kernel<D>, L::kDynamic) || !set_smem_limit(bwd_rows_kernel<D>, RowsSmem<D, false>::kDynamic) ||
+            !set_smem_limit(bwd_rows_kernel<D, true>, RowsSmem<D, true>::kDynamic))
+            return MODA_ERR_CUDA;
         configured_dev = dev;
     }
     float* delta = static_cast<float*>(a.workspace);
@@ -389,29 +405,45 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     const bool split_depth = G > 1 && a.l > 0;             // depth part by the per-position kernel after the finish kernel
     const unsigned tiles = unsigned(B) * H * num_tiles(T);
     constexpr int kRowThreads = kTileRows * (D / 32);
+    bool beside_rows = false;
     if (stages & 1) {
-        RowsParams r;
-        r.Q = static_cast<const __nv_bfloat16*>(a.Q);
-        r.O = static_cast<const __nv_bfloat16*>(a.O);
-        r.dO = static_cast<const __nv_bfloat16*>(a.dO);
-        r.depth_kv = a.depth_kv;
-        r.d_depth_kv = static_cast<__nv_bfloat16*>(a.d_depth_kv);
-        r.LSE = a.LSE; r.delta = delta; r.dq_acc = dq_acc;
-        r.B = B; r.T = T; r.H = H; r.l = split_depth ? 0 : a.l;
-        r.accumulate = a.accumulate_depth ? 1 : 0;
-        r.scale = a.scale; r.scale_log2 = a.scale * kLog2e;
-        if (a.fp8_cache) bwd_rows_kernel<D, true><<<tiles, kRowThreads, 0, stream>>>(r);
-        else bwd_rows_kernel<D><<<tiles, kRowThreads, 0, stream>>>(r);
+        bwd_prep_kernel<D><<<tiles, kRowThreads, 0, stream>>>(static_cast<const __nv_bfloat16*>(a.O), static_cast<const __nv_bfloat16*>(a.dO),
+                                                             delta, dq_acc, B, T, H);
         if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
+        if (a.l > 0 && !split_depth) {
+            RowsParams r;
+            r.depth_kv = a.depth_kv;
+            r.d_depth_kv = static_cast<__nv_bfloat16*>(a.d_depth_kv);
+            r.LSE = a.LSE; r.delta = delta; r.dq_acc = dq_acc;
+            r.B = B; r.T = T; r.H = H; r.l = a.l;
+            r.accumulate = a.accumulate_depth ? 1 : 0;
+            r.scale = a.scale; r.scale_log2 = a.scale * kLog2e;
+            // asked for alone, the depth part gets every SM; beside the sequence part, its share
+            beside_rows = (stages & 2) != 0;
+            const unsigned units = (tiles + 128 / D - 1) / (128 / D);
+            const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, a.fp8_cache, units) : std::min(units, 148u);
+            if (a.fp8_cache) bwd_rows_kernel<D, true><<<grid, 512, RowsSmem<D, true>::kDynamic, stream>>>(mQ, mdO, r);
+            else bwd_rows_kernel<D><<<grid, 512, RowsSmem<D, false>::kDynamic, stream>>>(mQ, mdO, r);
+            if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
+        }
     }
     if (stages & 2) {
         FusedParams f;
         f.LSE = a.LSE; f.delta = delta; f.dq_acc = dq_acc;
         f.B = B; f.T = T; f.H = H; f.G = G;
         f.scale = a.scale; f.scale_log2 = a.scale * kLog2e;
-        const unsigned grid = unsigned(B) * Hk * num_tiles(T);
-        moda_bwd_fused_kernel<D><<<grid, L::kThreads, L::kDynamic, stream>>>(mK, mV, mQ, mdO, mdK, mdV, f);
-        if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
+        f.beside_rows = beside_rows ? 1 : 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(unsigned(B) * Hk * num_tiles(T), 1, 1);
+        cfg.blockDim = dim3(L::kThreads, 1, 1);
+        cfg.dynamicSmemBytes = L::kDynamic;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = beside_rows ? 1 : 0;
+        if (!cuda_ok(cudaLaunchKernelEx(&cfg, moda_bwd_fused_kernel<D>, mK, mV, mQ, mdO, mdK, mdV, f))) return MODA_ERR_CUDA;
     }
     if (stages & 4) {
         bwd_dq_finish_kernel<D><<<tiles, kRowThreads, 0, stream>>>(dq_acc, static_cast<__nv_bfloat16*>(a.dQ), B, T, H, a.scale);

@@ -53,15 +53,10 @@ inline size_t bwd_workspace_bytes_gqa(int B, int T, int H, int Hk, int l) {
 }
 
 __device__ __forceinline__ float dot8_bf16(const uint4& a, const uint4& b) {
-    float acc = bf16_lo_to_f32(a.x) * bf16_lo_to_f32(b.x);
-    acc = fmaf(bf16_hi_to_f32(a.x), bf16_hi_to_f32(b.x), acc);
-    acc = fmaf(bf16_lo_to_f32(a.y), bf16_lo_to_f32(b.y), acc);
-    acc = fmaf(bf16_hi_to_f32(a.y), bf16_hi_to_f32(b.y), acc);
-    acc = fmaf(bf16_lo_to_f32(a.z), bf16_lo_to_f32(b.z), acc);
-    acc = fmaf(bf16_hi_to_f32(a.z), bf16_hi_to_f32(b.z), acc);
-    acc = fmaf(bf16_lo_to_f32(a.w), bf16_lo_to_f32(b.w), acc);
-    acc = fmaf(bf16_hi_to_f32(a.w), bf16_hi_to_f32(b.w), acc);
-    return acc;
+    float acc = fma_bf16x2(a.x, b.x, 0.f);
+    acc = fma_bf16x2(a.y, b.y, acc);
+    acc = fma_bf16x2(a.z, b.z, acc);
+    return fma_bf16x2(a.w, b.w, acc);
 }
 
 // D_t = <dO_t, O_t>, one group of d/8 lanes per row of the [B][T][H] row space; written as [B][H][T].

@@ -7,11 +7,11 @@
 //   dQ = scale (dS K + sum_i dU_i Kd_i)     dK = scale dS^T Q     dV = P^T dO
 //   dKd_i = scale dU_i Q                    dVd_i = R_i dO        (row-local)
 //
-// Three launches on the caller's stream:
-//   1. bwd_rows_kernel        everything that is local to a query row: D_t, and for every depth slot
-//                             R_i, dU_i, dKd_i, dVd_i (written in cache layout) and the row's depth share
-//                             of dQ, which initialises an fp32 dQ accumulator in the workspace.  Streams the
-//                             depth cache exactly once; bound by HBM.
+// Four launches on the caller's stream:
+//   0. bwd_prep_kernel        D_t, and a cleared fp32 dQ accumulator in the workspace.
+//   1. bwd_rows_kernel        (l > 0) the depth part, local to a query row: for every depth slot R_i, dU_i, dKd_i, dVd_i
+//                             (written in cache layout), and the row's depth share of dQ, added to the accumulator.
+//                             Streams the depth cache exactly once, on a share of the SMs while 2. has the others.
 //   2. moda_bwd_fused_kernel  one CTA per 128-key tile, looping over the 128-query tiles at or below the
 //                             diagonal.  Per pair of tiles: S^T = K Q^T and dP^T = V dO^T (tcgen05, operands
 //                             in shared memory; one extra k-step each adds the per-query terms -LSE / scale and
@@ -50,206 +50,38 @@ inline size_t bwd_fused_workspace_bytes(int B, int T, int H, int d) {
 }
 
 // =====================================================================================
-// 1. Row-local part: D_t, depth gradients, depth share of dQ
+// 1. Row terms D_t = <dO_t, O_t>, and a cleared dQ accumulator
 // =====================================================================================
-// One CTA per (b, h, 128-row tile); D / 32 threads per row, each owning 32 features (four 16-byte
-// chunks of every depth row).  Lanes of a row are adjacent, so the two dot products of a slot are
-// finished with shuffles; lanes with the same feature part own consecutive rows, so every warp access
-// to the cache is a set of 128-byte (d = 128) or 256-byte (d = 64) runs.  q and dO stay packed in
-// registers; a slot's key and value chunks are read once and used for everything the slot needs.
-struct RowsParams {
-    const __nv_bfloat16 *Q, *O, *dO;
-    const void* depth_kv;   // bf16 cache, or e4m3 codes + row scales (FP8 instantiation); gradients are bf16 either way
-    __nv_bfloat16* d_depth_kv;
-    const float* LSE;
-    float* delta;        // [B][H][T]
-    float* dq_acc;       // accumulator layout above; every element is written (zeros when l == 0)
-    int B, T, H, l;
-    int accumulate;      // nonzero: depth gradients are added to d_depth_kv (bf16 adds in L2)
-    float scale, scale_log2;
-};
-
-template <int D, bool FP8 = false>
-__global__ void __launch_bounds__(kTileRows * (D / 32), 512 / (kTileRows * (D / 32)))
-bwd_rows_kernel(const RowsParams p) {
+// One CTA per (b, h, 128-row tile); D / 32 threads per row, each owning 32 features.  Bound by HBM: O and dO in, the
+// fp32 accumulator out.
+template <int D>
+__global__ void __launch_bounds__(kTileRows * (D / 32))
+bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO, float* __restrict__ delta,
+                float* __restrict__ dq_acc, int B, int T, int H) {
     constexpr int PARTS = D / 32;                 // threads per row
     constexpr int CH = D / 8;                     // 16-byte chunks per row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int part = lane % PARTS;
     const int r = warp * (32 / PARTS) + lane / PARTS;
-    const int nq = num_tiles(p.T);
+    const int nq = num_tiles(T);
     const int qt = blockIdx.x % nq;
     const int bh = blockIdx.x / nq;
-    const int b = bh / p.H, h = bh % p.H;
+    const int b = bh / H, h = bh % H;
     const int t = qt * kTileRows + r;
-    const bool valid = t < p.T;
-
-    uint4 q4[4], g4[4];
     float dpart = 0.f;
-    if (valid) {
-        const size_t row = ((size_t(b) * p.T + t) * p.H + h) * CH + part * 4;
-        const uint4* Q = reinterpret_cast<const uint4*>(p.Q) + row;
-        const uint4* O = reinterpret_cast<const uint4*>(p.O) + row;
-        const uint4* G = reinterpret_cast<const uint4*>(p.dO) + row;
+    if (t < T) {
+        const size_t row = ((size_t(b) * T + t) * H + h) * CH + part * 4;
+        const uint4* o = reinterpret_cast<const uint4*>(O) + row;
+        const uint4* g = reinterpret_cast<const uint4*>(dO) + row;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            q4[j] = Q[j];
-            g4[j] = G[j];
-            dpart += dot8_bf16(O[j], g4[j]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) q4[j] = g4[j] = make_uint4(0, 0, 0, 0);
+        for (int j = 0; j < 4; ++j) dpart += dot8_bf16(o[j], g[j]);
     }
 #pragma unroll
     for (int off = 1; off < PARTS; off <<= 1) dpart += __shfl_xor_sync(0xffffffffu, dpart, off);
-    const float delta = dpart;
-    const size_t row_idx = (size_t(b) * p.H + h) * p.T + t;
-    const float neg_lse2 = valid ? -p.LSE[row_idx] * kLog2e : -INFINITY;   // rows past T: R = 0, zero gradients
-    if (valid && part == 0) p.delta[row_idx] = delta;
-
-    float acc[32];
+    if (t < T && part == 0) delta[(size_t(b) * H + h) * T + t] = dpart;
+    float4* dst = reinterpret_cast<float4*>(dq_acc) + size_t(blockIdx.x) * (D / 4) * kTileRows + threadIdx.x;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-
-    if (FP8 && p.l > 0) {
-        // e4m3 cache: this thread's 32 features are two 16-byte chunks of codes; the row's scale is one float per slot
-        // for K and one for V.  Gradients are taken with respect to the dequantised keys and values.
-        const size_t slot_stride = cache_slot_elems(p.B, p.T, p.H, D) / 8;                    // gradient cache, in uint4
-        const size_t gblk = (size_t(bh) * nq + qt) * 2 * (kTileRows * CH) + size_t(part * 4) * kTileRows + r;
-        uint4* gK = reinterpret_cast<uint4*>(p.d_depth_kv) + gblk;
-        uint4* gV = gK + kTileRows * CH;
-        const size_t slot_bytes8 = cache8_slot_bytes(p.B, p.T, p.H, D), blk_bytes8 = cache8_block_bytes(D);
-        const uint8_t* cK = reinterpret_cast<const uint8_t*>(p.depth_kv) + (size_t(bh) * nq + qt) * 2 * blk_bytes8;
-        const bool accumulate = p.accumulate != 0;
-#pragma unroll 1
-        for (int i = 0; i < p.l; ++i) {
-            const uint8_t* cV = cK + blk_bytes8;
-            uint4 k8[2], v8[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                k8[j] = __ldcs(reinterpret_cast<const uint4*>(cK) + size_t(part * 2 + j) * kTileRows + r);
-                v8[j] = __ldcs(reinterpret_cast<const uint4*>(cV) + size_t(part * 2 + j) * kTileRows + r);
-            }
-            const float sk = __ldcs(reinterpret_cast<const float*>(cK + size_t(kTileRows) * D) + r);
-            const float sv = __ldcs(reinterpret_cast<const float*>(cV + size_t(kTileRows) * D) + r);
-            float kf[32];
-            float u = 0.f, dr = 0.f;
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const uint32_t kw[4] = {k8[j].x, k8[j].y, k8[j].z, k8[j].w}, vw[4] = {v8[j].x, v8[j].y, v8[j].z, v8[j].w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float v0, v1, v2, v3;
-                    e4m3x4_to_f32(kw[k], kf[16 * j + 4 * k], kf[16 * j + 4 * k + 1], kf[16 * j + 4 * k + 2], kf[16 * j + 4 * k + 3]);
-                    e4m3x4_to_f32(vw[k], v0, v1, v2, v3);
-                    // features 16 j + 4 k .. + 3 of this thread = halves of the packed q / dO words 2 (4 j + k), 2 (4 j + k) + 1
-                    const uint32_t* qw = reinterpret_cast<const uint32_t*>(q4) + 2 * (4 * j + k);
-                    const uint32_t* gw = reinterpret_cast<const uint32_t*>(g4) + 2 * (4 * j + k);
-                    u = fmaf(bf16_lo_to_f32(qw[0]), kf[16 * j + 4 * k], u);
-                    u = fmaf(bf16_hi_to_f32(qw[0]), kf[16 * j + 4 * k + 1], u);
-                    u = fmaf(bf16_lo_to_f32(qw[1]), kf[16 * j + 4 * k + 2], u);
-                    u = fmaf(bf16_hi_to_f32(qw[1]), kf[16 * j + 4 * k + 3], u);
-                    dr = fmaf(bf16_lo_to_f32(gw[0]), v0, dr);
-                    dr = fmaf(bf16_hi_to_f32(gw[0]), v1, dr);
-                    dr = fmaf(bf16_lo_to_f32(gw[1]), v2, dr);
-                    dr = fmaf(bf16_hi_to_f32(gw[1]), v3, dr);
-                }
-            }
-#pragma unroll
-            for (int off = 1; off < PARTS; off <<= 1) {
-                u += __shfl_xor_sync(0xffffffffu, u, off);
-                dr += __shfl_xor_sync(0xffffffffu, dr, off);
-            }
-            const float R = fast_exp2(fmaf(u * sk, p.scale_log2, neg_lse2));
-            const float dU = R * (dr * sv - delta);
-            const uint32_t r2 = pack_bf16x2(R, R);
-            const float sdu = dU * p.scale;
-            const uint32_t sdu2 = pack_bf16x2(sdu, sdu);
-            const float duk = dU * sk;                        // dQ share: dU * (scale_k * code)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                uint4 ov, ok;
-                ov.x = mul_bf16x2(g4[j].x, r2); ov.y = mul_bf16x2(g4[j].y, r2);
-                ov.z = mul_bf16x2(g4[j].z, r2); ov.w = mul_bf16x2(g4[j].w, r2);
-                ok.x = mul_bf16x2(q4[j].x, sdu2); ok.y = mul_bf16x2(q4[j].y, sdu2);
-                ok.z = mul_bf16x2(q4[j].z, sdu2); ok.w = mul_bf16x2(q4[j].w, sdu2);
-                if (accumulate) {
-                    red_add_bf16x2_v4(gV + j * kTileRows, ov);
-                    red_add_bf16x2_v4(gK + j * kTileRows, ok);
-                } else {
-                    __stcs(gV + j * kTileRows, ov);
-                    __stcs(gK + j * kTileRows, ok);
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[8 * j + e] = fmaf(duk, kf[8 * j + e], acc[8 * j + e]);
-            }
-            cK += slot_bytes8; gK += slot_stride; gV += slot_stride;
-        }
-    } else
-    if (p.l > 0) {
-        const size_t slot_stride = cache_slot_elems(p.B, p.T, p.H, D) / 8;                    // in uint4
-        const size_t blk = (size_t(bh) * nq + qt) * 2 * (kTileRows * CH) + size_t(part * 4) * kTileRows + r;
-        const uint4* cK = reinterpret_cast<const uint4*>(p.depth_kv) + blk;
-        const uint4* cV = cK + kTileRows * CH;
-        uint4* gK = reinterpret_cast<uint4*>(p.d_depth_kv) + blk;
-        uint4* gV = gK + kTileRows * CH;
-        const bool accumulate = p.accumulate != 0;
-#pragma unroll 1
-        for (int i = 0; i < p.l; ++i) {
-            uint4 kc[4], vc[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                kc[j] = __ldcs(cK + j * kTileRows);          // streamed: every byte of the cache is used once
-                vc[j] = __ldcs(cV + j * kTileRows);
-            }
-            float u = 0.f, dr = 0.f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                u += dot8_bf16(q4[j], kc[j]);
-                dr += dot8_bf16(g4[j], vc[j]);
-            }
-#pragma unroll
-            for (int off = 1; off < PARTS; off <<= 1) {
-                u += __shfl_xor_sync(0xffffffffu, u, off);
-                dr += __shfl_xor_sync(0xffffffffu, dr, off);
-            }
-            const float R = fast_exp2(fmaf(u, p.scale_log2, neg_lse2));   // the forward's LSE covers both key sets
-            const float dU = R * (dr - delta);
-            const uint32_t r2 = pack_bf16x2(R, R);
-            const float sdu = dU * p.scale;
-            const uint32_t sdu2 = pack_bf16x2(sdu, sdu);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                uint4 ov, ok;
-                ov.x = mul_bf16x2(g4[j].x, r2); ov.y = mul_bf16x2(g4[j].y, r2);
-                ov.z = mul_bf16x2(g4[j].z, r2); ov.w = mul_bf16x2(g4[j].w, r2);
-                ok.x = mul_bf16x2(q4[j].x, sdu2); ok.y = mul_bf16x2(q4[j].y, sdu2);
-                ok.z = mul_bf16x2(q4[j].z, sdu2); ok.w = mul_bf16x2(q4[j].w, sdu2);
-                if (accumulate) {
-                    red_add_bf16x2_v4(gV + j * kTileRows, ov);
-                    red_add_bf16x2_v4(gK + j * kTileRows, ok);
-                } else {
-                    __stcs(gV + j * kTileRows, ov);
-                    __stcs(gK + j * kTileRows, ok);
-                }
-                acc[8 * j + 0] = fmaf(dU, bf16_lo_to_f32(kc[j].x), acc[8 * j + 0]);
-                acc[8 * j + 1] = fmaf(dU, bf16_hi_to_f32(kc[j].x), acc[8 * j + 1]);
-                acc[8 * j + 2] = fmaf(dU, bf16_lo_to_f32(kc[j].y), acc[8 * j + 2]);
-                acc[8 * j + 3] = fmaf(dU, bf16_hi_to_f32(kc[j].y), acc[8 * j + 3]);
-                acc[8 * j + 4] = fmaf(dU, bf16_lo_to_f32(kc[j].z), acc[8 * j + 4]);
-                acc[8 * j + 5] = fmaf(dU, bf16_hi_to_f32(kc[j].z), acc[8 * j + 5]);
-                acc[8 * j + 6] = fmaf(dU, bf16_lo_to_f32(kc[j].w), acc[8 * j + 6]);
-                acc[8 * j + 7] = fmaf(dU, bf16_hi_to_f32(kc[j].w), acc[8 * j + 7]);
-            }
-            cK += slot_stride; cV += slot_stride; gK += slot_stride; gV += slot_stride;
-        }
-    }
-    // depth share of dQ (unscaled) -> accumulator; the fused kernel adds the sequence share on top
-    float4* dst = reinterpret_cast<float4*>(p.dq_acc) + (size_t(bh) * nq + qt) * (D / 4) * kTileRows + size_t(part * 8) * kTileRows + r;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        dst[j * kTileRows] = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+    for (int j = 0; j < 8; ++j) dst[j * (kTileRows * PARTS)] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // =====================================================================================
@@ -283,7 +115,288 @@ bwd_dq_finish_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict
 }
 
 // =====================================================================================
-// 2. Sequence part: dK, dV and the dQ tiles
+// 2a. Row-local depth part: depth gradients and the depth share of dQ
+// =====================================================================================
+// A persistent grid of a share of the SMs (the host chooses it so that both parts end together).  It lets the next grid of
+// the stream, the sequence part, start at once: this part moves every byte of the depth cache and of its gradient cache
+// once and is bound by HBM, the sequence part by the tensor cores and L2, so one after the other leaves each resource idle
+// in turn.  Both only add to the dQ accumulator; the sequence grid ends after this one has.
+// Backward, ms, one after the other -> side by side: T = 4096, l = 23, d = 128, B = 4: 1.96 -> 1.64; T = 8192, l = 16,
+// B = 2: 2.27 -> 2.04; T = 5000, l = 23, e4m3: 1.24 -> 1.02; T = 32768, l = 32, d = 64, H = 32: 16.9 -> 16.3.
+//
+// A CTA walks units of 128 rows (d = 128; two tiles of 128 rows at d = 64, whose blocks are neighbours in the cache).
+// Per unit the ring brings the Q and dO rows (TMA, 64 KiB) and then, slot by slot, the unit's K and V blocks (one
+// contiguous run of the cache: 64 KiB in bf16, 33-34 KiB in e4m3).  A stage is released as soon as its bytes are in
+// registers, so nearly the whole ring is in flight all the time.  D / 32 threads per row, each owning 32 features;
+// lanes of a quarter warp own consecutive rows of one feature part: 128 contiguous bytes per access in the stage and
+// in the gradient cache.  The two dot products of a slot are finished with shuffles; their terms are mixed-precision FMAs
+// (unpacking the bf16 factors first made the arithmetic the bound: 2.7 us per 64 KiB in, 64 KiB out and SM against 1.55;
+// 1.05 without the stores, which are the bound now).
+struct RowsParams {
+    const void* depth_kv;   // bf16 cache, or e4m3 codes + row scales (FP8 instantiation); gradients are bf16 either way
+    __nv_bfloat16* d_depth_kv;
+    const float *LSE, *delta;
+    float* dq_acc;          // accumulator layout above; the depth share is added
+    int B, T, H, l;
+    int accumulate;         // nonzero: depth gradients are added to d_depth_kv (bf16 adds in L2)
+    float scale, scale_log2;
+};
+
+template <int D, bool FP8>
+struct RowsSmem {
+    static constexpr int kTilesPerUnit = 128 / D;                        // 512 threads, 32 features each
+    static constexpr int kQBytes = 4 * kTileRows * 128;                  // Q and dO rows of a unit: 64 KiB at either width
+    static constexpr int kTileKV = FP8 ? 2 * (kTileRows * D + kTileRows * 4) : 2 * kTileRows * D * 2;   // K and V blocks of a tile
+    static constexpr int kStages = 3;                                    // the Q, dO entry sets the stage size
+    static constexpr int kStageBytes = 65536 + (FP8 ? 4096 : 0);
+    static constexpr int kBars = kStages * kStageBytes;
+    static constexpr int kMisc = kBars + 2 * kStages * 8;
+    static constexpr int kTotal = kMisc + 16;
+    static constexpr int kDynamic = kTotal + 1024;
+    static_assert(kDynamic > 233472 / 2, "one CTA per SM: the sequence part beside it needs whole SMs too");
+    static_assert(kTilesPerUnit * kTileKV <= kStageBytes && kQBytes <= kStageBytes, "a ring stage holds either kind of entry");
+};
+
+template <int D, bool FP8 = false>
+__global__ void __launch_bounds__(512, 1)
+bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapdO, const RowsParams p) {
+    using R = RowsSmem<D, FP8>;
+    constexpr int PARTS = D / 32, TPU = R::kTilesPerUnit, NSUB = D / 64;
+    constexpr int RW = 32 / PARTS;                     // rows per warp
+    constexpr int CH = D / 8;
+    grid_launch_dependents();                          // the sequence part may take the SMs that this grid leaves
+    if (g_moda_status != 0) return;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = aligned_dynamic_smem(smem_raw, R::kTotal);
+    if (smem == nullptr) {
+        if (threadIdx.x == 0) atomicCAS(&g_moda_status, 0, kStatusSmemLayout);
+        return;
+    }
+    const uint32_t sbase = smem_u32(smem);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + R::kMisc);
+    const int B = p.B, T = p.T, H = p.H, row_ctas = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int hf = (TPU == 2) ? tid >> 8 : 0;          // which tile of the unit
+    const int part = lane / RW;
+    const int r = ((tid >> 5) & (4 * PARTS - 1)) * RW + lane % RW;
+    const int nq = num_tiles(T);
+    const int tiles = B * H * nq;
+    const int units = (tiles + TPU - 1) / TPU;
+    const int cta = blockIdx.x;
+    const int my_units = (units - cta + row_ctas - 1) / row_ctas;
+    const int n_total = my_units * (p.l + 1);          // ring entries: per unit one of Q, dO and l of K, V
+    if (tid == 0) {
+        *abort_flag = 0;
+        for (int s = 0; s < R::kStages; ++s) {
+            mbar_init(sbase + R::kBars + 8 * s, 1);
+            mbar_init(sbase + R::kBars + 8 * (R::kStages + s), 16);
+        }
+        fence_mbar_init();
+    }
+    __syncthreads();
+    const size_t slot_bytes = FP8 ? cache8_slot_bytes(B, T, H, D) : cache_slot_elems(B, T, H, D) * 2;
+    const uint64_t policy = l2_policy_evict_first();
+    // entry (unit index u, slot i; i = -1: Q and dO) into stage st
+    auto issue = [&](int u, int i, int st) {
+        const int first = (cta + u * row_ctas) * TPU;
+        const int cnt = (TPU == 1 || first + 1 < tiles) ? TPU : 1;
+        const uint32_t full = sbase + R::kBars + 8 * st, dst = sbase + st * R::kStageBytes;
+        if (i < 0) {
+            mbar_arrive_expect_tx(full, uint32_t(cnt) * (2 * kTileRows * D * 2));
+            for (int k = 0; k < cnt; ++k) {
+                const int bh = (first + k) / nq, qt = (first + k) % nq;
+#pragma unroll
+                for (int s = 0; s < NSUB; ++s) {
+                    tma_load_4d(dst + k * (kTileRows * D * 4) + s * (kTileRows * 128), &mapQ, full, s * 64, bh % H, qt * kTileRows, bh / H);
+                    tma_load_4d(dst + k * (kTileRows * D * 4) + (NSUB + s) * (kTileRows * 128), &mapdO, full, s * 64, bh % H, qt * kTileRows, bh / H);
+                }
+            }
+        } else {
+            const uint32_t bytes = uint32_t(cnt) * R::kTileKV;
+            mbar_arrive_expect_tx(full, bytes);
+            bulk_load(dst, static_cast<const uint8_t*>(p.depth_kv) + size_t(i) * slot_bytes + size_t(first) * R::kTileKV, bytes, full, policy);
+        }
+    };
+    int iu = 0, ii = -1;                               // next entry to issue (thread 0)
+    if (tid == 0) {
+        tma_prefetch_desc(&mapQ);
+        tma_prefetch_desc(&mapdO);
+        for (int n = 0; n < R::kStages && n < n_total; ++n) {
+            issue(iu, ii, n);
+            if (++ii == p.l) { ii = -1; ++iu; }
+        }
+    }
+    // row terms of the thread's row in unit u; rows past T: R = 0, zero gradients
+    auto row_terms = [&](int u, float& neg_lse2, float& delta) {
+        const int lt = (cta + u * row_ctas) * TPU + hf;
+        neg_lse2 = -INFINITY;
+        delta = 0.f;
+        if (u < my_units && lt < tiles) {
+            const int t = (lt % nq) * kTileRows + r;
+            if (t < T) {
+                const size_t idx = size_t(lt / nq) * T + t;
+                neg_lse2 = -p.LSE[idx] * kLog2e;
+                delta = p.delta[idx];
+            }
+        }
+    };
+    const size_t grad_stride = cache_slot_elems(B, T, H, D) / 8;         // slot of the gradient cache, in uint4
+    const bool accumulate = p.accumulate != 0;
+    float next_lse, next_delta;
+    row_terms(0, next_lse, next_delta);
+    int st = 0, phase = 0;
+    for (int u = 0; u < my_units; ++u) {
+        const int lt = (cta + u * row_ctas) * TPU + hf;
+        const bool have = TPU == 1 || lt < tiles;      // the last unit of an odd number of tiles has one tile
+        const float neg_lse2 = next_lse, delta = next_delta;
+        row_terms(u + 1, next_lse, next_delta);
+        uint4* gK = reinterpret_cast<uint4*>(p.d_depth_kv) + (size_t(lt) * 2 * CH + part * 4) * kTileRows + r;
+        uint4 q4[4], g4[4];
+        float acc[32];
+        for (int i = -1; i < p.l; ++i) {
+            const uint32_t full = sbase + R::kBars + 8 * st, empty = sbase + R::kBars + 8 * (R::kStages + st);
+            const uint8_t* stage = smem + st * R::kStageBytes;
+            mbar_wait(full, phase, abort_flag, 150);
+            if (i < 0) {
+                const uint8_t* qs = stage + hf * (kTileRows * D * 4);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    q4[j] = *reinterpret_cast<const uint4*>(qs + swz_chunk_offset(r, part * 4 + j));
+                    g4[j] = *reinterpret_cast<const uint4*>(qs + kTileRows * D * 2 + swz_chunk_offset(r, part * 4 + j));
+                }
+                fence_proxy_async_smem();              // the refill (async proxy) comes after these loads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty);
+#pragma unroll
+                for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+            } else {
+                float u_s = 0.f, dr = 0.f;
+                float kf[FP8 ? 32 : 1];
+                uint4 kc[FP8 ? 1 : 4];
+                float sk = 1.f;
+                if constexpr (FP8) {
+                    const uint8_t* ks = stage + hf * R::kTileKV;
+                    const uint8_t* vs = ks + kTileRows * D + kTileRows * 4;
+                    uint4 k8[2], v8[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        k8[j] = *reinterpret_cast<const uint4*>(ks + ((part * 2 + j) * kTileRows + r) * 16);
+                        v8[j] = *reinterpret_cast<const uint4*>(vs + ((part * 2 + j) * kTileRows + r) * 16);
+                    }
+                    sk = *reinterpret_cast<const float*>(ks + kTileRows * D + r * 4);
+                    const float sv = *reinterpret_cast<const float*>(vs + kTileRows * D + r * 4);
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const uint32_t kw[4] = {k8[j].x, k8[j].y, k8[j].z, k8[j].w}, vw[4] = {v8[j].x, v8[j].y, v8[j].z, v8[j].w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float v0, v1, v2, v3;
+                            e4m3x4_to_f32(kw[k], kf[16 * j + 4 * k], kf[16 * j + 4 * k + 1], kf[16 * j + 4 * k + 2], kf[16 * j + 4 * k + 3]);
+                            e4m3x4_to_f32(vw[k], v0, v1, v2, v3);
+                            // features 16 j + 4 k .. + 3 of this thread = halves of the packed q / dO words 2 (4 j + k), 2 (4 j + k) + 1
+                            const uint32_t* qw = reinterpret_cast<const uint32_t*>(q4) + 2 * (4 * j + k);
+                            const uint32_t* gw = reinterpret_cast<const uint32_t*>(g4) + 2 * (4 * j + k);
+                            u_s = fmaf(bf16_lo_to_f32(qw[0]), kf[16 * j + 4 * k], u_s);
+                            u_s = fmaf(bf16_hi_to_f32(qw[0]), kf[16 * j + 4 * k + 1], u_s);
+                            u_s = fmaf(bf16_lo_to_f32(qw[1]), kf[16 * j + 4 * k + 2], u_s);
+                            u_s = fmaf(bf16_hi_to_f32(qw[1]), kf[16 * j + 4 * k + 3], u_s);
+                            dr = fmaf(bf16_lo_to_f32(gw[0]), v0, dr);
+                            dr = fmaf(bf16_hi_to_f32(gw[0]), v1, dr);
+                            dr = fmaf(bf16_lo_to_f32(gw[1]), v2, dr);
+                            dr = fmaf(bf16_hi_to_f32(gw[1]), v3, dr);
+                        }
+                    }
+#pragma unroll
+                    for (int off = RW; off < 32; off <<= 1) {
+                        u_s += __shfl_xor_sync(0xffffffffu, u_s, off);
+                        dr += __shfl_xor_sync(0xffffffffu, dr, off);
+                    }
+                    u_s *= sk;
+                    dr *= sv;
+                } else {
+                    const uint4* ks = reinterpret_cast<const uint4*>(stage) + (hf * 2 * CH + part * 4) * kTileRows + r;
+                    uint4 vc[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        kc[j] = ks[j * kTileRows];
+                        vc[j] = ks[(CH + j) * kTileRows];
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        u_s += dot8_bf16(q4[j], kc[j]);
+                        dr += dot8_bf16(g4[j], vc[j]);
+                    }
+#pragma unroll
+                    for (int off = RW; off < 32; off <<= 1) {
+                        u_s += __shfl_xor_sync(0xffffffffu, u_s, off);
+                        dr += __shfl_xor_sync(0xffffffffu, dr, off);
+                    }
+                }
+                const float Rp = fast_exp2(fmaf(u_s, p.scale_log2, neg_lse2));       // the forward's LSE covers both key sets
+                const float dU = Rp * (dr - delta);
+                const uint32_t r2 = pack_bf16x2(Rp, Rp);
+                const float sdu = dU * p.scale;
+                const uint32_t sdu2 = pack_bf16x2(sdu, sdu);
+                const float duk = dU * sk;                 // dQ share: dU * (scale_k * code)
+                uint4* gV = gK + CH * kTileRows;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    uint4 ov, ok;
+                    ov.x = mul_bf16x2(g4[j].x, r2); ov.y = mul_bf16x2(g4[j].y, r2);
+                    ov.z = mul_bf16x2(g4[j].z, r2); ov.w = mul_bf16x2(g4[j].w, r2);
+                    ok.x = mul_bf16x2(q4[j].x, sdu2); ok.y = mul_bf16x2(q4[j].y, sdu2);
+                    ok.z = mul_bf16x2(q4[j].z, sdu2); ok.w = mul_bf16x2(q4[j].w, sdu2);
+                    if (have) {
+                        if (accumulate) {
+                            red_add_bf16x2_v4(gV + j * kTileRows, ov);
+                            red_add_bf16x2_v4(gK + j * kTileRows, ok);
+                        } else {
+                            __stcs(gV + j * kTileRows, ov);
+                            __stcs(gK + j * kTileRows, ok);
+                        }
+                    }
+                    if constexpr (FP8) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) acc[8 * j + e] = fmaf(duk, kf[8 * j + e], acc[8 * j + e]);
+                    } else {
+                        axpy_bf16x2(duk, kc[j].x, acc[8 * j + 0], acc[8 * j + 1]);
+                        axpy_bf16x2(duk, kc[j].y, acc[8 * j + 2], acc[8 * j + 3]);
+                        axpy_bf16x2(duk, kc[j].z, acc[8 * j + 4], acc[8 * j + 5]);
+                        axpy_bf16x2(duk, kc[j].w, acc[8 * j + 6], acc[8 * j + 7]);
+                    }
+                }
+                gK += grad_stride;
+            }
+            if (tid == 0 && iu < my_units) {
+                mbar_wait(empty, phase, abort_flag, 151);
+                issue(iu, ii, st);
+                if (++ii == p.l) { ii = -1; ++iu; }
+            }
+            if (++st == R::kStages) { st = 0; phase ^= 1; }
+        }
+        if (have) {
+            // the depth share of dQ (unscaled) joins the accumulator that the sequence part adds to
+            float* dst = p.dq_acc + ((size_t(lt) * (D / 4) + part * 8) * kTileRows + r) * 4;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                red_add_f32_v4(dst + j * kTileRows * 4, acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+        }
+    }
+    __syncthreads();
+    if (*abort_flag != 0) {                            // copies still in flight land before the CTA gives its memory up
+        const uint64_t t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 2000000ull) {}
+    }
+}
+
+// =====================================================================================
+// 2b. Sequence part: dK, dV and the dQ tiles
 // =====================================================================================
 // 512 threads (in warp order):
 //   row warps    two warpgroups: a thread owns one key row (= tensor-memory lane) and 64 of the 128 query columns of
@@ -382,6 +495,7 @@ struct FusedParams {
     int B, T, H;        // H = number of query heads
     int G;              // query heads per key/value head; dK, dV sum over the G heads of a group
     float scale, scale_log2;
+    int beside_rows;    // launched beside bwd_rows_kernel (which has not finished): the grid must not end before it
 };
 
 template <int D>
@@ -682,7 +796,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             for (int j = 0; j < 4; ++j) {
                 const int c = qrow0 + 4 * lane + j;
                 const float nl = (c < p.T) ? -p.LSE[row_base + c] * inv_scale : -1.0e30f;
-                const float nd = (c < p.T) ? -p.delta[row_base + c] : 0.f;
+                const float nd = (c < p.T) ? -__ldcg(p.delta + row_base + c) : 0.f;
                 av[j] = make_uint4(0u, 0u, 0u, 0u);
                 split3_bf16(nl, av[j].x, av[j].y);
                 split3_bf16(nd, av[j].z, av[j].w);
@@ -803,6 +917,8 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     }
     __syncthreads();
     if (warp == W_S) tmem_dealloc(tmem, kTmemCols);
+    // what follows on the stream reads the accumulator and the depth gradients: this grid ends after the rows kernel has
+    if (p.beside_rows && blockIdx.x == gridDim.x - 1) grid_dependency_wait();
 }
 
 }  // namespace moda

@@ -59,6 +59,12 @@ __device__ __forceinline__ bool elect_one() {
     return pred != 0;
 }
 
+// Programmatic dependent launch.  The first lets the next grid of the stream start (if it was launched to) once every CTA
+// of this one has said so or ended; the second returns when the grids that this one was launched beside have ended and
+// their writes are visible.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Warpgroup-wide register re-allocation (all 128 threads of the warpgroup execute it).
 template <int N>
 __device__ __forceinline__ void setmaxnreg_inc() {
@@ -454,6 +460,9 @@ __device__ __forceinline__ void red_add_bf16x2_v4(void* gptr, const uint4& v) {
     asm volatile("red.global.add.noftz.v4.bf16x2 [%0], {%1, %2, %3, %4};"
                  :: "l"(gptr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
+__device__ __forceinline__ void red_add_f32_v4(float* gptr, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(gptr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
 __device__ __forceinline__ void red_add_bf16x2_v2(void* gptr, const uint2& v) {
     asm volatile("red.global.add.noftz.v2.bf16x2 [%0], {%1, %2};" :: "l"(gptr), "r"(v.x), "r"(v.y) : "memory");
 }
@@ -465,6 +474,30 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
+}
+// acc + lo(a) lo(b) + hi(a) hi(b), in this order: two mixed-precision FMAs (bf16 factors, fp32 sum), each rounded once like
+// fmaf on the unpacked values, without the four instructions that unpack them.
+__device__ __forceinline__ float fma_bf16x2(uint32_t a, uint32_t b, float acc) {
+    asm("{\n"
+        ".reg .b16 al, ah, bl, bh;\n"
+        "mov.b32 {al, ah}, %1;\n"
+        "mov.b32 {bl, bh}, %2;\n"
+        "fma.rn.f32.bf16 %0, al, bl, %0;\n"
+        "fma.rn.f32.bf16 %0, ah, bh, %0;\n"
+        "}\n" : "+f"(acc) : "r"(a), "r"(b));
+    return acc;
+}
+// (y0, y1) += a * (lo(x), hi(x)): one packed fp32 FMA, each half rounded like fmaf.
+__device__ __forceinline__ void axpy_bf16x2(float a, uint32_t x, float& y0, float& y1) {
+    const uint32_t lo = x << 16, hi = x & 0xffff0000u;
+    asm("{\n"
+        ".reg .b64 aa, xx, yy;\n"
+        "mov.b64 aa, {%2, %2};\n"
+        "mov.b64 xx, {%3, %4};\n"
+        "mov.b64 yy, {%0, %1};\n"
+        "fma.rn.f32x2 yy, aa, xx, yy;\n"
+        "mov.b64 {%0, %1}, yy;\n"
+        "}\n" : "+f"(y0), "+f"(y1) : "f"(a), "r"(lo), "r"(hi));
 }
 // Four e4m3 bytes (lowest byte first) -> four floats.  Two hardware conversions to f16 pairs (exact: every e4m3 value is
 // an f16 value), then to f32.

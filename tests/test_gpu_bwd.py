@@ -179,3 +179,50 @@ def test_small_and_large_scales(scale):
     assert moda.moda_last_status() == 0
     dKd, dVd = unpack_cache(dcache, w.l, w.B, w.T, w.H, w.d)
     assert_grads_close((dQ, dK, dV, dKd, dVd), oracle_backward(x, scale), f"scale {scale}")
+
+
+# The depth part walks units of 128 rows (two tiles at d = 64) on a share of the SMs beside the sequence part.  Several units
+# per CTA, a last unit of one tile (d = 64, odd number of tiles), a ragged last tile; a depth cache in bf16 and in e4m3; and
+# the launches asked for one by one, where the depth part has every SM to itself.
+@pytest.mark.parametrize("B,T,H,d,l", [(1, 1100, 8, 128, 2), (1, 2400, 7, 64, 3), (3, 129, 1, 64, 1), (1, 3000, 3, 128, 24)])
+@pytest.mark.parametrize("e4m3", [False, True])
+def test_depth_part_beside_the_sequence_part(B, T, H, d, l, e4m3):
+    from oracle import moda_oracle as orc
+    w = synthetic.Workload("units", B, T, H, d, l)
+    x = synthetic.make(w, seed=61, device="cuda")
+    Kd, Vd = f64(x["Kd"]), f64(x["Vd"])
+    if e4m3:
+        cache = moda.alloc_depth_cache_e4m3(B, T, H, d, l, "cuda")
+        for i in range(l):
+            moda.moda_depth_cache_append_e4m3(cache, i, x["Kd"][i].contiguous(), x["Vd"][i].contiguous())
+        Kd, Vd = (orc.dequantize_e4m3_rows(*orc.quantize_e4m3_rows(y)) for y in (Kd, Vd))
+        fwd, bwd = moda.moda_attn_fwd_e4m3, moda.moda_attn_bwd_e4m3
+    else:
+        cache = build_cache(x["Kd"], x["Vd"])
+        fwd, bwd = moda.moda_attn_fwd, moda.moda_attn_bwd
+    ref = orc.backward(f64(x["Q"]), f64(x["K"]), f64(x["V"]), Kd, Vd, f64(x["dO"]), w.scale)
+    O, LSE = fwd(x["Q"], x["K"], x["V"], cache, l, w.scale)
+    dcache = moda.alloc_depth_cache(B, T, H, d, l).fill_(5.0)
+    dQ, dK, dV, dcache = bwd(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, w.scale, d_depth_kv=dcache)
+    assert moda.moda_last_status() == 0
+    got = (dQ, dK, dV, *unpack_cache(dcache, l, B, T, H, d))
+    rdQ, rdK, rdV, rdKd, rdVd = ref
+    assert_grads_close(got, (rdQ, rdK, rdV, rdKd[:0], rdVd), f"{(B, T, H, d, l, e4m3)}")
+    # dKd_i = scale R_i (<dO, vd_i> - D) q row by row: D = <dO, O> is formed from the bf16 O, which is off by up to 2^-9 of
+    # itself from its rounding and as much from the bf16 P behind it, so dU_i is off by up to R_i 2^-8 sum |dO O|; the factor
+    # and the product are rounded to bf16 once each.  Where few keys are visible the two terms of dU_i cancel and the row
+    # itself may be far below that error.
+    g, o, q = f64(x["dO"]), f64(O), f64(x["Q"])
+    norm = lambda a: np.linalg.norm(a, axis=-1)
+    R = norm(rdVd) / norm(g)
+    bound = w.scale * norm(q) * R * 2.0 ** -8 * np.abs(g * o).sum(-1) + 2.0 ** -7 * norm(rdKd) + 1e-6
+    worst = float((norm(f64(got[3]) - rdKd) / bound).max())
+    assert worst <= 1.0, f"dKd row error over its bound: {worst}"
+    assert rel_l2(f64(got[3]), rdKd) <= TOL_GRAD_REL_L2
+    if not e4m3:
+        ws = torch.empty(moda.moda_bwd_workspace_bytes(B, T, H, d, l), dtype=torch.uint8, device="cuda")
+        again = moda.alloc_depth_cache(B, T, H, d, l).fill_(5.0)
+        out = [torch.empty_like(t) for t in (dQ, dK, dV)]
+        for stage in (1, 2, 4):
+            bwd(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, w.scale, *out, again, workspace=ws, stages=stage)
+        assert_same_gradients((*got[:3], dcache), (*out, again), "stage by stage")
