@@ -584,15 +584,9 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                 // ---- depth scores u_i = <q, kd_i>, 64 features per sweep ----
 #pragma unroll 1
                 for (int half = 0; half < NSUB; ++half) {
-                    float q[64];
+                    uint4 q[8];                              // stays packed: the products are mixed-precision FMAs
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint4 v = qvalid ? __ldg(qrow + half * 8 + c) : make_uint4(0u, 0u, 0u, 0u);
-                        q[8 * c + 0] = bf16_lo_to_f32(v.x); q[8 * c + 1] = bf16_hi_to_f32(v.x);
-                        q[8 * c + 2] = bf16_lo_to_f32(v.y); q[8 * c + 3] = bf16_hi_to_f32(v.y);
-                        q[8 * c + 4] = bf16_lo_to_f32(v.z); q[8 * c + 5] = bf16_hi_to_f32(v.z);
-                        q[8 * c + 6] = bf16_lo_to_f32(v.w); q[8 * c + 7] = bf16_hi_to_f32(v.w);
-                    }
+                    for (int c = 0; c < 8; ++c) q[c] = qvalid ? __ldg(qrow + half * 8 + c) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
                     for (int i = 0; i < gl; ++i) {
                         uint4 cur[8];
@@ -600,14 +594,10 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
-                            a0 = fmaf(q[8 * c + 0], bf16_lo_to_f32(cur[c].x), a0);
-                            a1 = fmaf(q[8 * c + 1], bf16_hi_to_f32(cur[c].x), a1);
-                            a2 = fmaf(q[8 * c + 2], bf16_lo_to_f32(cur[c].y), a2);
-                            a3 = fmaf(q[8 * c + 3], bf16_hi_to_f32(cur[c].y), a3);
-                            a0 = fmaf(q[8 * c + 4], bf16_lo_to_f32(cur[c].z), a0);
-                            a1 = fmaf(q[8 * c + 5], bf16_hi_to_f32(cur[c].z), a1);
-                            a2 = fmaf(q[8 * c + 6], bf16_lo_to_f32(cur[c].w), a2);
-                            a3 = fmaf(q[8 * c + 7], bf16_hi_to_f32(cur[c].w), a3);
+                            fma2_bf16x2(q[c].x, cur[c].x, a0, a1);
+                            fma2_bf16x2(q[c].y, cur[c].y, a2, a3);
+                            fma2_bf16x2(q[c].z, cur[c].z, a0, a1);
+                            fma2_bf16x2(q[c].w, cur[c].w, a2, a3);
                         }
                         const float part = (a0 + a1) + (a2 + a3);
                         if (half == 0) sU[i * kTileRows + r] = part;
@@ -649,14 +639,10 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                         const float w = sU[i * kTileRows + r];
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
-                            acc[8 * c + 0] = fmaf(w, bf16_lo_to_f32(cur[c].x), acc[8 * c + 0]);
-                            acc[8 * c + 1] = fmaf(w, bf16_hi_to_f32(cur[c].x), acc[8 * c + 1]);
-                            acc[8 * c + 2] = fmaf(w, bf16_lo_to_f32(cur[c].y), acc[8 * c + 2]);
-                            acc[8 * c + 3] = fmaf(w, bf16_hi_to_f32(cur[c].y), acc[8 * c + 3]);
-                            acc[8 * c + 4] = fmaf(w, bf16_lo_to_f32(cur[c].z), acc[8 * c + 4]);
-                            acc[8 * c + 5] = fmaf(w, bf16_hi_to_f32(cur[c].z), acc[8 * c + 5]);
-                            acc[8 * c + 6] = fmaf(w, bf16_lo_to_f32(cur[c].w), acc[8 * c + 6]);
-                            acc[8 * c + 7] = fmaf(w, bf16_hi_to_f32(cur[c].w), acc[8 * c + 7]);
+                            axpy_bf16x2(w, cur[c].x, acc[8 * c + 0], acc[8 * c + 1]);
+                            axpy_bf16x2(w, cur[c].y, acc[8 * c + 2], acc[8 * c + 3]);
+                            axpy_bf16x2(w, cur[c].z, acc[8 * c + 4], acc[8 * c + 5]);
+                            axpy_bf16x2(w, cur[c].w, acc[8 * c + 6], acc[8 * c + 7]);
                         }
                     }
                     if (g0 == 0 && half == 0) wait_previous_tile();

@@ -487,6 +487,16 @@ __device__ __forceinline__ float fma_bf16x2(uint32_t a, uint32_t b, float acc) {
         "}\n" : "+f"(acc) : "r"(a), "r"(b));
     return acc;
 }
+// The same into two sums: acc_lo + lo(a) lo(b), acc_hi + hi(a) hi(b).
+__device__ __forceinline__ void fma2_bf16x2(uint32_t a, uint32_t b, float& acc_lo, float& acc_hi) {
+    asm("{\n"
+        ".reg .b16 al, ah, bl, bh;\n"
+        "mov.b32 {al, ah}, %2;\n"
+        "mov.b32 {bl, bh}, %3;\n"
+        "fma.rn.f32.bf16 %0, al, bl, %0;\n"
+        "fma.rn.f32.bf16 %1, ah, bh, %1;\n"
+        "}\n" : "+f"(acc_lo), "+f"(acc_hi) : "r"(a), "r"(b));
+}
 // (y0, y1) += a * (lo(x), hi(x)): one packed fp32 FMA, each half rounded like fmaf.
 __device__ __forceinline__ void axpy_bf16x2(float a, uint32_t x, float& y0, float& y1) {
     const uint32_t lo = x << 16, hi = x & 0xffff0000u;
