@@ -5,20 +5,25 @@
 // The step reads every cached K and V row once and does 4 G d FLOPs per row, so it is bound by
 // HBM; G <= 8 query rows share a key, too few for a tcgen05 tile (64 or 128 rows).
 //
-//   decode_split_tma_kernel  persistent, one CTA per SM, over work items (batch, kv head, split of the key
-//                         range).  A producer lane keeps a ring of TMA stages (64 keys: their K rows and V
+//   decode_split_tma_kernel  one CTA per SM, in teams of up to eight CTAs for adjacent kv heads, whose rows are adjacent in the
+//                         cache.  The stages (64 keys) of all (batch, kv heads of a team) groups, in this order, are cut
+//                         into equal runs, one per team, by the lengths that the sequences have: a CTA works on the
+//                         piece of each group that its run covers.  (Pieces of a fixed number of keys, dealt out in
+//                         turn, left SMs idle when lengths differ: B = 32, uniform in [1, 8192], paged, G = 4, d = 128:
+//                         146 -> 103 us; equal lengths, B = 1, T = 8192: 16.1 -> 13.7.)  A producer lane keeps a ring of TMA stages (64 keys: their K rows and V
 //                         rows as 128-byte-swizzled boxes) in flight, 128 KiB per SM, and runs ahead into
-//                         the CTA's next work item, so the HBM stream does not stop at item boundaries.
+//                         the CTA's next piece, so the HBM stream does not stop at their boundaries.
 //                         Eight consumer warps, 32 keys of a stage each: scores and weighted values with
 //                         warp-level MMAs whose 16-row operand holds the G <= 8 heads of the group (the
 //                         CUDA-core form of the same arithmetic is issue-bound from G = 4 on); K pieces
 //                         and, through transposing matrix loads, V pieces come from the swizzled stage.
 //                         Each warp keeps an online-softmax state (m, l, o) per head; at the end of an
-//                         item the warps are merged through shared memory and the CTA writes one partial
+//                         piece the warps are merged through shared memory and the CTA writes one partial
 //                         (m, l, o[d]) per head.
-//   decode_merge_kernel   grid (query head, batch): merges the partials of all splits with the l
+//   decode_merge_kernel   grid (query head, batch): merges the partials of all pieces of a group with the l
 //                         depth pairs of the token (scored here: l d-length dot products) and writes
-//                         O (bf16) and LSE (natural log).
+//                         O (bf16) and LSE (natural log).  It starts beside the split kernel (programmatic dependent
+//                         launch) and scores the depth pairs while that runs (1 to 3 us of a step).
 #pragma once
 
 #include <cstdint>
@@ -32,8 +37,8 @@ namespace moda {
 
 constexpr int kDecodeWarps = 8;
 constexpr int kDecodeThreads = kDecodeWarps * 32;
-constexpr int kDecodeKeysPerPass = kDecodeWarps * 32;      // keys one CTA scores per pass
-constexpr int kDecodeMaxSplits = 128;
+constexpr int kDecodeStageKeys = 64;
+constexpr int kDecodeMaxSplits = 128;                      // partials of a group that the workspace holds
 constexpr float kDecodeLog2e = 1.4426950408889634f;
 constexpr float kDecodeLn2 = 0.6931471805599453f;
 
@@ -44,10 +49,11 @@ struct DecodeParams {
     const __nv_bfloat16* depth;   // [l][B][Hk][2][d]: key row then value row of (slot, b, kv head)
     __nv_bfloat16* O;             // [B][H][d]
     float* LSE;                   // [B][H]
-    float* part;                  // [B][Hk][S][G][d + 2]: m (log2 domain), l, o[d]
+    float* part;                  // [B][Hk][kDecodeMaxSplits][G][d + 2]: m (log2 domain), l, o[d]; with seq_lens the last
+                                  // one of a group starts with the number of its partials
     int B, T_kv, T_cap, H, Hk, l;
-    int S, keys_per_split;        // keys_per_split is a multiple of kDecodeKeysPerPass
-    int num_sms;
+    int min_run;                  // fewest stages of a CTA's run
+    int team, teams;              // CTAs of a team (divides Hk); teams that the SMs hold
     int kv_rep;                   // groups of more than 8 query heads run as kv_rep groups of 8 on the same K, V head
     const int* seq_lens;          // [B] cached positions per sequence (each 1 .. T_kv), or null: T_kv for all
     const int* block_table;       // paged cache: [B][max_blocks] page of every block of page_size positions, or null
@@ -55,25 +61,24 @@ struct DecodeParams {
     float scale_log2;             // scale * log2(e)
 };
 
-// Split of the key range of every (batch, kv head) group into S work items of `passes_per_split`
-// passes (256 keys) each.  The persistent CTAs take items round-robin, so the step lasts as long as the
-// CTA with the most work: ceil(items / SMs) items of passes_per_split passes plus a fixed cost per item
-// (merge, partial write; about a third of a pass).  The plan with the smallest such estimate wins.
-struct DecodePlan { int S, keys_per_split; };
-inline DecodePlan decode_plan(int B, int Hk, int T_kv, int num_sms) {
-    const int passes = (T_kv + kDecodeKeysPerPass - 1) / kDecodeKeysPerPass;
-    const long long groups = (long long)B * Hk;
-    DecodePlan best{1, passes * kDecodeKeysPerPass};
-    double best_cost = 1e300;
-    for (int pp = passes; pp >= 1; --pp) {
-        const int S = (passes + pp - 1) / pp;
-        if (S > kDecodeMaxSplits) break;
-        const long long items = groups * S;
-        const long long rounds = (items + num_sms - 1) / num_sms;
-        const double cost = double(rounds) * (pp + 0.35);
-        if (cost < best_cost - 1e-9) { best_cost = cost; best = DecodePlan{S, pp * kDecodeKeysPerPass}; }
-    }
-    return best;
+// Stages of a CTA's run.  At least four, one for each pair of consumer warps (a shorter run takes as long), and enough
+// that no group is cut into more than kDecodeMaxSplits - 1 pieces.
+__host__ __device__ inline int decode_stages(int len) { return (len + kDecodeStageKeys - 1) / kDecodeStageKeys; }
+__host__ __device__ inline int decode_run(int total_stages, int teams, int min_run) {
+    const int run = (total_stages + teams - 1) / teams;
+    return run > min_run ? run : min_run;
+}
+inline int decode_min_run(int T_kv, bool equal, int groups, int teams) {
+    const int ns = decode_stages(T_kv);
+    const int cap = (ns + kDecodeMaxSplits - 3) / (kDecodeMaxSplits - 2);
+    const int least = cap > 4 ? cap : 4;
+    if (!equal) return least;
+    // equal lengths: a run that cuts every group at the same places leaves one piece per CTA where a cheaper run that crosses
+    // groups leaves two; a piece costs about a stage and a half
+    const int run = decode_run(groups * ns, teams, least);
+    const int cuts = (ns + run - 1) / run > 1 ? ns / run : 1;
+    const int even = (ns + cuts - 1) / cuts;
+    return (long long)groups * cuts <= teams && even <= run + 1 + run / 8 ? even : least;
 }
 inline size_t decode_workspace_bytes(int B, int H, int d) {
     return size_t(B) * H * kDecodeMaxSplits * (d + 2) * 4;
@@ -92,7 +97,6 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t smem_addr, uint32_t& 
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_addr) : "memory");
 }
 
-constexpr int kDecodeStageKeys = 64;
 constexpr int kDecodeConsumerWarps = 8;
 constexpr int kDecodeConsumerThreads = kDecodeConsumerWarps * 32;
 constexpr int kDecodeTmaThreads = kDecodeConsumerThreads + 32;
@@ -140,30 +144,107 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
     auto empty_bar = [&](int st) { return bars + (8 + st) * 8; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_items = p.B * p.Hk * p.S;
-    // work item -> (batch, kv head, split) and its key range
-    struct Item { int b, hk, split, k_begin, k_end, n_stage; };
-    auto item_of = [&](int it) {
-        Item w;
-        // split-major order: a CTA's items (it, it + grid, ...) then come from all parts of the key range, so
-        // the empty late splits of short sequences spread over the CTAs instead of emptying some of them
-        const int groups = p.B * p.Hk;
-        w.split = it / groups;
-        const int bh = it - w.split * groups;
-        w.hk = bh % p.Hk;
-        w.b = bh / p.Hk;
-        w.k_begin = w.split * p.keys_per_split;
-        const int len = p.seq_lens ? min(max(p.seq_lens[w.b], 1), p.T_kv) : p.T_kv;   // this sequence's cached positions
-        w.k_end = min(len, w.k_begin + p.keys_per_split);
-        w.n_stage = max(0, (w.k_end - w.k_begin + kDecodeStageKeys - 1) / kDecodeStageKeys);
-        return w;
-    };
+    auto len_of = [&](int b) { return p.seq_lens ? min(max(p.seq_lens[b], 1), p.T_kv) : p.T_kv; };   // cached positions of a sequence
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         for (int st = 0; st < L::kStages; ++st) { mbar_init(full_bar(st), 1); mbar_init(empty_bar(st), 2); }
         fence_mbar_init();
     }
+    grid_launch_dependents();                                           // the merge kernel may come up and score its depth pairs
+    // ---- this CTA's run of stages, and where it starts: sequence, kv head, stage of that group ----
+    const int my_team = int(blockIdx.x) / p.team, heads = p.Hk / p.team;   // heads: kv heads that one CTA of a team takes in turn
+    const int head_in_team = int(blockIdx.x) % p.team;
+    int total, b0 = 0, before = 0;                                      // stages in all; first sequence; stages per head before it
+    if (p.seq_lens == nullptr) {
+        total = p.B * heads * decode_stages(p.T_kv);
+    } else {
+        // Sums over the lengths, a block of them at a time.  Once for the total, which gives the run's length, and once
+        // for the sequence that the run starts in.
+        __shared__ int s_sum[kDecodeTmaThreads / 32], s_at[3];
+        auto block_scan = [&](int v, int& block_total) {                // sum over the threads before this one
+            int incl = v;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += up;
+            }
+            __syncthreads();
+            if (lane == 31) s_sum[warp] = incl;
+            __syncthreads();
+            int base = 0;
+            block_total = 0;
+#pragma unroll
+            for (int w = 0; w < kDecodeTmaThreads / 32; ++w) {
+                if (w < warp) base += s_sum[w];
+                block_total += s_sum[w];
+            }
+            return base + incl - v;
+        };
+        int sum = 0, part_sum, v = 0, pre = 0;
+        for (int b = threadIdx.x; b - int(threadIdx.x) < p.B; b += kDecodeTmaThreads) {
+            v = b < p.B ? decode_stages(len_of(b)) : 0;
+            pre = block_scan(v, part_sum) + sum;
+            sum += part_sum;
+        }
+        total = sum * heads;
+        const int first = my_team * decode_run(total, p.teams, p.min_run);
+        int carry = 0;
+        for (int b = threadIdx.x; b - int(threadIdx.x) < p.B; b += kDecodeTmaThreads) {
+            if (p.B > kDecodeTmaThreads) {                              // else the values of the first pass still stand
+                v = b < p.B ? decode_stages(len_of(b)) : 0;
+                pre = block_scan(v, part_sum) + carry;
+                carry += part_sum;
+            }
+            if (first >= pre * heads && first < (pre + v) * heads) { s_at[0] = b; s_at[1] = pre; }
+        }
+        __syncthreads();
+        if (first < total) { b0 = s_at[0]; before = s_at[1]; }
+    }
+    const int run = decode_run(total, p.teams, p.min_run);
+    const int run_begin = my_team * run, run_end = min(total, run_begin + run);
+    // the pieces of the run, one group after the other
+    struct Item { int b, hk, k_begin, k_end, n_stage, index, pieces; };   // index: of this piece in its group
+    struct Walk { int b, hk, ns, start, at; };                            // group (hk: team of heads), its stages, its first stage and ours in the order of all
+    auto walk_begin = [&]() {
+        Walk k;
+        k.at = run_begin;
+        if (p.seq_lens == nullptr) {
+            k.ns = decode_stages(p.T_kv);
+            const int group = run_begin / k.ns;
+            k.b = group / heads;
+            k.hk = group % heads;
+            k.start = group * k.ns;
+        } else {
+            k.b = b0;
+            k.ns = run_begin < total ? decode_stages(len_of(b0)) : 1;
+            k.hk = (run_begin - before * heads) / k.ns;
+            k.start = before * heads + k.hk * k.ns;
+        }
+        return k;
+    };
+    auto walk_item = [&](const Walk& k) {
+        Item w;
+        const int len = len_of(k.b);
+        const int s0 = k.at - k.start, s1 = min(k.ns, run_end - k.start);
+        w.b = k.b; w.hk = k.hk * p.team + head_in_team;
+        w.k_begin = s0 * kDecodeStageKeys;
+        w.k_end = min(len, s1 * kDecodeStageKeys);
+        w.n_stage = s1 - s0;
+        const int first_cta = k.start / run;
+        w.index = my_team - first_cta;
+        w.pieces = (k.start + k.ns - 1) / run - first_cta + 1;
+        return w;
+    };
+    auto walk_next = [&](Walk& k) {                                       // to the next group; past the run's end: at >= run_end
+        k.start += k.ns;
+        k.at = k.start;
+        if (++k.hk == heads) {
+            k.hk = 0;
+            ++k.b;
+            if (k.at < run_end) k.ns = decode_stages(len_of(k.b));
+        }
+    };
     __syncthreads();
 
     int n_issued = 0;                                                   // producer lane: stages requested so far
@@ -172,8 +253,8 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         if (lane == 0) {
             tma_prefetch_desc(&mapK);
             tma_prefetch_desc(&mapV);
-            for (int it = blockIdx.x; it < n_items && *abort_flag == 0; it += gridDim.x) {
-                const Item w = item_of(it);
+            for (Walk k = walk_begin(); k.at < run_end && *abort_flag == 0; walk_next(k)) {
+                const Item w = walk_item(k);
                 // paged cache: the page of a stage's 64 positions comes from the sequence's block table; the
                 // entry of the next stage is requested before this stage's wait, so its latency is hidden
                 const int* table = p.block_table ? p.block_table + size_t(w.b) * p.max_blocks : nullptr;
@@ -209,11 +290,11 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         const int g = lane >> 2, t = lane & 3;
         const int ctid = threadIdx.x;                                    // 0 .. 255
         // q rows (bf16, heads 0..7, zero beyond G) of an item: one 16-byte piece per thread
-        auto fetch_q = [&](const Item& w) {
+        auto fetch_q = [&](const Walk& w) {
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             const int row = ctid / CH, piece = ctid % CH;
             if (ctid < 8 * CH && row < G)
-                v = *reinterpret_cast<const uint4*>(p.q + (size_t(w.b) * p.H + w.hk * G + row) * D + piece * 8);
+                v = *reinterpret_cast<const uint4*>(p.q + (size_t(w.b) * p.H + (w.hk * p.team + head_in_team) * G + row) * D + piece * 8);
             return v;
         };
         auto store_q = [&](int buf, const uint4& v) {
@@ -221,14 +302,16 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         };
         int qb = 0;
         int gi0 = 0;                                                     // running stage index at the start of the item
-        if (blockIdx.x < n_items) store_q(0, fetch_q(item_of(blockIdx.x)));
+        Walk k = walk_begin();
+        if (k.at < run_end) store_q(0, fetch_q(k));
         decode_consumer_sync();
 #pragma unroll 1
-        for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-            const Item w = item_of(it);
-            const bool has_next = it + gridDim.x < n_items;
+        while (k.at < run_end) {
+            const Item w = walk_item(k);
+            walk_next(k);
+            const bool has_next = k.at < run_end;
             uint4 qnext = make_uint4(0u, 0u, 0u, 0u);
-            if (has_next) qnext = fetch_q(item_of(it + gridDim.x));       // lands while this item is processed
+            if (has_next) qnext = fetch_q(k);                             // lands while this piece is processed
             // A fragments of q: for every 32 features, this lane's 8 features of head g (the same 8 features
             // that it takes from a key row below, so the pairing inside the MMA is consistent)
             uint4 qf[D / 32];
@@ -333,7 +416,9 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             }
             if (has_next) store_q(qb ^ 1, qnext);
             decode_consumer_sync();
-            float* out = p.part + ((size_t(w.b) * p.Hk + w.hk) * p.S + w.split) * G * (D + 2);
+            float* out = p.part + ((size_t(w.b) * p.Hk + w.hk) * kDecodeMaxSplits + w.index) * G * (D + 2);
+            if (p.seq_lens && w.index == 0 && ctid == 0)
+                out[size_t(kDecodeMaxSplits - 1) * G * (D + 2)] = __int_as_float(w.pieces);
             for (int e = ctid; e < G * D; e += kDecodeConsumerThreads) {
                 const int hg = e / D, c = e - hg * D;
                 float mx = -INFINITY;
@@ -418,11 +503,22 @@ decode_merge_kernel(const DecodeParams p) {
         }
     }
     __syncthreads();
-    const float* part = p.part + ((size_t(b) * p.Hk + hk) * p.S * G + g) * (D + 2);   // + split * G * (D + 2)
+    // ---- from here on: what the split kernel wrote ----
+    grid_dependency_wait();
+    const float* group = p.part + (size_t(b) * p.Hk + hk) * kDecodeMaxSplits * G * (D + 2);
+    const float* part = group + g * (D + 2);                                        // + piece * G * (D + 2)
     const size_t split_stride = size_t(G) * (D + 2);
+    int S;                                                                          // pieces of the group
+    if (p.seq_lens) {
+        S = __float_as_int(__ldcg(group + (kDecodeMaxSplits - 1) * split_stride));
+    } else {
+        const int ns = decode_stages(p.T_kv), heads = p.Hk / p.team;
+        const int run = decode_run(p.B * heads * ns, p.teams, p.min_run), start = (b * heads + hk / p.team) * ns;
+        S = (start + ns - 1) / run - start / run + 1;
+    }
     // ---- global maximum over the split maxima and the depth scores ----
     float mx = -INFINITY;
-    for (int s = tid; s < p.S; s += kDecodeMergeThreads) mx = fmaxf(mx, part[s * split_stride]);
+    for (int s = tid; s < S; s += kDecodeMergeThreads) mx = fmaxf(mx, __ldcg(part + s * split_stride));
     for (int i = tid; i < p.l; i += kDecodeMergeThreads) mx = fmaxf(mx, s_d[i]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
@@ -434,11 +530,11 @@ decode_merge_kernel(const DecodeParams p) {
     __syncthreads();
     // ---- weights and the row sum ----
     float lt = 0.f;
-    for (int s = tid; s < p.S; s += kDecodeMergeThreads) {
-        const float ms = part[s * split_stride];
+    for (int s = tid; s < S; s += kDecodeMergeThreads) {
+        const float ms = __ldcg(part + s * split_stride);
         const float f = ms == -INFINITY ? 0.f : fast_exp2(ms - mx);
         s_w[s] = f;
-        lt = fmaf(f, part[s * split_stride + 1], lt);
+        lt = fmaf(f, __ldcg(part + s * split_stride + 1), lt);
     }
     for (int i = tid; i < p.l; i += kDecodeMergeThreads) {
         const float w = fast_exp2(s_d[i] - mx);
@@ -456,18 +552,18 @@ decode_merge_kernel(const DecodeParams p) {
     float acc[FPL];
 #pragma unroll
     for (int c = 0; c < FPL; ++c) acc[c] = 0.f;
-    for (int s0 = warp; s0 < p.S; s0 += NW * UN) {
+    for (int s0 = warp; s0 < S; s0 += NW * UN) {
         float x[UN][FPL];
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
-            const int s = min(s0 + u * NW, p.S - 1);
+            const int s = min(s0 + u * NW, S - 1);
             const float* src = part + s * split_stride + 2 + lane * FPL;
 #pragma unroll
-            for (int c = 0; c < FPL; ++c) x[u][c] = src[c];
+            for (int c = 0; c < FPL; ++c) x[u][c] = __ldcg(src + c);
         }
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
-            const float w = s0 + u * NW < p.S ? s_w[s0 + u * NW] : 0.f;
+            const float w = s0 + u * NW < S ? s_w[s0 + u * NW] : 0.f;
 #pragma unroll
             for (int c = 0; c < FPL; ++c) acc[c] = fmaf(w, x[u][c], acc[c]);
         }

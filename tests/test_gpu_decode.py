@@ -157,3 +157,26 @@ def test_decode_over_a_paged_cache(B, T_max, H, Hk, d, l, page):
     # the contiguous entry point with the same lengths gives the same bits
     O2, LSE2 = moda.moda_attn_decode_varlen(x["q"], x["K"], x["V"], seq_lens, x["depth"] if l else None, T_max, l, scale)
     assert torch.equal(O, O2) and torch.equal(LSE, LSE2)
+
+
+# Equal runs of stages per CTA: a run of several short sequences, one long sequence among short ones, a run that starts inside a
+# group, more sequences than the split kernel has threads (its sums over the lengths then take several rounds), one group over all
+# SMs (the run's length is set by the number of partials that the workspace holds).
+@pytest.mark.parametrize("B,T_max,H,Hk,d,l,kind", [(300, 200, 4, 2, 64, 2, "random"), (620, 70, 2, 1, 128, 1, "random"), (40, 6000, 8, 2, 128, 3, "one long"),
+                                                   (40, 6000, 4, 4, 64, 0, "all one"), (1, 40000, 2, 1, 64, 5, "full"), (3, 9000, 16, 1, 128, 4, "full")])
+def test_runs_of_stages_over_unequal_lengths(B, T_max, H, Hk, d, l, kind):
+    x = synthetic.make_decode(B, T_max, H, Hk, d, l, seed=41, device="cuda")
+    rng = np.random.default_rng(B)
+    lens = {"random": [int(v) for v in rng.integers(1, T_max + 1, size=B)], "one long": [63] * (B // 2) + [T_max] + [1] * (B - B // 2 - 1),
+            "all one": [1] * B, "full": [T_max] * B}[kind]
+    seq_lens = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    scale = d ** -0.5
+    O, LSE = moda.moda_attn_decode_varlen(x["q"], x["K"], x["V"], seq_lens, x["depth"] if l else None, T_max, l, scale)
+    assert moda.moda_last_status() == 0
+    o_ref, lse_ref = oracle_rows(x, lens, l, scale)
+    assert rel_l2(f64(O), o_ref) <= TOL_O_REL_L2
+    assert np.abs(f64(LSE) - lse_ref).max() <= TOL_LSE_ABS
+    if kind == "full":                                       # the entry point without lengths may cut the stages at other places
+        O2, LSE2 = run(x, T_max, l, scale)
+        assert rel_l2(f64(O2), o_ref) <= TOL_O_REL_L2
+        assert np.abs(f64(LSE2) - lse_ref).max() <= TOL_LSE_ABS
