@@ -120,6 +120,11 @@ int moda_depth_cache_append(void* cache, int B, int T, int H, int d, int slot,
 int moda_depth_cache_unpack(const void* cache, int B, int T, int H, int d, int slot,
                             void* K_i, void* V_i, void* stream);
 
+/* The same, added: K_i += slot's keys, V_i += its values (each sum rounded to bf16 once; either may be null).  A layer's
+ * K, V gradient is its own plus what later layers sent to its slot of the gradient cache. */
+int moda_depth_cache_unpack_add(const void* cache, int B, int T, int H, int d, int slot,
+                                void* K_i, void* V_i, void* stream);
+
 /*
  * Forward (Sec. 2.2 definition; Alg. 1 computes the same values with an online
  * softmax).  depth_kv holds at least l slots in the cache layout (may be null when

@@ -43,6 +43,7 @@ from .binding import (  # noqa: F401
     moda_depth_cache_e4m3_bytes,
     moda_depth_cache_bytes,
     moda_depth_cache_unpack,
+    moda_depth_cache_unpack_add,
     moda_depth_cache_unpack_pm,
     moda_kv_project_append,
     moda_kv_project_append_e4m3,

@@ -22,6 +22,7 @@ class _ModaAttention(torch.autograd.Function):
         ctx.save_for_backward(Q, K, V, depth_kv if l > 0 else None, O, LSE)
         ctx.l, ctx.scale = int(l), float(scale)
         ctx.mark_non_differentiable(LSE)
+        ctx.set_materialize_grads(False)                       # nothing to fill for LSE
         return O, LSE
 
     @staticmethod
@@ -30,10 +31,15 @@ class _ModaAttention(torch.autograd.Function):
         B, T, H, d = Q.shape
         Hk = K.shape[2]
         l = ctx.l
+        if dO is None:
+            dO = torch.zeros_like(O)
         d_cache = None
         if l > 0:
-            # slots >= l of the caller's cache get no gradient: start from zeros of the cache's size
-            d_cache = torch.zeros_like(depth_kv)
+            # the kernels write every element of slots < l; later slots of the caller's cache get no gradient
+            d_cache = torch.empty_like(depth_kv)
+            slots = binding.moda_depth_cache_bytes(B, T, Hk, d, l) // 2
+            if slots < depth_kv.numel():
+                d_cache.view(-1)[slots:].zero_()
         dQ, dK, dV, _ = binding.moda_attn_bwd_gqa(Q, K, V, depth_kv, O, dO.contiguous(), LSE, l, ctx.scale,
                                                   d_depth_kv=d_cache)
         return dQ, dK, dV, d_cache, None, None

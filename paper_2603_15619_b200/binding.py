@@ -18,7 +18,7 @@ LIB_PATH = os.path.join(_PKG, "libmoda_b200.so")
 MODA_MAX_DEPTH = 256
 SYMBOLS = (
     "moda_version", "moda_strerror", "moda_last_cuda_error", "moda_last_status", "moda_selftest_wait_timeout",
-    "moda_depth_cache_bytes", "moda_depth_cache_append", "moda_depth_cache_unpack",
+    "moda_depth_cache_bytes", "moda_depth_cache_append", "moda_depth_cache_unpack", "moda_depth_cache_unpack_add",
     "moda_attn_fwd", "moda_bwd_workspace_bytes", "moda_attn_bwd", "moda_attn_bwd_stages",
     "moda_attn_bwd_static_scratch",
     "moda_attn_fwd_gqa", "moda_bwd_workspace_bytes_gqa", "moda_attn_bwd_gqa", "moda_attn_bwd_gqa_stages",
@@ -74,6 +74,8 @@ def load() -> ctypes.CDLL:
     lib.moda_depth_cache_append.argtypes = [vp, ci, ci, ci, ci, ci, vp, vp, vp]
     lib.moda_depth_cache_unpack.restype = ci
     lib.moda_depth_cache_unpack.argtypes = [vp, ci, ci, ci, ci, ci, vp, vp, vp]
+    lib.moda_depth_cache_unpack_add.restype = ci
+    lib.moda_depth_cache_unpack_add.argtypes = [vp, ci, ci, ci, ci, ci, vp, vp, vp]
     lib.moda_attn_fwd.restype = ci
     lib.moda_attn_fwd.argtypes = [vp, vp, vp, vp, ci, ci, ci, ci, ci, cf, vp, vp, vp]
     lib.moda_bwd_workspace_bytes.restype = sz
@@ -141,13 +143,16 @@ def _ptr(t):
         raise ValueError("device (CUDA) tensors required")
     if not t.is_contiguous():
         raise ValueError("contiguous tensors required")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    # the current device's current stream, without the Stream object around it
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _new(shape, dtype, device, stream):
@@ -162,6 +167,8 @@ def _new(shape, dtype, device, stream):
 
 
 def _new_like(t, stream):
+    if stream is None:
+        return torch.empty_like(t, memory_format=torch.contiguous_format)
     return _new(t.shape, t.dtype, t.device, stream)
 
 
@@ -242,6 +249,14 @@ def moda_depth_cache_unpack(cache, slot, K_i, V_i, stream=None):
     B, T, H, d = _bthd(ref, "K_i/V_i")
     _check(load().moda_depth_cache_unpack(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
            "moda_depth_cache_unpack")
+
+
+def moda_depth_cache_unpack_add(cache, slot, K_i, V_i, stream=None):
+    """K_i, V_i += slot ``slot`` of a (gradient) cache, each sum rounded to bf16 once."""
+    ref = K_i if K_i is not None else V_i
+    B, T, H, d = _bthd(ref, "K_i/V_i")
+    _check(load().moda_depth_cache_unpack_add(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+           "moda_depth_cache_unpack_add")
 
 
 def moda_depth_cache_e4m3_bytes(B, T, H, d, l_max) -> int:

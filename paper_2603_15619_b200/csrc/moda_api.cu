@@ -141,6 +141,8 @@ int check_device(bool may_allocate = true) {
     if (dev != cached_dev) {
         int major = 0;
         if (!cuda_ok(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev))) return MODA_ERR_CUDA;
+        // a thread whose first CUDA call this is (an autograd worker) has no context yet, and encoding a tensor map needs one
+        if (!cuda_ok(cudaSetDevice(dev))) return MODA_ERR_CUDA;
         cached_dev = dev;
         cached_rc = (major == 10) ? MODA_OK : MODA_ERR_DEVICE;
     }
@@ -559,11 +561,11 @@ int launch_bwd(const BwdArgs& a, int stages, cudaStream_t stream) {
     return MODA_OK;
 }
 
-template <int D, bool kToCache>
+template <int D, bool kToCache, bool kAdd = false>
 int launch_cache_copy(void* cache, int B, int T, int H, int slot, void* Xk, void* Xv, cudaStream_t stream) {
     uint4* slot_base = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(cache) + size_t(slot) * cache_slot_elems(B, T, H, D));
     const unsigned grid = unsigned(B) * H * num_tiles(T) * 2;
-    depth_cache_copy_kernel<D, kToCache><<<grid, 256, 0, stream>>>(slot_base, static_cast<uint4*>(Xk), static_cast<uint4*>(Xv), T, H);
+    depth_cache_copy_kernel<D, kToCache, kAdd><<<grid, 256, 0, stream>>>(slot_base, static_cast<uint4*>(Xk), static_cast<uint4*>(Xv), T, H);
     return cuda_ok(cudaGetLastError()) ? MODA_OK : MODA_ERR_CUDA;
 }
 
@@ -835,6 +837,18 @@ int moda_depth_cache_unpack(const void* cache, int B, int T, int H, int d, int s
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return d == 128 ? launch_cache_copy<128, false>(const_cast<void*>(cache), B, T, H, slot, K_i, V_i, st)
                     : launch_cache_copy<64, false>(const_cast<void*>(cache), B, T, H, slot, K_i, V_i, st);
+}
+
+int moda_depth_cache_unpack_add(const void* cache, int B, int T, int H, int d, int slot,
+                                void* K_i, void* V_i, void* stream) {
+    if (int rc = check_shape(B, T, H, d)) return rc;
+    if (slot < 0 || slot >= MODA_MAX_DEPTH) return MODA_ERR_BAD_SLOT;
+    if (!cache || (!K_i && !V_i)) return MODA_ERR_NULL_POINTER;
+    if (!aligned16(cache) || !aligned16(K_i) || !aligned16(V_i)) return MODA_ERR_MISALIGNED;
+    if (int rc = check_device()) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    return d == 128 ? launch_cache_copy<128, false, true>(const_cast<void*>(cache), B, T, H, slot, K_i, V_i, st)
+                    : launch_cache_copy<64, false, true>(const_cast<void*>(cache), B, T, H, slot, K_i, V_i, st);
 }
 
 int moda_attn_fwd(const void* Q, const void* K, const void* V, const void* depth_kv,

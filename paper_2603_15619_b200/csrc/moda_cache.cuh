@@ -26,11 +26,18 @@ __host__ __device__ inline size_t cache_block_offset(int B, int T, int H, int d,
            (((size_t(b) * H + h) * num_tiles(T) + tile) * 2 + kv) * cache_block_elems(d);
 }
 
+// Packed bf16 sum, each half rounded to nearest even.
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // One CTA moves one (b, h, tile, kv) block between [B][T][H][d] and the cache, through a
 // shared-memory tile so that both the global reads and the global writes are 16-byte
 // accesses on consecutive addresses across a warp.
-//   kToCache = true : X -> cache (append);  false : cache -> X (unpack)
-template <int D, bool kToCache>
+//   kToCache = true : X -> cache (append);  false : cache -> X (unpack; kAdd: X += cache)
+template <int D, bool kToCache, bool kAdd = false>
 __global__ void __launch_bounds__(256)
 depth_cache_copy_kernel(uint4* __restrict__ cache_slot,            // base of the slot
                         uint4* __restrict__ Xk, uint4* __restrict__ Xv,  // [B][T][H][d]
@@ -67,7 +74,15 @@ depth_cache_copy_kernel(uint4* __restrict__ cache_slot,            // base of th
         __syncthreads();
         for (int i = threadIdx.x; i < kTileRows * CH; i += 256) {
             const int row = i / CH, ch = i % CH;
-            if (t0 + row < T) X[((size_t(b) * T + t0 + row) * H + h) * CH + ch] = tile[row * (CH + 1) + ch];
+            if (t0 + row < T) {
+                uint4* x = X + ((size_t(b) * T + t0 + row) * H + h) * CH + ch;
+                uint4 v = tile[row * (CH + 1) + ch];
+                if constexpr (kAdd) {
+                    const uint4 o = *x;
+                    v = make_uint4(add_bf16x2(o.x, v.x), add_bf16x2(o.y, v.y), add_bf16x2(o.z, v.z), add_bf16x2(o.w, v.w));
+                }
+                *x = v;
+            }
         }
     }
 }

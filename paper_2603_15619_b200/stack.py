@@ -4,9 +4,9 @@ In a MoDA model (paper Sec. 2.2, the "write" step) every attention layer appends
 the depth stream after attending, and layer l attends to the l slots written before it.  So K_i, V_i
 of layer i receive gradient from layer i's own sequence attention and, as depth slot i, from every
 later layer.  ``DepthStream`` owns the depth cache and one gradient cache of the same layout and
-wires those contributions together around the C-ABI calls (the backward call's accumulate flag adds
-each layer's depth gradients into the shared gradient cache); it is plumbing: no arithmetic of the
-operator happens here beyond adding a slot's gradient to its layer's K, V gradient.
+wires those contributions together around the C-ABI calls (the first layer of a backward pass writes its
+depth gradients into the shared gradient cache, the backward call's accumulate flag adds those of the
+others); it is plumbing: no arithmetic of the operator happens here.
 
     stream = DepthStream(B, T, H_kv, d, n_layers)
     for layer in layers:
@@ -34,7 +34,7 @@ class _Attend(torch.autograd.Function):
         O, LSE = binding.moda_attn_fwd_append(Q, K, V, stream.cache if l > 0 else None, l, scale, stream.cache, l)
         ctx.save_for_backward(Q, K, V, O, LSE)
         ctx.stream, ctx.l, ctx.scale = stream, l, scale
-        return O, token + 0
+        return O, torch.empty_like(token)
 
     @staticmethod
     def backward(ctx, dO, dtoken):
@@ -42,17 +42,13 @@ class _Attend(torch.autograd.Function):
         stream, l = ctx.stream, ctx.l
         B, T, H, d = Q.shape
         Hk = K.shape[2]
-        # slots < l of the gradient cache receive this layer's share (added in place by the kernel)
+        # slots < l of the gradient cache receive this layer's share
         dQ, dK, dV, _ = binding.moda_attn_bwd_gqa(
             Q, K, V, stream.cache if l > 0 else None, O, dO.contiguous(), LSE, l, ctx.scale,
-            d_depth_kv=stream.grad_cache if l > 0 else None,
-            stages=binding.MODA_BWD_ALL_STAGES | binding.MODA_BWD_ACCUMULATE_DEPTH)
+            d_depth_kv=stream.grads if l > 0 else None,
+            stages=binding.MODA_BWD_ALL_STAGES | (binding.MODA_BWD_ACCUMULATE_DEPTH if stream.add_to_slots(l) else 0))
         if stream.slot_has_grad(l):                                     # later layers attended to slot l
-            dKs = torch.empty_like(K)
-            dVs = torch.empty_like(V)
-            binding.moda_depth_cache_unpack(stream.grad_cache, l, dKs, dVs)
-            dK += dKs
-            dV += dVs
+            binding.moda_depth_cache_unpack_add(stream.grads, l, dK, dV)
         return dQ, dK, dV, dtoken, None, None, None
 
 
@@ -66,14 +62,14 @@ class _Write(torch.autograd.Function):
         binding.moda_depth_cache_append(stream.cache, slot, K, V)
         ctx.stream, ctx.slot = stream, slot
         ctx.save_for_backward(K, V)
-        return token + 0
+        return torch.empty_like(token)
 
     @staticmethod
     def backward(ctx, dtoken):
         K, V = ctx.saved_tensors
         dK, dV = torch.zeros_like(K), torch.zeros_like(V)
         if ctx.stream.slot_has_grad(ctx.slot):
-            binding.moda_depth_cache_unpack(ctx.stream.grad_cache, ctx.slot, dK, dV)
+            binding.moda_depth_cache_unpack(ctx.stream.grads, ctx.slot, dK, dV)
         return dK, dV, dtoken, None, None
 
 
@@ -88,7 +84,7 @@ class _ProjectWrite(torch.autograd.Function):
         binding.moda_kv_project_append(X, Wk, Wv, stream.shape[2], cache=stream.cache, slot=slot, store_kv=False)
         ctx.stream, ctx.slot = stream, slot
         ctx.save_for_backward(X, Wk, Wv)
-        return token + 0
+        return torch.empty_like(token)
 
     @staticmethod
     def backward(ctx, dtoken):
@@ -98,10 +94,40 @@ class _ProjectWrite(torch.autograd.Function):
             return torch.zeros_like(X), torch.zeros_like(Wk), torch.zeros_like(Wv), dtoken, None, None
         dK = torch.empty((B, T, Hk, d), dtype=X.dtype, device=X.device)
         dV = torch.empty_like(dK)
-        binding.moda_depth_cache_unpack(ctx.stream.grad_cache, ctx.slot, dK, dV)
+        binding.moda_depth_cache_unpack(ctx.stream.grads, ctx.slot, dK, dV)
         dK2, dV2, X2 = dK.view(B * T, Hk * d), dV.view(B * T, Hk * d), X.view(B * T, -1)
-        dX = torch.addmm(dK2 @ Wk, dV2, Wv).view_as(X)
+        dX = (dK2 @ Wk).addmm_(dV2, Wv).view_as(X)
         return dX, dK2.t() @ X2, dV2.t() @ X2, dtoken, None, None
+
+
+class _Slots:
+    """What a stream's autograd nodes share: the two caches and how far the gradient cache is filled.  Kept apart from the
+    DepthStream, whose token leads back to the nodes: a node that held the stream itself would close a reference cycle,
+    and the caches would then live until the garbage collector happens to run."""
+
+    def __init__(self, B, T, H_kv, d, n_layers, device):
+        self.shape = (B, T, H_kv, d)
+        self.n_layers = n_layers
+        self.cache = binding.alloc_depth_cache(B, T, H_kv, d, n_layers, device)
+        self.grads = torch.empty_like(self.cache)              # slots < grad_slots hold gradients, the others nothing yet
+        self.grad_slots = 0
+
+    def zero_slots(self, first, end):
+        binding.depth_cache_window(self.grads, *self.shape, first, end - first).zero_()
+
+    def add_to_slots(self, l):
+        """Whether a layer that attended to slots < l adds its depth gradients to what the gradient cache holds, or is the
+        first of a backward pass and writes them."""
+        if self.grad_slots == 0:
+            self.grad_slots = l
+            return False
+        if l > self.grad_slots:                                # an earlier pass began at a lower layer
+            self.zero_slots(self.grad_slots, l)
+            self.grad_slots = l
+        return True
+
+    def slot_has_grad(self, l):
+        return l < self.grad_slots
 
 
 class DepthStream:
@@ -110,13 +136,20 @@ class DepthStream:
     def __init__(self, B, T, H_kv, d, n_layers, device="cuda"):
         self.shape = (B, T, H_kv, d)
         self.n_layers = int(n_layers)
-        self.cache = binding.alloc_depth_cache(B, T, H_kv, d, n_layers, device)
-        self.grad_cache = torch.zeros_like(self.cache)
+        self._slots = _Slots(B, T, H_kv, d, self.n_layers, device)
+        self.cache = self._slots.cache
         self.n_written = 0
         self.token = torch.zeros((), device=device, requires_grad=True)
 
+    @property
+    def grad_cache(self):
+        """Gradient cache; zero in the slots that no backward pass has reached."""
+        if self._slots.grad_slots < self.n_layers:
+            self._slots.zero_slots(self._slots.grad_slots, self.n_layers)
+        return self._slots.grads
+
     def slot_has_grad(self, l):
-        return l < self.n_written - 1
+        return self._slots.slot_has_grad(l)
 
     def attend(self, Q, K, V, scale=None):
         """MoDA attention of the next layer: attends to the slots written so far, then appends K, V."""
@@ -125,7 +158,7 @@ class DepthStream:
             raise ValueError("more layers than the stream was sized for")
         if scale is None:
             scale = Q.shape[-1] ** -0.5
-        O, self.token = _Attend.apply(Q, K, V, self.token, self, l, float(scale))
+        O, self.token = _Attend.apply(Q, K, V, self.token, self._slots, l, float(scale))
         self.n_written = l + 1
         return O
 
@@ -134,7 +167,7 @@ class DepthStream:
         slot = self.n_written
         if slot >= self.n_layers:
             raise ValueError("more slots than the stream was sized for")
-        self.token = _Write.apply(K, V, self.token, self, slot)
+        self.token = _Write.apply(K, V, self.token, self._slots, slot)
         self.n_written = slot + 1
 
     def project_write(self, X, Wk, Wv):
@@ -143,5 +176,5 @@ class DepthStream:
         slot = self.n_written
         if slot >= self.n_layers:
             raise ValueError("more slots than the stream was sized for")
-        self.token = _ProjectWrite.apply(X, Wk, Wv, self.token, self, slot)
+        self.token = _ProjectWrite.apply(X, Wk, Wv, self.token, self._slots, slot)
         self.n_written = slot + 1

@@ -31,3 +31,15 @@ def test_append_layout_and_round_trip(B, T, H, d, l):
         moda.moda_depth_cache_unpack(cache, i, Kd2[i], Vd2[i])
     assert torch.equal(Kd2, x["Kd"]) and torch.equal(Vd2, x["Vd"])
     assert moda.moda_last_status() == 0
+
+
+@pytest.mark.parametrize("B,T,H,d", [(1, 1, 1, 64), (2, 129, 3, 128), (1, 300, 2, 64)])
+def test_unpack_add_rounds_the_sum_once(B, T, H, d):
+    g = torch.Generator(device="cuda").manual_seed(7)
+    new = lambda: torch.randn((B, T, H, d), generator=g, device="cuda").to(torch.bfloat16)
+    K, V, k, v = new(), new(), new(), new()
+    cache = moda.alloc_depth_cache(B, T, H, d, 2)
+    moda.moda_depth_cache_append(cache, 1, K, V)
+    k2, v2 = k.clone(), v.clone()
+    moda.moda_depth_cache_unpack_add(cache, 1, k2, v2)
+    assert torch.equal(k2, (k.float() + K.float()).to(torch.bfloat16)) and torch.equal(v2, (v.float() + V.float()).to(torch.bfloat16))

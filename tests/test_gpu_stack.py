@@ -162,3 +162,52 @@ def test_window_of_the_last_slots_is_the_operator_on_those_slots(B, T, H, Hk, d,
     assert float(dKd[:l - S].abs().max()) == 0.0 and float(dVd[:l - S].abs().max()) == 0.0     # slots outside the window untouched
     for got, want in ((dQ, refs[0]), (dK, refs[1]), (dV, refs[2]), (dKd[l - S:], refs[3]), (dVd[l - S:], refs[4])):
         assert rel_l2(f64(got), want) <= TOL_GRAD_REL_L2
+
+
+def test_passes_that_begin_at_different_layers_and_a_stream_that_is_dropped():
+    """A backward pass writes the slots below the first layer that it meets and adds to them from there on; a later pass
+    that begins higher finds zeros in the slots above.  The stream's caches go with its last reference."""
+    import weakref
+    B, T, H, d, n = 1, 200, 2, 64, 4
+    xs = [synthetic.make_gqa(B, T, H, H, d, 0, seed=60 + i, device="cuda") for i in range(n)]
+
+    def stack():
+        layers = [{k: x[k].clone().requires_grad_(k != "dO") for k in ("Q", "K", "V", "dO")} for x in xs]
+        stream = moda.DepthStream(B, T, H, d, n)
+        return layers, stream, [stream.attend(L["Q"], L["K"], L["V"]) for L in layers]
+
+    # the lowest layer that attends to anything first, then the whole stack: the second pass's gradients are what one pass gives,
+    # apart from slot 0, which holds the first pass's share as well
+    layers, stream, outs = stack()
+    first = torch.autograd.grad(outs[1], [layers[0]["K"]], layers[1]["dO"], retain_graph=True)[0]
+    both = torch.autograd.grad(outs, [L["K"] for L in layers], [L["dO"] for L in layers])
+    layers1, stream1, outs1 = stack()
+    once = torch.autograd.grad(outs1, [L["K"] for L in layers1], [L["dO"] for L in layers1])
+    for i in range(1, n):
+        assert torch.equal(both[i], once[i]), i
+    assert rel_l2(f64(both[0]), f64(once[0]) + f64(first)) <= TOL_GRAD_REL_L2
+    assert bool((stream1.grad_cache.view(n, -1)[n - 1] == 0).all())
+    assert moda.moda_last_status() == 0
+    gone = weakref.ref(stream1._slots)
+    del layers1, stream1, outs1, once
+    assert gone() is None, "a reference cycle keeps the caches"
+
+
+def test_a_thread_whose_first_cuda_call_is_ours():
+    import threading
+    B, T, H, d = 1, 130, 1, 64
+    x = synthetic.make_gqa(B, T, H, H, d, 0, seed=3, device="cuda")
+    want, _ = moda.moda_attn_fwd(x["Q"], x["K"], x["V"], None, 0, d ** -0.5)
+    O, LSE = torch.empty_like(x["Q"]), torch.empty((B, H, T), dtype=torch.float32, device="cuda")
+    failed = []
+
+    def work():
+        try:
+            moda.moda_attn_fwd(x["Q"], x["K"], x["V"], None, 0, d ** -0.5, O=O, LSE=LSE)
+        except Exception as e:                                 # noqa: BLE001
+            failed.append(e)
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert not failed and torch.equal(O, want), failed
