@@ -1034,15 +1034,12 @@ int moda_attn_fwd_append_e4m3(const void* Q, const void* K, const void* V, const
     if (l > 0 && append_cache_e4m3 == depth_kv_e4m3 && append_slot < l && H_kv != H) return MODA_ERR_BAD_SLOT;
     if (int rc = check_device()) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    void* slot = static_cast<uint8_t*>(append_cache_e4m3) + size_t(append_slot) * cache8_slot_bytes(B, T, H_kv, d);
-    // Quantising a row costs the depth warps about as many instructions as eight depth slots do.  On long sequences that
-    // disappears under the key loop (64K: + 0.07 ms against 0.19 ms for a separate pass); on short ones the depth warps
-    // set the pace and the separate HBM-bound pass is cheaper (8K, l = 16: 0.06 ms against + 0.14 ms), so the quantiser
-    // then runs as its own launch behind the forward (same bytes; still after every read of the cache by this call).
-    const bool fused = T >= 32768;
-    const int rc = d == 128 ? launch_fwd<128>(Q, K, V, depth_kv_e4m3, B, T, T, H, H_kv, l, scale, O, LSE, fused ? slot : nullptr, st, kCacheE4m3)
-                            : launch_fwd<64>(Q, K, V, depth_kv_e4m3, B, T, T, H, H_kv, l, scale, O, LSE, fused ? slot : nullptr, st, kCacheE4m3);
-    if (rc != MODA_OK || fused) return rc;
+    // The quantiser runs as its own launch behind the forward, after every read of the cache by this call.  Inside the
+    // forward's depth warps it costs about as many instructions as eight depth slots (l = 8, d = 128, ms, inside -> behind:
+    // T = 32768 4.64 -> 4.50, 65536 17.40 -> 17.21; B = 2, T = 5000 0.53 -> 0.36).
+    const int rc = d == 128 ? launch_fwd<128>(Q, K, V, depth_kv_e4m3, B, T, T, H, H_kv, l, scale, O, LSE, nullptr, st, kCacheE4m3)
+                            : launch_fwd<64>(Q, K, V, depth_kv_e4m3, B, T, T, H, H_kv, l, scale, O, LSE, nullptr, st, kCacheE4m3);
+    if (rc != MODA_OK) return rc;
     return moda_depth_cache_append_e4m3(append_cache_e4m3, B, T, H_kv, d, append_slot, K, V, stream);
 }
 

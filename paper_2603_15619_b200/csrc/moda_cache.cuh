@@ -170,14 +170,16 @@ __device__ __forceinline__ float div_rn(float x, const RowDivider& d) {
     return q0 == 0.f ? q0 : fmaf(e, d.r, q0);      // a zero keeps the sign of x, as the IEEE quotient does (-0 has its own code)
 }
 
-// One CTA quantises one (b, h, tile, kv) block of a [B][T][H][d] tensor into a slot.  256 threads: thread
-// (row r, half hf) owns d/2 features of its row; the two halves of a row meet in shared memory for the row maximum.
+// One CTA quantises one (b, h, tile, kv) block of a [B][T][H][d] tensor into a slot.  d / 16 lanes per row, 16 features and
+// one 16-byte chunk of codes each; the row maximum is a few shuffles, and a thread's rows are all requested before the first
+// is used.  Bound by HBM (2 d bytes in, d + 4 out per row): T = 16384, 16 heads of 128: 111 -> 41 us (4.9 TB/s) against a
+// version that turned the tile in shared memory, and T = 65536: 473 -> 147 us.
 template <int D>
 __global__ void __launch_bounds__(256)
 depth_cache_quant_kernel(uint8_t* __restrict__ slot_base, const uint4* __restrict__ Xk, const uint4* __restrict__ Xv, int T, int H) {
     constexpr int CH = D / 8;                       // 16-byte chunks (8 bf16) per input row
-    __shared__ uint4 tile[kTileRows * (CH + 1)];
-    __shared__ float amax2[2][kTileRows];
+    constexpr int LPR = D / 16, RPW = 32 / LPR;     // lanes per row, rows per warp at a time
+    constexpr int PASSES = kTileRows / (8 * RPW);
     const int ntile = num_tiles(T);
     int bid = blockIdx.x;
     const int kv = bid & 1; bid >>= 1;
@@ -187,47 +189,48 @@ depth_cache_quant_kernel(uint8_t* __restrict__ slot_base, const uint4* __restric
     const uint4* X = kv ? Xv : Xk;
     uint8_t* blk = slot_base + (((size_t(b) * H + h) * ntile + tl) * 2 + kv) * cache8_block_bytes(D);
     const int t0 = tl * kTileRows;
-    for (int i = threadIdx.x; i < kTileRows * CH; i += 256) {
-        const int row = i / CH, ch = i % CH;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (t0 + row < T) v = X[((size_t(b) * T + t0 + row) * H + h) * CH + ch];
-        tile[row * (CH + 1) + ch] = v;
-    }
-    __syncthreads();
-    const int r = threadIdx.x & 127, hf = threadIdx.x >> 7;
-    constexpr int HCH = CH / 2;                     // input chunks of this thread's half row
-    float x[D / 2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = lane / RPW, r0 = warp * (PASSES * RPW) + lane % RPW;       // feature chunk, first row
+    uint4 in[PASSES][2];
 #pragma unroll
-    for (int c = 0; c < HCH; ++c) {
-        const uint4 v = tile[r * (CH + 1) + hf * HCH + c];
-        x[8 * c + 0] = __uint_as_float(v.x << 16); x[8 * c + 1] = __uint_as_float(v.x & 0xffff0000u);
-        x[8 * c + 2] = __uint_as_float(v.y << 16); x[8 * c + 3] = __uint_as_float(v.y & 0xffff0000u);
-        x[8 * c + 4] = __uint_as_float(v.z << 16); x[8 * c + 5] = __uint_as_float(v.z & 0xffff0000u);
-        x[8 * c + 6] = __uint_as_float(v.w << 16); x[8 * c + 7] = __uint_as_float(v.w & 0xffff0000u);
+    for (int i = 0; i < PASSES; ++i) {
+        const int t = t0 + r0 + i * RPW;
+        in[i][0] = in[i][1] = make_uint4(0, 0, 0, 0);
+        if (t < T) {
+            const uint4* src = X + ((size_t(b) * T + t) * H + h) * CH + 2 * c;
+            in[i][0] = src[0];
+            in[i][1] = src[1];
+        }
     }
-    float am = 0.f;
-#pragma unroll
-    for (int i = 0; i < D / 2; ++i) am = fmaxf(am, fabsf(x[i]));
-    amax2[hf][r] = am;
-    __syncthreads();
-    am = fmaxf(amax2[0][r], amax2[1][r]);
-    const float scale = am > 0.f ? __fdiv_rn(am, 448.f) : 1.f;
-    const RowDivider dv = make_row_divider(scale);
     uint4* codes = reinterpret_cast<uint4*>(blk);
 #pragma unroll
-    for (int g = 0; g < D / 32; ++g) {              // 16 features per output chunk
+    for (int i = 0; i < PASSES; ++i) {
+        const uint32_t w8[8] = {in[i][0].x, in[i][0].y, in[i][0].z, in[i][0].w, in[i][1].x, in[i][1].y, in[i][1].z, in[i][1].w};
+        float x[16];
+        float am = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            x[2 * k] = __uint_as_float(w8[k] << 16);
+            x[2 * k + 1] = __uint_as_float(w8[k] & 0xffff0000u);
+            am = fmaxf(am, fmaxf(fabsf(x[2 * k]), fabsf(x[2 * k + 1])));
+        }
+#pragma unroll
+        for (int off = RPW; off < 32; off <<= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, off));
+        const float scale = am > 0.f ? __fdiv_rn(am, 448.f) : 1.f;
+        const RowDivider dv = make_row_divider(scale);
         uint32_t w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float* xx = x + 16 * g + 4 * k;
+            const float* xx = x + 4 * k;
             uint16_t lo, hi;
             asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(lo) : "f"(div_rn(xx[1], dv)), "f"(div_rn(xx[0], dv)));
             asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(hi) : "f"(div_rn(xx[3], dv)), "f"(div_rn(xx[2], dv)));
             w[k] = uint32_t(lo) | (uint32_t(hi) << 16);
         }
-        codes[size_t(hf * (D / 32) + g) * kTileRows + r] = make_uint4(w[0], w[1], w[2], w[3]);
+        const int r = r0 + i * RPW;
+        codes[c * kTileRows + r] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (c == 0) reinterpret_cast<float*>(blk + size_t(kTileRows) * D)[r] = scale;
     }
-    if (hf == 0) reinterpret_cast<float*>(blk + size_t(kTileRows) * D)[r] = scale;
 }
 
 }  // namespace moda

@@ -113,7 +113,7 @@ struct FwdParams {
     // "Write" step of the depth stream fused into the forward: when not null, the base of one cache slot
     // (H / G heads) into which every CTA copies the K and V rows of its own positions (append_rows_from_global).
     // Only with kv_off == 0; the first head of a group writes.
-    void* append_slot;               // bf16 slot, or (e4m3 instantiations) a slot of codes + row scales
+    void* append_slot;               // bf16 slot (an e4m3 slot is written by its own kernel behind the forward)
 };
 
 // Which (batch, query head, key/value head, query tile) a CTA works on.  The G query heads that
@@ -156,10 +156,8 @@ __device__ __forceinline__ uint32_t swz_chunk_offset(int r, int c) {
 // contiguous bytes per chunk.  The rows are read from global memory (the key loop loads the same rows as its diagonal
 // tile, so they come from L2 or cost one more read of 4 d bytes per position), which lets the depth warps do this as
 // soon as they have finished reading the cache, off the path of the key loop and the epilogue.  Rows past T are written
-// as zeros (e4m3: code 0, scale 1), which is what the cache wants in its tail rows.
-// FP8: the slot is in the e4m3 layout (moda_cache.cuh) and the row is quantised exactly as depth_cache_quant_kernel does
-// (row maximum / 448 as the scale, correctly rounded quotients, round to nearest even, saturating; a zero row has scale 1).
-template <int D, bool FP8>
+// as zeros, which is what the cache wants in its tail rows.
+template <int D>
 __device__ __forceinline__ void append_rows_from_global(void* slot, const __nv_bfloat16* K, const __nv_bfloat16* V,
                                                         int b, int hk, int Hk, int T, int nq, int qt, int r) {
     constexpr int CH = D / 8;
@@ -173,42 +171,9 @@ __device__ __forceinline__ void append_rows_from_global(void* slot, const __nv_b
         uint4 x[CH];
 #pragma unroll
         for (int c = 0; c < CH; ++c) x[c] = valid ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
-        if constexpr (!FP8) {
-            uint4* dst = reinterpret_cast<uint4*>(slot) + (block_index * 2 + kv) * (kTileRows * CH) + r;
+        uint4* dst = reinterpret_cast<uint4*>(slot) + (block_index * 2 + kv) * (kTileRows * CH) + r;
 #pragma unroll
-            for (int c = 0; c < CH; ++c) dst[c * kTileRows] = x[c];
-        } else {
-            uint8_t* blk = static_cast<uint8_t*>(slot) + (block_index * 2 + kv) * cache8_block_bytes(D);
-            float am = 0.f;
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                const uint32_t w[4] = {x[c].x, x[c].y, x[c].z, x[c].w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) am = fmaxf(am, fmaxf(fabsf(bf16_lo_to_f32(w[k])), fabsf(bf16_hi_to_f32(w[k]))));
-            }
-            const float scale = am > 0.f ? __fdiv_rn(am, 448.f) : 1.f;
-            const RowDivider dv = make_row_divider(scale);
-            uint4* codes = reinterpret_cast<uint4*>(blk) + r;
-#pragma unroll
-            for (int g = 0; g < D / 16; ++g) {            // 16 features per chunk of codes = two 16-byte bf16 chunks
-                uint32_t cw[4];
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const uint32_t w[4] = {x[2 * g + half].x, x[2 * g + half].y, x[2 * g + half].z, x[2 * g + half].w};
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        uint16_t lo, hi;
-                        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(lo)
-                            : "f"(div_rn(bf16_hi_to_f32(w[2 * k]), dv)), "f"(div_rn(bf16_lo_to_f32(w[2 * k]), dv)));
-                        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(hi)
-                            : "f"(div_rn(bf16_hi_to_f32(w[2 * k + 1]), dv)), "f"(div_rn(bf16_lo_to_f32(w[2 * k + 1]), dv)));
-                        cw[2 * half + k] = uint32_t(lo) | (uint32_t(hi) << 16);
-                    }
-                }
-                codes[g * kTileRows] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-            }
-            reinterpret_cast<float*>(blk + size_t(kTileRows) * D)[r] = scale;
-        }
+        for (int c = 0; c < CH; ++c) dst[c * kTileRows] = x[c];
     }
 }
 
@@ -664,10 +629,10 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             mbar_arrive(bar(kBarDepth));
             }
         }
-        if (p.append_slot != nullptr && h == hk * p.G) {
+        if (!FP8 && p.append_slot != nullptr && h == hk * p.G) {
             // the write step: every read of the depth cache by this CTA is complete here, so the slot may be one that was read
             for (int t = 0; t < n_tiles; ++t)
-                append_rows_from_global<D, FP8>(p.append_slot, p.K, p.V, b, hk, Hk, p.T, nq, tile_qt(t), tid - 128);
+                append_rows_from_global<D>(p.append_slot, p.K, p.V, b, hk, Hk, p.T, nq, tile_qt(t), tid - 128);
         }
     } else {
       setmaxnreg_dec<72>();   // one instruction for the whole producer warpgroup (warps 8-11)

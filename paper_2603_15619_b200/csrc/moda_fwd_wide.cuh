@@ -549,9 +549,9 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             tc_fence_before_sync();
             mbar_arrive(bar(k2BarDepth));
         }
-        if (p.append_slot != nullptr && h == hk * p.G) {
+        if (!FP8 && p.append_slot != nullptr && h == hk * p.G) {
             // the "write" step of the depth stream (see moda_fwd_kernel): after this CTA's reads of the depth cache
-            append_rows_from_global<D, FP8>(p.append_slot, p.K, p.V, b, hk, p.H / p.G, p.T, nq, qt, tid - 256);
+            append_rows_from_global<D>(p.append_slot, p.K, p.V, b, hk, p.H / p.G, p.T, nq, qt, tid - 256);
         }
     } else {
       setmaxnreg_dec<40>();   // one instruction for the whole producer warpgroup (warps 12-15)
