@@ -3,9 +3,9 @@
 
 A "step" is one pass of the whole hot path for one attention layer over one batch of
 synthetic inputs that are already resident in HBM: the forward kernel, which also does the
-depth-cache "write" of the layer's own K, V (one slot), and the three backward launches (row-local part:
-row terms, depth gradients, depth share of dQ; sequence part: dK, dV and the dQ tiles; dQ
-finish).  `value` is forward+backward TFLOP/s with the FLOP convention of
+depth-cache "write" of the layer's own K, V (one slot), and the backward (row terms; depth part: depth
+gradients, depth share of dQ, which runs beside the sequence part: dK, dV and the dQ tiles; dQ
+finish).  The per-kernel times of the detail come from its stages launched one after the other.  `value` is forward+backward TFLOP/s with the FLOP convention of
 paper_2603_15619_b200/flops.py (causal-halved sequence part + depth part, backward =
 2.5 x forward).  Default workload: c4 (B=1, T=65536, H=16, d=128, l=24), the largest
 configured workload at d = 128 and the one the 64K ratio target is stated on.
@@ -223,8 +223,9 @@ class Layer:
         return {
             # the forward's own bytes plus the slot it writes (K and V once more, in cache layout)
             "fwd_append": {"bytes": flops.fwd_bytes(w.B, w.T, w.H, w.d, w.l) + 2.0 * 2 * E, "flops": f_fwd},
-            # reads Q O dO (bf16), LSE and the depth cache; writes the row terms, the depth gradients and the fp32 dQ accumulator
-            "bwd_rows": {"bytes": 2.0 * (3 * E + 4 * w.l * E) + 4.0 * E + 8.0 * rows, "flops": 2.0 * E + 2.5 * dep},
+            # reads O dO, then Q dO (bf16), LSE, D and the depth cache; writes the row terms, the depth gradients and the fp32 dQ
+            # accumulator (cleared; the depth share is added)
+            "bwd_rows": {"bytes": 2.0 * (4 * E + 4 * w.l * E) + 8.0 * E + 12.0 * rows, "flops": 2.0 * E + 2.5 * dep},
             # reads Q K V dO + LSE, D; writes dK dV; reads and writes the fp32 dQ accumulator; the five sequence contractions
             "bwd_seq": {"bytes": 2.0 * 6 * E + 2 * 4.0 * E + 8.0 * rows, "flops": 2.5 * seq},
             "bwd_finish": {"bytes": 4.0 * E + 2.0 * E, "flops": 0.0},
@@ -329,7 +330,7 @@ def run_moda(args, rank, world, device):
                    "l2_policy": "inputs larger than L2 (depth cache %.2f GiB + 4 x %.0f MiB activations per step)"
                                 % (flops.depth_bytes_fwd(w.B, w.T, w.H, w.d, w.l) / 2 ** 30, w.B * w.T * w.H * w.d * 2 / 2 ** 20),
                    "parallelism": f"independent batch shards x{world}, no collective"},
-        "roofline": roof, "clocks": clocks, "gpu_launches": 4 * K, "detail": detail,
+        "roofline": roof, "clocks": clocks, "gpu_launches": ((5 if w.l else 4) + (1 if layer.e4m3 else 0)) * K, "detail": detail,
     }
 
     headline = {"fwd_ms": per_kernel["fwd_append"], "bwd_ms": bwd_ms}

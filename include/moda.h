@@ -188,11 +188,12 @@ int moda_attn_bwd(const void* Q, const void* K, const void* V, const void* depth
                   void* workspace, size_t workspace_bytes, void* stream);
 
 /*
- * moda_attn_bwd is three launches; this entry point runs a subset of them so that each can
- * be timed or profiled on its own.  `stages` is a bit mask of the launches in the order above:
- *     MODA_BWD_STAGE_ROWS      (1) row terms, depth gradients, start of the dQ accumulator
+ * moda_attn_bwd has three stages; this entry point runs a subset of them so that each can
+ * be timed or profiled on its own.  `stages` is a bit mask in the order above:
+ *     MODA_BWD_STAGE_ROWS      (1) row terms, cleared dQ accumulator; depth gradients, depth part of dQ
  *     MODA_BWD_STAGE_SEQ       (2) dK, dV and the dQ tiles (reads D_t, adds to the accumulator)
  *     MODA_BWD_STAGE_FINISH    (3) dQ from the accumulator
+ * With (1) and (2) in one call the depth part runs beside the sequence part on a share of the SMs.
  * moda_attn_bwd(...) is moda_attn_bwd_stages(..., MODA_BWD_ALL_STAGES, stream).
  * MODA_BWD_DETERMINISTIC selects the split form of the backward instead: no floating-point
  * atomics, every output bit-reproducible, at the price of seven contractions for five and two
