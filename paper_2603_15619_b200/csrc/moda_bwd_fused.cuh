@@ -517,12 +517,17 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     constexpr uint32_t kColX = 0, kColY = 128 * XB, kColdK = kColY + 128, kColdV = kColdK + D;
     static_assert(kColdV + D <= kTmemCols, "tensor-memory plan too large");
 
-    if (g_moda_status != 0) return;
+    const bool last_cta = p.beside_rows && blockIdx.x == gridDim.x - 1;   // ends the grid after the rows kernel, on every path
+    if (g_moda_status != 0) {
+        if (last_cta) grid_dependency_wait();
+        return;
+    }
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = aligned_dynamic_smem(smem_raw, L::kTotal);
     if (smem == nullptr) {
         if (threadIdx.x == 0) atomicCAS(&g_moda_status, 0, kStatusSmemLayout);
+        if (last_cta) grid_dependency_wait();
         return;
     }
     const uint32_t sbase = smem_u32(smem);
@@ -918,7 +923,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     __syncthreads();
     if (warp == W_S) tmem_dealloc(tmem, kTmemCols);
     // what follows on the stream reads the accumulator and the depth gradients: this grid ends after the rows kernel has
-    if (p.beside_rows && blockIdx.x == gridDim.x - 1) grid_dependency_wait();
+    if (last_cta) grid_dependency_wait();
 }
 
 }  // namespace moda
