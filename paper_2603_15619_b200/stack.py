@@ -3,10 +3,8 @@
 In a MoDA model (paper Sec. 2.2, the "write" step) every attention layer appends its own K, V to
 the depth stream after attending, and layer l attends to the l slots written before it.  So K_i, V_i
 of layer i receive gradient from layer i's own sequence attention and, as depth slot i, from every
-later layer.  ``DepthStream`` owns the depth cache and one gradient cache of the same layout and
-wires those contributions together around the C-ABI calls (the first layer of a backward pass writes its
-depth gradients into the shared gradient cache, the backward call's accumulate flag adds those of the
-others); it is plumbing: no arithmetic of the operator happens here.
+later layer.  ``DepthStream`` owns the depth cache and wires those contributions together around the
+C-ABI calls; it is plumbing: no arithmetic of the operator happens here.
 
     stream = DepthStream(B, T, H_kv, d, n_layers)
     for layer in layers:
@@ -14,10 +12,12 @@ others); it is plumbing: no arithmetic of the operator happens here.
         o = stream.attend(q, k, v)               # attends to the slots so far, then appends k, v
         x = layer.rest(x, o)
 
-Backward runs the layers in reverse (a token tensor chains the calls so that autograd keeps that
-order even if the layers' inputs are unrelated): layer l adds its depth gradients into slots < l of
-the gradient cache, and the gradient of its own K, V is its sequence-attention gradient plus slot l
-of that cache, which by then holds the contributions of all later layers.
+A token tensor chains the calls: the token behind slot l stands for the first l + 1 slots of the depth
+cache, and its gradient is a gradient cache of that many slots.  Backward runs the layers in reverse.
+The first layer of a pass writes its depth gradients into a new buffer, every layer below adds its own to
+slots < l of that buffer in place (the backward call's accumulate flag) and takes slot l, which by then
+holds the contributions of all later layers, as part of the gradient of its own K, V.  Because the buffer
+travels as a gradient, passes over one stream do not see each other, also when one failed half way.
 """
 from __future__ import annotations
 
@@ -28,28 +28,28 @@ from . import binding
 
 class _Attend(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, Q, K, V, token, stream, l, scale):
+    def forward(ctx, Q, K, V, token, slots, l, scale):
         Q, K, V = Q.contiguous(), K.contiguous(), V.contiguous()
         # attention and the "write" step (slot l = this layer's K, V) in one launch
-        O, LSE = binding.moda_attn_fwd_append(Q, K, V, stream.cache if l > 0 else None, l, scale, stream.cache, l)
+        O, LSE = binding.moda_attn_fwd_append(Q, K, V, slots.cache if l > 0 else None, l, scale, slots.cache, l)
         ctx.save_for_backward(Q, K, V, O, LSE)
-        ctx.stream, ctx.l, ctx.scale = stream, l, scale
-        return O, torch.empty_like(token)
+        ctx.slots, ctx.l, ctx.scale = slots, l, scale
+        ctx.set_materialize_grads(False)                       # a token without a gradient is the start of a pass
+        return O, slots.token(l + 1)
 
     @staticmethod
     def backward(ctx, dO, dtoken):
         Q, K, V, O, LSE = ctx.saved_tensors
-        stream, l = ctx.stream, ctx.l
-        B, T, H, d = Q.shape
-        Hk = K.shape[2]
+        slots, l = ctx.slots, ctx.l
+        dO = torch.zeros_like(O) if dO is None else dO.contiguous()
         # slots < l of the gradient cache receive this layer's share
+        grads, filled = slots.open(dtoken, l)
         dQ, dK, dV, _ = binding.moda_attn_bwd_gqa(
-            Q, K, V, stream.cache if l > 0 else None, O, dO.contiguous(), LSE, l, ctx.scale,
-            d_depth_kv=stream.grads if l > 0 else None,
-            stages=binding.MODA_BWD_ALL_STAGES | (binding.MODA_BWD_ACCUMULATE_DEPTH if stream.add_to_slots(l) else 0))
-        if stream.slot_has_grad(l):                                     # later layers attended to slot l
-            binding.moda_depth_cache_unpack_add(stream.grads, l, dK, dV)
-        return dQ, dK, dV, dtoken, None, None, None
+            Q, K, V, slots.cache if l > 0 else None, O, dO, LSE, l, ctx.scale, d_depth_kv=grads if l > 0 else None,
+            stages=binding.MODA_BWD_ALL_STAGES | (binding.MODA_BWD_ACCUMULATE_DEPTH if filled else 0))
+        if filled:                                             # later layers attended to slot l
+            binding.moda_depth_cache_unpack_add(grads, l, dK, dV)
+        return dQ, dK, dV, slots.close(grads, filled, l), None, None, None
 
 
 class _Write(torch.autograd.Function):
@@ -57,20 +57,23 @@ class _Write(torch.autograd.Function):
     slot of the gradient cache that the later layers filled."""
 
     @staticmethod
-    def forward(ctx, K, V, token, stream, slot):
+    def forward(ctx, K, V, token, slots, slot):
         K, V = K.contiguous(), V.contiguous()
-        binding.moda_depth_cache_append(stream.cache, slot, K, V)
-        ctx.stream, ctx.slot = stream, slot
+        binding.moda_depth_cache_append(slots.cache, slot, K, V)
+        ctx.slots, ctx.slot = slots, slot
         ctx.save_for_backward(K, V)
-        return torch.empty_like(token)
+        ctx.set_materialize_grads(False)
+        return slots.token(slot + 1)
 
     @staticmethod
     def backward(ctx, dtoken):
         K, V = ctx.saved_tensors
+        slots, slot = ctx.slots, ctx.slot
         dK, dV = torch.zeros_like(K), torch.zeros_like(V)
-        if ctx.stream.slot_has_grad(ctx.slot):
-            binding.moda_depth_cache_unpack(ctx.stream.grads, ctx.slot, dK, dV)
-        return dK, dV, dtoken, None, None
+        grads, filled = slots.open(dtoken, slot)
+        if filled:
+            binding.moda_depth_cache_unpack(grads, slot, dK, dV)
+        return dK, dV, slots.close(grads, filled, slot) if filled else None, None, None
 
 
 class _ProjectWrite(torch.autograd.Function):
@@ -79,59 +82,68 @@ class _ProjectWrite(torch.autograd.Function):
     the slot of the gradient cache is dK, dV; dX = dK Wk + dV Wv and dW = dK^T X are plain library GEMMs."""
 
     @staticmethod
-    def forward(ctx, X, Wk, Wv, token, stream, slot):
+    def forward(ctx, X, Wk, Wv, token, slots, slot):
         X, Wk, Wv = X.contiguous(), Wk.contiguous(), Wv.contiguous()
-        binding.moda_kv_project_append(X, Wk, Wv, stream.shape[2], cache=stream.cache, slot=slot, store_kv=False)
-        ctx.stream, ctx.slot = stream, slot
+        binding.moda_kv_project_append(X, Wk, Wv, slots.shape[2], cache=slots.cache, slot=slot, store_kv=False)
+        ctx.slots, ctx.slot = slots, slot
         ctx.save_for_backward(X, Wk, Wv)
-        return torch.empty_like(token)
+        ctx.set_materialize_grads(False)
+        return slots.token(slot + 1)
 
     @staticmethod
     def backward(ctx, dtoken):
         X, Wk, Wv = ctx.saved_tensors
-        B, T, Hk, d = ctx.stream.shape
-        if not ctx.stream.slot_has_grad(ctx.slot):
-            return torch.zeros_like(X), torch.zeros_like(Wk), torch.zeros_like(Wv), dtoken, None, None
+        slots, slot = ctx.slots, ctx.slot
+        B, T, Hk, d = slots.shape
+        grads, filled = slots.open(dtoken, slot)
+        if not filled:
+            return torch.zeros_like(X), torch.zeros_like(Wk), torch.zeros_like(Wv), None, None, None
         dK = torch.empty((B, T, Hk, d), dtype=X.dtype, device=X.device)
         dV = torch.empty_like(dK)
-        binding.moda_depth_cache_unpack(ctx.stream.grads, ctx.slot, dK, dV)
+        binding.moda_depth_cache_unpack(grads, slot, dK, dV)
         dK2, dV2, X2 = dK.view(B * T, Hk * d), dV.view(B * T, Hk * d), X.view(B * T, -1)
         dX = (dK2 @ Wk).addmm_(dV2, Wv).view_as(X)
-        return dX, dK2.t() @ X2, dV2.t() @ X2, dtoken, None, None
+        return dX, dK2.t() @ X2, dV2.t() @ X2, slots.close(grads, filled, slot), None, None
 
 
 class _Slots:
-    """What a stream's autograd nodes share: the two caches and how far the gradient cache is filled.  Kept apart from the
+    """What a stream's autograd nodes share: the depth cache, and the gradient cache of the latest pass.  Kept apart from the
     DepthStream, whose token leads back to the nodes: a node that held the stream itself would close a reference cycle,
     and the caches would then live until the garbage collector happens to run."""
 
     def __init__(self, B, T, H_kv, d, n_layers, device):
         self.shape = (B, T, H_kv, d)
         self.n_layers = n_layers
+        self.slot_elems = binding.moda_depth_cache_bytes(B, T, H_kv, d, 1) // 2
         self.cache = binding.alloc_depth_cache(B, T, H_kv, d, n_layers, device)
-        self.grads = torch.empty_like(self.cache)              # slots < grad_slots hold gradients, the others nothing yet
-        self.grad_slots = 0
+        self.grads = None                                      # gradient cache of the latest pass
+        self.grad_slots = 0                                    # slots of it that hold something
 
-    def zero_slots(self, first, end):
-        binding.depth_cache_window(self.grads, *self.shape, first, end - first).zero_()
+    def token(self, n):
+        """A tensor of the first n slots' shape without their memory."""
+        return torch.empty_strided((n * self.slot_elems,), (0,), dtype=self.cache.dtype, device=self.cache.device)
 
-    def add_to_slots(self, l):
-        """Whether a layer that attended to slots < l adds its depth gradients to what the gradient cache holds, or is the
-        first of a backward pass and writes them."""
-        if self.grad_slots == 0:
-            self.grad_slots = l
-            return False
-        if l > self.grad_slots:                                # an earlier pass began at a lower layer
-            self.zero_slots(self.grad_slots, l)
-            self.grad_slots = l
-        return True
+    def open(self, dtoken, slot):
+        """(buffer, filled) for the node of slot ``slot``: a gradient cache that it may write in place, and whether slots
+        0 .. ``slot`` of it hold gradients.  ``dtoken`` is what the nodes above passed down, None at the start of a pass."""
+        if dtoken is None:
+            self.grads, self.grad_slots = None, 0              # the previous pass's: its memory may serve this one
+            return torch.empty_like(self.cache) if slot > 0 else None, False
+        if self.grads is not None and dtoken.data_ptr() == self.grads.data_ptr():
+            return self.grads, True
+        grads = torch.empty_like(self.cache)                   # a gradient from elsewhere: not ours to write to
+        grads[:dtoken.numel()].copy_(dtoken)
+        return grads, True
 
-    def slot_has_grad(self, l):
-        return l < self.grad_slots
+    def close(self, grads, filled, slot):
+        """The gradient of the token below slot ``slot``, once the node's own share is in ``grads``."""
+        if grads is not self.grads:
+            self.grads, self.grad_slots = grads, slot + 1 if filled else slot
+        return grads[:slot * self.slot_elems] if slot > 0 else None
 
 
 class DepthStream:
-    """Depth cache of one forward pass through a stack (and its gradient cache)."""
+    """Depth cache of one forward pass through a stack, and the gradient of its slots."""
 
     def __init__(self, B, T, H_kv, d, n_layers, device="cuda"):
         self.shape = (B, T, H_kv, d)
@@ -139,17 +151,21 @@ class DepthStream:
         self._slots = _Slots(B, T, H_kv, d, self.n_layers, device)
         self.cache = self._slots.cache
         self.n_written = 0
-        self.token = torch.zeros((), device=device, requires_grad=True)
+        self.token = self._slots.token(0).requires_grad_()
 
     @property
     def grad_cache(self):
-        """Gradient cache; zero in the slots that no backward pass has reached."""
-        if self._slots.grad_slots < self.n_layers:
-            self._slots.zero_slots(self._slots.grad_slots, self.n_layers)
-        return self._slots.grads
+        """Gradient cache of the latest backward pass, zero in the slots that it did not reach."""
+        s = self._slots
+        if s.grads is None:
+            s.grads = torch.zeros_like(s.cache)
+        elif s.grad_slots < self.n_layers:
+            s.grads[s.grad_slots * s.slot_elems:].zero_()
+            s.grad_slots = self.n_layers
+        return s.grads
 
     def slot_has_grad(self, l):
-        return self._slots.slot_has_grad(l)
+        return l < self.n_written - 1
 
     def attend(self, Q, K, V, scale=None):
         """MoDA attention of the next layer: attends to the slots written so far, then appends K, V."""
