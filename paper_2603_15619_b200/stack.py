@@ -118,6 +118,7 @@ class _Slots:
         self.cache = binding.alloc_depth_cache(B, T, H_kv, d, n_layers, device)
         self.grads = None                                      # gradient cache of the latest pass
         self.grad_slots = 0                                    # slots of it that hold something
+        self.seeded = False                                    # it is the caller's: the next pass adds to it
 
     def token(self, n):
         """A tensor of the first n slots' shape without their memory."""
@@ -127,6 +128,8 @@ class _Slots:
         """(buffer, filled) for the node of slot ``slot``: a gradient cache that it may write in place, and whether slots
         0 .. ``slot`` of it hold gradients.  ``dtoken`` is what the nodes above passed down, None at the start of a pass."""
         if dtoken is None:
+            if self.seeded:
+                return self.grads, True
             self.grads, self.grad_slots = None, 0              # the previous pass's: its memory may serve this one
             return torch.empty_like(self.cache) if slot > 0 else None, False
         if self.grads is not None and dtoken.data_ptr() == self.grads.data_ptr():
@@ -139,30 +142,47 @@ class _Slots:
         """The gradient of the token below slot ``slot``, once the node's own share is in ``grads``."""
         if grads is not self.grads:
             self.grads, self.grad_slots = grads, slot + 1 if filled else slot
+        self.seeded = False
         return grads[:slot * self.slot_elems] if slot > 0 else None
 
 
 class DepthStream:
-    """Depth cache of one forward pass through a stack, and the gradient of its slots."""
+    """Depth cache of one forward pass through a stack, and the gradient of its slots.
+
+    ``cache`` may be replaced by another depth cache of the same size.  ``grad_cache`` is the gradient cache of the latest
+    backward pass; before the first one it is zero, and what the caller adds to it then, or a gradient cache that the caller
+    assigns, is where the next pass starts from."""
 
     def __init__(self, B, T, H_kv, d, n_layers, device="cuda"):
         self.shape = (B, T, H_kv, d)
         self.n_layers = int(n_layers)
         self._slots = _Slots(B, T, H_kv, d, self.n_layers, device)
-        self.cache = self._slots.cache
         self.n_written = 0
         self.token = self._slots.token(0).requires_grad_()
+
+    @property
+    def cache(self):
+        return self._slots.cache
+
+    @cache.setter
+    def cache(self, cache):
+        self._slots.cache = cache
 
     @property
     def grad_cache(self):
         """Gradient cache of the latest backward pass, zero in the slots that it did not reach."""
         s = self._slots
         if s.grads is None:
-            s.grads = torch.zeros_like(s.cache)
+            self.grad_cache = torch.zeros_like(s.cache)
         elif s.grad_slots < self.n_layers:
             s.grads[s.grad_slots * s.slot_elems:].zero_()
             s.grad_slots = self.n_layers
         return s.grads
+
+    @grad_cache.setter
+    def grad_cache(self, grads):
+        s = self._slots
+        s.grads, s.grad_slots, s.seeded = grads, self.n_layers, True
 
     def slot_has_grad(self, l):
         return l < self.n_written - 1

@@ -169,6 +169,34 @@ def test_a_pass_inside_another(op):
     check([torch.zeros(x.shape) if g is None else g for x, g in zip(stack.leaves, inner)], want)
 
 
+def test_caches_that_the_caller_reads_replaces_or_fills(op):
+    stack = Stack()
+    stream, outs = stack.run()
+    n = len(KINDS)
+    mine = stream.cache.clone()
+    stream.cache = mine                                    # the nodes use it from now on
+    assert stream._slots.cache is mine and stream.cache is mine
+    assert torch.equal(stream.grad_cache, torch.zeros(n * SLOT))
+    slots_of(stream.grad_cache)[1].fill_(3.0)              # a gradient from elsewhere for the slot of the first write
+    got = run_pass(stack, outs, (0, 1, 2), retain_graph=True)
+    want = [w.clone() for w in stack.grads((0, 1, 2))]
+    for i in (3, 4):
+        want[i] += 3.0
+    check(got, want)
+    check(run_pass(stack, outs, (0, 1, 2), retain_graph=True), stack.grads((0, 1, 2)))
+    full = slots_of(stream.grad_cache)
+    assert bool((full[4:] == 0).all()) and torch.equal(full[3, 0].float(), coef(4, 3) * stack.dO[2].float())
+    assert stream.slot_has_grad(n - 2) and not stream.slot_has_grad(n - 1)
+    seed = torch.zeros(n * SLOT, dtype=torch.bfloat16)
+    slots_of(seed)[1].fill_(-2.0)
+    stream.grad_cache = seed
+    want = [w.clone() for w in stack.grads((0, 1, 2))]
+    for i in (3, 4):
+        want[i] -= 2.0
+    check(run_pass(stack, outs, (0, 1, 2)), want)
+    assert stream.grad_cache is seed
+
+
 def test_one_layer_alone(op):
     stream = moda.DepthStream(B, T, H, D, 1, device="cpu")
     x = [torch.ones(B, T, H, D, dtype=torch.bfloat16, requires_grad=True) for _ in range(3)]
