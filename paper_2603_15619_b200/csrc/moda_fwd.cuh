@@ -437,7 +437,8 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             float m_d = -INFINITY, l_d = 0.f;
             if constexpr (FP8) {
                 // e4m3 cache: a unit holds all D features of one slot's keys (values) for the tile's rows, its row
-                // scales sit beside it; codes are widened to fp32 in registers, everything else as below.
+                // scales sit beside it; codes are widened to fp32 in registers, everything else as below.  Packed fp32 FMAs
+                // (T = 8192, B = 2, 16 heads, us: l = 8 694 -> 670, l = 16 793 -> 732, l = 32 972 -> 859).
                 constexpr int C8 = D / 16;                    // 16-byte chunks (16 codes) of a row
                 const float* sScale = reinterpret_cast<const float*>(smem + L::kScale);
                 auto take_unit8 = [&](uint4 (&dst)[C8], float& sc) {
@@ -477,10 +478,8 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                                 for (int k = 0; k < 4; ++k) {
                                     float f0, f1, f2, f3;
                                     e4m3x4_to_f32(w[k], f0, f1, f2, f3);
-                                    a0 = fmaf(q[16 * c + 4 * k + 0], f0, a0);
-                                    a1 = fmaf(q[16 * c + 4 * k + 1], f1, a1);
-                                    a2 = fmaf(q[16 * c + 4 * k + 2], f2, a2);
-                                    a3 = fmaf(q[16 * c + 4 * k + 3], f3, a3);
+                                    fma2_f32(q[16 * c + 4 * k + 0], q[16 * c + 4 * k + 1], f0, f1, a0, a1);
+                                    fma2_f32(q[16 * c + 4 * k + 2], q[16 * c + 4 * k + 3], f2, f3, a2, a3);
                                 }
                             }
                             sU[i * kTileRows + r] = ((a0 + a1) + (a2 + a3)) * sc;
@@ -524,10 +523,8 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                                 for (int k = 0; k < 4; ++k) {
                                     float f0, f1, f2, f3;
                                     e4m3x4_to_f32(ww[k], f0, f1, f2, f3);
-                                    acc[16 * c + 4 * k + 0] = fmaf(w, f0, acc[16 * c + 4 * k + 0]);
-                                    acc[16 * c + 4 * k + 1] = fmaf(w, f1, acc[16 * c + 4 * k + 1]);
-                                    acc[16 * c + 4 * k + 2] = fmaf(w, f2, acc[16 * c + 4 * k + 2]);
-                                    acc[16 * c + 4 * k + 3] = fmaf(w, f3, acc[16 * c + 4 * k + 3]);
+                                    fma2_f32(w, w, f0, f1, acc[16 * c + 4 * k + 0], acc[16 * c + 4 * k + 1]);
+                                    fma2_f32(w, w, f2, f3, acc[16 * c + 4 * k + 2], acc[16 * c + 4 * k + 3]);
                                 }
                             }
                         }

@@ -82,7 +82,7 @@ enum Fwd2Bar : int {
     k2BarDrain = 27,
     k2BarRef = 28,     // +(j & 1): the reference maximum for tile j has been published
     k2BarDFull = 30,   // +ring stage (<= 6): depth unit landed
-    k2BarDEmpty = 36,  // +ring stage (<= 6): all 128 depth threads have read the unit
+    k2BarDEmpty = 36,  // +ring stage (<= 6): the 128 depth threads (e4m3: their 4 warps) have read the unit
 };
 
 
@@ -145,7 +145,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         mbar_init(bar(k2BarDrain), 1);
         for (int s = 0; s < L::kRingStages; ++s) {
             mbar_init(bar(k2BarDFull + s), 1);
-            mbar_init(bar(k2BarDEmpty + s), 128);
+            mbar_init(bar(k2BarDEmpty + s), FP8 ? 4 : 128);
         }
         fence_mbar_init();
     }
@@ -360,7 +360,11 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             // group raises the maximum.  Up to 32 slots are one group.
             float m_d = -INFINITY, l_d = 0.f;
             if constexpr (FP8) {
-                // e4m3 cache (see moda_fwd_kernel): a unit = all D features of one slot for the tile's rows + row scales
+                // e4m3 cache (see moda_fwd_kernel): a unit = all D features of one slot for the tile's rows + row scales.
+                // Widening the codes makes these loops twice as long as the bf16 ones, and they share the issue slots with
+                // the softmax warps: packed fp32 FMAs, the running maximum inside the score loop, a stage handed back by
+                // warps.  32 heads, us, scalar FMAs and 128 arrivals -> this: T = 8192, l = 8 994 -> 916, l = 32 1275 -> 1221;
+                // T = 32768, l = 8 6111 -> 6047, l = 32 6820 -> 6517.  Arrivals by warps cost the bf16 loop below 1 to 2 %.
                 constexpr int C8 = D / 16;
                 const float* sScale = reinterpret_cast<const float*>(smem + L::kScale);
                 auto take_unit8 = [&](uint4 (&dst)[C8], float& sc) {
@@ -371,12 +375,14 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                     for (int c = 0; c < C8; ++c) dst[c] = *reinterpret_cast<const uint4*>(src + c * (kTileRows * 16));
                     sc = sScale[st * kTileRows + r];
                     fence_proxy_async_smem();
-                    mbar_arrive(bar(k2BarDEmpty + st));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(k2BarDEmpty + st));
                     ++unit;
                 };
 #pragma unroll 1
                 for (int g0 = 0; g0 < p.l; g0 += kFwdDepthGroup) {
                     const int gl = min(kFwdDepthGroup, p.l - g0);
+                    float m_new = m_d;
                     {
                         float q[D];
 #pragma unroll
@@ -400,17 +406,15 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                                 for (int k = 0; k < 4; ++k) {
                                     float f0, f1, f2, f3;
                                     e4m3x4_to_f32(w[k], f0, f1, f2, f3);
-                                    a0 = fmaf(q[16 * c + 4 * k + 0], f0, a0);
-                                    a1 = fmaf(q[16 * c + 4 * k + 1], f1, a1);
-                                    a2 = fmaf(q[16 * c + 4 * k + 2], f2, a2);
-                                    a3 = fmaf(q[16 * c + 4 * k + 3], f3, a3);
+                                    fma2_f32(q[16 * c + 4 * k + 0], q[16 * c + 4 * k + 1], f0, f1, a0, a1);
+                                    fma2_f32(q[16 * c + 4 * k + 2], q[16 * c + 4 * k + 3], f2, f3, a2, a3);
                                 }
                             }
-                            sU[i * kTileRows + r] = ((a0 + a1) + (a2 + a3)) * sc;
+                            const float u = ((a0 + a1) + (a2 + a3)) * sc;
+                            sU[i * kTileRows + r] = u;
+                            m_new = fmaxf(m_new, u * p.scale_log2);
                         }
                     }
-                    float m_new = m_d;
-                    for (int i = 0; i < gl; ++i) m_new = fmaxf(m_new, sU[i * kTileRows + r] * p.scale_log2);
                     const float f = fast_exp2(m_d - m_new);
                     l_d *= f;
                     for (int i = 0; i < gl; ++i) {
@@ -447,10 +451,8 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                                 for (int k = 0; k < 4; ++k) {
                                     float f0, f1, f2, f3;
                                     e4m3x4_to_f32(ww[k], f0, f1, f2, f3);
-                                    acc[16 * c + 4 * k + 0] = fmaf(w, f0, acc[16 * c + 4 * k + 0]);
-                                    acc[16 * c + 4 * k + 1] = fmaf(w, f1, acc[16 * c + 4 * k + 1]);
-                                    acc[16 * c + 4 * k + 2] = fmaf(w, f2, acc[16 * c + 4 * k + 2]);
-                                    acc[16 * c + 4 * k + 3] = fmaf(w, f3, acc[16 * c + 4 * k + 3]);
+                                    fma2_f32(w, w, f0, f1, acc[16 * c + 4 * k + 0], acc[16 * c + 4 * k + 1]);
+                                    fma2_f32(w, w, f2, f3, acc[16 * c + 4 * k + 2], acc[16 * c + 4 * k + 3]);
                                 }
                             }
                         }

@@ -509,6 +509,17 @@ __device__ __forceinline__ void axpy_bf16x2(float a, uint32_t x, float& y0, floa
         "mov.b64 {%0, %1}, yy;\n"
         "}\n" : "+f"(y0), "+f"(y1) : "f"(a), "r"(lo), "r"(hi));
 }
+// (y0, y1) += (a0, a1) * (b0, b1): one packed fp32 FMA, each half rounded like fmaf.
+__device__ __forceinline__ void fma2_f32(float a0, float a1, float b0, float b1, float& y0, float& y1) {
+    asm("{\n"
+        ".reg .b64 aa, bb, yy;\n"
+        "mov.b64 aa, {%2, %3};\n"
+        "mov.b64 bb, {%4, %5};\n"
+        "mov.b64 yy, {%0, %1};\n"
+        "fma.rn.f32x2 yy, aa, bb, yy;\n"
+        "mov.b64 {%0, %1}, yy;\n"
+        "}\n" : "+f"(y0), "+f"(y1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
 // Four e4m3 bytes (lowest byte first) -> four floats.  Two hardware conversions to f16 pairs (exact: every e4m3 value is
 // an f16 value), then to f32.
 __device__ __forceinline__ void e4m3x4_to_f32(uint32_t w, float& f0, float& f1, float& f2, float& f3) {
