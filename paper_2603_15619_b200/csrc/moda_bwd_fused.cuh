@@ -121,8 +121,9 @@ bwd_dq_finish_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict
 // the stream, the sequence part, start at once: this part moves every byte of the depth cache and of its gradient cache
 // once and is bound by HBM, the sequence part by the tensor cores and L2, so one after the other leaves each resource idle
 // in turn.  Both only add to the dQ accumulator; the sequence grid ends after this one has.
-// Backward, ms, one after the other -> side by side: T = 4096, l = 23, d = 128, B = 4: 1.96 -> 1.64; T = 8192, l = 16,
-// B = 2: 2.27 -> 2.04; T = 5000, l = 23, e4m3: 1.24 -> 1.02; T = 32768, l = 32, d = 64, H = 32: 16.9 -> 16.3.
+// Whole backward, ms, short runs, one after the other -> side by side: T = 4096, l = 23, d = 128, B = 4: 2.11 -> 1.66; T = 8192,
+// l = 16, B = 2: 2.53 -> 2.15, e4m3 2.39 -> 2.01; T = 5000, l = 23, e4m3: 1.42 -> 1.11; T = 32768, l = 32, d = 64, 32 heads:
+// 17.8 -> 16.6, e4m3 17.0 -> 15.9.
 //
 // A CTA walks units of 128 rows (d = 128; two tiles of 128 rows at d = 64, whose blocks are neighbours in the cache).
 // Per unit the ring brings the Q and dO rows (TMA, 64 KiB) and then, slot by slot, the unit's K and V blocks (one
@@ -131,7 +132,9 @@ bwd_dq_finish_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict
 // lanes of a quarter warp own consecutive rows of one feature part: 128 contiguous bytes per access in the stage and
 // in the gradient cache.  The two dot products of a slot are finished with shuffles; their terms are mixed-precision FMAs
 // (unpacking the bf16 factors first made the arithmetic the bound: 2.7 us per 64 KiB in, 64 KiB out and SM against 1.55;
-// 1.05 without the stores, which are the bound now).
+// 1.05 without the stores, which are the bound now).  With e4m3 codes they are packed fp32 FMAs, values before keys so that
+// only the widened keys stay in registers: an entry takes 1.75 to 2.0 us as in bf16, against 2.2 (d = 128) and 2.7 (d = 64) with a
+// scalar FMA per element.
 struct RowsParams {
     const void* depth_kv;   // bf16 cache, or e4m3 codes + row scales (FP8 instantiation); gradients are bf16 either way
     __nv_bfloat16* d_depth_kv;
@@ -288,27 +291,27 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(empty);
+                    // features 16 j + 4 k .. + 3 of this thread = halves of the packed q / dO words 2 (4 j + k), 2 (4 j + k) + 1; values
+                    // first, so that only the widened keys (needed again for dQ) stay in registers
+                    const uint32_t* qw = reinterpret_cast<const uint32_t*>(q4);
+                    const uint32_t* gw = reinterpret_cast<const uint32_t*>(g4);
+                    float u1 = 0.f, dr1 = 0.f;
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const uint32_t kw[4] = {k8[j].x, k8[j].y, k8[j].z, k8[j].w}, vw[4] = {v8[j].x, v8[j].y, v8[j].z, v8[j].w};
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            float v0, v1, v2, v3;
-                            e4m3x4_to_f32(kw[k], kf[16 * j + 4 * k], kf[16 * j + 4 * k + 1], kf[16 * j + 4 * k + 2], kf[16 * j + 4 * k + 3]);
-                            e4m3x4_to_f32(vw[k], v0, v1, v2, v3);
-                            // features 16 j + 4 k .. + 3 of this thread = halves of the packed q / dO words 2 (4 j + k), 2 (4 j + k) + 1
-                            const uint32_t* qw = reinterpret_cast<const uint32_t*>(q4) + 2 * (4 * j + k);
-                            const uint32_t* gw = reinterpret_cast<const uint32_t*>(g4) + 2 * (4 * j + k);
-                            u_s = fmaf(bf16_lo_to_f32(qw[0]), kf[16 * j + 4 * k], u_s);
-                            u_s = fmaf(bf16_hi_to_f32(qw[0]), kf[16 * j + 4 * k + 1], u_s);
-                            u_s = fmaf(bf16_lo_to_f32(qw[1]), kf[16 * j + 4 * k + 2], u_s);
-                            u_s = fmaf(bf16_hi_to_f32(qw[1]), kf[16 * j + 4 * k + 3], u_s);
-                            dr = fmaf(bf16_lo_to_f32(gw[0]), v0, dr);
-                            dr = fmaf(bf16_hi_to_f32(gw[0]), v1, dr);
-                            dr = fmaf(bf16_lo_to_f32(gw[1]), v2, dr);
-                            dr = fmaf(bf16_hi_to_f32(gw[1]), v3, dr);
-                        }
+                    for (int m = 0; m < 8; ++m) {
+                        float f0, f1, f2, f3;
+                        e4m3x4_to_f32(reinterpret_cast<const uint32_t*>(v8)[m], f0, f1, f2, f3);
+                        fma2_f32(bf16_lo_to_f32(gw[2 * m]), bf16_hi_to_f32(gw[2 * m]), f0, f1, dr, dr1);
+                        fma2_f32(bf16_lo_to_f32(gw[2 * m + 1]), bf16_hi_to_f32(gw[2 * m + 1]), f2, f3, dr, dr1);
                     }
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) {
+                        float* f = kf + 4 * m;
+                        e4m3x4_to_f32(reinterpret_cast<const uint32_t*>(k8)[m], f[0], f[1], f[2], f[3]);
+                        fma2_f32(bf16_lo_to_f32(qw[2 * m]), bf16_hi_to_f32(qw[2 * m]), f[0], f[1], u_s, u1);
+                        fma2_f32(bf16_lo_to_f32(qw[2 * m + 1]), bf16_hi_to_f32(qw[2 * m + 1]), f[2], f[3], u_s, u1);
+                    }
+                    u_s += u1;
+                    dr += dr1;
 #pragma unroll
                     for (int off = RW; off < 32; off <<= 1) {
                         u_s += __shfl_xor_sync(0xffffffffu, u_s, off);
@@ -363,7 +366,7 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                     }
                     if constexpr (FP8) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) acc[8 * j + e] = fmaf(duk, kf[8 * j + e], acc[8 * j + e]);
+                        for (int e = 0; e < 8; e += 2) fma2_f32(duk, duk, kf[8 * j + e], kf[8 * j + e + 1], acc[8 * j + e], acc[8 * j + e + 1]);
                     } else {
                         axpy_bf16x2(duk, kc[j].x, acc[8 * j + 0], acc[8 * j + 1]);
                         axpy_bf16x2(duk, kc[j].y, acc[8 * j + 2], acc[8 * j + 3]);
