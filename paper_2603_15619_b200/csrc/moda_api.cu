@@ -158,6 +158,19 @@ int check_device(bool may_allocate = true) {
     return MODA_OK;
 }
 
+int device_sm_count(int* out) {
+    static thread_local int cached_dev = -1, cached_sms = 0;
+    int dev = 0;
+    if (!cuda_ok(cudaGetDevice(&dev))) return MODA_ERR_CUDA;
+    if (dev != cached_dev) {
+        int sms = 0;
+        if (!cuda_ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return MODA_ERR_CUDA;
+        cached_dev = dev; cached_sms = sms;
+    }
+    *out = cached_sms;
+    return MODA_OK;
+}
+
 template <typename Kernel>
 bool set_smem_limit(Kernel k, int bytes) {
     return cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -371,17 +384,21 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
 }
 
 // How many SMs the depth part of a fused backward gets beside the sequence part.  Measured SM time: an entry of the row
-// ring 1.7 us (2.2 us for e4m3 codes at d = 64); an iteration of the sequence part 2.9 us (d = 64: 1.9 us) and 5 us (7 us)
-// per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both parts end together; a few SMs
-// more than that cost less than a few too few, because SMs that the depth part leaves go on with the sequence part
-// (T = 8192, l = 16, d = 128, whole backward: 24 SMs 2.53 ms, 32 2.09, 36 2.04, 48 2.12, 88 2.25; x = 33), and below
-// 16 SMs the tail of the depth part shows (T = 65536, l = 24: 12 SMs 47.0 ms, 16 46.9, 40 46.7; x = 8).
-inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, bool fp8, unsigned units) {
+// ring 1.75 us (16 SMs at it) to 2.0 us (50), bf16 and e4m3 at either width alike; an iteration of the sequence part 2.9 us
+// (d = 64: 1.9 us) and 5 us (7 us) per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both
+// parts end together; a few SMs more than that cost less than a few too few, because SMs that the depth part leaves go on
+// with the sequence part, and below 16 its tail shows.  The number is even: with an odd one a CTA shares its pair of SMs
+// with a CTA of the sequence part, and the whole depth part waits for that one.
+// Whole backward, us, by SMs: T = 8192, l = 16, d = 128 (x = 33): e4m3 24 2551, 32 2006, 34 1963, 36 1946, 37 2238, 38 2007,
+// 64 2090; bf16 32 2131, 35 2223, 36 2046, 37 2135, 38 2045, 64 2164.  T = 32768, l = 32, d = 64, e4m3 (x = 15): 16 16342,
+// 17 19585, 18 16372, 20 16166, 21 16892, 40 16330.  T = 4096, l = 23, B = 4 (x = 65): 60 1698, 68 1536, 72 1570, 80 1657.
+inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms) {
     const double nq = num_tiles(T);
-    const double depth = double(units) * (l + 1) * (fp8 && d == 64 ? 2.2 : 1.7);
+    const double depth = double(units) * (l + 1) * 1.7;
     const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.45 * (nq + 1) : 7.0 + 0.95 * (nq + 1));
-    const double x = 148.0 * depth / (depth + seq);
-    return std::min(units, unsigned(std::min(148.0, std::max(16.0, std::ceil(1.06 * x + 1.0)))));
+    const double x = sms * depth / (depth + seq);
+    const unsigned share = std::max(16u, 2 * unsigned(std::ceil((1.06 * x + 1.0) / 2)));
+    return std::min(units, std::min(share, sms));
 }
 
 template <int D>
@@ -423,7 +440,9 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
             // asked for alone, the depth part gets every SM; beside the sequence part, its share
             beside_rows = (stages & 2) != 0;
             const unsigned units = (tiles + 128 / D - 1) / (128 / D);
-            const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, a.fp8_cache, units) : std::min(units, 148u);
+            int sms = 0;
+            if (int rc = device_sm_count(&sms)) return rc;
+            const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, units, unsigned(sms)) : std::min(units, unsigned(sms));
             if (a.fp8_cache) bwd_rows_kernel<D, true><<<grid, 512, RowsSmem<D, true>::kDynamic, stream>>>(mQ, mdO, r);
             else bwd_rows_kernel<D><<<grid, 512, RowsSmem<D, false>::kDynamic, stream>>>(mQ, mdO, r);
             if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
@@ -672,19 +691,6 @@ int launch_decode(const DecodeParams& p, cudaStream_t stream) {
         case 8: return launch_decode_g<D, 8>(p, stream);
         default: return MODA_ERR_BAD_GROUP;
     }
-}
-
-int device_sm_count(int* out) {
-    static thread_local int cached_dev = -1, cached_sms = 0;
-    int dev = 0;
-    if (!cuda_ok(cudaGetDevice(&dev))) return MODA_ERR_CUDA;
-    if (dev != cached_dev) {
-        int sms = 0;
-        if (!cuda_ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return MODA_ERR_CUDA;
-        cached_dev = dev; cached_sms = sms;
-    }
-    *out = cached_sms;
-    return MODA_OK;
 }
 
 // The decode step behind its three entry points: contiguous cache with one length, contiguous cache with a
