@@ -302,7 +302,7 @@ int moda_attn_fwd_prefill(const void* Q, const void* K, const void* V, const voi
  * Two launches on `stream`: a kernel that streams the KV cache once per key/value head (the key
  * range is split over enough CTAs to fill the device) and a merge kernel that adds the depth pairs.
  * All pointers are device pointers owned by the caller; validation, asynchrony and error codes are
- * as for moda_attn_fwd.  The reduction order depends only on (B, H_kv, T_kv) and the device's SM
+ * as for moda_attn_fwd.  The reduction order depends only on (B, H, H_kv, d, T_kv) and the device's SM
  * count, so results are bit-reproducible on one device type.
  */
 size_t moda_decode_workspace_bytes(int B, int H, int d);
@@ -326,6 +326,10 @@ int moda_attn_decode(const void* q, const void* K, const void* V, const void* de
  *     seq_lens         : device int32 [B] as above; max_blocks_per_seq * page_size >= max_seq_len
  * Everything else (q, depth_kv_token, O, LSE, workspace, groups, validation, launches) is as for
  * moda_attn_decode.  Positions of a page past the sequence's length may hold anything.
+ * The key range is cut by the lengths that the batch has, so the reduction order of a sequence depends on
+ * the lengths of all of them (and on max_seq_len): the same call gives the same bits, but the last bits of a
+ * sequence's result may change with its neighbours, by no more than its distance from the exact result (both
+ * cuts round the probabilities of a piece to bf16 against the piece's own maximum).
  */
 int moda_attn_decode_varlen(const void* q, const void* K, const void* V, const int* seq_lens,
                             const void* depth_kv_token,

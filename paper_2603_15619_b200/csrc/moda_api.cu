@@ -644,6 +644,16 @@ int launch_kv_project(const void* X, const void* Wk, const void* Wv, int B, int 
     return cuda_ok(cudaLaunchKernelEx(&cfg, moda_kv_project_kernel<D, NH, FP8>, mX, mWk, mWv, mK, mV, p)) ? MODA_OK : MODA_ERR_CUDA;
 }
 
+// Shared memory that a merge CTA asks for beyond its own, so that an SM takes at most four (8, 12) of them.  They are placed
+// while the split kernel still holds most SMs, and without a limit they pile up on the few that it leaves or has left, where a
+// dozen of them take turns.  Where there are more than twelve per SM they fill every SM anyway.  us, no limit / 12 / 8 / 4 per SM:
+// 256 CTAs (B = 32, T = 8192, 1 head, G = 8, d = 64) 19.9 / 19.9 / 18.1 / 16.9; 48 CTAs (B = 3, T = 2000, 16 heads, d = 128) 14.1 / 14.8 /
+// 13.4 / 11.6; 1024 CTAs (B = 128, T = 1000, 1 head, G = 8, d = 64) 16.0 / 15.6 / 13.4 / 15.1; 1536 CTAs (B = 48, T = 1000, 8 heads, G = 4,
+// d = 64) 27.5 / 25.9 / 27.4; 2048 CTAs (B = 128, 4 heads, G = 4) 33.2 / 32.7 / 33.8 / 40.2.
+inline size_t decode_merge_reserve(long long ctas, int sms) {
+    return ctas <= 4ll * sms ? 44000 : ctas <= 8ll * sms ? 24000 : ctas <= 12ll * sms ? 16000 : 0;
+}
+
 // Decode step: a split kernel over the KV cache and a merge kernel that adds the depth pairs.
 template <int D, int G>
 int launch_decode_g(const DecodeParams& p, cudaStream_t stream) {
@@ -661,14 +671,18 @@ int launch_decode_g(const DecodeParams& p, cudaStream_t stream) {
         if (!set_smem_limit(decode_split_tma_kernel<D, G>, L::kDynamic)) return MODA_ERR_CUDA;
         configured_dev = dev;
     }
-    // one CTA per SM, or per run of stages when there are fewer
-    const long long runs = ((long long)p.B * (p.Hk / p.team) * decode_stages(p.T_kv) + p.min_run - 1) / p.min_run;
+    // one CTA per SM, or per run when there are fewer (with lengths: at least as many as there can be runs)
+    const long long groups = (long long)p.B * (p.Hk / p.team), units = decode_units(p.T_kv, p.unit_log2);
+    const int shortest = p.seq_lens ? p.min_run : p.cut.run;
+    const long long runs = !p.seq_lens && !p.cut.aligned ? (groups * units + shortest - 1) / shortest
+                                                         : groups * ((units + shortest - 1) / shortest);
     const unsigned grid = unsigned((runs < p.teams ? runs : p.teams) * p.team);
     decode_split_tma_kernel<D, G><<<grid, kDecodeTmaThreads, L::kDynamic, stream>>>(mK, mV, p);
     if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(p.H), unsigned(p.B), 1);
     cfg.blockDim = dim3(kDecodeMergeThreads, 1, 1);
+    cfg.dynamicSmemBytes = decode_merge_reserve((long long)p.H * p.B, p.team * p.teams);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -731,10 +745,19 @@ int decode_common(const void* q, const void* K, const void* V, const int* seq_le
     p.seq_lens = seq_lens; p.block_table = block_table; p.page_size = page_size; p.max_blocks = max_blocks;
     // Heads that are adjacent in memory are read at the same time by the CTAs of a team: one CTA per head in turn reads the
     // cache in pieces of 128 or 256 bytes, which costs d = 64 a third of the HBM rate (B = 64, T = 8192, 8 heads, us: teams of
-    // 1 235, of 4 160, of 8 162; d = 128, B = 32: 167, 174, 164).
-    p.team = p.Hk % 8 == 0 ? 8 : p.Hk % 4 == 0 ? 4 : p.Hk % 2 == 0 ? 2 : 1;
+    // 1 235, of 4 160, of 8 162; d = 128, B = 32: 167, 174, 164).  So a team takes the largest divisor of the heads up to 8 (B = 32,
+    // T = 8192, 7 heads, G = 2, d = 64, us: teams of 1 105, of 7 74), at d = 64 rather 4 than 5 to 7, whose teams leave more SMs
+    // without one (12 heads: teams of 4 127, of 6 133; d = 128: 249, 247).
+    p.team = 8;
+    while (p.Hk % p.team != 0) --p.team;
+    if (d == 64 && p.team < 8 && p.Hk % 4 == 0) p.team = 4;
     p.teams = sms / p.team;
-    p.min_run = decode_min_run(T_kv, seq_lens == nullptr, B * (p.Hk / p.team), p.teams);
+    const int heads = p.Hk / p.team;
+    p.unit_log2 = decode_unit_log2((long long)B * heads, T_kv);
+    p.min_run = decode_min_run(T_kv, p.unit_log2);
+    p.cut = decode_cut_equal(B * heads, T_kv, p.unit_log2, p.teams, H / p.Hk);
+    p.stride = DecodeWalk::stride_of(decode_units(T_kv, p.unit_log2), p.cut);
+    p.max_pieces = std::min(kDecodeMaxSplits - 1, decode_units(T_kv, p.unit_log2) / p.min_run + 2);
     p.scale_log2 = scale * kDecodeLog2e;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return d == 128 ? launch_decode<128>(p, st) : launch_decode<64>(p, st);

@@ -7,26 +7,29 @@
 //
 //   decode_split_tma_kernel  one CTA per SM, in teams of up to eight CTAs for adjacent kv heads, whose rows are adjacent in the
 //                         cache.  The stages (64 keys) of all (batch, kv heads of a team) groups, in this order, are cut
-//                         into equal runs, one per team, by the lengths that the sequences have: a CTA works on the
-//                         piece of each group that its run covers.  (Pieces of a fixed number of keys, dealt out in
-//                         turn, left SMs idle when lengths differ: B = 32, uniform in [1, 8192], paged, G = 4, d = 128:
-//                         146 -> 103 us; equal lengths, B = 1, T = 8192: 16.1 -> 13.7.)  A producer lane keeps a ring of TMA stages (64 keys: their K rows and V
-//                         rows as 128-byte-swizzled boxes) in flight, 128 KiB per SM, and runs ahead into
-//                         the CTA's next piece, so the HBM stream does not stop at their boundaries.
+//                         into equal runs, one per team, by the lengths that the sequences have (decode_plan.h): a CTA works
+//                         on the piece of each group that its run covers, on one piece only where the teams suffice.  (Pieces
+//                         of a fixed number of keys, dealt out in turn, left SMs idle when lengths differ: B = 32, uniform in
+//                         [1, 8192], paged, G = 4, d = 128: 138 -> 100 us.)  A producer lane keeps a ring of TMA stages (64
+//                         keys: their K rows and V rows as 128-byte-swizzled boxes) in flight, 128 KiB per SM, and runs ahead
+//                         into the CTA's next piece, so the HBM stream does not stop at their boundaries.
 //                         Eight consumer warps, 32 keys of a stage each: scores and weighted values with
 //                         warp-level MMAs whose 16-row operand holds the G <= 8 heads of the group (the
 //                         CUDA-core form of the same arithmetic is issue-bound from G = 4 on); K pieces
 //                         and, through transposing matrix loads, V pieces come from the swizzled stage.
-//                         Each warp keeps an online-softmax state (m, l, o) per head; at the end of an
+//                         Each warp keeps an online-softmax state (m, l, o) per head; at the end of a
 //                         piece the warps are merged through shared memory and the CTA writes one partial
 //                         (m, l, o[d]) per head.
 //   decode_merge_kernel   grid (query head, batch): merges the partials of all pieces of a group with the l
 //                         depth pairs of the token (scored here: l d-length dot products) and writes
 //                         O (bf16) and LSE (natural log).  It starts beside the split kernel (programmatic dependent
-//                         launch) and scores the depth pairs while that runs (1 to 3 us of a step).
+//                         launch) once every producer has requested its last stage, and scores the depth pairs while the
+//                         last stages are worked on (about 1 us of a step; from the split kernel's start on it took issue
+//                         slots from it: B = 8, T = 4096, 6 heads, G = 2, d = 128: 20.0 -> 18.3 us).
 #pragma once
 
 #include <cstdint>
+#include "decode_plan.h"
 #include <cuda_bf16.h>
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -35,10 +38,6 @@
 
 namespace moda {
 
-constexpr int kDecodeWarps = 8;
-constexpr int kDecodeThreads = kDecodeWarps * 32;
-constexpr int kDecodeStageKeys = 64;
-constexpr int kDecodeMaxSplits = 128;                      // partials of a group that the workspace holds
 constexpr float kDecodeLog2e = 1.4426950408889634f;
 constexpr float kDecodeLn2 = 0.6931471805599453f;
 
@@ -52,7 +51,10 @@ struct DecodeParams {
     float* part;                  // [B][Hk][kDecodeMaxSplits][G][d + 2]: m (log2 domain), l, o[d]; with seq_lens the last
                                   // one of a group starts with the number of its partials
     int B, T_kv, T_cap, H, Hk, l;
-    int min_run;                  // fewest stages of a CTA's run
+    int unit_log2, min_run;       // keys of a unit; fewest units of a run (decode_plan.h)
+    DecodeCut cut;                // without seq_lens (with them the kernel works it out)
+    int stride;                   // units that a group takes in the order, without seq_lens
+    int max_pieces;               // of any group
     int team, teams;              // CTAs of a team (divides Hk); teams that the SMs hold
     int kv_rep;                   // groups of more than 8 query heads run as kv_rep groups of 8 on the same K, V head
     const int* seq_lens;          // [B] cached positions per sequence (each 1 .. T_kv), or null: T_kv for all
@@ -61,25 +63,6 @@ struct DecodeParams {
     float scale_log2;             // scale * log2(e)
 };
 
-// Stages of a CTA's run.  At least four, one for each pair of consumer warps (a shorter run takes as long), and enough
-// that no group is cut into more than kDecodeMaxSplits - 1 pieces.
-__host__ __device__ inline int decode_stages(int len) { return (len + kDecodeStageKeys - 1) / kDecodeStageKeys; }
-__host__ __device__ inline int decode_run(int total_stages, int teams, int min_run) {
-    const int run = (total_stages + teams - 1) / teams;
-    return run > min_run ? run : min_run;
-}
-inline int decode_min_run(int T_kv, bool equal, int groups, int teams) {
-    const int ns = decode_stages(T_kv);
-    const int cap = (ns + kDecodeMaxSplits - 3) / (kDecodeMaxSplits - 2);
-    const int least = cap > 4 ? cap : 4;
-    if (!equal) return least;
-    // equal lengths: a run that cuts every group at the same places leaves one piece per CTA where a cheaper run that crosses
-    // groups leaves two; a piece costs about a stage and a half
-    const int run = decode_run(groups * ns, teams, least);
-    const int cuts = (ns + run - 1) / run > 1 ? ns / run : 1;
-    const int even = (ns + cuts - 1) / cuts;
-    return (long long)groups * cuts <= teams && even <= run + 1 + run / 8 ? even : least;
-}
 inline size_t decode_workspace_bytes(int B, int H, int d) {
     return size_t(B) * H * kDecodeMaxSplits * (d + 2) * 4;
 }
@@ -151,16 +134,40 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         for (int st = 0; st < L::kStages; ++st) { mbar_init(full_bar(st), 1); mbar_init(empty_bar(st), 2); }
         fence_mbar_init();
     }
-    grid_launch_dependents();                                           // the merge kernel may come up and score its depth pairs
-    // ---- this CTA's run of stages, and where it starts: sequence, kv head, stage of that group ----
+    // ---- this CTA's run, and where it starts: sequence, and units per team of heads before it ----
     const int my_team = int(blockIdx.x) / p.team, heads = p.Hk / p.team;   // heads: kv heads that one CTA of a team takes in turn
     const int head_in_team = int(blockIdx.x) % p.team;
-    int total, b0 = 0, before = 0;                                      // stages in all; first sequence; stages per head before it
+    DecodeCut cut = p.cut;
+    int total, b0, before;
     if (p.seq_lens == nullptr) {
-        total = p.B * heads * decode_stages(p.T_kv);
+        total = p.B * heads * p.stride;
+        b0 = my_team * cut.run / (heads * p.stride);                    // past the last one for a team without a run
+        before = b0 * p.stride;
+    } else if (p.B <= 32) {
+        // every warp for itself, a lane per sequence
+        int v = lane < p.B ? decode_units(len_of(lane), p.unit_log2) : 0;
+        cut = DecodeCut{decode_run(int(__reduce_add_sync(0xffffffffu, v)) * heads, p.teams, p.min_run), 0};
+        if (p.B * heads <= p.teams) {
+            const int longer = decode_aligned_run(cut.run, 1), longest = decode_aligned_run(cut.run, G);
+            if (int(__reduce_add_sync(0xffffffffu, decode_ceil_div(v, cut.run))) * heads <= p.teams) cut.aligned = 1;
+            else if (int(__reduce_add_sync(0xffffffffu, decode_ceil_div(v, longer))) * heads <= p.teams) cut = DecodeCut{longer, 1};
+            else if (int(__reduce_add_sync(0xffffffffu, decode_ceil_div(v, longest))) * heads <= p.teams) cut = DecodeCut{longest, 1};
+            v = DecodeWalk::stride_of(v, cut);
+        }
+        int upto = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, upto, off);
+            if (lane >= off) upto += up;
+        }
+        total = __shfl_sync(0xffffffffu, upto, 31) * heads;
+        const int first = my_team * cut.run;
+        const uint32_t here = __ballot_sync(0xffffffffu, first >= (upto - v) * heads && first < upto * heads);
+        b0 = here ? __ffs(here) - 1 : 0;
+        before = __shfl_sync(0xffffffffu, upto - v, b0);
     } else {
-        // Sums over the lengths, a block of them at a time.  Once for the total, which gives the run's length, and once
-        // for the sequence that the run starts in.
+        // Sums over the lengths, a block of them at a time: once for the total, which gives the run, and once for the
+        // sequence that the run starts in.
         __shared__ int s_sum[kDecodeTmaThreads / 32], s_at[3];
         auto block_scan = [&](int v, int& block_total) {                // sum over the threads before this one
             int incl = v;
@@ -183,68 +190,44 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         };
         int sum = 0, part_sum, v = 0, pre = 0;
         for (int b = threadIdx.x; b - int(threadIdx.x) < p.B; b += kDecodeTmaThreads) {
-            v = b < p.B ? decode_stages(len_of(b)) : 0;
+            v = b < p.B ? decode_units(len_of(b), p.unit_log2) : 0;
             pre = block_scan(v, part_sum) + sum;
             sum += part_sum;
         }
+        cut = DecodeCut{decode_run(sum * heads, p.teams, p.min_run), 0};
+        if (p.B * heads <= p.teams && p.B <= kDecodeTmaThreads) {       // one sequence per thread; at most 127 pieces each
+            const int longer = decode_aligned_run(cut.run, 1), longest = decode_aligned_run(cut.run, G);
+            block_scan(decode_ceil_div(v, longer) | decode_ceil_div(v, longest) << 16, part_sum);
+            if ((part_sum & 0xffff) * heads <= p.teams) cut = DecodeCut{longer, 1};
+            else if ((part_sum >> 16) * heads <= p.teams) cut = DecodeCut{longest, 1};
+            if (cut.aligned) {
+                v = DecodeWalk::stride_of(v, cut);
+                pre = block_scan(v, sum);
+            }
+        }
         total = sum * heads;
-        const int first = my_team * decode_run(total, p.teams, p.min_run);
+        const int first = my_team * cut.run;
         int carry = 0;
         for (int b = threadIdx.x; b - int(threadIdx.x) < p.B; b += kDecodeTmaThreads) {
             if (p.B > kDecodeTmaThreads) {                              // else the values of the first pass still stand
-                v = b < p.B ? decode_stages(len_of(b)) : 0;
+                v = b < p.B ? decode_units(len_of(b), p.unit_log2) : 0;
                 pre = block_scan(v, part_sum) + carry;
                 carry += part_sum;
             }
             if (first >= pre * heads && first < (pre + v) * heads) { s_at[0] = b; s_at[1] = pre; }
         }
         __syncthreads();
-        if (first < total) { b0 = s_at[0]; before = s_at[1]; }
+        b0 = first < total ? s_at[0] : 0;
+        before = first < total ? s_at[1] : 0;
     }
-    const int run = decode_run(total, p.teams, p.min_run);
-    const int run_begin = my_team * run, run_end = min(total, run_begin + run);
-    // the pieces of the run, one group after the other
-    struct Item { int b, hk, k_begin, k_end, n_stage, index, pieces; };   // index: of this piece in its group
-    struct Walk { int b, hk, ns, start, at; };                            // group (hk: team of heads), its stages, its first stage and ours in the order of all
     auto walk_begin = [&]() {
-        Walk k;
-        k.at = run_begin;
-        if (p.seq_lens == nullptr) {
-            k.ns = decode_stages(p.T_kv);
-            const int group = run_begin / k.ns;
-            k.b = group / heads;
-            k.hk = group % heads;
-            k.start = group * k.ns;
-        } else {
-            k.b = b0;
-            k.ns = run_begin < total ? decode_stages(len_of(b0)) : 1;
-            k.hk = (run_begin - before * heads) / k.ns;
-            k.start = before * heads + k.hk * k.ns;
-        }
+        DecodeWalk k;
+        k.begin(cut, my_team, total, heads, p.unit_log2, b0, before, len_of);
         return k;
     };
-    auto walk_item = [&](const Walk& k) {
-        Item w;
-        const int len = len_of(k.b);
-        const int s0 = k.at - k.start, s1 = min(k.ns, run_end - k.start);
-        w.b = k.b; w.hk = k.hk * p.team + head_in_team;
-        w.k_begin = s0 * kDecodeStageKeys;
-        w.k_end = min(len, s1 * kDecodeStageKeys);
-        w.n_stage = s1 - s0;
-        const int first_cta = k.start / run;
-        w.index = my_team - first_cta;
-        w.pieces = (k.start + k.ns - 1) / run - first_cta + 1;
-        return w;
-    };
-    auto walk_next = [&](Walk& k) {                                       // to the next group; past the run's end: at >= run_end
-        k.start += k.ns;
-        k.at = k.start;
-        if (++k.hk == heads) {
-            k.hk = 0;
-            ++k.b;
-            if (k.at < run_end) k.ns = decode_stages(len_of(k.b));
-        }
-    };
+    // kv head of a piece for this CTA of the team, and its 64-key stages
+    auto head_of = [&](int head_team) { return head_team * p.team + head_in_team; };
+    auto stages_of = [](const DecodePiece& w) { return (w.k_end - w.k_begin + kDecodeStageKeys - 1) / kDecodeStageKeys; };
     __syncthreads();
 
     int n_issued = 0;                                                   // producer lane: stages requested so far
@@ -253,18 +236,19 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         if (lane == 0) {
             tma_prefetch_desc(&mapK);
             tma_prefetch_desc(&mapV);
-            for (Walk k = walk_begin(); k.at < run_end && *abort_flag == 0; walk_next(k)) {
-                const Item w = walk_item(k);
+            for (DecodeWalk k = walk_begin(); !k.done() && *abort_flag == 0; k.next(cut, heads, p.unit_log2, len_of)) {
+                const DecodePiece w = k.piece(cut, my_team, p.unit_log2, len_of);
+                const int n_stage = stages_of(w), kv_head = head_of(w.head_team) / p.kv_rep;
                 // paged cache: the page of a stage's 64 positions comes from the sequence's block table; the
                 // entry of the next stage is requested before this stage's wait, so its latency is hidden
                 const int* table = p.block_table ? p.block_table + size_t(w.b) * p.max_blocks : nullptr;
-                int page_next = (table && w.n_stage > 0) ? table[w.k_begin / p.page_size] : 0;
-                for (int i = 0; i < w.n_stage; ++i) {
+                int page_next = table ? table[w.k_begin / p.page_size] : 0;
+                for (int i = 0; i < n_stage; ++i) {
                     const int gi = n_issued;
                     const int st = gi % L::kStages;
                     const int t0 = w.k_begin + i * kDecodeStageKeys;
                     const int page = page_next;
-                    if (table && i + 1 < w.n_stage) page_next = table[(t0 + kDecodeStageKeys) / p.page_size];
+                    if (table && i + 1 < n_stage) page_next = table[(t0 + kDecodeStageKeys) / p.page_size];
                     if (gi >= L::kStages) mbar_wait(empty_bar(st), ((gi / L::kStages) - 1) & 1, abort_flag, 70);
                     if (*abort_flag != 0) break;
                     const uint32_t dst = smem_u32(smem + L::kRing + st * L::kStageBytes);
@@ -273,12 +257,13 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
                     const int c3 = table ? page : w.b;                     // page / batch index
 #pragma unroll
                     for (int h = 0; h < NH; ++h) {
-                        tma_load_4d(dst + h * kBoxBytes, &mapK, full_bar(st), 64 * h, w.hk / p.kv_rep, c2, c3);
-                        tma_load_4d(dst + (NH + h) * kBoxBytes, &mapV, full_bar(st), 64 * h, w.hk / p.kv_rep, c2, c3);
+                        tma_load_4d(dst + h * kBoxBytes, &mapK, full_bar(st), 64 * h, kv_head, c2, c3);
+                        tma_load_4d(dst + (NH + h) * kBoxBytes, &mapV, full_bar(st), 64 * h, kv_head, c2, c3);
                     }
                     n_issued = gi + 1;
                 }
             }
+            grid_launch_dependents();                                   // the merge kernel may come up and score its depth pairs
         }
     } else {
         // ---- consumers: warp pair `pair` takes the stages whose running index is pair mod 4 (always the
@@ -290,11 +275,11 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         const int g = lane >> 2, t = lane & 3;
         const int ctid = threadIdx.x;                                    // 0 .. 255
         // q rows (bf16, heads 0..7, zero beyond G) of an item: one 16-byte piece per thread
-        auto fetch_q = [&](const Walk& w) {
+        auto fetch_q = [&](const DecodeWalk& w) {
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             const int row = ctid / CH, piece = ctid % CH;
             if (ctid < 8 * CH && row < G)
-                v = *reinterpret_cast<const uint4*>(p.q + (size_t(w.b) * p.H + (w.hk * p.team + head_in_team) * G + row) * D + piece * 8);
+                v = *reinterpret_cast<const uint4*>(p.q + (size_t(w.b) * p.H + head_of(w.head_team) * G + row) * D + piece * 8);
             return v;
         };
         auto store_q = [&](int buf, const uint4& v) {
@@ -302,16 +287,24 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
         };
         int qb = 0;
         int gi0 = 0;                                                     // running stage index at the start of the item
-        Walk k = walk_begin();
-        if (k.at < run_end) store_q(0, fetch_q(k));
+        DecodeWalk k = walk_begin();
+        if (!k.done()) store_q(0, fetch_q(k));
         decode_consumer_sync();
 #pragma unroll 1
-        while (k.at < run_end) {
-            const Item w = walk_item(k);
-            walk_next(k);
-            const bool has_next = k.at < run_end;
+        while (!k.done()) {
+            int k_begin, k_end, n_stage;
+            bool has_next;
             uint4 qnext = make_uint4(0u, 0u, 0u, 0u);
-            if (has_next) qnext = fetch_q(k);                             // lands while this piece is processed
+            {
+                const DecodePiece w = k.piece(cut, my_team, p.unit_log2, len_of);
+                k_begin = w.k_begin;
+                k_end = w.k_end;
+                n_stage = stages_of(w);
+                DecodeWalk next = k;
+                next.next(cut, heads, p.unit_log2, len_of);
+                has_next = !next.done();
+                if (has_next) qnext = fetch_q(next);                      // lands while this piece is processed
+            }
             // A fragments of q: for every 32 features, this lane's 8 features of head g (the same 8 features
             // that it takes from a key row below, so the pairing inside the MMA is consistent)
             uint4 qf[D / 32];
@@ -325,15 +318,15 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
 
             const int first = (pair - (gi0 % kDecodePairs) + kDecodePairs) % kDecodePairs;
 #pragma unroll 1
-            for (int i = first; i < w.n_stage; i += kDecodePairs) {
+            for (int i = first; i < n_stage; i += kDecodePairs) {
                 const int gi = gi0 + i;
                 const int st = gi % L::kStages;
                 mbar_wait(full_bar(st), (gi / L::kStages) & 1, abort_flag, 71);
                 // After a wait has given up every later wait returns at once; the loops still run to their
                 // ends (without touching the data) so that all warps meet at the barriers below.
                 const bool live = __shfl_sync(0xffffffffu, *abort_flag, 0) == 0;
-                const int k0 = w.k_begin + i * kDecodeStageKeys + half * 32;   // first key of this warp
-                const int n = min(32, w.k_end - k0);                           // <= 0: second half of a short last stage
+                const int k0 = k_begin + i * kDecodeStageKeys + half * 32;   // first key of this warp
+                const int n = min(32, k_end - k0);                           // <= 0: second half of a short last stage
                 if (live && n > 0) {
                     uint8_t* sK = smem + L::kRing + st * L::kStageBytes;
                     uint8_t* sV = sK + NH * kBoxBytes;
@@ -403,7 +396,7 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty_bar(st));
             }
-            gi0 += w.n_stage;
+            gi0 += n_stage;
 
             // ---- merge the eight warps, write the item's partial ----
             lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
@@ -416,7 +409,10 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             }
             if (has_next) store_q(qb ^ 1, qnext);
             decode_consumer_sync();
-            float* out = p.part + ((size_t(w.b) * p.Hk + w.hk) * kDecodeMaxSplits + w.index) * G * (D + 2);
+            asm volatile("" : "+r"(cut.run));                              // nothing of the piece's place is kept over the key loop
+            const DecodePiece w = k.piece(cut, my_team, p.unit_log2, len_of);
+            k.next(cut, heads, p.unit_log2, len_of);
+            float* out = p.part + ((size_t(w.b) * p.Hk + head_of(w.head_team)) * kDecodeMaxSplits + w.index) * G * (D + 2);
             if (p.seq_lens && w.index == 0 && ctid == 0)
                 out[size_t(kDecodeMaxSplits - 1) * G * (D + 2)] = __int_as_float(w.pieces);
             for (int e = ctid; e < G * D; e += kDecodeConsumerThreads) {
@@ -503,22 +499,24 @@ decode_merge_kernel(const DecodeParams p) {
         }
     }
     __syncthreads();
+    int S = p.seq_lens ? p.max_pieces                                               // pieces of the group
+                       : decode_pieces_equal(p.cut, b * (p.Hk / p.team) + hk / p.team, p.T_kv, p.unit_log2);
     // ---- from here on: what the split kernel wrote ----
     grid_dependency_wait();
     const float* group = p.part + (size_t(b) * p.Hk + hk) * kDecodeMaxSplits * G * (D + 2);
     const float* part = group + g * (D + 2);                                        // + piece * G * (D + 2)
     const size_t split_stride = size_t(G) * (D + 2);
-    int S;                                                                          // pieces of the group
+    // a thread per piece: its maximum and row sum, requested together with the number of pieces (slots past that number hold
+    // nothing yet and are not used)
+    static_assert(kDecodeMergeThreads >= kDecodeMaxSplits, "a thread per piece");
+    float2 piece = make_float2(-INFINITY, 0.f);
+    if (tid < S) piece = __ldcg(reinterpret_cast<const float2*>(part + tid * split_stride));
     if (p.seq_lens) {
-        S = __float_as_int(__ldcg(group + (kDecodeMaxSplits - 1) * split_stride));
-    } else {
-        const int ns = decode_stages(p.T_kv), heads = p.Hk / p.team;
-        const int run = decode_run(p.B * heads * ns, p.teams, p.min_run), start = (b * heads + hk / p.team) * ns;
-        S = (start + ns - 1) / run - start / run + 1;
+        S = min(max(__float_as_int(__ldcg(group + (kDecodeMaxSplits - 1) * split_stride)), 1), S);
+        if (tid >= S) piece = make_float2(-INFINITY, 0.f);
     }
     // ---- global maximum over the split maxima and the depth scores ----
-    float mx = -INFINITY;
-    for (int s = tid; s < S; s += kDecodeMergeThreads) mx = fmaxf(mx, __ldcg(part + s * split_stride));
+    float mx = piece.x;
     for (int i = tid; i < p.l; i += kDecodeMergeThreads) mx = fmaxf(mx, s_d[i]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
@@ -530,11 +528,10 @@ decode_merge_kernel(const DecodeParams p) {
     __syncthreads();
     // ---- weights and the row sum ----
     float lt = 0.f;
-    for (int s = tid; s < S; s += kDecodeMergeThreads) {
-        const float ms = __ldcg(part + s * split_stride);
-        const float f = ms == -INFINITY ? 0.f : fast_exp2(ms - mx);
-        s_w[s] = f;
-        lt = fmaf(f, __ldcg(part + s * split_stride + 1), lt);
+    if (tid < S) {
+        const float f = piece.x == -INFINITY ? 0.f : fast_exp2(piece.x - mx);
+        s_w[tid] = f;
+        lt = f * piece.y;
     }
     for (int i = tid; i < p.l; i += kDecodeMergeThreads) {
         const float w = fast_exp2(s_d[i] - mx);

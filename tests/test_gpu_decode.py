@@ -163,7 +163,12 @@ def test_decode_over_a_paged_cache(B, T_max, H, Hk, d, l, page):
 # group, more sequences than the split kernel has threads (its sums over the lengths then take several rounds), one group over all
 # SMs (the run's length is set by the number of partials that the workspace holds).
 @pytest.mark.parametrize("B,T_max,H,Hk,d,l,kind", [(300, 200, 4, 2, 64, 2, "random"), (620, 70, 2, 1, 128, 1, "random"), (40, 6000, 8, 2, 128, 3, "one long"),
-                                                   (40, 6000, 4, 4, 64, 0, "all one"), (1, 40000, 2, 1, 64, 5, "full"), (3, 9000, 16, 1, 128, 4, "full")])
+                                                   (40, 6000, 4, 4, 64, 0, "all one"), (1, 40000, 2, 1, 64, 5, "full"), (3, 9000, 16, 1, 128, 4, "full"),
+                                                   # a piece per team, a warp or the whole block adding up the lengths; teams of 5, 7, 6 and 4 heads; 8 heads
+                                                   # to a group, where one long piece is preferred to two; merge CTAs at 4 and 8 per SM
+                                                   (8, 4096, 4, 1, 128, 2, "random"), (33, 900, 5, 5, 64, 1, "random"), (3, 2000, 14, 7, 128, 3, "random"),
+                                                   (16, 2048, 12, 6, 64, 1, "full"), (5, 1500, 12, 12, 64, 0, "random"), (120, 1000, 8, 1, 128, 2, "random"),
+                                                   (37, 300, 32, 8, 64, 33, "random")])
 def test_runs_of_stages_over_unequal_lengths(B, T_max, H, Hk, d, l, kind):
     x = synthetic.make_decode(B, T_max, H, Hk, d, l, seed=41, device="cuda")
     rng = np.random.default_rng(B)
