@@ -226,3 +226,36 @@ def test_depth_part_beside_the_sequence_part(B, T, H, d, l, e4m3):
         for stage in (1, 2, 4):
             bwd(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, w.scale, *out, again, workspace=ws, stages=stage)
         assert_same_gradients((*got[:3], dcache), (*out, again), "stage by stage")
+
+
+# Captured in a graph: the depth part and the sequence part are two branches of the launch, and what follows the call (here a
+# copy of every gradient) comes after both.
+@pytest.mark.parametrize("B,T,H,d,l,e4m3", [(1, 1100, 8, 128, 9, False), (1, 2400, 7, 64, 12, True)])
+def test_forward_and_backward_replayed_from_a_graph(B, T, H, d, l, e4m3):
+    x = synthetic.make(synthetic.Workload("graph", B, T, H, d, l), seed=62, device="cuda")
+    scale = d ** -0.5
+    if e4m3:
+        cache = moda.alloc_depth_cache_e4m3(B, T, H, d, l, "cuda")
+        for i in range(l):
+            moda.moda_depth_cache_append_e4m3(cache, i, x["Kd"][i].contiguous(), x["Vd"][i].contiguous())
+        fwd, bwd = moda.moda_attn_fwd_e4m3, moda.moda_attn_bwd_e4m3
+    else:
+        cache = build_cache(x["Kd"], x["Vd"])
+        fwd, bwd = moda.moda_attn_fwd, moda.moda_attn_bwd
+    dcache = moda.alloc_depth_cache(B, T, H, d, l)
+
+    def step():
+        O, LSE = fwd(x["Q"], x["K"], x["V"], cache, l, scale)
+        dQ, dK, dV, _ = bwd(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, scale, d_depth_kv=dcache)
+        return [t.clone() for t in (dQ, dK, dV, dcache)]
+    want = step()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = step()
+    for _ in range(3):
+        for t in (dcache, *got):
+            t.fill_(7.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert moda.moda_last_status() == 0
+        assert_same_gradients(got, want, f"{(B, T, H, d, l, e4m3)}")
