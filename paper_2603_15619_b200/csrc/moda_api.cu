@@ -61,6 +61,21 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 
+// Whether a context is current on the calling thread.
+bool has_context() {
+    using Fn = CUresult (*)(CUcontext*);
+    static Fn fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuCtxGetCurrent", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<Fn>(p);
+    });
+    CUcontext current = nullptr;
+    return fn != nullptr && fn(&current) == CUDA_SUCCESS && current != nullptr;
+}
+
 // Tensor map over a contiguous bf16 [B][T][H][d] tensor; one box = 128 positions x 64
 // features of one (b, h), written to shared memory with the 128-byte swizzle.
 // Out-of-range rows (ragged last tile) read as zero and are dropped on store.
@@ -141,8 +156,9 @@ int check_device(bool may_allocate = true) {
     if (dev != cached_dev) {
         int major = 0;
         if (!cuda_ok(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev))) return MODA_ERR_CUDA;
-        // a thread whose first CUDA call this is (an autograd worker) has no context yet, and encoding a tensor map needs one
-        if (!cuda_ok(cudaSetDevice(dev))) return MODA_ERR_CUDA;
+        // a thread whose first CUDA call this is (an autograd worker) has no context yet, and encoding a tensor map needs one;
+        // a context that the caller has made current stays
+        if (!has_context() && !cuda_ok(cudaSetDevice(dev))) return MODA_ERR_CUDA;
         cached_dev = dev;
         cached_rc = (major == 10) ? MODA_OK : MODA_ERR_DEVICE;
     }

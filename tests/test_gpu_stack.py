@@ -244,3 +244,32 @@ def test_a_thread_whose_first_cuda_call_is_ours():
     t.join()
     torch.cuda.synchronize()
     assert not failed and torch.equal(O, want), failed
+
+
+def test_a_context_that_the_caller_made_current_stays():
+    """A thread with a CUDA context of its own (not the one that the runtime shares) calls the library on memory of that context."""
+    import threading
+    from cuda.bindings import driver
+    seen = []
+
+    def ok(res):
+        assert res[0] == driver.CUresult.CUDA_SUCCESS, res[0]
+        return res[1] if len(res) > 1 else None
+
+    def work():
+        ctx = ok(driver.cuCtxCreate(0, 0))
+        try:
+            B, T, H, d = 1, 5, 1, 64
+            lib = moda.binding.load()
+            k, v = (ok(driver.cuMemAlloc(B * T * H * d * 2)) for _ in range(2))
+            cache = ok(driver.cuMemAlloc(int(lib.moda_depth_cache_bytes(B, T, H, d, 1))))
+            rc = lib.moda_depth_cache_append(int(cache), B, T, H, d, 0, int(k), int(v), None)
+            seen.append((rc, int(ok(driver.cuCtxGetCurrent())) == int(ctx)))
+            ok(driver.cuCtxSynchronize())
+        finally:
+            ok(driver.cuCtxDestroy(ctx))
+    torch.cuda.synchronize()
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert seen == [(0, True)]
