@@ -374,10 +374,11 @@ int moda_attn_bwd_static_scratch(const void* Q, const void* K, const void* V, co
 
 /*
  * moda_attn_fwd_e4m3 that also writes the layer's own K, V as slot `append_slot` of an e4m3 cache
- * (the write step of Sec. 2.2 fused into the forward, as moda_attn_fwd_append does for a bf16
- * cache).  The slot receives byte for byte what moda_depth_cache_append_e4m3(append_cache_e4m3, ..., append_slot, K, V)
- * stores.  Rules for writing a slot that the call also reads as in moda_attn_fwd_append.  One launch for T >= 32768; on
- * shorter sequences the quantiser runs as a second launch behind the forward (cheaper there), with the same result.
+ * (the write step of Sec. 2.2 in the same call, as moda_attn_fwd_append does for a bf16 cache).  The slot
+ * receives byte for byte what moda_depth_cache_append_e4m3(append_cache_e4m3, ..., append_slot, K, V)
+ * stores.  Two launches: the forward, then the quantiser, after every read of the cache by the call.  The rules
+ * for a slot that the call also reads are those of moda_attn_fwd_append, grouped heads (MODA_ERR_BAD_SLOT)
+ * included, so that a caller may hold either kind of cache.
  */
 int moda_attn_fwd_append_e4m3(const void* Q, const void* K, const void* V, const void* depth_kv_e4m3,
                               int B, int T, int H, int H_kv, int d, int l, float scale,

@@ -293,7 +293,7 @@ def moda_attn_fwd_e4m3(Q, K, V, depth_kv_e4m3, l, scale, O=None, LSE=None, strea
 
 
 def moda_attn_fwd_append_e4m3(Q, K, V, depth_kv_e4m3, l, scale, append_cache_e4m3, append_slot, O=None, LSE=None, stream=None):
-    """moda_attn_fwd_e4m3 that also quantises K, V into slot ``append_slot`` of an e4m3 cache in the same launch."""
+    """moda_attn_fwd_e4m3 that also quantises K, V into slot ``append_slot`` of an e4m3 cache (a second launch behind it)."""
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
     if O is None:
         O = _new_like(Q, stream)

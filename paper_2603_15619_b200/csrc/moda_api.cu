@@ -1080,8 +1080,9 @@ int moda_attn_fwd_append_e4m3(const void* Q, const void* K, const void* V, const
     if (int rc = check_device()) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // The quantiser runs as its own launch behind the forward, after every read of the cache by this call.  Inside the
-    // forward's depth warps it costs about as many instructions as eight depth slots (l = 8, d = 128, ms, inside -> behind:
-    // T = 32768 4.64 -> 4.50, 65536 17.40 -> 17.21; B = 2, T = 5000 0.53 -> 0.36).
+    // forward's depth warps it cost about as many instructions as eight depth slots.  Forward with the write step, us, inside ->
+    // behind: d = 128, 16 heads, B = 2, T = 8192, l = 8 811 -> 722, l = 32 1091 -> 929; T = 32768, l = 8 4843 -> 4689; d = 64, 32 heads, B = 2,
+    // T = 1000, l = 4 49.6 -> 48.4, T = 8192, l = 8 994 -> 963, l = 32 1346 -> 1321; T = 32768, l = 8 6231 -> 6034.
     const int rc = d == 128 ? launch_fwd<128>(Q, K, V, depth_kv_e4m3, B, T, T, H, H_kv, l, scale, O, LSE, nullptr, st, kCacheE4m3)
                             : launch_fwd<64>(Q, K, V, depth_kv_e4m3, B, T, T, H, H_kv, l, scale, O, LSE, nullptr, st, kCacheE4m3);
     if (rc != MODA_OK) return rc;
