@@ -23,9 +23,9 @@ using namespace moda;
 
 thread_local int tl_last_cuda_error = 0;
 
-// One thread waits on an mbarrier that nothing arrives at; the bounded wait gives up after `limit_ns`
+// One thread waits on an mbarrier that nothing arrives at; the bounded wait gives up after `limit_cycles`
 // and records (MODA_SELFTEST_WAIT_SITE << 8) | 1 exactly as a production kernel's wait would.
-__global__ void wait_timeout_selftest_kernel(uint64_t limit_ns) {
+__global__ void wait_timeout_selftest_kernel(uint32_t limit_cycles) {
     __shared__ __align__(8) uint64_t bar_word;
     __shared__ int abort_word;
     if (threadIdx.x == 0) {
@@ -34,7 +34,10 @@ __global__ void wait_timeout_selftest_kernel(uint64_t limit_ns) {
         fence_mbar_init();
     }
     __syncthreads();
-    if (threadIdx.x == 0) mbar_wait(smem_u32(&bar_word), 0, &abort_word, MODA_SELFTEST_WAIT_SITE, limit_ns);
+    if (threadIdx.x == 0) {
+        mbar_wait(smem_u32(&bar_word), 0, &abort_word, MODA_SELFTEST_WAIT_SITE, limit_cycles);
+        if (abort_word != 0) report_abort(&abort_word);
+    }
 }
 
 inline bool cuda_ok(cudaError_t e) {
@@ -400,18 +403,19 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
 }
 
 // How many SMs the depth part of a fused backward gets beside the sequence part.  Measured SM time: an entry of the row
-// ring 1.75 us (16 SMs at it) to 2.0 us (50), bf16 and e4m3 at either width alike; an iteration of the sequence part 2.9 us
-// (d = 64: 1.9 us) and 5 us (7 us) per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both
+// ring 1.75 us (16 SMs at it) to 2.0 us (50), e4m3 a tenth more; an iteration of the sequence part 2.7 us
+// (d = 64: 1.75 us) and 5 us (7 us) per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both
 // parts end together; a few SMs more than that cost less than a few too few, because SMs that the depth part leaves go on
 // with the sequence part, and below 16 its tail shows.  The number is even: with an odd one a CTA shares its pair of SMs
 // with a CTA of the sequence part, and the whole depth part waits for that one.
-// Whole backward, us, by SMs: T = 8192, l = 16, d = 128 (x = 33): e4m3 24 2551, 32 2006, 34 1963, 36 1946, 37 2238, 38 2007,
-// 64 2090; bf16 32 2131, 35 2223, 36 2046, 37 2135, 38 2045, 64 2164.  T = 32768, l = 32, d = 64, e4m3 (x = 15): 16 16342,
-// 17 19585, 18 16372, 20 16166, 21 16892, 40 16330.  T = 4096, l = 23, B = 4 (x = 65): 60 1698, 68 1536, 72 1570, 80 1657.
-inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms) {
+// Whole backward, us, by SMs: T = 8192, l = 16, B = 2, d = 128: 28 2325, 32 2182, 36 2000, 40 1935, 44 2122 (taken: 40);
+// T = 4096, l = 23, B = 4: d = 128 64 1698, 72 1653, 80 1720 (72), d = 64 52 1914, 56 1797, 60 1821 (58); T = 8192, l = 16,
+// d = 64, 32 heads: 24 2521, 28 2359, 32 2410 (30).  e4m3, T = 5000, l = 23, B = 2: d = 128 62 1184, 66 1138, 72 1118 (70); d = 64
+// 50 1366, 54 1301, 58 1269, 64 1276 (56).
+inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms, bool fp8) {
     const double nq = num_tiles(T);
-    const double depth = double(units) * (l + 1) * 1.7;
-    const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.45 * (nq + 1) : 7.0 + 0.95 * (nq + 1));
+    const double depth = double(units) * (l + 1) * (fp8 ? 1.9 : 1.7);
+    const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.36 * (nq + 1) : 7.0 + 0.88 * (nq + 1));
     const double x = sms * depth / (depth + seq);
     const unsigned share = std::max(16u, 2 * unsigned(std::ceil((1.06 * x + 1.0) / 2)));
     return std::min(units, std::min(share, sms));
@@ -458,7 +462,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
             const unsigned units = (tiles + 128 / D - 1) / (128 / D);
             int sms = 0;
             if (int rc = device_sm_count(&sms)) return rc;
-            const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, units, unsigned(sms)) : std::min(units, unsigned(sms));
+            const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, units, unsigned(sms), a.fp8_cache) : std::min(units, unsigned(sms));
             if (a.fp8_cache) bwd_rows_kernel<D, true><<<grid, 512, RowsSmem<D, true>::kDynamic, stream>>>(mQ, mdO, r);
             else bwd_rows_kernel<D><<<grid, 512, RowsSmem<D, false>::kDynamic, stream>>>(mQ, mdO, r);
             if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
@@ -837,7 +841,7 @@ int moda_last_cuda_error(void) { return tl_last_cuda_error; }
 
 int moda_selftest_wait_timeout(void* stream) {
     if (int rc = check_device()) return rc;
-    wait_timeout_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(1000000ull);
+    wait_timeout_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(2000000u);
     return cuda_ok(cudaGetLastError()) ? MODA_OK : MODA_ERR_CUDA;
 }
 

@@ -239,6 +239,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         const size_t row_idx = (size_t(b) * p.H + h) * p.T + q0 + r;
         const float neg_lse2 = valid ? -p.LSE[row_idx] * kLog2e : -INFINITY;   // invalid rows get P = 0
         const float delta = valid ? p.delta[row_idx] : 0.f;
+#pragma unroll 1
         for (int j = 0; j < n_kv; ++j) {
             const int buf = j & 1;
             mbar_wait(bar(kDqBarSFull + buf), (j >> 1) & 1, abort_flag, 50);
@@ -306,7 +307,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
 #pragma unroll
             for (int s = 0; s < NSUB; ++s) tma_store_4d(&mapdQ, sbase + L::kQ + s * L::kSubBytes, s * 64, h, q0, b);
             tma_store_commit();
-            tma_store_wait_all();
+            tma_store_wait_read();
         }
     } else if (warp < 12) {
         // =========================== depth backward (row-local) ===========================
@@ -388,6 +389,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     }
                 }
                 // R_i = exp(u_i - LSE): the forward's LSE already covers sequence and depth keys.
+#pragma unroll 1
                 for (int ii = 0; ii < gl; ++ii)
                     sU[ii * kTileRows + r] = fast_exp2(fmaf(sU[ii * kTileRows + r], p.scale_log2, neg_lse2));
 
@@ -420,9 +422,11 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     }
                 }
                 // dU_i = R_i (<dO, vd_i> - D)
+#pragma unroll 1
                 for (int ii = 0; ii < gl; ++ii)
                     sDr[ii * kTileRows + r] = sU[ii * kTileRows + r] * (sDr[ii * kTileRows + r] - delta);
                 if (!store_grads) {
+#pragma unroll 1
                     for (int ii = 0; ii < gl; ++ii) {
                         float* dst = rt_row + size_t(g0 + ii) * 2 * (kTileRows * p.G);
                         dst[0] = sU[ii * kTileRows + r];
@@ -509,6 +513,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     tma_load_4d(sbase + L::kQ + s * L::kSubBytes, &mapQ, bar(kDqBarQ), s * 64, h, q0, b);
                     tma_load_4d(sbase + L::kdO + s * L::kSubBytes, &mapdO, bar(kDqBarQ), s * 64, h, q0, b);
                 }
+#pragma unroll 1
                 for (int j = 0; j < n_kv; ++j) {
                     const int st = j % L::kStages;
                     if (j >= L::kStages)
@@ -537,11 +542,14 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 // fetch and the values are not needed again (evict_first)
                 const uint64_t keep = l2_policy_evict_last();
                 int unit = 0;
+#pragma unroll 1
                 for (int g0 = 0; g0 < p.l; g0 += kDepthGroup) {
                     const int gl = min(kDepthGroup, p.l - g0);
                     for (int pass = 0; pass < 3; ++pass) {
                         const int kv = (pass == 1) ? 1 : 0;
+#pragma unroll 1
                         for (int half = 0; half < NSUB; ++half)
+#pragma unroll 1
                             for (int ii = 0; ii < gl; ++ii, ++unit) {
                                 const int st = unit % L::kRingStages;
                                 if (unit >= L::kRingStages)
@@ -569,6 +577,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 for (int kk = 0; kk < D / 16; ++kk) da[kk] = desc_kmajor_sw128(a_tile + (kk >> 2) * L::kSubBytes, kk & 3);
                 const uint64_t db0 = desc_kmajor_sw128(sbase + L::kKV + (is_s ? 0 : L::kHalfTileBytes), 0);
                 mbar_wait(bar(kDqBarQ), 0, abort_flag, 81);
+#pragma unroll 1
                 for (int j = 0; j < n_kv; ++j) {
                     const int st = j % L::kStages, buf = j & 1;
                     if (j >= 2) {
@@ -594,6 +603,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             {   // whole warp: operands are warp-uniform, one elected lane issues
                 constexpr uint32_t idesc_dq = make_idesc_bf16(128, D, false, true);
                 const uint64_t db0 = desc_mnmajor_sw128(sbase + L::kKV, 0, L::kHalfSubBytes);
+#pragma unroll 1
                 for (int j = 0; j < n_kv; ++j) {
                     const int st = j % L::kStages, buf = j & 1;
                     mbar_wait(bar(kDqBarPFull + buf), (j >> 1) & 1, abort_flag, 82);
@@ -614,6 +624,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0 && tid == 256) {
+        report_abort(abort_flag);
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) {}
     }
@@ -850,6 +861,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
         const int hc = warp >> 2;                            // which 32 query columns of every iteration
         const int r = tid & 127;                             // key row inside the tile = TMEM lane
         const uint32_t lane_addr = uint32_t((warp & 3) * 32) << 16;
+#pragma unroll 1
         for (int it = 0; it < n_it; ++it) {
             const int st = it % L::kStages, buf = it & 1;
             const int qoff = (i_first + it % n_per) * kKeyTile - k0;  // query of column c sees key row r iff qoff + c >= r
@@ -920,7 +932,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
                 tma_store_4d(&mapdV, sbase + L::kV + s * L::kSubBytes, s * 64, h, k0, b);
             }
             tma_store_commit();
-            tma_store_wait_all();
+            tma_store_wait_read();
         }
     } else if (warp < 12) {
       setmaxnreg_dec<64>();
@@ -938,6 +950,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
                 tma_load_4d(sbase + L::kV + s * L::kSubBytes, &mapV, bar(kDkvBarKV), s * 64, h, k0, b);
             }
         }
+#pragma unroll 1
         for (int it = 0; it < n_it; ++it) {
             const int st = it % L::kStages;
             const int hq = h * p.G + it / n_per;
@@ -981,6 +994,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
             for (int kk = 0; kk < D / 16; ++kk) da[kk] = desc_kmajor_sw128(a_tile + (kk >> 2) * L::kSubBytes, kk & 3);
             const uint64_t db0 = desc_kmajor_sw128(sbase + L::kQdO + (is_s ? 0 : L::kHalfTileBytes), 0);
             mbar_wait(bar(kDkvBarKV), 0, abort_flag, 111);
+#pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
                 const int st = it % L::kStages, buf = it & 1;
                 mbar_wait(bar(kDkvBarQFull + st), (it / L::kStages) & 1, abort_flag, 110);
@@ -1000,6 +1014,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
         {   // whole warp: operands are warp-uniform, one elected lane issues
             constexpr uint32_t idesc_acc = make_idesc_bf16(128, D, false, true);
             const uint64_t db0 = desc_mnmajor_sw128(sbase + L::kQdO + L::kHalfTileBytes, 0, L::kHalfSubBytes);
+#pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
                 const int st = it % L::kStages, buf = it & 1;
                 mbar_wait(bar(kDkvBarPFull + buf), (it >> 1) & 1, abort_flag, 112);
@@ -1022,6 +1037,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
         {   // whole warp: operands are warp-uniform, one elected lane issues
             constexpr uint32_t idesc_acc = make_idesc_bf16(128, D, false, true);
             const uint64_t db0 = desc_mnmajor_sw128(sbase + L::kQdO, 0, L::kHalfSubBytes);
+#pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
                 const int st = it % L::kStages, buf = it & 1;
                 mbar_wait(bar(kDkvBarPFull + buf), (it >> 1) & 1, abort_flag, 114);
@@ -1042,6 +1058,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0 && tid == 128) {
+        report_abort(abort_flag);
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) {}
     }

@@ -248,6 +248,7 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     float next_lse, next_delta;
     row_terms(0, next_lse, next_delta);
     int st = 0, phase = 0;
+#pragma unroll 1
     for (int u = 0; u < my_units; ++u) {
         const int lt = (cta + u * row_ctas) * TPU + hf;
         const bool have = TPU == 1 || lt < tiles;      // the last unit of an odd number of tiles has one tile
@@ -256,6 +257,7 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         uint4* gK = reinterpret_cast<uint4*>(p.d_depth_kv) + (size_t(lt) * 2 * CH + part * 4) * kTileRows + r;
         uint4 q4[4], g4[4];
         float acc[32];
+#pragma unroll 1
         for (int i = -1; i < p.l; ++i) {
             const uint32_t full = sbase + R::kBars + 8 * st, empty = sbase + R::kBars + 8 * (R::kStages + st);
             const uint8_t* stage = smem + st * R::kStageBytes;
@@ -393,6 +395,7 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     }
     __syncthreads();
     if (*abort_flag != 0) {                            // copies still in flight land before the CTA gives its memory up
+        report_abort(abort_flag);
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) {}
     }
@@ -624,9 +627,8 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         // this thread's row of dS^T: sub-tile of its 64-column half, 128-byte rows, its first 16-byte chunk
         uint8_t* ds_row = smem + L::kdS + ((hc * COLS) >> 6) * L::kSubBytes + r * 128;
         const int ds_chunk0 = ((hc * COLS) & 63) >> 3;
-        for (int it = 0; it < n_it; ++it) {
-            const int st = it % L::kStages;
-            const bool diag = (it % n_per) == 0;             // the query tile is the key tile itself: causal mask
+#pragma unroll 1
+        for (int it = 0, qi = kt; it < n_it; ++it, qi = (qi + 1 < nk) ? qi + 1 : kt) {
             uint32_t pk[COLS / 2];                           // P_i^T of this thread: COLS values, bf16 pairs
             // ---- P_i^T ----
             const int xb = it % XB;
@@ -647,15 +649,16 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                     float e1 = fast_exp2(__uint_as_float(sv[4 * i4 + 1]) * p.scale_log2);
                     float e2 = fast_exp2(__uint_as_float(sv[4 * i4 + 2]) * p.scale_log2);
                     float e3 = fast_exp2(__uint_as_float(sv[4 * i4 + 3]) * p.scale_log2);
-                    if (diag) {                               // query column c sees key row r iff c >= r
-                        const int c = hc * COLS + 4 * i4;
-                        if (c + 0 < r) e0 = 0.f;
-                        if (c + 1 < r) e1 = 0.f;
-                        if (c + 2 < r) e2 = 0.f;
-                        if (c + 3 < r) e3 = 0.f;
-                    }
                     pk[2 * i4] = pack_bf16x2(e0, e1);
                     pk[2 * i4 + 1] = pack_bf16x2(e2, e3);
+                }
+            }
+            if (qi == kt) {                                  // the query tile is the key tile itself: column c sees key row r iff c >= r
+                const int first = r - hc * COLS;             // (masked here and not in the loop above: it stays off the path of every other tile)
+#pragma unroll
+                for (int j = 0; j < COLS / 2; ++j) {
+                    if (2 * j < first) pk[j] &= 0xffff0000u;
+                    if (2 * j + 1 < first) pk[j] &= 0x0000ffffu;
                 }
             }
             // P^T (bf16, two per column) overlays the first half of the columns this thread has read
@@ -728,7 +731,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 tma_store_4d(&mapdV, sbase + L::kdO + s * L::kSubBytes, s * 64, h, k0, b);
             }
             tma_store_commit();
-            tma_store_wait_all();
+            tma_store_wait_read();
         }
         }
     } else if (warp < W_LOAD) {
@@ -741,10 +744,10 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         const int r = tid & 127;                             // query row inside the tile = TMEM lane
         const uint32_t tY = tmem + (uint32_t((warp & 3) * 32) << 16) + kColY;
         float4* stg = reinterpret_cast<float4*>(smem + L::kStg) + r;          // [feature / 4 (16)][row 128] float4
-        for (int it = 0; it < n_it; ++it) {
-            const int hq = h * p.G + it / n_per;
-            const int qi = kt + it % n_per;
-            float* dst = p.dq_acc + ((size_t(b) * p.H + hq) * nk + qi) * (size_t(kTileRows) * D);
+        float* dst = p.dq_acc + ((size_t(b) * p.H + h * p.G) * nk + kt) * (size_t(kTileRows) * D);
+        int slot = 0;
+#pragma unroll 1
+        for (int it = 0, qi = kt; it < n_it; ++it) {
             mbar_wait(bar(kFBardQFull), it & 1, abort_flag, 120);
             tc_fence_after_sync();
             uint32_t o[D];
@@ -758,7 +761,6 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             // all but one of the ring's reductions stay in flight and L2, not this loop, sets the pace.
 #pragma unroll
             for (int ch = 0; ch < D / 16; ++ch) {
-                const int slot = (it * (D / 16) + ch) % L::kStgSlots;      // the ring runs on across iterations
                 if (tid == NROW) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(L::kStgSlots - 1) : "memory");
                 asm volatile("bar.sync 2, 128;" ::: "memory");
 #pragma unroll
@@ -772,9 +774,15 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                                  ::"l"(dst + ch * (16 * kTileRows)), "r"(sbase + L::kStg + slot * (16 * kTileRows * 4)), "r"(16 * kTileRows * 4) : "memory");
                     tma_store_commit();
                 }
+                slot = (slot + 1 == L::kStgSlots) ? 0 : slot + 1;          // the ring runs on across iterations
+            }
+            dst += kTileRows * D;
+            if (++qi == nk) {                                // the next query head of the group
+                qi = kt;
+                dst += size_t(kt) * (kTileRows * D);
             }
         }
-        if (tid == NROW) tma_store_wait_all();               // every addition has been performed before the CTA retires
+        if (tid == NROW) tma_store_wait_read();              // the staging chunks have been read
     } else {
       setmaxnreg_dec<kRegsOther>();
       if (warp == W_LOAD) {
@@ -792,11 +800,11 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             }
         }
         const float inv_scale = 1.f / p.scale;
+        int hq = h * p.G, qrow0 = k0;
+#pragma unroll 1
         for (int it = 0; it < n_it; ++it) {
             const int st = it % L::kStages;
-            const int hq = h * p.G + it / n_per;
             const size_t row_base = (size_t(b) * p.H + hq) * p.T;
-            const int qrow0 = (kt + it % n_per) * kTileRows;
             // lane handles query columns 4 lane .. 4 lane + 3: for each, -LSE / scale and -D_t as three bf16 parts
             // (hi + mid + lo = the fp32 value); queries past T get a large negative first term so that P = 0
             uint4 av[4];
@@ -828,6 +836,11 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             } else {
                 mbar_arrive(bar(kFBarQFull + st));
             }
+            qrow0 += kTileRows;
+            if (qrow0 >= nk * kTileRows) {                   // the next query head of the group
+                qrow0 = k0;
+                ++hq;
+            }
         }
       } else if (warp == W_S || warp == W_DP) {
         // ============ MMA issuers: S^T = K Q^T (warp 13, into X), dP^T = V dO^T (warp 14, into Y) ============
@@ -848,6 +861,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             const uint64_t db_aug0 = make_smem_desc_noswz(sbase + L::kAug, uint32_t(L::kAugChunk), 128u);
             mbar_wait(bar(kFBarKV), 0, abort_flag, 140);
             const int nst = is_s ? L::kStages : L::kdOStages;
+#pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
                 const int st = it % nst;
                 // the accumulator buffer still holds P of its previous tile (until that dV completes) / dQ_{i-1} (until
@@ -862,10 +876,12 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 if (!is_s) mbar_wait(bar(kFBarQFull + qst), (it / L::kStages) & 1, abort_flag, 147);
                 tc_fence_after_sync();
                 const uint64_t db = db0 + uint64_t((st * L::kTileBytes) >> 4);
+#pragma unroll 1
+                for (int c = 0; c < NSUB; ++c) {
+                    const uint64_t ca = da0 + uint64_t(c * (L::kSubBytes >> 4)), cb = db + uint64_t(c * (L::kSubBytes >> 4));
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk)
-                    umma_ss(tmem + col, da0 + uint64_t(((kk >> 2) * L::kSubBytes + (kk & 3) * 32) >> 4),
-                            db + uint64_t(((kk >> 2) * L::kSubBytes + (kk & 3) * 32) >> 4), idesc_s, kk > 0);
+                    for (int kk = 0; kk < 4; ++kk) umma_ss(tmem + col, ca + uint64_t(kk * 2), cb + uint64_t(kk * 2), idesc_s, (c > 0 || kk > 0) ? 1u : 0u);
+                }
                 umma_ss(tmem + col, da_aug, db_aug0 + uint64_t((qst * L::kAugChunk) >> 4), idesc_s, 1u);
                 umma_commit(bar(is_s ? kFBarSFull + xb : kFBardPFull));
                 if (!is_s) umma_commit(bar(kFBardOEmpty + st));
@@ -887,12 +903,13 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             const uint64_t dqb0 = desc_mnmajor_sw128(sbase + L::kK, 0, L::kSubBytes);
             const uint64_t dka0 = desc_kmajor_sw128(sbase + L::kdS, 0);
             const uint64_t dkb0 = desc_mnmajor_sw128(sbase + L::kQ, 0, L::kSubBytes);
+#pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
                 const int st = it % L::kStages, dst = it % L::kdOStages, xb = it % XB;
                 mbar_wait2(bar(kFBarPFull + xb), (it / XB) & 1, bar(kFBardOFull + dst), (it / L::kdOStages) & 1, abort_flag, 144, 145);
                 tc_fence_after_sync();
                 const uint64_t dvb = dvb0 + uint64_t((dst * L::kTileBytes) >> 4);
-#pragma unroll
+#pragma unroll 4
                 for (int kk = 0; kk < kTileRows / 16; ++kk)  // 16 queries per k-step: 8 columns, in the block of the row warpgroup that owns them
                     umma_ts(tmem + kColdV, tmem + kColX + xb * 128 + (kk / (COLS / 16)) * COLS + (kk % (COLS / 16)) * 8, dvb + uint64_t(kk * 128),
                             idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
@@ -900,12 +917,12 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 umma_commit(bar(kFBardOEmpty + dst));
                 mbar_wait(bar(kFBardSFull), it & 1, abort_flag, 146);
                 tc_fence_after_sync();
-#pragma unroll
+#pragma unroll 4
                 for (int kk = 0; kk < kTileRows / 16; ++kk)
                     umma_ss(tmem + kColY, dqa0 + uint64_t(kk * 128), dqb0 + uint64_t(kk * 128), idesc_dq, kk > 0);
                 umma_commit(bar(kFBardQFull));
                 const uint64_t dkb = dkb0 + uint64_t((st * L::kTileBytes) >> 4);
-#pragma unroll
+#pragma unroll 4
                 for (int kk = 0; kk < kTileRows / 16; ++kk)
                     umma_ss(tmem + kColdK, dka0 + uint64_t(((kk >> 2) * L::kSubBytes + (kk & 3) * 32) >> 4), dkb + uint64_t(kk * 128),
                             idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
@@ -920,6 +937,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0 && tid == 256) {
+        report_abort(abort_flag);
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) {}
     }

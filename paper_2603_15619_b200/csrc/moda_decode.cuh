@@ -437,6 +437,7 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
 
     __syncthreads();
     if (*abort_flag != 0 && threadIdx.x == kDecodeConsumerThreads) {
+        report_abort(abort_flag);
         // a wait gave up: the copies requested last may still be in flight; let them land (bounded wait on
         // the latest use of each slot) before the CTA's shared memory is released
         for (int i = max(0, n_issued - L::kStages); i < n_issued; ++i)

@@ -258,10 +258,12 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         const int r = tid;                               // query row inside the tile = TMEM lane
         const uint32_t lane_addr = uint32_t(warp * 32) << 16;
         int jbase = 0;                                   // key tiles of the CTA's earlier query tiles: the rings run on
+#pragma unroll 1
         for (int t = 0; t < n_tiles; ++t) {
         const int qt = tile_qt(t), q0 = qt * kTileRows, n_kv = tile_nkv(t);
         float m_ref = -INFINITY;                         // reference maximum (log2 domain) the stored P, O use
         float l_sum = 0.f;
+#pragma unroll 1
         for (int j = 0; j < n_kv; ++j) {
             const int jj = jbase + j;
             const int buf = jj & 1;
@@ -394,7 +396,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             for (int s = 0; s < NSUB; ++s)
                 tma_store_4d(&mapO, sbase + L::kQ + s * L::kSubBytes, s * 64, h, q0, b);
             tma_store_commit();
-            tma_store_wait_all();
+            tma_store_wait_read();
         }
         // The tile is done: the Q buffer (output staging), O and the depth partial in tensor memory may be reused for the
         // CTA's next tile.
@@ -426,6 +428,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             // The slots are handled in groups of kFwdDepthGroup (the score scratch holds one group): an
             // online softmax over the groups, with the partial output o_d rescaled in TMEM when a later
             // group raises the maximum.  Up to 32 slots are one group.
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t) {
             const int qt = tile_qt(t), q0 = qt * kTileRows;
             // this thread's query row (zeros past T, as the TMA-loaded tile has them)
@@ -486,9 +489,11 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                         }
                     }
                     float m_new = m_d;
+#pragma unroll 1
                     for (int i = 0; i < gl; ++i) m_new = fmaxf(m_new, sU[i * kTileRows + r] * p.scale_log2);
                     const float f = fast_exp2(m_d - m_new);       // first group: exp2(-inf) = 0
                     l_d *= f;
+#pragma unroll 1
                     for (int i = 0; i < gl; ++i) {
                         const float w = fast_exp2(fmaf(sU[i * kTileRows + r], p.scale_log2, -m_new));
                         sU[i * kTileRows + r] = w;
@@ -568,9 +573,11 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                 }
                 // ---- partial softmax over the depth scores seen so far ----
                 float m_new = m_d;
+#pragma unroll 1
                 for (int i = 0; i < gl; ++i) m_new = fmaxf(m_new, sU[i * kTileRows + r] * p.scale_log2);
                 const float f = fast_exp2(m_d - m_new);       // first group: exp2(-inf) = 0
                 l_d *= f;
+#pragma unroll 1
                 for (int i = 0; i < gl; ++i) {
                     const float w = fast_exp2(fmaf(sU[i * kTileRows + r], p.scale_log2, -m_new));
                     sU[i * kTileRows + r] = w;
@@ -628,6 +635,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         }
         if (!FP8 && p.append_slot != nullptr && h == hk * p.G) {
             // the write step: every read of the depth cache by this CTA is complete here, so the slot may be one that was read
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t)
                 append_rows_from_global<D>(p.append_slot, p.K, p.V, b, hk, Hk, p.T, nq, tile_qt(t), tid - 128);
         }
@@ -640,6 +648,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             tma_prefetch_desc(&mapK);
             tma_prefetch_desc(&mapV);
             int jbase = 0;
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t) {
                 const int q0 = tile_qt(t) * kTileRows, n_kv = tile_nkv(t);
                 // the Q buffer doubles as the output staging of the previous tile
@@ -648,6 +657,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 #pragma unroll
                 for (int s = 0; s < NSUB; ++s)
                     tma_load_4d(sbase + L::kQ + s * L::kSubBytes, &mapQ, bar(kBarQ), s * 64, h, q0, b);
+#pragma unroll 1
                 for (int j = 0; j < n_kv; ++j) {
                     const int jj = jbase + j;
                     const int st = jj & 1, kst = jj % KST;
@@ -679,9 +689,11 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             for (int kk = 0; kk < D / 16; ++kk) dq[kk] = desc_kmajor_sw128(sbase + L::kQ + (kk >> 2) * L::kSubBytes, kk & 3);
             const uint64_t dk0 = desc_kmajor_sw128(sbase + L::kK, 0);
             int jbase = 0;
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t) {
             const int n_kv = tile_nkv(t);
             mbar_wait(bar(kBarQ), t & 1, abort_flag, 41);
+#pragma unroll 1
             for (int j = 0; j < n_kv; ++j) {
                 const int jj = jbase + j;
                 const int st = jj & 1, kst = jj % KST;
@@ -711,8 +723,10 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             constexpr uint32_t idesc_o = make_idesc_bf16(128, D, false, true);
             const uint64_t dv0 = desc_mnmajor_sw128(sbase + L::kV, 0, L::kSubBytes);
             int jbase = 0;
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t) {
             const int n_kv = tile_nkv(t);
+#pragma unroll 1
             for (int j = 0; j < n_kv; ++j) {
                 const int jj = jbase + j;
                 const int st = jj & 1;
@@ -748,11 +762,15 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             const size_t slot_bytes = cache8_slot_bytes(p.B, p.T, Hk, D);
             const size_t blk_bytes = cache8_block_bytes(D);
             int unit = 0;
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t) {
             const uint8_t* blk = reinterpret_cast<const uint8_t*>(p.depth_kv) + (((size_t(b) * Hk + hk) * nq + tile_qt(t)) * 2) * blk_bytes;
+#pragma unroll 1
             for (int g0 = 0; g0 < p.l; g0 += kFwdDepthGroup) {
                 const int gl = min(kFwdDepthGroup, p.l - g0);
+#pragma unroll 1
                 for (int kv = 0; kv < 2; ++kv)
+#pragma unroll 1
                     for (int i = 0; i < gl; ++i, ++unit) {
                         const int st = unit % L::kRingStages;
                         if (unit >= L::kRingStages)
@@ -768,13 +786,18 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
             const uint64_t policy = l2_policy_evict_first();          // the depth cache is read exactly once
             const size_t slot_bytes = cache_slot_elems(p.B, p.T, Hk, D) * 2;
             int unit = 0;
+#pragma unroll 1
             for (int t = 0; t < n_tiles; ++t) {
             const uint8_t* blk = reinterpret_cast<const uint8_t*>(p.depth_kv) +
                                  (((size_t(b) * Hk + hk) * nq + tile_qt(t)) * 2) * (size_t(kTileRows) * D * 2);
+#pragma unroll 1
             for (int g0 = 0; g0 < p.l; g0 += kFwdDepthGroup) {
                 const int gl = min(kFwdDepthGroup, p.l - g0);
+#pragma unroll 1
                 for (int kv = 0; kv < 2; ++kv)
+#pragma unroll 1
                     for (int half = 0; half < NSUB; ++half)
+#pragma unroll 1
                         for (int i = 0; i < gl; ++i, ++unit) {
                             const int st = unit % L::kRingStages;
                             if (unit >= L::kRingStages)
@@ -793,6 +816,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0 && tid == 256) {
+        report_abort(abort_flag);
         // Abort path only: give bulk copies still in flight a bounded time to land before the CTA's
         // shared memory is handed to another CTA.
         const uint64_t t0 = globaltimer_ns();

@@ -168,6 +168,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         const uint32_t lane_addr = uint32_t((warp & 3) * 32) << 16;
         float my_ref = -INFINITY;                        // reference maximum (log2 domain) l_part is expressed in
         float l_part = 0.f;                              // this warpgroup's share of the row sum
+#pragma unroll 1
         for (int j = wg; j < n_kv; j += 2) {
             const int buf = j % L::kStages;
             const uint32_t par = (j / L::kStages) & 1;
@@ -332,7 +333,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             for (int s = 0; s < NSUB; ++s)
                 tma_store_4d(&mapO, sbase + L::kQ + s * L::kSubBytes, s * 64, h, q0, b);
             tma_store_commit();
-            tma_store_wait_all();
+            tma_store_wait_read();
         }
     } else if (warp < 12) {
         // =========================== depth partial state ===========================
@@ -417,6 +418,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                     }
                     const float f = fast_exp2(m_d - m_new);
                     l_d *= f;
+#pragma unroll 1
                     for (int i = 0; i < gl; ++i) {
                         const float w = fast_exp2(fmaf(sU[i * kTileRows + r], p.scale_log2, -m_new));
                         sU[i * kTileRows + r] = w;
@@ -495,9 +497,11 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                 }
                 // ---- partial softmax over the depth scores seen so far ----
                 float m_new = m_d;
+#pragma unroll 1
                 for (int i = 0; i < gl; ++i) m_new = fmaxf(m_new, sU[i * kTileRows + r] * p.scale_log2);
                 const float f = fast_exp2(m_d - m_new);       // first group: exp2(-inf) = 0
                 l_d *= f;
+#pragma unroll 1
                 for (int i = 0; i < gl; ++i) {
                     const float w = fast_exp2(fmaf(sU[i * kTileRows + r], p.scale_log2, -m_new));
                     sU[i * kTileRows + r] = w;
@@ -567,6 +571,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
 #pragma unroll
             for (int s = 0; s < NSUB; ++s)
                 tma_load_4d(sbase + L::kQ + s * L::kSubBytes, &mapQ, bar(k2BarQ), s * 64, h, q0, b);
+#pragma unroll 1
             for (int j = 0; j < n_kv; ++j) {
                 const int st = j % L::kStages;
                 const uint32_t par = ((j / L::kStages) - 1) & 1;
@@ -595,6 +600,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             for (int kk = 0; kk < D / 16; ++kk) dq[kk] = desc_kmajor_sw128(sbase + L::kQ + (kk >> 2) * L::kSubBytes, kk & 3);
             const uint64_t dk0 = desc_kmajor_sw128(sbase + L::kK, 0);
             mbar_wait(bar(k2BarQ), 0, abort_flag, 41);
+#pragma unroll 1
             for (int j = 0; j < n_kv; ++j) {
                 const int st = j % L::kStages;
                 // score buffer st still holds P_{j-stages} until that tile's PV has completed
@@ -623,6 +629,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         {   // whole warp: operands are warp-uniform, one elected lane issues
             constexpr uint32_t idesc_o = make_idesc_bf16(128, D, false, true);
             const uint64_t dv0 = desc_mnmajor_sw128(sbase + L::kV, 0, L::kKeySubBytes);
+#pragma unroll 1
             for (int j = 0; j < n_kv; ++j) {
                 const int st = j % L::kStages;
                 const uint32_t par = (j / L::kStages) & 1;
@@ -655,9 +662,12 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             const size_t blk_bytes = cache8_block_bytes(D);
             const uint8_t* blk = reinterpret_cast<const uint8_t*>(p.depth_kv) + (((size_t(b) * Hk + hk) * nq + qt) * 2) * blk_bytes;
             int unit = 0;
+#pragma unroll 1
             for (int g0 = 0; g0 < p.l; g0 += kFwdDepthGroup) {
                 const int gl = min(kFwdDepthGroup, p.l - g0);
+#pragma unroll 1
                 for (int kv = 0; kv < 2; ++kv)
+#pragma unroll 1
                     for (int i = 0; i < gl; ++i, ++unit) {
                         const int st = unit % L::kRingStages;
                         if (unit >= L::kRingStages)
@@ -674,10 +684,14 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             const uint8_t* blk = reinterpret_cast<const uint8_t*>(p.depth_kv) +
                                  (((size_t(b) * Hk + hk) * nq + qt) * 2) * (size_t(kTileRows) * D * 2);
             int unit = 0;
+#pragma unroll 1
             for (int g0 = 0; g0 < p.l; g0 += kFwdDepthGroup) {
                 const int gl = min(kFwdDepthGroup, p.l - g0);
+#pragma unroll 1
                 for (int kv = 0; kv < 2; ++kv)
+#pragma unroll 1
                     for (int half = 0; half < NSUB; ++half)
+#pragma unroll 1
                         for (int i = 0; i < gl; ++i, ++unit) {
                             const int st = unit % L::kRingStages;
                             if (unit >= L::kRingStages)
@@ -695,6 +709,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0 && tid == 256) {
+        report_abort(abort_flag);
         // Abort path only: give bulk copies still in flight a bounded time to land before the CTA's
         // shared memory is handed to another CTA.
         const uint64_t t0 = globaltimer_ns();

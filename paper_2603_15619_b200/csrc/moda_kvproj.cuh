@@ -136,10 +136,12 @@ moda_kv_project_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_co
             tma_prefetch_desc(&mapX);
             tma_prefetch_desc(mapW);
             int n = 0;                                         // stages filled so far
+#pragma unroll 1
             for (int item = cl; item < n_items; item += n_clusters) {
                 const int hk0 = (item % hgroups) * NH;
                 const int t0 = (((item / hgroups) % npairs) * 2 + int(rank)) * kTileRows;   // may lie past T: zeros
                 const int b = item / (hgroups * npairs);
+#pragma unroll 1
                 for (int k = 0; k < n_k; ++k, ++n) {
                     const int st = n % L::kStages;
                     if (n >= L::kStages) mbar_wait(bar_empty(st), ((n / L::kStages) - 1) & 1, abort_flag, 163);
@@ -161,6 +163,7 @@ moda_kv_project_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_co
         if (rank == 0) {
             constexpr uint32_t idesc = make_idesc_bf16(256, 2 * NW, false, false);
             int n = 0, i = 0;
+#pragma unroll 1
             for (int item = cl; item < n_items; item += n_clusters, ++i) {
                 const int set = i & 1;
                 if (i >= 2) {
@@ -168,6 +171,7 @@ moda_kv_project_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_co
                     tc_fence_after_sync();
                 }
                 const uint32_t acc = tmem + uint32_t(set * 2 * NW);
+#pragma unroll 1
                 for (int k = 0; k < n_k; ++k, ++n) {
                     const int st = n % L::kStages;
                     mbar_wait(bar_full(st), (n / L::kStages) & 1, abort_flag, 164);
@@ -194,6 +198,7 @@ moda_kv_project_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_co
         const uint32_t lane_addr = uint32_t((warp & 3) * 32) << 16;
         constexpr int CH = D / 8;
         int i = 0;
+#pragma unroll 1
         for (int item = cl; item < n_items; item += n_clusters, ++i) {
             const int set = i & 1;
             const int hk0 = (item % hgroups) * NH;
@@ -300,6 +305,7 @@ moda_kv_project_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_co
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag != 0 && tid == 0) {
+        report_abort(abort_flag);
         const uint64_t t_start = globaltimer_ns();
         while (globaltimer_ns() - t_start < 2000000ull) {}     // abort path only: let copies in flight land
     }

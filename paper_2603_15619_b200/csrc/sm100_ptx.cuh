@@ -104,11 +104,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait.  `abort_flag` is a CTA-wide word in shared memory: once any waiter of the
-// CTA has timed out, every later wait returns at once so that the CTA can reach its
-// tear-down (TMEM release) instead of spinning.  Limit: ~1 s of wall time.
-__device__ __forceinline__ void report_wait_timeout(int site) {
-    const int code = kStatusWaitTimeout | (site << 8);
+// Bounded wait.  `abort_flag` is a CTA-wide word in shared memory: a wait that runs out writes its site's code there, and
+// from then on every wait of the CTA gives up after a few probes so that the CTA can reach its tear-down (TMEM release)
+// instead of spinning; there report_abort passes the code on.  Limit: 2e9 cycles, about 1 s (the cycle counter: a read of
+// the global timer takes about a microsecond, which every wait that has to wait would pay).
+//
+// What a wait site costs in code matters: a kernel here has ten to thirty of them in its loops.  With the clock in 64
+// bits, a spin counter and the report in line (some 45 instructions a site), and the loops around them unrolled by the
+// compiler, the kernels were 63 to 94 KB, the code that all warp roles run per iteration no longer fitted the
+// instruction cache of an SM, and warps stood for a fifth of their time without an instruction to issue
+// (smsp__average_warps_issue_stalled_no_instruction of the fused backward: 2.9 of 13.9).  So: one asm block whose usual
+// path is a few instructions, loops over tiles marked `unroll 1`, and code that few iterations need kept off their path.
+__device__ __forceinline__ void report_abort(volatile int* abort_flag) {
+    const int code = *abort_flag;
     if (atomicCAS(&g_moda_status, 0, code) == 0) {
         int* host = g_moda_status_host;
         if (host != nullptr) {
@@ -118,20 +126,36 @@ __device__ __forceinline__ void report_wait_timeout(int site) {
     }
 }
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int site,
-                                          uint64_t limit_ns = 1000000000ull) {
-    if (mbar_try_wait(bar, parity)) return;
-    const uint64_t t0 = globaltimer_ns();
-    uint32_t spins = 0;
-    while (!mbar_try_wait(bar, parity)) {
-        if ((++spins & 0xffu) == 0) {
-            if (*abort_flag != 0) return;
-            if (globaltimer_ns() - t0 > limit_ns) {
-                *abort_flag = 1;
-                report_wait_timeout(site);
-                return;
-            }
-        }
-    }
+                                          uint32_t limit_cycles = 2000000000u) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        ".reg .b32 t0, t;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n"
+        "@p bra DONE_%=;\n"
+        "mov.u32 t, 32;\n"
+        "PROBE_%=:\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n"
+        "@p bra DONE_%=;\n"
+        "sub.u32 t, t, 1;\n"
+        "setp.ne.u32 p, t, 0;\n"
+        "@p bra PROBE_%=;\n"
+        "mov.u32 t0, %%clock;\n"
+        "LONG_%=:\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n"
+        "@p bra DONE_%=;\n"
+        "ld.volatile.shared.b32 t, [%2];\n"
+        "setp.ne.b32 p, t, 0;\n"
+        "@p bra DONE_%=;\n"
+        "mov.u32 t, %%clock;\n"
+        "sub.u32 t, t, t0;\n"
+        "setp.lt.u32 p, t, %4;\n"
+        "@p bra LONG_%=;\n"
+        "st.volatile.shared.b32 [%2], %3;\n"
+        "DONE_%=:\n"
+        "}\n"
+        ::"r"(bar), "r"(parity), "r"(smem_u32(const_cast<const int*>(abort_flag))), "r"(kStatusWaitTimeout | (site << 8)), "r"(limit_cycles)
+        : "memory");
 }
 
 // Bounded wait on two barriers.  Both probes are issued before either result is used, so their
@@ -195,6 +219,11 @@ __device__ __forceinline__ void tma_store_commit() {
 }
 __device__ __forceinline__ void tma_store_wait_all() {
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+// The same up to the point where the sources have been read: what a CTA needs before it gives its shared memory up (the
+// writes belong to the grid, which ends after them).
+__device__ __forceinline__ void tma_store_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // Plain (untiled) bulk copy global -> shared; both addresses 16-byte aligned, size a multiple
