@@ -644,11 +644,15 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 tmem_wait_ld();
 #pragma unroll
                 for (int i4 = 0; i4 < COLS / 4; ++i4) {
-                    // the contraction has already subtracted LSE / scale from every score of the query's column
-                    float e0 = fast_exp2(__uint_as_float(sv[4 * i4 + 0]) * p.scale_log2);
-                    float e1 = fast_exp2(__uint_as_float(sv[4 * i4 + 1]) * p.scale_log2);
-                    float e2 = fast_exp2(__uint_as_float(sv[4 * i4 + 2]) * p.scale_log2);
-                    float e3 = fast_exp2(__uint_as_float(sv[4 * i4 + 3]) * p.scale_log2);
+                    // the contraction has already subtracted LSE / scale from every score of the query's column (packed
+                    // products, here and for dS^T: 64 instructions fewer per tile, the same bits; d = 64 1-2 % faster)
+                    float e0, e1, e2, e3;
+                    mul2_f32(__uint_as_float(sv[4 * i4 + 0]), __uint_as_float(sv[4 * i4 + 1]), p.scale_log2, p.scale_log2, e0, e1);
+                    mul2_f32(__uint_as_float(sv[4 * i4 + 2]), __uint_as_float(sv[4 * i4 + 3]), p.scale_log2, p.scale_log2, e2, e3);
+                    e0 = fast_exp2(e0);
+                    e1 = fast_exp2(e1);
+                    e2 = fast_exp2(e2);
+                    e3 = fast_exp2(e3);
                     pk[2 * i4] = pack_bf16x2(e0, e1);
                     pk[2 * i4 + 1] = pack_bf16x2(e2, e3);
                 }
@@ -680,16 +684,15 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 tmem_wait_ld();
 #pragma unroll
                 for (int g = 0; g < COLS / 8; ++g) {         // 8 query columns = one 16-byte chunk of the row
-                    const uint32_t* pp = pk + 4 * g;         // gv holds dP - D_t already (subtracted by the contraction)
-                    uint4 v;
-                    v.x = pack_bf16x2(bf16_lo_to_f32(pp[0]) * __uint_as_float(gv[8 * g + 0]),
-                                      bf16_hi_to_f32(pp[0]) * __uint_as_float(gv[8 * g + 1]));
-                    v.y = pack_bf16x2(bf16_lo_to_f32(pp[1]) * __uint_as_float(gv[8 * g + 2]),
-                                      bf16_hi_to_f32(pp[1]) * __uint_as_float(gv[8 * g + 3]));
-                    v.z = pack_bf16x2(bf16_lo_to_f32(pp[2]) * __uint_as_float(gv[8 * g + 4]),
-                                      bf16_hi_to_f32(pp[2]) * __uint_as_float(gv[8 * g + 5]));
-                    v.w = pack_bf16x2(bf16_lo_to_f32(pp[3]) * __uint_as_float(gv[8 * g + 6]),
-                                      bf16_hi_to_f32(pp[3]) * __uint_as_float(gv[8 * g + 7]));
+                    uint32_t w[4];                           // gv holds dP - D_t already (subtracted by the contraction)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        float x0, x1;
+                        mul2_f32(bf16_lo_to_f32(pk[4 * g + k]), bf16_hi_to_f32(pk[4 * g + k]), __uint_as_float(gv[8 * g + 2 * k]),
+                                 __uint_as_float(gv[8 * g + 2 * k + 1]), x0, x1);
+                        w[k] = pack_bf16x2(x0, x1);
+                    }
+                    const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
                     *reinterpret_cast<uint4*>(ds_row + (((ds_chunk0 + g) ^ (r & 7)) << 4)) = v;
                 }
             }

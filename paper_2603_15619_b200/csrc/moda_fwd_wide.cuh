@@ -242,17 +242,21 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             const float neg_m = -m_ref;
             // P_j (bf16, two per column) overlays the first half of S_j's columns: one 32-column block of
             // scores at a time, stored as soon as it is converted.
-            float sum0 = 0.f, sum1 = 0.f;
+            // (packed fp32 FMAs and additions for a shorter loop: forwards 1-3 % faster)
+            float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
             auto exp_block = [&](const uint32_t (&sv)[32], uint32_t col) {
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; i += 2) {
-                    const float a0 = fast_exp2(fmaf(__uint_as_float(sv[2 * i]), p.scale_log2, neg_m));
-                    const float a1 = fast_exp2(fmaf(__uint_as_float(sv[2 * i + 1]), p.scale_log2, neg_m));
-                    const float b0 = fast_exp2(fmaf(__uint_as_float(sv[2 * i + 2]), p.scale_log2, neg_m));
-                    const float b1 = fast_exp2(fmaf(__uint_as_float(sv[2 * i + 3]), p.scale_log2, neg_m));
-                    sum0 += a0 + a1;
-                    sum1 += b0 + b1;
+                    float a0, a1, b0, b1;
+                    fma2_scale(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1]), p.scale_log2, neg_m, a0, a1);
+                    fma2_scale(__uint_as_float(sv[2 * i + 2]), __uint_as_float(sv[2 * i + 3]), p.scale_log2, neg_m, b0, b1);
+                    a0 = fast_exp2(a0);
+                    a1 = fast_exp2(a1);
+                    b0 = fast_exp2(b0);
+                    b1 = fast_exp2(b1);
+                    add2_f32(a0, a1, sum0, sum1);
+                    add2_f32(b0, b1, sum2, sum3);
                     pk[i] = pack_bf16x2(a0, a1);
                     pk[i + 1] = pack_bf16x2(b0, b1);
                 }
@@ -260,7 +264,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             };
 #pragma unroll
             for (int c = 0; c < NB; ++c) exp_block(sv[c], c * 16);
-            l_part += sum0 + sum1;
+            l_part += (sum0 + sum1) + (sum2 + sum3);
             tmem_wait_st();
             tc_fence_before_sync();
             mbar_arrive(bar(k2BarPFull + buf));
