@@ -108,6 +108,26 @@ __device__ __forceinline__ void decode_consumer_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kDecodeConsumerThreads) : "memory");
 }
 
+// The bounded wait of this kernel, which has two of them: as compiler-visible code, with the abort word and the time looked
+// at on every 256th probe only, and the report where the wait runs out.  mbar_wait looks at both on every probe and, being one asm block, moves the register
+// allocation of the whole kernel: d = 128, G = 1 spilled 8 bytes instead of none, G = 2 52 instead of 48.  Code size, which mbar_wait
+// is made for, is no matter here.  mbar_wait -> this form, us, graph replays in turn: B = 1, T = 8192, G = 2 10.04 -> 9.94,
+// G = 1 13.21 -> 13.03; B = 8, 8 heads, G = 1 49.18 -> 47.88; paged, B = 32, T = 4096, G = 1 91.56 -> 90.22; d = 64 the same.
+__device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int site) {
+    if (mbar_try_wait(bar, parity)) return;
+    const uint64_t t0 = globaltimer_ns();
+    uint32_t spins = 0;
+    while (!mbar_try_wait(bar, parity)) {
+        if ((++spins & 0xffu) != 0) continue;
+        if (*abort_flag != 0) return;
+        if (globaltimer_ns() - t0 > 1000000000ull) {
+            *abort_flag = kStatusWaitTimeout | (site << 8);
+            report_abort(abort_flag);
+            return;
+        }
+    }
+}
+
 template <int D, int G>
 __global__ void __launch_bounds__(kDecodeTmaThreads, 1)
 decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
@@ -249,7 +269,7 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
                     const int t0 = w.k_begin + i * kDecodeStageKeys;
                     const int page = page_next;
                     if (table && i + 1 < n_stage) page_next = table[(t0 + kDecodeStageKeys) / p.page_size];
-                    if (gi >= L::kStages) mbar_wait(empty_bar(st), ((gi / L::kStages) - 1) & 1, abort_flag, 70);
+                    if (gi >= L::kStages) decode_wait(empty_bar(st), ((gi / L::kStages) - 1) & 1, abort_flag, 70);
                     if (*abort_flag != 0) break;
                     const uint32_t dst = smem_u32(smem + L::kRing + st * L::kStageBytes);
                     mbar_arrive_expect_tx(full_bar(st), L::kStageBytes);
@@ -321,7 +341,7 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
             for (int i = first; i < n_stage; i += kDecodePairs) {
                 const int gi = gi0 + i;
                 const int st = gi % L::kStages;
-                mbar_wait(full_bar(st), (gi / L::kStages) & 1, abort_flag, 71);
+                decode_wait(full_bar(st), (gi / L::kStages) & 1, abort_flag, 71);
                 // After a wait has given up every later wait returns at once; the loops still run to their
                 // ends (without touching the data) so that all warps meet at the barriers below.
                 const bool live = __shfl_sync(0xffffffffu, *abort_flag, 0) == 0;
@@ -437,7 +457,6 @@ decode_split_tma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_c
 
     __syncthreads();
     if (*abort_flag != 0 && threadIdx.x == kDecodeConsumerThreads) {
-        report_abort(abort_flag);
         // a wait gave up: the copies requested last may still be in flight; let them land (bounded wait on
         // the latest use of each slot) before the CTA's shared memory is released
         for (int i = max(0, n_issued - L::kStages); i < n_issued; ++i)
