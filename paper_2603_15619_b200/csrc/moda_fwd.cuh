@@ -250,11 +250,16 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     tc_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
 
-    // Register budget: the launch gives every warp 168 registers (3 warps per scheduler);
-    // the producer warpgroup hands most of its share to the two compute warpgroups.
+    // Register budget: the launch gives every warp 168 registers (3 warps per scheduler), and setmaxnreg.inc takes what the
+    // producer warpgroup gives up.  208 + 208 + 88: the issuing and loading warps need more than 72 (with 216 + 216 + 72 they
+    // reloaded descriptors from local memory in their loops, 16 bytes of spills), the compute warps no more than 208.
+    // 72 -> 88, us: T = 8192, l = 0 587 -> 571, with l = 16 812 -> 774, T = 32768, l = 8 4583 -> 4465, T = 65536, l = 24 18503 -> 17949,
+    // prefill of 2000 over 15000 1075 -> 1039.
+    constexpr int kRegsCompute = 208, kRegsProducer = 88;
+    static_assert(2 * kRegsCompute + kRegsProducer <= 3 * 168, "register shares of the three warpgroups");
     if (warp < 4) {
         // =========================== softmax + epilogue ===========================
-        setmaxnreg_inc<216>();
+        setmaxnreg_inc<kRegsCompute>();
         const int r = tid;                               // query row inside the tile = TMEM lane
         const uint32_t lane_addr = uint32_t(warp * 32) << 16;
         int jbase = 0;                                   // key tiles of the CTA's earlier query tiles: the rings run on
@@ -419,7 +424,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         }
     } else if (warp < 8) {
         // =========================== depth partial state ===========================
-        setmaxnreg_inc<216>();
+        setmaxnreg_inc<kRegsCompute>();
         if (p.l > 0) {
             const int r = tid - 128;
             const uint32_t lane_addr = uint32_t((warp & 3) * 32) << 16;
@@ -652,7 +657,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                 append_rows_from_global<D>(p.append_slot, p.K, p.V, b, hk, Hk, p.T, nq, tile_qt(t), tid - 128);
         }
     } else {
-      setmaxnreg_dec<72>();   // one instruction for the whole producer warpgroup (warps 8-11)
+      setmaxnreg_dec<kRegsProducer>();   // one instruction for the whole producer warpgroup (warps 8-11)
       if (warp == 8) {
         // =========================== TMA producer ===========================
         if (lane == 0) {

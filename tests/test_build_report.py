@@ -13,6 +13,9 @@ REPORT = os.path.join(build.PKG, "build_ptxas.log")
 LIMITS = {
     "decode_split_tma_kernel<128, 1>": (0, 0),
     "decode_split_tma_kernel<128, 2>": (48, 60),
+    "moda_fwd_kernel<128, 2, false>": (0, 0),
+    "moda_fwd_kernel<128, 2, true>": (0, 0),
+    "moda_fwd_kernel<128, 1, false>": (0, 0),
 }
 
 
