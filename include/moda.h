@@ -77,10 +77,13 @@ int moda_last_cuda_error(void);
 
 /*
  * Reads (and optionally clears) the device status word.  Every wait inside the kernels
- * is bounded; a wait that runs out stores (site << 8) | 1 here and the kernel tears
- * down normally, leaving its outputs undefined.  0 means no kernel has reported a
- * problem.  This call synchronises the device.  Returns the status word (>= 0) or a
- * negative MODA_ERR_CUDA.
+ * is bounded (about 1 s); when one runs out, the CTA keeps (site << 8) | 1 of the first
+ * that did, walks what is left of its work with every further wait giving up at once,
+ * stores the code here when it comes to its end (the decode kernel: right away), and the
+ * kernel ends normally, leaving its outputs undefined.  Of several CTAs the first to store
+ * is kept.  0 means no kernel has reported a problem.  This call synchronises the device,
+ * so it sees the code of every kernel launched before.  Returns the status word (>= 0) or
+ * a negative MODA_ERR_CUDA.
  *
  * The same code is also written to four bytes of pinned host memory that the library maps
  * into the device on its first launching call on that device (the only memory the library

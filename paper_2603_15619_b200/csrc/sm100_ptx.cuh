@@ -104,8 +104,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait.  `abort_flag` is a CTA-wide word in shared memory: a wait that runs out writes its site's code there, and
-// from then on every wait of the CTA gives up after two probes so that the CTA can reach its tear-down (TMEM release)
+// Bounded wait.  `abort_flag` is a CTA-wide word in shared memory: the first wait that runs out leaves its site's code there,
+// and from then on every wait of the CTA gives up after two probes so that the CTA can reach its tear-down (TMEM release)
 // instead of spinning; there report_abort passes the code on.  Limit: 2e9 cycles, about 1 s (the cycle counter: a read of
 // the global timer takes about a microsecond, which every wait that has to wait would pay).
 //
@@ -145,7 +145,7 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatil
         "sub.u32 t, t, t0;\n"
         "setp.lt.u32 p, t, %4;\n"
         "@p bra LONG_%=;\n"
-        "st.volatile.shared.b32 [%2], %3;\n"
+        "atom.shared.cas.b32 t, [%2], 0, %3;\n"
         "DONE_%=:\n"
         "}\n"
         ::"r"(bar), "r"(parity), "r"(smem_u32(const_cast<const int*>(abort_flag))), "r"(kStatusWaitTimeout | (site << 8)), "r"(limit_cycles)
