@@ -34,10 +34,10 @@ __global__ void wait_timeout_selftest_kernel(uint32_t limit_cycles) {
         fence_mbar_init();
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        mbar_wait(smem_u32(&bar_word), 0, &abort_word, MODA_SELFTEST_WAIT_SITE, limit_cycles);
-        if (abort_word != 0) report_abort(&abort_word);
-    }
+    if (threadIdx.x == 0) mbar_wait(smem_u32(&bar_word), 0, &abort_word, MODA_SELFTEST_WAIT_SITE, limit_cycles);
+    __syncthreads();
+    abort_teardown(&abort_word, 0);
+    __syncthreads();
 }
 
 inline bool cuda_ok(cudaError_t e) {

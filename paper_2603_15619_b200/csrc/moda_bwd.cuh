@@ -623,11 +623,7 @@ moda_bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
 
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag != 0 && tid == 256) {
-        report_abort(abort_flag);
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 2000000ull) {}
-    }
+    abort_teardown(abort_flag, 256);
     __syncthreads();
     if (warp == 16) tmem_dealloc(tmem, kTmemCols);
 }
@@ -1057,11 +1053,7 @@ moda_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_cons
 
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag != 0 && tid == 128) {
-        report_abort(abort_flag);
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 2000000ull) {}
-    }
+    abort_teardown(abort_flag, 128);
     __syncthreads();
     if (warp == 9) tmem_dealloc(tmem, kTmemCols);
 }

@@ -394,11 +394,8 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
         }
     }
     __syncthreads();
-    if (*abort_flag != 0) {                            // copies still in flight land before the CTA gives its memory up
-        report_abort(abort_flag);
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 2000000ull) {}
-    }
+    abort_teardown(abort_flag, 0);
+    __syncthreads();
 }
 
 // =====================================================================================
@@ -939,11 +936,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag != 0 && tid == 256) {
-        report_abort(abort_flag);
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 2000000ull) {}
-    }
+    abort_teardown(abort_flag, 256);
     __syncthreads();
     if (warp == W_S) tmem_dealloc(tmem, kTmemCols);
     // what follows on the stream reads the accumulator and the depth gradients: this grid ends after the rows kernel has

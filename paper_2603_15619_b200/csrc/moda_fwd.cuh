@@ -832,13 +832,7 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag != 0 && tid == 256) {
-        report_abort(abort_flag);
-        // Abort path only: give bulk copies still in flight a bounded time to land before the CTA's
-        // shared memory is handed to another CTA.
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 2000000ull) {}
-    }
+    abort_teardown(abort_flag, 256);
     __syncthreads();
     if (warp == 9) tmem_dealloc(tmem, kTmemCols);
 }

@@ -304,11 +304,7 @@ moda_kv_project_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_co
 
     tc_fence_before_sync();
     __syncthreads();
-    if (*abort_flag != 0 && tid == 0) {
-        report_abort(abort_flag);
-        const uint64_t t_start = globaltimer_ns();
-        while (globaltimer_ns() - t_start < 2000000ull) {}     // abort path only: let copies in flight land
-    }
+    abort_teardown(abort_flag, 0);
     // neither CTA leaves (or frees tensor memory) while the other may still read its accumulator or have loads in flight
     cluster_sync_all();
     if (warp == 1) tmem_dealloc_pair(tmem, kTmemCols);

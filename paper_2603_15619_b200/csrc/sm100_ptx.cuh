@@ -106,7 +106,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 
 // Bounded wait.  `abort_flag` is a CTA-wide word in shared memory: the first wait that runs out leaves its site's code there,
 // and from then on every wait of the CTA gives up after two probes so that the CTA can reach its tear-down (TMEM release)
-// instead of spinning; there report_abort passes the code on.  Limit: 2e9 cycles, about 1 s (the cycle counter: a read of
+// instead of spinning; there abort_teardown passes the code on.  Limit: 2e9 cycles, about 1 s (the cycle counter: a read of
 // the global timer takes about a microsecond, which every wait that has to wait would pay).
 //
 // What a wait site costs in code matters: a kernel here has ten to thirty of them in its loops.  With the clock in 64
@@ -124,6 +124,19 @@ __device__ __forceinline__ void report_abort(volatile int* abort_flag) {
             *reinterpret_cast<volatile int*>(host) = code;
             __threadfence_system();
         }
+    }
+}
+// Every kernel that waits with mbar_wait calls this at its end, all threads, behind a CTA-wide barrier; another CTA-wide
+// barrier follows, so that no thread leaves before the one that is named here.  If a wait gave up, that thread reports it
+// and gives bulk copies still in flight a bounded time to land before the CTA's shared memory is handed on.  (The thread
+// index is read again: kept over the kernel's loops it cost bwd_rows_kernel a register and 1-2 % with an e4m3 cache.)
+__device__ __forceinline__ void abort_teardown(volatile int* abort_flag, uint32_t thread) {
+    uint32_t tid;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    if (*abort_flag != 0 && tid == thread) {
+        report_abort(abort_flag);
+        const uint64_t t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 2000000ull) {}
     }
 }
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int site,
