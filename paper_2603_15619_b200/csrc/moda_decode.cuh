@@ -121,8 +121,8 @@ __device__ __forceinline__ void decode_wait(uint32_t bar, uint32_t parity, volat
         if ((++spins & 0xffu) != 0) continue;
         if (*abort_flag != 0) return;
         if (globaltimer_ns() - t0 > 1000000000ull) {
-            atomicCAS(const_cast<int*>(abort_flag), 0, kStatusWaitTimeout | (site << 8));
-            report_abort(abort_flag);
+            *abort_flag = 1;
+            report_abort(kStatusWaitTimeout | (site << 8));
             return;
         }
     }

@@ -116,8 +116,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // (smsp__average_warps_issue_stalled_no_instruction of the fused backward: 2.9 of 13.9).  So: one asm block whose usual
 // path is a few instructions, loops over tiles marked `unroll 1`, and code that few iterations need kept off their path.
 // (32 probes without the clock before the bounded loop: 0-4 % slower forwards at d = 64 than this shorter form.)
-__device__ __forceinline__ void report_abort(volatile int* abort_flag) {
-    const int code = *abort_flag;
+__device__ __forceinline__ void report_abort(int code) {
     if (atomicCAS(&g_moda_status, 0, code) == 0) {
         int* host = g_moda_status_host;
         if (host != nullptr) {
@@ -134,7 +133,7 @@ __device__ __forceinline__ void abort_teardown(volatile int* abort_flag, uint32_
     uint32_t tid;
     asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
     if (*abort_flag != 0 && tid == thread) {
-        report_abort(abort_flag);
+        report_abort(*abort_flag);
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) {}
     }
