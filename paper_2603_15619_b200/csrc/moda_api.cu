@@ -406,12 +406,15 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
 // ring 1.75 us (16 SMs at it) to 2.0 us (50), e4m3 a tenth more; an iteration of the sequence part 2.7 us
 // (d = 64: 1.75 us) and 5 us (7 us) per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both
 // parts end together; a few SMs more than that cost less than a few too few, because SMs that the depth part leaves go on
-// with the sequence part, and below 16 its tail shows.  The number is even: with an odd one a CTA shares its pair of SMs
-// with a CTA of the sequence part, and the whole depth part waits for that one.
-// Whole backward, us, by SMs: T = 8192, l = 16, B = 2, d = 128: 28 2325, 32 2182, 36 2000, 40 1935, 44 2122 (taken: 40);
-// T = 4096, l = 23, B = 4: d = 128 64 1698, 72 1653, 80 1720 (72), d = 64 52 1914, 56 1797, 60 1821 (58); T = 8192, l = 16,
-// d = 64, 32 heads: 24 2521, 28 2359, 32 2410 (30).  e4m3, T = 5000, l = 23, B = 2: d = 128 62 1184, 66 1138, 72 1118 (70); d = 64
-// 50 1366, 54 1301, 58 1269, 64 1276 (56).
+// with the sequence part.  The number is even: with an odd one a CTA shares its pair of SMs with a CTA of the sequence part,
+// and the whole depth part waits for that one.
+// Whole backward, us, by SMs (of 38 shapes; rounds of one count differ by 4-8 %).  bf16:
+// T = 8192, l = 16, B = 2, d = 128: 34 2167, 36 2057, 38 1979, 40 2000, 44 1994 (taken: 40); T = 4096, l = 23, B = 4, d = 128: 66 1664,
+// 70 1602, 74 1619, 78 1634 (72); T = 32768, l = 32, d = 64: 16 14505, 18 13163, 20 13545, 24 15269 (18).  e4m3: T = 5000, l = 23, B = 2:
+// d = 128 64 1111, 68 1075, 72 1086, 76 1099 (70), d = 64 50 1256, 56 1158, 60 1205 (56); T = 8192, l = 16, d = 128: 38 1962, 42 1882,
+// 46 1965 (42); T = 32768, l = 24, d = 128: 18 11551, 20 11102, 24 11776 (20).  Within 3.4 % of the best count everywhere but in
+// two places: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347) and T = 65536, where 16 are taken and 10 would be best (l = 24,
+// d = 128: 45.3 against 43.8 ms; at T = 32768, l = 8 16 and 12 are 11.1 and 10.9).
 inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms, bool fp8) {
     const double nq = num_tiles(T);
     const double depth = double(units) * (l + 1) * (fp8 ? 1.9 : 1.7);

@@ -322,10 +322,13 @@ moda_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
                 m_ref = m_new;
             }
             const float neg_m = -m_ref;
-            // Packed fp32 FMAs and additions: the pipes take as long for them as for twice as many scalar ones, but the loop is
-            // 190 instructions shorter, and it is fetched again for every tile beside the code of eleven other warps (unrolled by
-            // two it is 20 % slower).  Scalar -> packed, us: l = 0 T = 8192 604 -> 585, T = 32768 4628 -> 4465, prefill of 2000 over 15000
-            // 1078 -> 1040.
+            // Packed fp32 FMAs and additions: the pipes take as long for them as for twice as many scalar ones, but a tile takes
+            // 128 instructions fewer (64 FMAs, 64 additions), and the loop is fetched again for every tile beside the code of
+            // eleven other warps (unrolled by two it is 20 % slower).  With shorter waits and the rolled branch above, the kernel
+            // alone, in turn, us: l = 0 T = 8192 600 -> 576, T = 32768, l = 8 4641 -> 4496, prefill of 2000 over 15000 1106 -> 1069.
+            // Eight sums, because adding neighbours first and keeping four, as the scalar code did, costs the instructions
+            // again or register moves for packed ones: T = 8192 563 -> 575 or 594.  A chain of additions is 16 long either way,
+            // and LSE is as far from 64 bits (rms 2.5e-7 to 9.6e-7 over T = 256 ... 12000, both the same to 2 %).
             float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f, sum4 = 0.f, sum5 = 0.f, sum6 = 0.f, sum7 = 0.f;
             uint32_t pk0[16], pk1[16], pk2[16], pk3[16];
 #pragma unroll

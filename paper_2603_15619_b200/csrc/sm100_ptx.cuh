@@ -112,9 +112,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // What a wait site costs in code matters: a kernel here has ten to thirty of them in its loops.  With the clock in 64
 // bits, a spin counter and the report in line (some 45 instructions a site), and the loops around them unrolled by the
 // compiler, the kernels were 63 to 94 KB, the code that all warp roles run per iteration no longer fitted the
-// instruction cache of an SM, and warps stood for a fifth of their time without an instruction to issue
-// (smsp__average_warps_issue_stalled_no_instruction of the fused backward: 2.9 of 13.9).  So: one asm block whose usual
-// path is a few instructions, loops over tiles marked `unroll 1`, and code that few iterations need kept off their path.
+// instruction cache of an SM: the fused backward missed it on every fifth request, and its warps stood for a tenth of their
+// time without an instruction to issue (smsp__average_warps_issue_stalled_no_instruction 1.28 of 12.2 per issue at T = 8192,
+// l = 0; now 0.27 of 12.4).  So: one asm block whose usual path is a few instructions, loops over tiles marked `unroll 1`,
+// and code that few iterations need kept off their path.
 // (32 probes without the clock before the bounded loop: 0-4 % slower forwards at d = 64 than this shorter form.)
 __device__ __forceinline__ void report_abort(int code) {
     if (atomicCAS(&g_moda_status, 0, code) == 0) {
