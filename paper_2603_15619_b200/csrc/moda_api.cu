@@ -403,24 +403,37 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
 }
 
 // How many SMs the depth part of a fused backward gets beside the sequence part.  Measured SM time: an entry of the row
-// ring 1.75 us (16 SMs at it) to 2.0 us (50), e4m3 a tenth more; an iteration of the sequence part 2.7 us
-// (d = 64: 1.75 us) and 5 us (7 us) per key tile around them.  With the share x = depth / (depth + sequence) of all SMs both
+// ring 1.75 us (16 SMs at it) to 2.0 us (50), e4m3 a tenth more; an iteration of the sequence part at d = 128 2.7 us
+// and 5 us per key tile around them; at d = 64 12 us per key tile and 1.33 us an iteration, rising to 1.5 us for the longest (their runs
+// last long enough for the clocks to come down, which the depth part, bound by HBM, does not feel).  With the share
+// x = depth / (depth + sequence) of all SMs both
 // parts end together; a few SMs more than that cost less than a few too few, because SMs that the depth part leaves go on
 // with the sequence part.  The number is even: with an odd one a CTA shares its pair of SMs with a CTA of the sequence part,
 // and the whole depth part waits for that one.
-// Whole backward, us, by SMs (of 38 shapes; rounds of one count differ by 4-8 %).  bf16:
-// T = 8192, l = 16, B = 2, d = 128: 34 2167, 36 2057, 38 1979, 40 2000, 44 1994 (taken: 40); T = 4096, l = 23, B = 4, d = 128: 66 1664,
-// 70 1602, 74 1619, 78 1634 (72); T = 32768, l = 32, d = 64: 16 14505, 18 13163, 20 13545, 24 15269 (18).  e4m3: T = 5000, l = 23, B = 2:
-// d = 128 64 1111, 68 1075, 72 1086, 76 1099 (70), d = 64 50 1256, 56 1158, 60 1205 (56); T = 8192, l = 16, d = 128: 38 1962, 42 1882,
-// 46 1965 (42); T = 32768, l = 24, d = 128: 18 11551, 20 11102, 24 11776 (20).  Within 3.4 % of the best count everywhere but in
-// two places: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347) and T = 65536, where 16 are taken and 10 would be best (l = 24,
-// d = 128: 45.3 against 43.8 ms; at T = 32768, l = 8 16 and 12 are 11.1 and 10.9).
+// Whole backward, us, by SMs (rounds of one count differ by 4-8 %).  d = 128, 26 shapes, bf16:
+// T = 8192, l = 16, B = 2: 34 2167, 36 2057, 38 1979, 40 2000, 44 1994 (taken: 40); T = 4096, l = 23, B = 4: 66 1664,
+// 70 1602, 74 1619, 78 1634 (72).  e4m3: T = 5000, l = 23, B = 2: 64 1111, 68 1075, 72 1086, 76 1099 (70); T = 8192, l = 16: 38 1962, 42 1882,
+// 46 1965 (42); T = 32768, l = 24: 18 11551, 20 11102, 24 11776 (20).  Within 3.4 % of the best count everywhere but in
+// two places: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347) and T = 65536, where 16 are taken and 10 would be best (l = 24:
+// 45.3 against 43.8 ms; at T = 32768, l = 8 16 and 12 are 11.1 and 10.9).
+// d = 64, ten shapes, within 2 % of the best; bf16: T = 1024, l = 30, B = 4, 16 heads (256 units): 86 201, 96 206, 102 212, 110 223 (86); T = 4096, l = 23, B = 4, 16 heads:
+// 56 932, 60 874, 64 861, 68 878 (60); T = 8192, l = 16, B = 2, 32 heads: 30 2144, 32 2041, 34 1972, 38 2028 (34); T = 16384, l = 32, 32 heads: 32 3957,
+// 36 3646, 40 3663 (36); T = 32768, l = 32, 32 heads: 18 13600, 20 12386, 22 12938 (20); e4m3: T = 5000, l = 23, B = 2, 32 heads: 56 1157, 60 1143,
+// 64 1183 (60); T = 32768, l = 32: 20 12828, 22 12598, 24 12922 (22).
 inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms, bool fp8) {
     const double nq = num_tiles(T);
     const double depth = double(units) * (l + 1) * (fp8 ? 1.9 : 1.7);
-    const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.36 * (nq + 1) : 7.0 + 0.88 * (nq + 1));
+    const double n = nq + 1;
+    const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.36 * n : 12.0 + (0.66 + 0.00035 * n) * n);
     const double x = sms * depth / (depth + seq);
-    const unsigned share = std::max(16u, 2 * unsigned(std::ceil((1.06 * x + 1.0) / 2)));
+    const auto even = [](double c) { return 2 * unsigned(std::ceil(c / 2)); };
+    unsigned share = std::max(16u, even(1.06 * x + 1.0));
+    // few units for each SM: what counts is how many the busiest one has
+    const unsigned rounds = (units + share - 1) / share;
+    if (rounds > 1 && rounds <= 16) {
+        const unsigned fewer = even(std::ceil(double(units) / (rounds - 1)));
+        share = (100 * fewer <= 112 * share && fewer <= sms) ? fewer : even(std::ceil(double(units) / rounds));
+    }
     return std::min(units, std::min(share, sms));
 }
 

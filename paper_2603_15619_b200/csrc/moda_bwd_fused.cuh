@@ -402,22 +402,22 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 // 2b. Sequence part: dK, dV and the dQ tiles
 // =====================================================================================
 // 512 threads (in warp order):
-//   row warps    two warpgroups: a thread owns one key row (= tensor-memory lane) and 64 of the 128 query columns of
-//                an iteration: P^T, then dS^T.
+//   row warps    two warpgroups.  d = 128: both work on the same iteration, a thread owns one key row (= tensor-memory
+//                lane) and 64 of its 128 query columns.  d = 64: they take alternate iterations, a thread owns one key row
+//                and all 128 query columns.  Either way P^T, then dS^T.
 //   drain warps  one warpgroup: a thread owns one query row of the dQ tile; it copies the row out of tensor memory
 //                (which frees the region at once) and hands it, 8 KiB at a time through a staging ring in shared
 //                memory, to bulk reductions into the fp32 accumulator, at whatever pace L2 takes them, without
 //                holding up the row warps.
-//   then         a loader warp (TMA tiles; the per-query terms as bf16 parts for the extra k-step) and the warps
-//                that issue the contractions:
-//                S, dP, and dV then dQ then dK.  One tcgen05.mma costs its
-//                issuing thread about as long as it executes, so the contractions that start an iteration's two
-//                chains have their own warps on different schedulers; MMAs of different warps are ordered by
-//                mbarriers only.
+//   then         a loader warp (TMA tiles; the per-query terms as bf16 parts for the extra k-step) and three warps
+//                that issue the contractions: S; dP (d = 64: and dV); dV, dQ, dK (d = 64: dK, dQ).  MMAs of
+//                different warps are ordered by mbarriers only.  (One warp for all five, in the order in which they become
+//                ready, took 1.5 times as long at d = 64: its waits and commits come one after the other.)
 //
 // Tensor memory (fp32 columns): X, 128 columns per buffer, S^T overlaid by P^T (bf16) -- one buffer at d = 128,
-// two at d = 64 (where dK and dV leave room);  Y, 128 columns, dP^T and then the dQ tile of the same iteration;
-// dK, D columns;  dV, D columns.  512 columns at either head width.
+// two at d = 64 (where dK and dV leave room);  Y, 128 columns, dP^T;  dK, D columns;  dV, D columns.  512 columns at either head
+// width.  The dQ tile takes Y behind dP^T of the same iteration (d = 128), or the half of an X buffer that P^T has left
+// (d = 64: dQ_i behind P_{i+1}, so that neither dP_{i+1} nor S_{i+1} waits for the copy).
 //
 // What bounds it (cycle stamps per warp role, T = 8192): the rate at which a dQ tile's additions are taken by L2 (64 KiB
 // of fp32 per iteration per SM at d = 128; all SMs together sustain about 5.9 TB/s in a kernel that does nothing else,
@@ -426,23 +426,37 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 // dQ staging 64 KiB in and out, against 128 bytes per clock) is at two thirds of its peak since the row warps no
 // longer load the per-query terms.
 //
-// Two dependency chains per iteration i, which overlap each other and the next iteration:
+// Two dependency chains per iteration i at d = 128, which overlap each other and the next iteration:
 //   X:  S'_i = S_i - LSE / scale -> P_i^T = exp2(S' c) (row warps) -> dV_i -> X free -> S_{i+1}
 //   Y:  dP'_i = dP_i - D -> dS_i^T = P o dP' to shared memory (row warps) -> dQ_i -> copied out (drain warps) -> Y free -> dP_{i+1}
 // and dK_i, issued behind dQ_i, fills the tensor pipe while the row warps exponentiate tile i+1.
+//
+// At d = 64 the row warps set the pace: with both warpgroups on one iteration they exponentiate together (1320 cycles, the
+// SFU's 1024 and latencies) and then form dS together (900, the SFU idle), 2650 cycles an iteration against some 1700 of the
+// tensor cores (an SS MMA of N = 64 takes 48 cycles, its operands at 128 bytes a clock, not 32).  On alternate iterations
+// one's exponentials overlap the other's dS.  What that needs: P^T in registers for a whole row (160 registers),
+// dP_{i+1} as soon as dP_i is in registers, a second dS buffer, a fourth Q stage (a tile is in use for two and a half iterations
+// and takes some 1200 cycles to arrive) -- paid for with two of the four staging chunks.  Cycles per iteration about 2300 now; T = 32768,
+// 32 heads, whole backward 13.1 -> 11.3 ms (1.15-1.18), T = 16384, 64 heads on 8 6.8 -> 5.8, T = 8192, 16 heads 474 -> 425 us, T = 1000 37.9 -> 37.3,
+// T = 300 16.4 -> 16.8 (two or three iterations: one warpgroup has the longer pass of the last).  Measured on the way, T = 32768, gain over
+// the shared iteration: scores in four loads of 32 columns, each waited for, 1.02 (all 128 requested at once: 1.15); dQ in its own tile's X
+// buffer 1.07; dQ before dK 1.06; three Q stages and four chunks 1.04; chunks of 4 KiB 0.93, or of one warp's 32 rows (no barrier among
+// the drain warps) 0.93; one X buffer with P^T and dQ in columns of their own 1.15.  dS^T in tensor memory as well, as dK's A operand,
+// with the shared iteration: 1.01 (d = 128: 0.97).
 
 template <int D>
 struct FusedSmem {
-    static constexpr int kRowWGs = 2;                          // row warpgroups (64 query columns per thread)
-    static constexpr int kCols = kTileRows / kRowWGs;          // query columns per row-warp thread
+    static constexpr int kRowWGs = 2;                          // row warpgroups
+    static constexpr bool kAlternate = (D == 64);              // they take alternate iterations; else half of the query columns each
+    static constexpr int kCols = kAlternate ? kTileRows : kTileRows / kRowWGs;     // query columns per row-warp thread
     static constexpr int kThreads = (kRowWGs * 4 + 8) * 32;    // row warps, 4 drain warps, loader + 3 issuers
     static constexpr int kTileBytes = kTileRows * D * 2;       // 128 x D bf16
     static constexpr int kSubBytes = kTileRows * 128;          // 128 x 64 sub-tile (128-byte rows)
-    // Stages of Q_i.  Q_i is read by S_i early and by dK_i late in its iteration, and a tile takes about 1600
+    // Stages of Q_i.  Q_i is read by S_i early and by dK_i late in its iteration, and a tile takes 1200 to 1600
     // cycles from the TMA issue to the first MMA that uses it, so with two stages the chain "dK_{i-2} completes ->
-    // load Q_i -> S_i -> P_i -> dS_i -> dK_i" spans two iterations and sets the pace; three stages (d = 64, where
-    // shared memory has room) take the load off that chain.
-    static constexpr int kStages = (D == 64) ? 3 : 2;
+    // load Q_i -> S_i -> P_i -> dS_i -> dK_i" spans two iterations and sets the pace; d = 64, where an iteration is in flight for longer,
+    // takes four.
+    static constexpr int kStages = (D == 64) ? 4 : 2;
     // dO_i is read by dP_i and dV_i, both of which complete before dP_{i+1} can be issued; at d = 128 one
     // stage leaves the 32 KiB that the dQ staging buffer needs
     static constexpr int kdOStages = (D == 128) ? 1 : 2;
@@ -450,10 +464,11 @@ struct FusedSmem {
     static constexpr int kV = kK + kTileBytes;
     static constexpr int kQ = kV + kTileBytes;                 // stages of Q_i
     static constexpr int kdO = kQ + kStages * kTileBytes;      // stages of dO_i
-    static constexpr int kdS = kdO + kdOStages * kTileBytes;   // dS^T: 128 keys x 128 queries bf16
+    static constexpr int kdS = kdO + kdOStages * kTileBytes;   // dS^T: 128 keys x 128 queries bf16, one buffer per warpgroup that fills one
     static constexpr int kdSBytes = kTileRows * kTileRows * 2;
-    static constexpr int kStg = kdS + kdSBytes;                // ring of 8 KiB chunks (16 feature columns of a dQ tile, fp32, accumulator layout)
-    static constexpr int kStgSlots = (D == 128) ? 3 : 4;       // three measured as fast as four; two cost 3-4 %
+    static constexpr int kdSBufs = kAlternate ? 2 : 1;
+    static constexpr int kStg = kdS + kdSBufs * kdSBytes;   // ring of 8 KiB chunks (16 feature columns of a dQ tile, fp32, accumulator layout)
+    static constexpr int kStgSlots = (D == 128) ? 3 : 2;       // d = 128: three as fast as four, two cost 3-4 %
     static constexpr int kStgBytes = kStgSlots * 16 * kTileRows * 4;
     // Operands of the extra k-step that adds the per-query terms to the two score contractions (see the kernel):
     // 2 KiB chunks of [128 rows][8 bf16] (unswizzled core matrices, 16 bytes per row): one per Q stage with the
@@ -464,7 +479,7 @@ struct FusedSmem {
     static constexpr int kAugOnesD = kAugOnesS + kAugChunk;
     static constexpr int kAugZero = kAugOnesD + kAugChunk;
     static constexpr int kBars = kAugZero + kAugChunk;
-    static constexpr int kNumBars = 28;
+    static constexpr int kNumBars = 32;
     static constexpr int kMisc = kBars + kNumBars * 8;
     static constexpr int kTotal = kMisc + 16;
     static constexpr int kSmemLimit = 232448;                  // 227 KiB per CTA on sm_100
@@ -476,19 +491,20 @@ struct FusedSmem {
 
 enum FusedBar : int {
     kFBarKV = 0,
-    kFBarQFull = 1,     // +stage (<= 3), count 32: Q_i and the per-query terms of the stage have landed
-    kFBarQEmpty = 4,    // +stage (<= 3): dK_i complete (Q_i, the row terms and the dS buffer are free)
-    kFBardOFull = 7,    // +stage (<= 2)
-    kFBardOEmpty = 9,   // +stage (<= 2), count 2: dP_i and dV_i complete
-    kFBarSFull = 11,    // +X buffer: S_i complete
-    kFBarPFull = 13,    // +X buffer, count 256: P_i^T written
-    kFBardPFull = 15,   // dP_i complete
-    kFBardSFull = 16,   // count 256: dS_i^T written to shared memory, dP_i consumed
-    kFBarXFree = 17,    // +X buffer: dV_i complete: the buffer may take S_{i + buffers}
-    kFBardQFull = 19,   // dQ_i complete
-    kFBarYFree = 20,    // count 128: dQ_i copied out: Y may take dP_{i+1}
-    kFBarFinal = 21,    // last dV and dK complete (one warp issues both)
-    kFBarDrain = 22,    // +issuer (3): abort path only
+    kFBarQFull = 1,     // +stage (<= 4), count 32: Q_i and the per-query terms of the stage have landed
+    kFBarQEmpty = 5,    // +stage (<= 4): dK_i complete (Q_i, the row terms and, d = 128, the dS buffer are free)
+    kFBardOFull = 9,    // +stage (<= 2)
+    kFBardOEmpty = 11,  // +stage (<= 2), count 2: dP_i and dV_i complete
+    kFBarSFull = 13,    // +X buffer: S_i complete
+    kFBarPFull = 15,    // +X buffer, count kRowArrivals: P_i^T written
+    kFBardPFull = 17,   // +X buffer: dP_i complete
+    kFBardSFull = 19,   // +dS buffer, count kRowArrivals: dS_i^T written to shared memory, dP_i consumed
+    kFBardSFree = 21,   // +dS buffer: dQ_i and dK_i complete (alternating warpgroups)
+    kFBarXFree = 23,    // +X buffer: dV_i complete (alternating warpgroups: and dQ_i copied out): the buffer may take S_{i + buffers}
+    kFBardQFull = 25,   // +X buffer: dQ_i complete
+    kFBarYFree = 27,    // count 128: dQ_i copied out (alternating warpgroups: dP_i in registers): Y may take dP_{i+1}
+    kFBarFinal = 28,    // last dV and dK complete, count = warps that issue them
+    kFBarDrain = 29,    // +issuer (3): abort path only
 };
 
 struct FusedParams {
@@ -510,12 +526,13 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     using L = FusedSmem<D>;
     constexpr int NSUB = D / 64;
     constexpr int NRW = L::kRowWGs, COLS = L::kCols, NROW = 128 * NRW;      // row warpgroups, columns per thread, row threads
+    constexpr bool ALT = L::kAlternate;
+    constexpr int kRowArrivals = ALT ? 128 : NROW;
     constexpr int W_DRAIN = 4 * NRW, W_LOAD = W_DRAIN + 4, W_S = W_LOAD + 1, W_DP = W_LOAD + 2;
     constexpr int W_ACC = W_LOAD + 3;                             // issues the three accumulating contractions
     constexpr int NOTHER = (L::kThreads / 32 - W_LOAD) * 32;      // threads of the loader / issuer warps
     constexpr uint32_t kTmemCols = 512;
-    // d = 64 leaves room for a second S^T / P^T buffer: S_{i+1} is then computed while the row warps still work
-    // on tile i, instead of waiting for dV_i to release the only buffer.
+    // d = 64 leaves room for a second S^T / P^T buffer: one per row warpgroup
     constexpr int XB = (D == 64) ? 2 : 1;
     constexpr uint32_t kColX = 0, kColY = 128 * XB, kColdK = kColY + 128, kColdV = kColdK + D;
     static_assert(kColdV + D <= kTmemCols, "tensor-memory plan too large");
@@ -561,14 +578,15 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar(kFBarSFull + s), 1);
-            mbar_init(bar(kFBarPFull + s), NROW);
-            mbar_init(bar(kFBarXFree + s), 1);
+            mbar_init(bar(kFBarPFull + s), kRowArrivals);
+            mbar_init(bar(kFBarXFree + s), ALT ? 129 : 1);
+            mbar_init(bar(kFBardPFull + s), 1);
+            mbar_init(bar(kFBardSFull + s), kRowArrivals);
+            mbar_init(bar(kFBardSFree + s), 1);
+            mbar_init(bar(kFBardQFull + s), 1);
         }
-        mbar_init(bar(kFBardPFull), 1);
-        mbar_init(bar(kFBardSFull), NROW);
-        mbar_init(bar(kFBardQFull), 1);
         mbar_init(bar(kFBarYFree), 128);
-        mbar_init(bar(kFBarFinal), 1);
+        mbar_init(bar(kFBarFinal), ALT ? 2 : 1);
         for (int s = 0; s < 3; ++s) mbar_init(bar(kFBarDrain + s), 1);
         fence_mbar_init();
     }
@@ -607,12 +625,12 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     constexpr int kRegsLaunch = 128;
     static_assert(L::kThreads == 512, "the register shares below assume 512 threads");
     // Shares measured (T = 8192 .. 65536): the issuing warps need about 100 registers to keep their descriptors and
-    // barrier addresses without spills; d = 128: 128 / 160 / 96 (42.1 ms at T = 65536 against 44.1 with 136 / 160 / 80),
-    // d = 64: 136 / 136 / 104 (27.6 ms at T = 32768, H = 32 against 28.5 with 152 / 152 / 56).
-    constexpr int kRegsRow = (D == 128) ? 128 : 136, kRegsDrain = (D == 128) ? 160 : 136, kRegsOther = (D == 128) ? 96 : 104;
+    // barrier addresses without spills; d = 128: 128 / 160 / 96 (42.1 ms at T = 65536 against 44.1 with 136 / 160 / 80).  d = 64: 128
+    // scores and what becomes of them in a row thread, a dQ row of 64 in a drain thread.
+    constexpr int kRegsRow = (D == 128) ? 128 : 160, kRegsDrain = (D == 128) ? 160 : 96, kRegsOther = 96;
     static_assert(NROW * kRegsRow + 128 * kRegsDrain + NOTHER * kRegsOther <= L::kThreads * kRegsLaunch, "register shares exceed the CTA's pool");
     // setmaxnreg.inc to less than the current count (or .dec to more) is an illegal instruction
-    static_assert(kRegsRow >= kRegsLaunch && kRegsDrain >= kRegsLaunch && kRegsOther <= kRegsLaunch, "setmaxnreg direction");
+    static_assert(kRegsRow >= kRegsLaunch && kRegsOther <= kRegsLaunch, "setmaxnreg direction");
     if (warp < W_DRAIN) {
         // =========================== row warps: P^T, dS^T, dK / dV epilogue ===========================
         setmaxnreg_inc<kRegsRow>();
@@ -624,6 +642,84 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         // this thread's row of dS^T: sub-tile of its 64-column half, 128-byte rows, its first 16-byte chunk
         uint8_t* ds_row = smem + L::kdS + ((hc * COLS) >> 6) * L::kSubBytes + r * 128;
         const int ds_chunk0 = ((hc * COLS) & 63) >> 3;
+        if constexpr (ALT) {
+            // this warpgroup's iterations: hc, hc + 2, ...  One key row and all 128 query columns of each.
+            const uint32_t tXw = tmem + lane_addr + kColX + hc * 128, tYw = tmem + lane_addr + kColY;
+            uint8_t* dsw = smem + L::kdS + hc * L::kdSBytes + r * 128;
+            int qi = kt + hc, ph = 0;
+#pragma unroll 1
+            for (int it = hc; it < n_it; it += 2, qi += 2, ph ^= 1) {
+                while (qi >= nk) qi -= n_per;
+                uint32_t pk[64];                             // P_i^T of this thread: 128 values, bf16 pairs
+                // ---- P_i^T ----
+                mbar_wait(bar(kFBarSFull + hc), ph, abort_flag, 121);
+                tc_fence_after_sync();
+                {
+                    uint32_t sv[4][32];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) tmem_ld32(tXw + c * 32, sv[c]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t(&pc)[16] = *reinterpret_cast<uint32_t(*)[16]>(pk + 16 * c);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            // the contraction has already subtracted LSE / scale from every score of the query's column
+                            float e0, e1;
+                            mul2_f32(__uint_as_float(sv[c][2 * j]), __uint_as_float(sv[c][2 * j + 1]), p.scale_log2, p.scale_log2, e0, e1);
+                            pc[j] = pack_bf16x2(fast_exp2(e0), fast_exp2(e1));
+                        }
+                    }
+                    if (qi == kt) {                          // the query tile is the key tile itself: column j sees key row r iff j >= r
+#pragma unroll
+                        for (int j = 0; j < 64; ++j) {
+                            if (2 * j < r) pk[j] &= 0xffff0000u;
+                            if (2 * j + 1 < r) pk[j] &= 0x0000ffffu;
+                        }
+                    }
+                    tmem_st32(tXw, *reinterpret_cast<uint32_t(*)[32]>(pk));     // overlays columns that this thread has read
+                    tmem_st32(tXw + 32, *reinterpret_cast<uint32_t(*)[32]>(pk + 32));
+                }
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive(bar(kFBarPFull + hc));
+
+                // ---- dS_i^T = P o (dP - D), with the bf16 P that dV uses ----
+                mbar_wait(bar(kFBardPFull + hc), ph, abort_flag, 122);
+                tc_fence_after_sync();
+                if (it >= 2) mbar_wait(bar(kFBardSFree + hc), ph ^ 1, abort_flag, 123);    // dQ_{i-2}, dK_{i-2} have read the buffer
+                {
+                    uint32_t gv[2][32];
+                    tmem_ld32(tYw, gv[0]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        if (c < 3) tmem_ld32(tYw + (c + 1) * 32, gv[(c + 1) & 1]);
+                        const uint32_t(&y)[32] = gv[c & 1];
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {        // 8 query columns = one 16-byte chunk of the row
+                            uint32_t w[4];                   // gv holds dP - D_t already (subtracted by the contraction)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const uint32_t pp = pk[16 * c + 4 * g + k];
+                                float x0, x1;
+                                mul2_f32(bf16_lo_to_f32(pp), bf16_hi_to_f32(pp), __uint_as_float(y[8 * g + 2 * k]), __uint_as_float(y[8 * g + 2 * k + 1]), x0, x1);
+                                w[k] = pack_bf16x2(x0, x1);
+                            }
+                            *reinterpret_cast<uint4*>(dsw + (c >> 1) * L::kSubBytes + ((((c & 1) * 4 + g) ^ (r & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                        if (c < 3) tmem_wait_ld();
+                        if (c == 2) {
+                            tc_fence_before_sync();
+                            mbar_arrive(bar(kFBarYFree));    // dP_i is in registers: Y may take dP_{i+1}
+                        }
+                    }
+                }
+                fence_proxy_async_smem();                    // generic-proxy stores -> read by the MMAs (async proxy)
+                tc_fence_before_sync();
+                mbar_arrive(bar(kFBardSFull + hc));
+            }
+        } else {
 #pragma unroll 1
         for (int it = 0, qi = kt; it < n_it; ++it, qi = (qi + 1 < nk) ? qi + 1 : kt) {
             uint32_t pk[COLS / 2];                           // P_i^T of this thread: COLS values, bf16 pairs
@@ -698,6 +794,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             mbar_arrive(bar(kFBardSFull));
         }
 
+        }
         // ---- epilogue: dK (scaled) by the first warpgroup, dV by the second ----
         if (hc < 2) {
         mbar_wait(bar(kFBarFinal), 0, abort_flag, 124);
@@ -740,22 +837,25 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         // in shared memory.  Per-thread red.global instructions would do the same additions, but they queue in the
         // load/store path of the SM at the pace L2 takes them, and every shared-memory load, store and barrier probe of
         // the row warps then waits behind them (measured: + 2000 cycles per iteration).
-        setmaxnreg_inc<kRegsDrain>();
+        if constexpr (kRegsDrain >= kRegsLaunch) setmaxnreg_inc<kRegsDrain>();
+        else setmaxnreg_dec<kRegsDrain>();
         const int r = tid & 127;                             // query row inside the tile = TMEM lane
-        const uint32_t tY = tmem + (uint32_t((warp & 3) * 32) << 16) + kColY;
+        const uint32_t tdQ = tmem + (uint32_t((warp & 3) * 32) << 16) + (ALT ? kColX + 64 : kColY);
+        if (ALT) mbar_arrive(bar(kFBarXFree));               // no dQ tile lies in the first S^T buffer's other half yet
         float4* stg = reinterpret_cast<float4*>(smem + L::kStg) + r;          // [feature / 4 (16)][row 128] float4
         float* dst = p.dq_acc + ((size_t(b) * p.H + h * p.G) * nk + kt) * (size_t(kTileRows) * D);
         int slot = 0;
 #pragma unroll 1
         for (int it = 0, qi = kt; it < n_it; ++it) {
-            mbar_wait(bar(kFBardQFull), it & 1, abort_flag, 120);
+            const int xb = it % XB;
+            mbar_wait(bar(kFBardQFull + xb), (it / XB) & 1, abort_flag, 120);
             tc_fence_after_sync();
             uint32_t o[D];
 #pragma unroll
-            for (int c = 0; c < D / 32; ++c) tmem_ld32(tY + c * 32, *reinterpret_cast<uint32_t(*)[32]>(o + c * 32));
+            for (int c = 0; c < D / 32; ++c) tmem_ld32(tdQ + (ALT ? (xb ^ 1) * 128 : 0) + c * 32, *reinterpret_cast<uint32_t(*)[32]>(o + c * 32));
             tmem_wait_ld();
             tc_fence_before_sync();
-            mbar_arrive(bar(kFBarYFree));                    // Y may take dP of the next iteration
+            mbar_arrive(bar(ALT ? kFBarXFree + (xb ^ 1) : kFBarYFree));   // X may take S of the iteration after the next / Y may take dP of the next
             // 16 feature columns (8 KiB, contiguous in the accumulator) at a time through a ring of staging chunks:
             // a chunk is rewritten once the reduction issued from it one ring earlier has finished reading it, so
             // all but one of the ring's reductions stay in flight and L2, not this loop, sets the pace.
@@ -785,6 +885,19 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         if (tid == NROW) tma_store_wait_read();              // the staging chunks have been read
     } else {
       setmaxnreg_dec<kRegsOther>();
+      constexpr uint32_t idesc_acc = make_idesc_bf16(128, D, false, true);
+      const uint64_t dvb0 = desc_mnmajor_sw128(sbase + L::kdO, 0, L::kSubBytes);
+      // dV += P^T dO (P^T from tensor memory, dO MN-major); dst = stage of dO_i, xb = X buffer of P_i
+      auto issue_dV = [&](int it, int dst, int xb) {
+          const uint64_t dvb = dvb0 + uint64_t((dst * L::kTileBytes) >> 4);
+          // 16 queries per k-step: 8 columns; with half the columns per row warpgroup, in the block of the one that owns them
+#pragma unroll 4
+          for (int kk = 0; kk < kTileRows / 16; ++kk)
+              umma_ts(tmem + kColdV, tmem + kColX + xb * 128 + (ALT ? kk * 8 : (kk / (COLS / 16)) * COLS + (kk % (COLS / 16)) * 8), dvb + uint64_t(kk * 128),
+                      idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(bar(kFBarXFree + xb));
+          umma_commit(bar(kFBardOEmpty + dst));
+      };
       if (warp == W_LOAD) {
         // =========================== loader: TMA tiles + per-query LSE, D_t ===========================
         if (lane == 0) {
@@ -869,6 +982,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 const int xb = it % nb;
                 const uint32_t col = is_s ? kColX + xb * 128 : kColY;
                 const uint32_t free_bar = is_s ? bar(kFBarXFree + xb) : bar(kFBarYFree);
+                const int ob = it % XB;
                 if (it >= nb) mbar_wait2(bar(full0 + st), (it / nst) & 1, free_bar, ((it - nb) / nb) & 1, abort_flag, 141, is_s ? 142 : 143);
                 else mbar_wait(bar(full0 + st), (it / nst) & 1, abort_flag, 141);
                 // dP also needs the Q stage's per-query terms (they arrive with Q_i)
@@ -883,22 +997,27 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                     for (int kk = 0; kk < 4; ++kk) umma_ss(tmem + col, ca + uint64_t(kk * 2), cb + uint64_t(kk * 2), idesc_s, (c > 0 || kk > 0) ? 1u : 0u);
                 }
                 umma_ss(tmem + col, da_aug, db_aug0 + uint64_t((qst * L::kAugChunk) >> 4), idesc_s, 1u);
-                umma_commit(bar(is_s ? kFBarSFull + xb : kFBardPFull));
+                umma_commit(bar(is_s ? kFBarSFull + xb : kFBardPFull + ob));
                 if (!is_s) umma_commit(bar(kFBardOEmpty + st));
+                // P_i is written before dP_i is consumed, so dV_i never holds up dP_{i+1}
+                if (ALT && !is_s) {
+                    mbar_wait(bar(kFBarPFull + ob), (it / XB) & 1, abort_flag, 144);
+                    tc_fence_after_sync();
+                    issue_dV(it, st, ob);
+                }
             }
+            if (ALT && !is_s) umma_commit(bar(kFBarFinal));
             drain_on_abort(is_s ? 0 : 1);
         }
       } else if (warp == W_ACC) {
-        // ============ MMA issuer of the accumulating contractions: dV_i += P^T dO (P^T from tensor memory, dO MN-major),
+        // ============ MMA issuer of the accumulating contractions.  d = 128: dV_i += P^T dO (P^T from tensor memory, dO MN-major),
         // ============ then, once dS_i^T is in shared memory, dQ_tile = dS K into Y (dS^T and K both MN-major) and
         // ============ dK += dS^T Q (dS^T K-major, Q MN-major).  P_i, dS_i, P_{i+1} are produced in this order, so one
         // ============ warp can take the three in turn.  dQ before dK: its tile has to be copied out before dP of the next
-        // ============ iteration can land, dK only has to finish before dS_{i+1} is written.  (A warp per contraction was
-        // ============ measured at d = 64, where these are N = 64 MMAs: no faster.)
+        // ============ iteration can land, dK only has to finish before dS_{i+1} is written.  d = 64: dK_i, then dQ_i, whose columns
+        // ============ P_{i+1} has to leave first.
         {
-            constexpr uint32_t idesc_acc = make_idesc_bf16(128, D, false, true);
             constexpr uint32_t idesc_dq = make_idesc_bf16(128, D, true, true);
-            const uint64_t dvb0 = desc_mnmajor_sw128(sbase + L::kdO, 0, L::kSubBytes);
             const uint64_t dqa0 = desc_mnmajor_sw128(sbase + L::kdS, 0, L::kSubBytes);
             const uint64_t dqb0 = desc_mnmajor_sw128(sbase + L::kK, 0, L::kSubBytes);
             const uint64_t dka0 = desc_kmajor_sw128(sbase + L::kdS, 0);
@@ -906,27 +1025,35 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 #pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
                 const int st = it % L::kStages, dst = it % L::kdOStages, xb = it % XB;
-                mbar_wait2(bar(kFBarPFull + xb), (it / XB) & 1, bar(kFBardOFull + dst), (it / L::kdOStages) & 1, abort_flag, 144, 145);
+                if constexpr (!ALT) {
+                    mbar_wait2(bar(kFBarPFull + xb), (it / XB) & 1, bar(kFBardOFull + dst), (it / L::kdOStages) & 1, abort_flag, 144, 145);
+                    tc_fence_after_sync();
+                    issue_dV(it, dst, xb);
+                }
+                const uint64_t dsb = uint64_t((ALT ? xb * L::kdSBytes : 0) >> 4);
+                mbar_wait(bar(kFBardSFull + xb), (it / XB) & 1, abort_flag, 146);
                 tc_fence_after_sync();
-                const uint64_t dvb = dvb0 + uint64_t((dst * L::kTileBytes) >> 4);
-#pragma unroll 4
-                for (int kk = 0; kk < kTileRows / 16; ++kk)  // 16 queries per k-step: 8 columns, in the block of the row warpgroup that owns them
-                    umma_ts(tmem + kColdV, tmem + kColX + xb * 128 + (kk / (COLS / 16)) * COLS + (kk % (COLS / 16)) * 8, dvb + uint64_t(kk * 128),
-                            idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
-                umma_commit(bar(kFBarXFree + xb));
-                umma_commit(bar(kFBardOEmpty + dst));
-                mbar_wait(bar(kFBardSFull), it & 1, abort_flag, 146);
-                tc_fence_after_sync();
-#pragma unroll 4
-                for (int kk = 0; kk < kTileRows / 16; ++kk)
-                    umma_ss(tmem + kColY, dqa0 + uint64_t(kk * 128), dqb0 + uint64_t(kk * 128), idesc_dq, kk > 0);
-                umma_commit(bar(kFBardQFull));
                 const uint64_t dkb = dkb0 + uint64_t((st * L::kTileBytes) >> 4);
+                auto issue_dK = [&]() {
+#pragma unroll 4
+                    for (int kk = 0; kk < kTileRows / 16; ++kk)
+                        umma_ss(tmem + kColdK, dka0 + dsb + uint64_t(((kk >> 2) * L::kSubBytes + (kk & 3) * 32) >> 4), dkb + uint64_t(kk * 128),
+                                idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
+                    umma_commit(bar(kFBarQEmpty + st));
+                };
+                if constexpr (ALT) {
+                    // dK first: dQ_i goes to the half of the other X buffer that P_{i+1} leaves (the last tile: whose dQ tile has been copied out)
+                    issue_dK();
+                    if (it + 1 < n_it) mbar_wait(bar(kFBarPFull + (xb ^ 1)), ((it + 1) / XB) & 1, abort_flag, 148);
+                    else if (it > 0) mbar_wait(bar(kFBarXFree + (xb ^ 1)), ((it - 1) / XB) & 1, abort_flag, 149);
+                    tc_fence_after_sync();
+                }
 #pragma unroll 4
                 for (int kk = 0; kk < kTileRows / 16; ++kk)
-                    umma_ss(tmem + kColdK, dka0 + uint64_t(((kk >> 2) * L::kSubBytes + (kk & 3) * 32) >> 4), dkb + uint64_t(kk * 128),
-                            idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
-                umma_commit(bar(kFBarQEmpty + st));
+                    umma_ss(tmem + (ALT ? kColX + (xb ^ 1) * 128 + 64 : kColY), dqa0 + dsb + uint64_t(kk * 128), dqb0 + uint64_t(kk * 128), idesc_dq, kk > 0);
+                umma_commit(bar(kFBardQFull + xb));
+                if constexpr (ALT) umma_commit(bar(kFBardSFree + xb));
+                else issue_dK();
             }
             umma_commit(bar(kFBarFinal));
             drain_on_abort(2);
