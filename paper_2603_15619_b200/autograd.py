@@ -55,6 +55,10 @@ def moda_attention(Q, K, V, depth_kv=None, l=0, scale=None):
         scale = Q.shape[-1] ** -0.5
     if l > 0 and depth_kv is None:
         raise ValueError("depth_kv is required when l > 0")
+    # the same two calls and saved tensors as a C++ node; None for anything but plain tensors outside of transforms, modes and tracers
+    out = binding.host().attention(Q, K, V, depth_kv, l, scale)
+    if out is not None:
+        return out
     if depth_kv is None:
         depth_kv = Q.new_empty(0)
     return _ModaAttention.apply(Q, K, V, depth_kv, int(l), float(scale))

@@ -8,12 +8,14 @@ call returns an error code, a ``ModaError`` is raised.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libmoda_b200.so")
+HOST_PATH = os.path.join(_PKG, "_host.so")
 
 MODA_MAX_DEPTH = 256
 SYMBOLS = (
@@ -134,6 +136,25 @@ def load() -> ctypes.CDLL:
     lib.moda_kv_project_append_e4m3.argtypes = [vp, vp, vp, ci, ci, ci, ci, ci, vp, vp, vp, ci, vp]
     _lib = lib
     return lib
+
+
+_host = None
+
+
+def host():
+    """The host path of the hot calls (csrc/moda_host.cpp): the same C calls without Python in between, for arguments that are
+    as documented and on the current stream.  Each of its functions returns None for anything else, which the code
+    below then takes."""
+    global _host
+    if _host is None:
+        if not os.path.exists(HOST_PATH):
+            raise ImportError(f"{HOST_PATH} is missing: build it with `python -m paper_2603_15619_b200.build` (or __graft_entry__.build())")
+        spec = importlib.util.spec_from_file_location(f"{__package__}._host", HOST_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        module.bind(load()._handle, _check)
+        _host = module
+    return _host
 
 
 def _ptr(t):
@@ -498,6 +519,8 @@ def moda_attn_fwd_gqa(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=None
     """Grouped-query forward: Q [B,T,H,d], K, V [B,T,H_kv,d], depth cache with H_kv heads.
 
     Returns O [B,T,H,d] bf16 and LSE [B,H,T] fp32 (allocated if not given)."""
+    if stream is None and (out := host().attn_fwd(Q, K, V, depth_kv, l, scale, None, 0, O, LSE)) is not None:
+        return out
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
     if O is None:
         O = _new_like(Q, stream)
@@ -512,6 +535,10 @@ def moda_attn_fwd_gqa(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=None
 def moda_attn_fwd_append(Q, K, V, depth_kv, l, scale, append_cache, append_slot, O=None, LSE=None, stream=None):
     """moda_attn_fwd_gqa that also stores K, V into slot ``append_slot`` of ``append_cache`` (cache layout, H_kv heads)
     in the same launch: the depth stream's write step without a separate pass over K and V."""
+    if stream is None and append_cache is not None:
+        out = host().attn_fwd(Q, K, V, depth_kv, l, scale, append_cache, append_slot, O, LSE)
+        if out is not None:
+            return out
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
     if O is None:
         O = _new_like(Q, stream)
@@ -529,6 +556,10 @@ def moda_attn_bwd_gqa(Q, K, V, depth_kv, O, dO, LSE, l, scale,
     """Grouped-query backward: dQ [B,T,H,d], dK, dV [B,T,H_kv,d], depth gradients (cache layout, H_kv heads).
 
     With ``stages`` (a MODA_BWD_STAGE_* mask) the call goes through moda_attn_bwd_gqa_stages."""
+    if stream is None:
+        out = host().attn_bwd(Q, K, V, depth_kv, O, dO, LSE, l, scale, dQ, dK, dV, d_depth_kv, workspace, stages)
+        if out is not None:
+            return out
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
     dQ = _new_like(Q, stream) if dQ is None else dQ
     dK = _new_like(K, stream) if dK is None else dK
@@ -560,6 +591,8 @@ def moda_decode_workspace_bytes(B, H, d) -> int:
 def moda_attn_decode(q, K, V, depth_kv_token, T_kv, l, scale, O=None, LSE=None, workspace=None, stream=None):
     """Decode step: q [B,H,d], K, V [B,T_cap,H_kv,d] (positions < T_kv read), depth pairs of the token
     [l,B,H_kv,2,d] (key row, value row).  Returns O [B,H,d] bf16 and LSE [B,H] fp32."""
+    if stream is None and (out := host().decode(q, K, V, None, None, depth_kv_token, T_kv, l, scale, O, LSE, workspace)) is not None:
+        return out
     if q.dtype != torch.bfloat16 or q.dim() != 3:
         raise ValueError("q must be a bf16 [B, H, d] tensor")
     B, H, d = q.shape
@@ -619,6 +652,8 @@ def _int32(t, name, shape):
 def moda_attn_decode_varlen(q, K, V, seq_lens, depth_kv_token, max_seq_len, l, scale, O=None, LSE=None,
                             workspace=None, stream=None):
     """Decode step with a length per sequence: seq_lens int32 [B] (device), each in [1, max_seq_len]."""
+    if stream is None and (out := host().decode(q, K, V, None, seq_lens, depth_kv_token, max_seq_len, l, scale, O, LSE, workspace)) is not None:
+        return out
     B, H, d = q.shape
     _, T_cap, Hk, _ = _bthd(K, "K")
     _int32(seq_lens, "seq_lens", (B,))
@@ -634,6 +669,9 @@ def moda_attn_decode_paged(q, K_pages, V_pages, block_table, seq_lens, depth_kv_
                            O=None, LSE=None, workspace=None, stream=None):
     """Decode step over a paged KV cache: K_pages, V_pages [num_pages, page_size, H_kv, d]; block_table int32
     [B, max_blocks]; seq_lens int32 [B]."""
+    if stream is None and (out := host().decode(q, K_pages, V_pages, block_table, seq_lens, depth_kv_token, max_seq_len, l, scale, O, LSE,
+                                                workspace)) is not None:
+        return out
     B, H, d = q.shape
     num_pages, page_size, Hk, _ = _bthd(K_pages, "K_pages")
     _int32(seq_lens, "seq_lens", (B,))

@@ -1,4 +1,4 @@
-"""Builds the CUDA library (libmoda_b200.so) in-tree with nvcc for sm_100a."""
+"""Builds the CUDA library (libmoda_b200.so, nvcc for sm_100a) and the host path of its hot calls (_host.so, g++) in-tree."""
 from __future__ import annotations
 
 import os
@@ -9,6 +9,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmoda_b200.so")
 SOURCES = [os.path.join(CSRC, "moda_api.cu")]
+HOST = os.path.join(PKG, "_host.so")
+HOST_SOURCE = os.path.join(CSRC, "moda_host.cpp")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-std=c++17", "-lineinfo",
@@ -44,5 +46,30 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_host(force: bool = False, verbose: bool = False) -> str:
+    """The CPython extension that moves the hot calls' host work out of Python (csrc/moda_host.cpp). Returns the .so path."""
+    deps = (HOST_SOURCE, os.path.join(PKG, "..", "include", "moda.h"))
+    if force or not os.path.exists(HOST) or any(os.path.getmtime(d) > os.path.getmtime(HOST) for d in deps):
+        import sysconfig
+
+        import torch
+        root = os.path.dirname(torch.__file__)
+        cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+        include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                   os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+        tmp = HOST + f".tmp{os.getpid()}"
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+        cmd += [f"-I{d}" for d in include] + ["-o", tmp, HOST_SOURCE, "-L" + os.path.join(root, "lib")]
+        cmd += ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if verbose or res.returncode != 0:
+            sys.stderr.write(res.stdout + res.stderr)
+        if res.returncode != 0:
+            raise RuntimeError("g++ failed building _host.so")
+        os.replace(tmp, HOST)
+    return HOST
+
+
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose=True))
+    print(build_host(force="--force" in sys.argv, verbose=True))

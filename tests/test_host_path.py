@@ -1,0 +1,248 @@
+"""The host path of the hot calls (csrc/moda_host.cpp): what it does not serve it hands back, and where it serves a call (GPU) the
+results and the autograd behaviour are those of the general path."""
+import pytest
+import torch
+
+import paper_2603_15619_b200 as moda
+from paper_2603_15619_b200 import autograd, binding
+
+gpu = pytest.mark.gpu
+BF16 = torch.bfloat16
+
+
+class _Refuses:
+    """Stands in for the extension: every call takes the general path."""
+
+    def __getattr__(self, name):
+        return lambda *a: None
+
+
+@pytest.fixture
+def general(monkeypatch):
+    """Runs a function on the general path."""
+    def run(f, *a, **k):
+        with monkeypatch.context() as m:
+            m.setattr(binding, "host", lambda: _Refuses())
+            return f(*a, **k)
+    return run
+
+
+def test_what_is_not_plain_is_handed_back():
+    host = binding.host()
+    x = torch.zeros(1, 4, 2, 64, dtype=BF16)
+    m = torch.empty(1, 4, 2, 64, dtype=BF16, device="meta")
+    for t in (x, m, None, 3):
+        assert host.attention(t, t, t, None, 0, 0.1) is None
+        assert host.attn_fwd(t, t, t, None, 0, 0.1, None, 0, None, None) is None
+        assert host.attn_bwd(t, t, t, None, t, t, t, 0, 0.1, None, None, None, None, None, None) is None
+        assert host.decode(t, t, t, None, None, None, 4, 0, 0.1, None, None, None) is None
+    assert host.decode() is None and host.attention() is None
+
+
+def _qkv(B, T, H, Hk, d, seed=0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    new = lambda *s: torch.randn(s, generator=g, device="cuda", dtype=BF16)
+    return new(B, T, H, d), new(B, T, Hk, d), new(B, T, Hk, d), new(B, T, H, d)
+
+
+def _cache(B, T, Hk, d, l, slots=None):
+    cache = moda.alloc_depth_cache(B, T, Hk, d, slots or max(l, 1))
+    for i in range(l):
+        _, K, V, _ = _qkv(B, T, Hk, Hk, d, 10 + i)
+        moda.moda_depth_cache_append(cache, i, K, V)
+    return cache
+
+
+def _same(a, b, loose=()):
+    assert len(a) == len(b)
+    for i, (x, y) in enumerate(zip(a, b)):
+        if x is None or y is None:
+            assert x is None and y is None
+        elif i in loose:                                   # dQ: the order of its fp32 additions is not fixed
+            assert (x.float() - y.float()).norm() <= 1e-3 * y.float().norm() + 1e-6
+        else:
+            assert torch.equal(x, y), i
+
+
+@gpu
+@pytest.mark.parametrize("B,T,H,Hk,d,l", [(1, 1, 1, 1, 64, 0), (2, 129, 4, 2, 64, 3), (1, 300, 2, 2, 128, 5)])
+def test_layer_calls_agree_with_the_general_path(general, B, T, H, Hk, d, l):
+    Q, K, V, dO = _qkv(B, T, H, Hk, d)
+    cache = _cache(B, T, Hk, d, l, l + 1)
+    other = cache.clone()
+    O, LSE = moda.moda_attn_fwd_append(Q, K, V, cache, l, 0.125, cache, l)
+    _same((O, LSE), general(moda.moda_attn_fwd_append, Q, K, V, other, l, 0.125, other, l))
+    assert torch.equal(cache[:other.numel()], other)
+    _same(moda.moda_attn_fwd_gqa(Q, K, V, cache, l, 0.125), (O, LSE))
+    given = torch.empty_like(O), torch.empty_like(LSE)
+    got = moda.moda_attn_fwd_gqa(Q, K, V, cache, l, 0.125, O=given[0], LSE=given[1])
+    assert got[0] is given[0] and got[1] is given[1] and torch.equal(given[0], O)
+    for stages in (None, moda.MODA_BWD_ALL_STAGES, moda.MODA_BWD_ALL_STAGES | moda.MODA_BWD_DETERMINISTIC):
+        a = moda.moda_attn_bwd_gqa(Q, K, V, cache, O, dO, LSE, l, 0.125, stages=stages)
+        b = general(moda.moda_attn_bwd_gqa, Q, K, V, cache, O, dO, LSE, l, 0.125, stages=stages)
+        _same(a, b, loose=(0,))
+    assert moda.moda_last_status() == 0
+
+
+@gpu
+@pytest.mark.parametrize("form", ["plain", "varlen", "paged"])
+def test_decode_agrees_with_the_general_path(general, form):
+    B, T, H, Hk, d, l = 3, 200, 4, 2, 64, 2
+    g = torch.Generator(device="cuda").manual_seed(1)
+    new = lambda *s: torch.randn(s, generator=g, device="cuda", dtype=BF16)
+    q, depth, lens = new(B, H, d), new(l, B, Hk, 2, d), torch.tensor([1, 77, 200], dtype=torch.int32, device="cuda")
+    if form == "paged":
+        args = (moda.moda_attn_decode_paged, q, new(12, 64, Hk, d), new(12, 64, Hk, d), torch.arange(12, dtype=torch.int32, device="cuda").view(3, 4), lens)
+    elif form == "varlen":
+        args = (moda.moda_attn_decode_varlen, q, new(B, T, Hk, d), new(B, T, Hk, d), lens)
+    else:
+        args = (moda.moda_attn_decode, q, new(B, T, Hk, d), new(B, T, Hk, d))
+    f, rest = args[0], (*args[1:], depth, T, l, 0.125)
+    _same(f(*rest), general(f, *rest))
+    with pytest.raises(moda.ModaError) as here:             # errors of the C call come as they did
+        f(*rest[:-1], -1.0)
+    with pytest.raises(moda.ModaError) as there:
+        general(f, *rest[:-1], -1.0)
+    assert here.value.code == there.value.code and str(here.value) == str(there.value)
+
+
+def _errors(f):
+    try:
+        f()
+    except Exception as e:
+        return type(e)
+    return None
+
+
+@gpu
+def test_wrong_arguments_are_refused_as_before(general):
+    Q, K, V, dO = _qkv(1, 64, 2, 2, 64)
+    bad = [lambda: moda.moda_attn_fwd_gqa(Q.float(), K, V, None, 0, 0.1), lambda: moda.moda_attn_fwd_gqa(Q.transpose(1, 2), K, V, None, 0, 0.1),
+           lambda: moda.moda_attn_fwd_gqa(Q, K[:, :32], V, None, 0, 0.1), lambda: moda.moda_attn_fwd_gqa(Q, K, V, None, 3, 0.1),
+           lambda: moda.moda_attn_fwd_gqa(Q, K.cpu(), V, None, 0, 0.1), lambda: moda.moda_attn_fwd_gqa(Q, K, V, None, 0, 0.0),
+           lambda: moda.moda_attn_fwd_gqa(Q.transpose(2, 3), K, V, None, 0, 0.1), lambda: moda.moda_attn_fwd_gqa(Q[..., :32], K[..., :32], V[..., :32], None, 0, 0.1),
+           lambda: moda.moda_attention(Q, K, V, None, 2), lambda: moda.moda_attention(Q, K.float(), V), lambda: moda.moda_attn_fwd_gqa(Q, K, V, None, -1, 0.1),
+           lambda: moda.moda_attn_fwd_append(Q, K, V, None, 0, 0.1, None, 0), lambda: moda.moda_attn_decode(Q[:, 0], K, V, None, 65, 0, 0.1)]
+    for i, f in enumerate(bad):
+        want = general(_errors, f)
+        assert want is not None and _errors(f) is want, (i, want, _errors(f))
+
+
+@gpu
+@pytest.mark.parametrize("l", [0, 2])
+def test_differentiable_call_behaves_as_the_general_one(general, l):
+    """Gradients, unused outputs, saved-tensor hooks, in-place changes, retained graphs, no_grad, inference mode, non-contiguous inputs,
+    second derivatives, transforms."""
+    def leaves():
+        Q, K, V, dO = _qkv(1, 130, 4, 2, 64)
+        x = [t.requires_grad_() for t in (Q, K, V)]
+        cache = _cache(1, 130, 2, 64, 2, 3).requires_grad_() if l else None
+        return x, cache, dO
+
+    def grads():
+        x, cache, dO = leaves()
+        O, LSE = moda.moda_attention(*x, cache, l)
+        assert O.requires_grad and not LSE.requires_grad
+        wrt = x + ([cache] if l else [])
+        first = torch.autograd.grad(O, wrt, dO, retain_graph=True)
+        again = torch.autograd.grad(O, wrt, dO)
+        with pytest.raises(RuntimeError, match="backward through the graph a second time"):
+            torch.autograd.grad(O, wrt, dO)
+        _same(first, again, loose=(0,))
+        return [O, LSE, *first]
+
+    _same(grads(), general(grads), loose=(2,))
+
+    def hooks():
+        x, cache, dO = leaves()
+        seen = []
+        with torch.autograd.graph.saved_tensors_hooks(lambda t: (seen.append(tuple(t.shape)), t.clone())[1], lambda t: t):
+            O, _ = moda.moda_attention(*x, cache, l)
+        O.backward(dO)
+        return sorted(seen), [t.grad for t in x]
+
+    a, b = hooks(), general(hooks)
+    assert a[0] == b[0] and len(a[0]) == (6 if l else 5)
+    _same(a[1], b[1], loose=(0,))
+
+    def changed():
+        x, cache, dO = leaves()
+        y = [t * 1 for t in x]
+        O, _ = moda.moda_attention(*y, cache, l)
+        y[1].add_(1)
+        O.backward(dO)
+
+    assert general(_errors, changed) is RuntimeError and _errors(changed) is RuntimeError
+
+    def others():
+        x, cache, dO = leaves()
+        with torch.no_grad():
+            assert not moda.moda_attention(*x, cache, l)[0].requires_grad
+        with torch.inference_mode():
+            a = moda.moda_attention(*x, cache, l)[0]
+            assert a.is_inference()
+        t = [u.transpose(1, 2).contiguous().transpose(1, 2) for u in x]       # not contiguous
+        b = moda.moda_attention(*t, cache, l)[0]
+        assert torch.equal(a, b)
+        g = torch.autograd.grad(moda.moda_attention(*x, cache, l)[0], x, dO, create_graph=True)
+        return [b, *g], [u.requires_grad for u in g]
+
+    a, b = others(), general(others)
+    _same(a[0], b[0], loose=(1,))
+    assert a[1] == b[1]
+
+    def mapped():
+        x, cache, dO = leaves()
+        torch.func.vmap(lambda q: moda.moda_attention(q, x[1], x[2], cache, l)[0])(x[0][None])
+
+    def dual():
+        x, cache, dO = leaves()
+        with torch.autograd.forward_ad.dual_level():
+            moda.moda_attention(torch.autograd.forward_ad.make_dual(x[0], dO), x[1], x[2], cache, l)
+
+    for f in (mapped, dual):
+        assert _errors(f) is general(_errors, f) and _errors(f) is not None
+
+    class Sub(torch.Tensor):
+        pass
+
+    def subclass():
+        x, cache, dO = leaves()
+        q = x[0].detach().as_subclass(Sub)
+        return [type(t) for t in moda.moda_attn_fwd_gqa(q, x[1].detach(), x[2].detach(), cache, l, 0.1)]
+
+    assert subclass() == general(subclass)
+    assert moda.moda_last_status() == 0
+
+
+@gpu
+def test_streams_and_threads():
+    """A call follows the current stream, in threads of their own too, and outputs belong to it."""
+    import threading
+    Q, K, V, dO = _qkv(1, 256, 2, 2, 64)
+    want = moda.moda_attn_fwd_gqa(Q, K, V, None, 0, 0.125)
+    torch.cuda.synchronize()
+    out, errors = {}, []
+
+    def work(i):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                leaves = [t.clone().requires_grad_() for t in (Q, K, V)]
+                for _ in range(20):
+                    O, LSE = moda.moda_attention(*leaves, None, 0, 0.125)
+                    g = torch.autograd.grad(O, leaves, dO)
+            s.synchronize()
+            out[i] = [O, LSE, *g]
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for i in range(4):
+        _same(out[i][:2], want)
+        _same(out[i], out[0], loose=(2,))
