@@ -13,6 +13,7 @@
 #include "moda_depth_gqa.cuh"
 #include "moda_fwd.cuh"
 #include "moda_fwd_wide.cuh"
+#include "moda_fwd_wide128.cuh"
 #include "moda_mass.cuh"
 #include "moda_kvproj.cuh"
 #include "sm100_ptx.cuh"
@@ -195,14 +196,25 @@ bool set_smem_limit(Kernel k, int bytes) {
     return cuda_ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
 }
 
-// d = 128 runs moda_fwd_kernel (one softmax warpgroup: the tensor pipe and the MMA issue rate set the
-// pace); d = 64 runs moda_fwd2_kernel (two softmax warpgroups, three score buffers: the exponentials do).
-// Which forward kernel at d = 128: one K stage and a five-unit depth ring when the depth stream
+// d = 64 runs moda_fwd2_kernel (two softmax warpgroups, three score buffers), d = 128 one with two softmax warpgroups as well
+// (moda_fwd_wide128.cuh) or, with many depth slots for the length, moda_fwd_kernel (see fwd_two_softmax).
+// Which form of moda_fwd_kernel: one K stage and a five-unit depth ring when the depth stream
 // outweighs the sequence work (measured: - 6 % at l d / T = 0.72, - 3 % at 0.5, slower below),
 // otherwise two K stages and a three-unit ring.
 inline bool fwd_depth_heavy(int T_q, int T_kv, int l, int d) {
     // against the mean number of key tiles of a query tile, (2 T_kv - T_q) / 256: with T_q = T_kv = T this is 2 l d >= T
     return d == 128 && l > 0 && 2ll * l * d >= 2ll * T_kv - T_q;
+}
+
+// Whether a d = 128 forward takes the kernel with two softmax warpgroups (moda_fwd_wide128.cuh).  It is the faster one where the key tiles
+// set the pace; where the depth slots do, its ring of three units against five and the smaller register share of its depth warps
+// cost it up to a fifth.  us, one warpgroup -> two (B = 2, 16 heads): l = 0: T = 128 7.2 -> 7.2, T = 1000 23.9 -> 22.2, T = 2048 57.7 -> 51.9,
+// T = 8192 552 -> 481, T = 16384 2339 -> 1964.  l = 4: T = 1000 27.1 -> 25.8, T = 512 11.4 -> 11.8.  l = 8: T = 4096 238 -> 223, T = 2048 84.0 -> 84.3,
+// T = 1000 33.1 -> 37.9.  l = 16: T = 8192 716 -> 714 and 719 -> 650, T = 4096 268 -> 291.  l = 24: T = 16384 2545 -> 2420, T = 8192 802 -> 842.  e4m3,
+// l = 8: T = 2048 73.6 -> 73.4, T = 1000 30.2 -> 33.8; l = 16: T = 8192 714 -> 631, T = 4096 235 -> 260.  2000 over 15000, l = 24, B = 4: 1192 -> 985.
+inline bool fwd_two_softmax(int T_q, int T_kv, int l) {
+    // against twice the mean number of keys of a query: 2 T_kv - T_q, T when T_q = T_kv = T
+    return 560ll * l <= 2ll * T_kv - T_q + 1120;
 }
 
 // Whether a grouped-query forward runs its depth part as the separate per-position kernel.  Measured at
@@ -284,7 +296,9 @@ int launch_fwd(const void* Q, const void* K, const void* V, const void* depth_kv
         bool ok;
         if constexpr (kWide) ok = set_smem_limit(moda_fwd2_kernel<D>, kSmem) && set_smem_limit(moda_fwd2_kernel<D, true>, kSmem8);
         else ok = set_smem_limit(moda_fwd_kernel<D, 2>, kSmem) && set_smem_limit(moda_fwd_kernel<128, 1>, kSmemDeep) &&
-                  set_smem_limit(moda_fwd_kernel<128, 2, true>, kSmem8);
+                  set_smem_limit(moda_fwd_kernel<128, 2, true>, kSmem8) &&
+                  set_smem_limit(d128::moda_fwd2_kernel<false>, d128::Fwd2Smem<false>::kDynamic) &&
+                  set_smem_limit(d128::moda_fwd2_kernel<true>, d128::Fwd2Smem<true>::kDynamic);
         if (!ok) return MODA_ERR_CUDA;
         configured_dev = dev;
     }
@@ -317,12 +331,19 @@ int launch_fwd(const void* Q, const void* K, const void* V, const void* depth_kv
     // A position-major cache is always read by the per-position kernel.
     const bool split_depth = pm ? l > 0 : (!fp8 && gqa_depth_split(D, p.G, l));
     if (split_depth) p.l = 0;
-    if (fp8) {
-        if constexpr (kWide) moda_fwd2_kernel<D, true><<<grid, kThreads, kSmem8, stream>>>(mQ, mK, mV, mO, p);
-        else moda_fwd_kernel<128, 2, true><<<grid, kThreads, kSmem8, stream>>>(mQ, mK, mV, mO, p);
-    } else if (kWide) moda_fwd2_kernel<D><<<grid, kThreads, kSmem, stream>>>(mQ, mK, mV, mO, p);
-    else if (!split_depth && fwd_depth_heavy(T, T_kv, l, D)) moda_fwd_kernel<128, 1><<<grid, kThreads, kSmemDeep, stream>>>(mQ, mK, mV, mO, p);
-    else moda_fwd_kernel<D, 2><<<grid, kThreads, kSmem, stream>>>(mQ, mK, mV, mO, p);
+    if constexpr (kWide) {
+        if (fp8) moda_fwd2_kernel<D, true><<<grid, kThreads, kSmem8, stream>>>(mQ, mK, mV, mO, p);
+        else moda_fwd2_kernel<D><<<grid, kThreads, kSmem, stream>>>(mQ, mK, mV, mO, p);
+    } else if (fwd_two_softmax(T, T_kv, p.l)) {
+        if (fp8) d128::moda_fwd2_kernel<true><<<grid, d128::kFwd2Threads, d128::Fwd2Smem<true>::kDynamic, stream>>>(mQ, mK, mV, mO, p);
+        else d128::moda_fwd2_kernel<false><<<grid, d128::kFwd2Threads, d128::Fwd2Smem<false>::kDynamic, stream>>>(mQ, mK, mV, mO, p);
+    } else if (fp8) {
+        moda_fwd_kernel<128, 2, true><<<grid, kThreads, kSmem8, stream>>>(mQ, mK, mV, mO, p);
+    } else if (!split_depth && fwd_depth_heavy(T, T_kv, l, D)) {
+        moda_fwd_kernel<128, 1><<<grid, kThreads, kSmemDeep, stream>>>(mQ, mK, mV, mO, p);
+    } else {
+        moda_fwd_kernel<128, 2><<<grid, kThreads, kSmem, stream>>>(mQ, mK, mV, mO, p);
+    }
     if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
     if (split_depth) {
         DepthMergeParams m;

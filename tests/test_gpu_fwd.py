@@ -125,3 +125,35 @@ def test_c2_full_size_sampled_rows_every_head():
     x = synthetic.make(w, seed=0, device="cuda")
     O, LSE = run_forward(x, w)
     check_sampled_rows(w, x, O, LSE)
+
+
+# d = 128, two softmax warpgroups on alternate key tiles (few slots for the length): one key tile, two, an odd number, one row in the last,
+# and key norms that grow or fall along the sequence, so that the reference maximum moves in either warpgroup, or never again.
+@pytest.mark.parametrize("direction", [0, 1, -1])
+@pytest.mark.parametrize("T,l", [(1, 0), (127, 1), (129, 0), (256, 1), (385, 1), (1153, 4), (1280, 4)])
+def test_two_softmax_warpgroups(T, l, direction):
+    w = synthetic.Workload("t", 1, T, 2, 128, l)
+    x = synthetic.make(w, seed=15, device="cuda")
+    if direction:
+        ramp = torch.linspace(0.2, 3.0, T, device="cuda")
+        ramp = ramp if direction > 0 else ramp.flip(0)
+        x["K"] = (x["K"].float() * ramp.view(1, T, 1, 1)).to(torch.bfloat16)
+    O, LSE = run_forward(x, w)
+    O_ref, LSE_ref = oracle_forward(x, w.scale)
+    assert_forward_close(O, LSE, O_ref, LSE_ref, f"{(T, l, direction)}")
+
+
+def test_two_softmax_warpgroups_with_two_groups_of_slots():
+    # 33 slots are two groups of the depth part's online softmax; so long a sequence is what brings them to this kernel
+    w = synthetic.Workload("g", 1, 17600, 1, 128, 33)
+    x = synthetic.make(w, seed=16, device="cuda")
+    O, LSE = run_forward(x, w)
+    check_sampled_rows(w, x, O, LSE, rows_per_head=60)
+    # the same through an e4m3 cache, against the rows' own dequantised slots
+    cache = moda.alloc_depth_cache_e4m3(w.B, w.T, w.H, w.d, w.l)
+    for i in range(w.l):
+        moda.moda_depth_cache_append_e4m3(cache, i, x["Kd"][i].contiguous(), x["Vd"][i].contiguous())
+    O8, LSE8 = moda.moda_attn_fwd_e4m3(x["Q"], x["K"], x["V"], cache, w.l, w.scale)
+    assert moda.moda_last_status() == 0
+    hat = [torch.from_numpy(orc.dequantize_e4m3_rows(*orc.quantize_e4m3_rows(f64(t)))) for t in (x["Kd"], x["Vd"])]
+    check_sampled_rows(w, dict(x, Kd=hat[0], Vd=hat[1]), O8, LSE8, rows_per_head=60)
