@@ -22,7 +22,9 @@ from .binding import (  # noqa: F401
     moda_attn_bwd_e4m3,
     moda_attn_bwd_gqa,
     moda_attn_bwd_gqa_pm,
+    moda_attn_bwd_gqa_slot,
     moda_attn_bwd_gqa_stages,
+    moda_attn_bwd_takes_slot,
     moda_attn_bwd_stages,
     moda_attn_bwd_static_scratch,
     moda_attn_decode,

@@ -24,6 +24,7 @@ SYMBOLS = (
     "moda_attn_fwd", "moda_bwd_workspace_bytes", "moda_attn_bwd", "moda_attn_bwd_stages",
     "moda_attn_bwd_static_scratch",
     "moda_attn_fwd_gqa", "moda_bwd_workspace_bytes_gqa", "moda_attn_bwd_gqa", "moda_attn_bwd_gqa_stages",
+    "moda_attn_bwd_gqa_slot", "moda_attn_bwd_takes_slot",
     "moda_decode_workspace_bytes", "moda_attn_decode", "moda_attn_fwd_prefill", "moda_attn_fwd_append",
     "moda_attn_decode_varlen", "moda_attn_decode_paged",
     "moda_depth_cache_e4m3_bytes", "moda_depth_cache_append_e4m3", "moda_attn_fwd_e4m3", "moda_attn_bwd_e4m3",
@@ -100,6 +101,10 @@ def load() -> ctypes.CDLL:
     lib.moda_attn_bwd_gqa.argtypes = [vp] * 7 + [ci] * 6 + [cf] + [vp] * 5 + [sz, vp]
     lib.moda_attn_bwd_gqa_stages.restype = ci
     lib.moda_attn_bwd_gqa_stages.argtypes = [vp] * 7 + [ci] * 6 + [cf] + [vp] * 5 + [sz, ci, vp]
+    lib.moda_attn_bwd_gqa_slot.restype = ci
+    lib.moda_attn_bwd_gqa_slot.argtypes = [vp] * 7 + [ci] * 6 + [cf] + [vp] * 5 + [sz, ci, vp]
+    lib.moda_attn_bwd_takes_slot.restype = ci
+    lib.moda_attn_bwd_takes_slot.argtypes = [ci] * 4
     lib.moda_attn_decode_varlen.restype = ci
     lib.moda_attn_decode_varlen.argtypes = [vp] * 5 + [ci] * 7 + [cf] + [vp] * 3 + [sz, vp]
     lib.moda_attn_decode_paged.restype = ci
@@ -582,6 +587,31 @@ def moda_attn_bwd_gqa(Q, K, V, depth_kv, O, dO, LSE, l, scale,
 def moda_attn_bwd_gqa_stages(*args, stages, **kwargs):
     """moda_attn_bwd_gqa restricted to the launches selected by the ``stages`` bit mask."""
     return moda_attn_bwd_gqa(*args, stages=stages, **kwargs)
+
+
+def moda_attn_bwd_takes_slot(H, Hk, d, l) -> bool:
+    return bool(load().moda_attn_bwd_takes_slot(int(H), int(Hk), int(d), int(l)))
+
+
+def moda_attn_bwd_gqa_slot(Q, K, V, depth_kv, O, dO, LSE, l, scale, d_depth_kv, slot,
+                           dQ=None, dK=None, dV=None, workspace=None, stream=None):
+    """Backward of a layer of a stack: depth gradients added to slots < l of d_depth_kv, slot ``slot`` >= l of it (the later
+    layers' gradient of this layer's K, V) added to dK, dV.  Returns dQ, dK, dV."""
+    if stream is None:
+        out = host().attn_bwd(Q, K, V, depth_kv, O, dO, LSE, l, scale, dQ, dK, dV, d_depth_kv, workspace, slot, True)
+        if out is not None:
+            return out[:3]
+    B, T, H, Hk, d = _gqa_shapes(Q, K, V)
+    dQ = _new_like(Q, stream) if dQ is None else dQ
+    dK = _new_like(K, stream) if dK is None else dK
+    dV = _new_like(V, stream) if dV is None else dV
+    if workspace is None:
+        workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
+    _check(load().moda_attn_bwd_gqa_slot(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None, _ptr(O), _ptr(dO), _ptr(LSE),
+                                         B, T, H, Hk, d, int(l), float(scale), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv),
+                                         _ptr(workspace), workspace.numel() * workspace.element_size(), int(slot), _stream(stream)),
+           "moda_attn_bwd_gqa_slot")
+    return dQ, dK, dV
 
 
 def moda_decode_workspace_bytes(B, H, d) -> int:

@@ -471,7 +471,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     int dev = 0;
     if (!cuda_ok(cudaGetDevice(&dev))) return MODA_ERR_CUDA;
     if (configured_dev != dev) {
-        if (!set_smem_limit(moda_bwd_fused_kernel<D>, L::kDynamic) || !set_smem_limit(bwd_rows_kernel<D>, RowsSmem<D, false>::kDynamic) ||
+        if (!set_smem_limit(moda_bwd_fused_kernel<D>, L::kDynamic) || !set_smem_limit(moda_bwd_fused_kernel<D, true>, L::kDynamic) || !set_smem_limit(bwd_rows_kernel<D>, RowsSmem<D, false>::kDynamic) ||
             !set_smem_limit(bwd_rows_kernel<D, true>, RowsSmem<D, true>::kDynamic))
             return MODA_ERR_CUDA;
         configured_dev = dev;
@@ -510,6 +510,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
         f.LSE = a.LSE; f.delta = delta; f.dq_acc = dq_acc;
         f.B = B; f.T = T; f.H = H; f.G = G;
         f.scale = a.scale; f.scale_log2 = a.scale * kLog2e;
+        f.slot_grad = static_cast<const uint4*>(a.slot_grad);
         f.beside_rows = beside_rows ? 1 : 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(unsigned(B) * Hk * num_tiles(T), 1, 1);
@@ -521,7 +522,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = beside_rows ? 1 : 0;
-        if (!cuda_ok(cudaLaunchKernelEx(&cfg, moda_bwd_fused_kernel<D>, mK, mV, mQ, mdO, mdK, mdV, f))) return MODA_ERR_CUDA;
+        if (!cuda_ok(cudaLaunchKernelEx(&cfg, a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true> : moda_bwd_fused_kernel<D, false>, mK, mV, mQ, mdO, mdK, mdV, f))) return MODA_ERR_CUDA;
     }
     if (stages & 4) {
         bwd_dq_finish_kernel<D><<<tiles, kRowThreads, 0, stream>>>(dq_acc, static_cast<__nv_bfloat16*>(a.dQ), B, T, H, a.scale);
@@ -849,6 +850,46 @@ int kv_project_common(const void* X, const void* Wk, const void* Wv, int B, int 
 }
 }  // namespace
 
+namespace {
+
+// The backward of every entry point that takes a plain cache; slot >= 0: dK, dV take up that slot of d_depth_kv as well.
+int bwd_gqa(const void* Q, const void* K, const void* V, const void* depth_kv, const void* O, const void* dO, const float* LSE,
+            int B, int T, int H, int H_kv, int d, int l, float scale, void* dQ, void* dK, void* dV, void* d_depth_kv,
+            void* workspace, size_t workspace_bytes, int stages, int slot, void* stream) {
+    if (int rc = check_shape(B, T, H, d)) return rc;
+    if (int rc = check_scale(scale)) return rc;
+    if (int rc = check_groups(H, H_kv)) return rc;
+    if ((stages & MODA_BWD_ALL_STAGES) == 0 || stages < 0 ||
+        stages > (MODA_BWD_ALL_STAGES | MODA_BWD_ACCUMULATE_DEPTH | MODA_BWD_DETERMINISTIC))
+        return MODA_ERR_BAD_SHAPE;
+    if (l < 0 || l > MODA_MAX_DEPTH) return MODA_ERR_BAD_DEPTH;
+    // slots < l are written by this call
+    if (slot >= 0 && (slot < l || slot >= MODA_MAX_DEPTH)) return MODA_ERR_BAD_SLOT;
+    if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV || (l > 0 && !depth_kv) || ((l > 0 || slot >= 0) && !d_depth_kv))
+        return MODA_ERR_NULL_POINTER;
+    if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(dO) || !aligned16(LSE) ||
+        !aligned16(dQ) || !aligned16(dK) || !aligned16(dV) ||
+        (l > 0 && !aligned16(depth_kv)) || ((l > 0 || slot >= 0) && !aligned16(d_depth_kv)))
+        return MODA_ERR_MISALIGNED;
+    const bool deterministic = (stages & MODA_BWD_DETERMINISTIC) != 0;
+    if (slot >= 0 && !bwd_uses_fused(d, H / H_kv, l, deterministic)) return MODA_ERR_BAD_GROUP;
+    const size_t need = bwd_uses_fused(d, H / H_kv, l, deterministic) ? bwd_fused_workspace_bytes(B, T, H, d)
+                                                                       : bwd_workspace_bytes_gqa(B, T, H, H_kv, l);
+    if (!workspace || !aligned16(workspace) || workspace_bytes < need) return MODA_ERR_WORKSPACE;
+    if (int rc = check_device()) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    BwdArgs a;
+    a.deterministic = deterministic;
+    a.Q = Q; a.K = K; a.V = V; a.depth_kv = depth_kv; a.O = O; a.dO = dO; a.LSE = LSE;
+    a.B = B; a.T = T; a.H = H; a.Hk = H_kv; a.l = l; a.scale = scale;
+    a.dQ = dQ; a.dK = dK; a.dV = dV; a.d_depth_kv = d_depth_kv; a.workspace = workspace;
+    a.accumulate_depth = (stages & MODA_BWD_ACCUMULATE_DEPTH) != 0;
+    if (slot >= 0) a.slot_grad = static_cast<const __nv_bfloat16*>(d_depth_kv) + size_t(slot) * cache_slot_elems(B, T, H_kv, d);
+    return d == 128 ? launch_bwd<128>(a, stages, st) : launch_bwd<64>(a, stages, st);
+}
+
+}  // namespace
+
 extern "C" {
 
 int moda_version(void) { return 100; }
@@ -1036,32 +1077,22 @@ int moda_attn_bwd_gqa_stages(const void* Q, const void* K, const void* V, const 
                              int B, int T, int H, int H_kv, int d, int l, float scale,
                              void* dQ, void* dK, void* dV, void* d_depth_kv,
                              void* workspace, size_t workspace_bytes, int stages, void* stream) {
-    if (int rc = check_shape(B, T, H, d)) return rc;
-    if (int rc = check_scale(scale)) return rc;
-    if (int rc = check_groups(H, H_kv)) return rc;
-    if ((stages & MODA_BWD_ALL_STAGES) == 0 || stages < 0 ||
-        stages > (MODA_BWD_ALL_STAGES | MODA_BWD_ACCUMULATE_DEPTH | MODA_BWD_DETERMINISTIC))
-        return MODA_ERR_BAD_SHAPE;
-    if (l < 0 || l > MODA_MAX_DEPTH) return MODA_ERR_BAD_DEPTH;
-    if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV || (l > 0 && (!depth_kv || !d_depth_kv)))
-        return MODA_ERR_NULL_POINTER;
-    if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || !aligned16(dO) || !aligned16(LSE) ||
-        !aligned16(dQ) || !aligned16(dK) || !aligned16(dV) ||
-        (l > 0 && (!aligned16(depth_kv) || !aligned16(d_depth_kv))))
-        return MODA_ERR_MISALIGNED;
-    const bool deterministic = (stages & MODA_BWD_DETERMINISTIC) != 0;
-    const size_t need = bwd_uses_fused(d, H / H_kv, l, deterministic) ? bwd_fused_workspace_bytes(B, T, H, d)
-                                                                       : bwd_workspace_bytes_gqa(B, T, H, H_kv, l);
-    if (!workspace || !aligned16(workspace) || workspace_bytes < need) return MODA_ERR_WORKSPACE;
-    if (int rc = check_device()) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    BwdArgs a;
-    a.deterministic = deterministic;
-    a.Q = Q; a.K = K; a.V = V; a.depth_kv = depth_kv; a.O = O; a.dO = dO; a.LSE = LSE;
-    a.B = B; a.T = T; a.H = H; a.Hk = H_kv; a.l = l; a.scale = scale;
-    a.dQ = dQ; a.dK = dK; a.dV = dV; a.d_depth_kv = d_depth_kv; a.workspace = workspace;
-    a.accumulate_depth = (stages & MODA_BWD_ACCUMULATE_DEPTH) != 0;
-    return d == 128 ? launch_bwd<128>(a, stages, st) : launch_bwd<64>(a, stages, st);
+    return bwd_gqa(Q, K, V, depth_kv, O, dO, LSE, B, T, H, H_kv, d, l, scale, dQ, dK, dV, d_depth_kv, workspace, workspace_bytes, stages, -1, stream);
+}
+
+int moda_attn_bwd_gqa_slot(const void* Q, const void* K, const void* V, const void* depth_kv,
+                           const void* O, const void* dO, const float* LSE,
+                           int B, int T, int H, int H_kv, int d, int l, float scale,
+                           void* dQ, void* dK, void* dV, void* d_depth_kv,
+                           void* workspace, size_t workspace_bytes, int slot, void* stream) {
+    if (slot < 0) return MODA_ERR_BAD_SLOT;
+    return bwd_gqa(Q, K, V, depth_kv, O, dO, LSE, B, T, H, H_kv, d, l, scale, dQ, dK, dV, d_depth_kv, workspace, workspace_bytes,
+                   MODA_BWD_ALL_STAGES | MODA_BWD_ACCUMULATE_DEPTH, slot, stream);
+}
+
+int moda_attn_bwd_takes_slot(int H, int H_kv, int d, int l) {
+    if (check_shape(1, 1, H, d) != MODA_OK || check_groups(H, H_kv) != MODA_OK || l < 0 || l > MODA_MAX_DEPTH) return 0;
+    return bwd_uses_fused(d, H / H_kv, l, false) ? 1 : 0;
 }
 
 // ---- depth cache in e4m3 with a scale per row ----

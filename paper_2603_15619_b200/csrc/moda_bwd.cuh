@@ -36,6 +36,7 @@ struct BwdArgs {
     int B, T, H, Hk, l;          // H query heads on Hk key/value heads
     float scale;
     void *dQ, *dK, *dV, *d_depth_kv, *workspace;
+    const void* slot_grad = nullptr; // slot of a gradient cache that dK, dV take up (fused form), or null
     bool accumulate_depth = false;   // add the depth gradients to d_depth_kv instead of overwriting it
     bool deterministic = false;      // split form (bit-reproducible) instead of the fused form
     bool pm_cache = false;           // depth_kv and d_depth_kv are position-major (grouped-query calls, fused form, per-position depth kernel)

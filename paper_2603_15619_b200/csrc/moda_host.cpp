@@ -31,7 +31,7 @@ using at::Tensor;
 
 // ---- the library: addresses from the handle that the binding has opened -----------------------------------------------
 #define MODA_HOST_CALLS(X)                                                                                              \
-    X(moda_attn_fwd_gqa) X(moda_attn_fwd_append) X(moda_attn_bwd_gqa) X(moda_attn_bwd_gqa_stages)                       \
+    X(moda_attn_fwd_gqa) X(moda_attn_fwd_append) X(moda_attn_bwd_gqa) X(moda_attn_bwd_gqa_stages) X(moda_attn_bwd_gqa_slot) \
     X(moda_bwd_workspace_bytes_gqa) X(moda_depth_cache_bytes) X(moda_attn_decode) X(moda_attn_decode_varlen)            \
     X(moda_attn_decode_paged) X(moda_decode_workspace_bytes)
 struct Library {
@@ -138,9 +138,10 @@ void forward(const Shape& s, const Tensor& Q, const Tensor& K, const Tensor& V, 
                                    O.data_ptr(), static_cast<float*>(LSE.data_ptr()), cache->data_ptr(), slot, stream());
     if (rc != 0) fail(rc, cache == nullptr ? "moda_attn_fwd_gqa" : "moda_attn_fwd_append");
 }
-// stages < 0: moda_attn_bwd_gqa, else the call with a mask
+// mode: moda_attn_bwd_gqa, the call with a mask, or the call with a slot
+enum Mode { kWhole, kMask, kSlot };
 void backward(const Shape& s, const Tensor& Q, const Tensor& K, const Tensor& V, const Tensor* depth, const Tensor& O, const Tensor& dO,
-              const Tensor& LSE, int l, float scale, int stages, Tensor& dQ, Tensor& dK, Tensor& dV, Tensor& dcache, Tensor& ws) {
+              const Tensor& LSE, int l, float scale, Mode mode, int arg, Tensor& dQ, Tensor& dK, Tensor& dV, Tensor& dcache, Tensor& ws) {
     if (!dQ.defined()) dQ = like(Q);
     if (!dK.defined()) dK = like(K);
     if (!dV.defined()) dV = like(V);
@@ -152,13 +153,19 @@ void backward(const Shape& s, const Tensor& Q, const Tensor& K, const Tensor& V,
     const void* dep = l > 0 ? ptr(depth) : nullptr;
     void* dc = l > 0 ? dcache.data_ptr() : nullptr;
     const float* lse = static_cast<const float*>(LSE.data_ptr());
-    const int rc = stages < 0
+    if (mode == kSlot) {
+        const int rc = lib.moda_attn_bwd_gqa_slot(Q.data_ptr(), K.data_ptr(), V.data_ptr(), dep, O.data_ptr(), dO.data_ptr(), lse, s.B, s.T, s.H, s.Hk, s.d, l,
+                                                  scale, dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), dcache.data_ptr(), ws.data_ptr(), bytes_of(ws), arg, stream());
+        if (rc != 0) fail(rc, "moda_attn_bwd_gqa_slot");
+        return;
+    }
+    const int rc = mode == kWhole
         ? lib.moda_attn_bwd_gqa(Q.data_ptr(), K.data_ptr(), V.data_ptr(), dep, O.data_ptr(), dO.data_ptr(), lse, s.B, s.T, s.H, s.Hk, s.d, l,
                                 scale, dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), dc, ws.data_ptr(), bytes_of(ws), stream())
         : lib.moda_attn_bwd_gqa_stages(Q.data_ptr(), K.data_ptr(), V.data_ptr(), dep, O.data_ptr(), dO.data_ptr(), lse, s.B, s.T, s.H, s.Hk,
-                                       s.d, l, scale, dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), dc, ws.data_ptr(), bytes_of(ws), stages,
+                                       s.d, l, scale, dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), dc, ws.data_ptr(), bytes_of(ws), arg,
                                        stream());
-    if (rc != 0) fail(rc, stages < 0 ? "moda_attn_bwd_gqa" : "moda_attn_bwd_gqa_stages");
+    if (rc != 0) fail(rc, mode == kWhole ? "moda_attn_bwd_gqa" : "moda_attn_bwd_gqa_stages");
 }
 
 // attn_fwd(Q, K, V, depth, l, scale, cache, slot, O, LSE) -> (O, LSE)
@@ -181,13 +188,15 @@ PyObject* attn_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
-// attn_bwd(Q, K, V, depth, O, dO, LSE, l, scale, dQ, dK, dV, dcache, workspace, stages or None) -> (dQ, dK, dV, dcache)
+// attn_bwd(Q, K, V, depth, O, dO, LSE, l, scale, dQ, dK, dV, dcache, workspace, stages or None) -> (dQ, dK, dV, dcache); with one argument more: the one before it is a slot
 PyObject* attn_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
-    int l, stages = -1;
+    int l, arg = -1;
     float scale;
-    if (n != 15 || !plain_thread() || !int_arg(a[7], l) || l < 0 || !float_arg(a[8], scale)) return none();
-    if (a[14] != Py_None && (!int_arg(a[14], stages) || stages < 0)) return none();
+    if (n < 15 || n > 16 || !plain_thread() || !int_arg(a[7], l) || l < 0 || !float_arg(a[8], scale)) return none();
+    if (a[14] != Py_None && (!int_arg(a[14], arg) || arg < 0)) return none();
+    const Mode mode = n == 16 ? kSlot : a[14] == Py_None ? kWhole : kMask;
+    if (mode == kSlot && (a[12] == Py_None || a[14] == Py_None)) return none();
     const Tensor *Q = dense(a[0], at::kBFloat16, 4), *K = dense(a[1], at::kBFloat16, 4), *V = dense(a[2], at::kBFloat16, 4);
     const Tensor *depth, *O, *dO, *LSE, *g[5];
     Shape s;
@@ -200,7 +209,7 @@ PyObject* attn_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (g[i] != nullptr) t[i] = *g[i];
     {
         NoGil nogil;
-        backward(s, *Q, *K, *V, depth, *O, *dO, *LSE, l, scale, stages, t[0], t[1], t[2], t[3], t[4]);
+        backward(s, *Q, *K, *V, depth, *O, *dO, *LSE, l, scale, mode, arg, t[0], t[1], t[2], t[3], t[4]);
     }
     return Py_BuildValue("NNNN", out(a[9], t[0]), out(a[10], t[1]), out(a[11], t[2]), t[3].defined() ? out(a[12], t[3]) : none());
     END_HANDLE_TH_ERRORS
@@ -237,7 +246,7 @@ struct Attention : torch::autograd::Function<Attention> {
             const int64_t slots = int64_t(lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l) / 2);
             if (slots < depth.numel()) dcache.view({-1}).slice(0, slots).zero_();
         }
-        ::backward(s, Q, K, V, l > 0 ? &depth : nullptr, O, dO, LSE, l, scale, -1, dQ, dK, dV, dcache, ws);
+        ::backward(s, Q, K, V, l > 0 ? &depth : nullptr, O, dO, LSE, l, scale, kWhole, 0, dQ, dK, dV, dcache, ws);
         return {dQ, dK, dV, dcache, Tensor(), Tensor()};
     }
 };

@@ -44,6 +44,10 @@ class _Attend(torch.autograd.Function):
         dO = torch.zeros_like(O) if dO is None else dO.contiguous()
         # slots < l of the gradient cache receive this layer's share
         grads, filled = slots.open(dtoken, l)
+        if filled and binding.moda_attn_bwd_takes_slot(Q.shape[2], K.shape[2], Q.shape[3], l):
+            # the fused backward adds slot l, which later layers attended to, where it stores dK, dV
+            dQ, dK, dV = binding.moda_attn_bwd_gqa_slot(Q, K, V, slots.cache if l > 0 else None, O, dO, LSE, l, ctx.scale, grads, l)
+            return dQ, dK, dV, slots.close(grads, filled, l), None, None, None
         dQ, dK, dV, _ = binding.moda_attn_bwd_gqa(
             Q, K, V, slots.cache if l > 0 else None, O, dO, LSE, l, ctx.scale, d_depth_kv=grads if l > 0 else None,
             stages=binding.MODA_BWD_ALL_STAGES | (binding.MODA_BWD_ACCUMULATE_DEPTH if filled else 0))

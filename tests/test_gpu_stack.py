@@ -89,6 +89,48 @@ def test_accumulate_flag_adds_the_depth_gradients_to_what_the_cache_holds(B, T, 
     assert rel_l2(acc.double().cpu().numpy(), want2.cpu().numpy()) < 1e-2
 
 
+@pytest.mark.parametrize("B,T,H,Hk,d,l,slot", [(1, 1, 1, 1, 64, 0, 0), (1, 127, 2, 2, 128, 0, 2), (2, 129, 3, 3, 128, 3, 3), (2, 257, 3, 3, 64, 2, 4),
+                                               (1, 1000, 2, 2, 128, 5, 6), (1, 700, 4, 4, 64, 9, 9), (1, 300, 8, 2, 128, 0, 1),
+                                               (1, 200, 8, 1, 64, 12, 12), (2, 130, 16, 1, 64, 9, 10)])
+def test_backward_that_takes_up_a_slot_of_the_gradient_cache(B, T, H, Hk, d, l, slot):
+    """moda_attn_bwd_gqa_slot = the accumulating backward with the slot added to dK, dV, rounded once."""
+    assert moda.moda_attn_bwd_takes_slot(H, Hk, d, l)
+    x = synthetic.make_gqa(B, T, H, Hk, d, l, seed=78, device="cuda")
+    scale = d ** -0.5
+    cache, grads = moda.alloc_depth_cache(B, T, Hk, d, max(l, 1)), moda.alloc_depth_cache(B, T, Hk, d, slot + 2)
+    for i in range(l):
+        moda.moda_depth_cache_append(cache, i, x["Kd"][i].contiguous(), x["Vd"][i].contiguous())
+    g = torch.Generator(device="cuda").manual_seed(6)
+    add = [torch.randn(B, T, Hk, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2 * (slot + 2))]
+    for i in range(slot + 2):
+        moda.moda_depth_cache_append(grads, i, add[2 * i], add[2 * i + 1])
+    other = grads.clone()
+    O, LSE = moda.moda_attn_fwd_gqa(x["Q"], x["K"], x["V"], cache, l, scale)
+    dQ, dK, dV, _ = moda.moda_attn_bwd_gqa(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, scale, d_depth_kv=other,
+                                           stages=moda.MODA_BWD_ALL_STAGES | moda.MODA_BWD_ACCUMULATE_DEPTH)
+    got = moda.moda_attn_bwd_gqa_slot(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, scale, grads, slot)
+    assert moda.moda_last_status() == 0
+    assert torch.equal(grads, other)                                         # slots < l alike, the others untouched
+    assert_same_gradients(got[:1], (dQ,), "dQ with and without a slot")
+    for new, plain, more in zip(got[1:], (dK, dV), add[2 * slot:]):
+        want = plain.double() + more.double()
+        # 8 significant bits: rounding the sum moves it by 2^-8 of itself at most, and so was the plain gradient rounded
+        bound = 1.02 * 2.0 ** -8 * (want.abs() + plain.double().abs())
+        assert bool(((new.double() - want).abs() <= bound).all())
+
+
+def test_calls_that_cannot_take_up_a_slot():
+    B, T, H, Hk, d, l = 1, 130, 4, 2, 128, 1
+    assert not moda.moda_attn_bwd_takes_slot(H, Hk, 96, 0) and not moda.moda_attn_bwd_takes_slot(4, 3, 64, 0)
+    x = synthetic.make_gqa(B, T, 2, 2, d, l, seed=79, device="cuda")
+    cache, grads = moda.alloc_depth_cache(B, T, 2, d, l), moda.alloc_depth_cache(B, T, 2, d, 2)
+    O, LSE = moda.moda_attn_fwd_gqa(x["Q"], x["K"], x["V"], cache, 0, 0.1)
+    for slot in (0, -1, 256):                                                # below l, no slot, past the largest
+        with pytest.raises(moda.ModaError):
+            moda.moda_attn_bwd_gqa_slot(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, 0.1, grads, slot)
+    assert moda.moda_last_status() == 0
+
+
 def test_slot_written_without_attending_gets_the_gradients_of_the_layers_after_it():
     B, T, H, Hk, d = 1, 200, 4, 2, 64
     scale = d ** -0.5
