@@ -458,6 +458,23 @@ inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, 
     return std::min(units, std::min(share, sms));
 }
 
+// A launch that may start before the grid in front of it has ended (that grid lets it, and it waits itself before it reads
+// what the grid writes), or a plain one.
+template <class... P, class... A>
+bool launch_beside(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, bool beside, cudaStream_t stream, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = beside ? 1 : 0;
+    return cuda_ok(cudaLaunchKernelEx(&cfg, kernel, args...));
+}
+
 template <int D>
 int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     const int B = a.B, T = a.T, H = a.H, Hk = a.Hk, G = a.H / a.Hk;
@@ -500,9 +517,8 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
             int sms = 0;
             if (int rc = device_sm_count(&sms)) return rc;
             const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, units, unsigned(sms), a.fp8_cache) : std::min(units, unsigned(sms));
-            if (a.fp8_cache) bwd_rows_kernel<D, true><<<grid, 512, RowsSmem<D, true>::kDynamic, stream>>>(mQ, mdO, r);
-            else bwd_rows_kernel<D><<<grid, 512, RowsSmem<D, false>::kDynamic, stream>>>(mQ, mdO, r);
-            if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
+            const size_t smem = a.fp8_cache ? RowsSmem<D, true>::kDynamic : RowsSmem<D, false>::kDynamic;
+            if (!launch_beside(a.fp8_cache ? bwd_rows_kernel<D, true> : bwd_rows_kernel<D, false>, grid, 512, smem, true, stream, mQ, mdO, r)) return MODA_ERR_CUDA;
         }
     }
     if (stages & 2) {
@@ -512,21 +528,12 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
         f.scale = a.scale; f.scale_log2 = a.scale * kLog2e;
         f.slot_grad = static_cast<const uint4*>(a.slot_grad);
         f.beside_rows = beside_rows ? 1 : 0;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(unsigned(B) * Hk * num_tiles(T), 1, 1);
-        cfg.blockDim = dim3(L::kThreads, 1, 1);
-        cfg.dynamicSmemBytes = L::kDynamic;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = beside_rows ? 1 : 0;
-        if (!cuda_ok(cudaLaunchKernelEx(&cfg, a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true> : moda_bwd_fused_kernel<D, false>, mK, mV, mQ, mdO, mdK, mdV, f))) return MODA_ERR_CUDA;
+        if (!launch_beside(a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true> : moda_bwd_fused_kernel<D, false>, unsigned(B) * Hk * num_tiles(T),
+                           L::kThreads, L::kDynamic, (stages & 1) != 0, stream, mK, mV, mQ, mdO, mdK, mdV, f)) return MODA_ERR_CUDA;
     }
     if (stages & 4) {
-        bwd_dq_finish_kernel<D><<<tiles, kRowThreads, 0, stream>>>(dq_acc, static_cast<__nv_bfloat16*>(a.dQ), B, T, H, a.scale);
-        if (!cuda_ok(cudaGetLastError())) return MODA_ERR_CUDA;
+        if (!launch_beside(bwd_dq_finish_kernel<D>, tiles, kRowThreads, 0, (stages & 2) != 0, stream, static_cast<const float*>(dq_acc),
+                           static_cast<__nv_bfloat16*>(a.dQ), B, T, H, a.scale)) return MODA_ERR_CUDA;
         if (split_depth) {
             DepthBwdParams m;
             m.Q = static_cast<const __nv_bfloat16*>(a.Q);

@@ -58,6 +58,7 @@ template <int D>
 __global__ void __launch_bounds__(kTileRows * (D / 32))
 bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO, float* __restrict__ delta,
                 float* __restrict__ dq_acc, int B, int T, int H) {
+    grid_launch_dependents();
     constexpr int PARTS = D / 32;                 // threads per row
     constexpr int CH = D / 8;                     // 16-byte chunks per row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -87,6 +88,12 @@ bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __rest
 // =====================================================================================
 // 3. dQ = bf16(scale * accumulator)
 // =====================================================================================
+// The launches of a backward overlap at their ends (programmatic dependent launch): a grid comes up while the one in front of
+// it finishes, and waits for it before it touches D_t, the accumulator or the depth gradients.  Whole backward, graph
+// replays, us, T = 100, l = 0, d = 64, 2 heads: 13.0 -> 10.9; 2 x 512, 16 heads, d = 128, l = 0: 24.0 -> 22.7; 2 x 1000, l = 0: 55.2 -> 54.1;
+// T = 2000, 16 heads on 4, d = 64, l = 12: 119.3 -> 116.2; with row-local slots between 0 and 1 us, from T = 4096 on nothing.  The
+// sequence part lets this kernel start at the END of its CTAs: from their start on, its CTAs filled the few SMs that
+// had no work in the last wave and did theirs there, four to an SM (2 x 1000, l = 0: 59.8; T = 512: 29.5).
 template <int D>
 __global__ void __launch_bounds__(kTileRows * (D / 32))
 bwd_dq_finish_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dQ, int B, int T, int H, float scale) {
@@ -100,6 +107,7 @@ bwd_dq_finish_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict
     const int bh = blockIdx.x / nq;
     const int b = bh / H, h = bh % H;
     const int t = qt * kTileRows + r;
+    grid_dependency_wait();                       // started beside the end of the sequence part
     if (t >= T) return;
     const float4* src = reinterpret_cast<const float4*>(dq_acc) + size_t(blockIdx.x) * (D / 4) * kTileRows + size_t(part * 8) * kTileRows + r;
     uint4* dst = reinterpret_cast<uint4*>(dQ) + ((size_t(b) * T + t) * H + h) * CH + part * 4;
@@ -167,6 +175,9 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     constexpr int PARTS = D / 32, TPU = R::kTilesPerUnit, NSUB = D / 64;
     constexpr int RW = 32 / PARTS;                     // rows per warp
     constexpr int CH = D / 8;
+    // D_t and the cleared accumulator.  Every thread, before anything else: the sequence part, which this lets start, then finds
+    // both, and no grid of a call ends before the one in front of it.  (The first ring loads ahead of the wait: no faster.)
+    grid_dependency_wait();
     grid_launch_dependents();                          // the sequence part may take the SMs that this grid leaves
     if (g_moda_status != 0) return;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -540,7 +551,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 
     const bool last_cta = p.beside_rows && blockIdx.x == gridDim.x - 1;   // ends the grid after the rows kernel, on every path
     if (g_moda_status != 0) {
-        if (last_cta) grid_dependency_wait();
+        grid_dependency_wait();
         return;
     }
 
@@ -548,7 +559,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     uint8_t* smem = aligned_dynamic_smem(smem_raw, L::kTotal);
     if (smem == nullptr) {
         if (threadIdx.x == 0) atomicCAS(&g_moda_status, 0, kStatusSmemLayout);
-        if (last_cta) grid_dependency_wait();
+        grid_dependency_wait();
         return;
     }
     const uint32_t sbase = smem_u32(smem);
@@ -903,7 +914,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 dst += size_t(kt) * (kTileRows * D);
             }
         }
-        if (tid == NROW) tma_store_wait_read();              // the staging chunks have been read
+        if (tid == NROW) tma_store_wait_all();               // the finish kernel may be up already: the sums are in place
     } else {
       setmaxnreg_dec<kRegsOther>();
       constexpr uint32_t idesc_acc = make_idesc_bf16(128, D, false, true);
@@ -933,6 +944,8 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 tma_load_4d(sbase + L::kV + s * L::kSubBytes, &mapV, bar(kFBarKV), s * 64, h, k0, b);
             }
         }
+        // without a depth part this grid starts beside the prep kernel, which writes D_t and clears the dQ accumulator
+        if (!p.beside_rows) grid_dependency_wait();
         const float inv_scale = 1.f / p.scale;
         int hq = h * p.G, qrow0 = k0;
 #pragma unroll 1
@@ -1084,6 +1097,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 
     tc_fence_before_sync();
     __syncthreads();
+    grid_launch_dependents();                          // the finish kernel may come up
     abort_teardown(abort_flag, 256);
     __syncthreads();
     if (warp == W_S) tmem_dealloc(tmem, kTmemCols);

@@ -259,3 +259,31 @@ def test_forward_and_backward_replayed_from_a_graph(B, T, H, d, l, e4m3):
         torch.cuda.synchronize()
         assert moda.moda_last_status() == 0
         assert_same_gradients(got, want, f"{(B, T, H, d, l, e4m3)}")
+
+
+@pytest.mark.parametrize("B,T,H,Hk,d,l", [(1, 1, 1, 1, 64, 0), (1, 100, 2, 2, 64, 0), (1, 129, 2, 2, 128, 0), (2, 512, 16, 16, 128, 0),
+                                          (2, 513, 8, 8, 128, 5), (4, 300, 16, 16, 64, 3), (1, 640, 8, 1, 64, 12), (2, 400, 4, 2, 128, 0)])
+def test_overlapping_launches_find_what_the_ones_in_front_of_them_write(B, T, H, Hk, d, l):
+    """The launches of a backward overlap at their ends; the stages called one by one do not.  The scratch holds NaN before each call."""
+    x = synthetic.make_gqa(B, T, H, Hk, d, l, seed=91, device="cuda")
+    cache = moda.alloc_depth_cache(B, T, Hk, d, max(l, 1))
+    for i in range(l):
+        moda.moda_depth_cache_append(cache, i, x["Kd"][i].contiguous(), x["Vd"][i].contiguous())
+    scale = d ** -0.5
+    O, LSE = moda.moda_attn_fwd_gqa(x["Q"], x["K"], x["V"], cache, l, scale)
+    ws = torch.empty(moda.moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l) // 4, dtype=torch.float32, device="cuda")
+    grads = [moda.alloc_depth_cache(B, T, Hk, d, max(l, 1)).zero_() for _ in range(2)]
+    call = lambda out, **kw: moda.moda_attn_bwd_gqa(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, scale, workspace=ws, **out, **kw)
+    want = dict(dQ=torch.empty_like(x["Q"]), dK=torch.empty_like(x["K"]), dV=torch.empty_like(x["V"]), d_depth_kv=grads[0])
+    ws.fill_(float("nan"))
+    for stage in (1, 2, 4):
+        call(want, stages=stage)
+    for repeat in range(10):
+        got = {k: torch.full_like(v, float("nan")) for k, v in want.items() if k != "d_depth_kv"}
+        got["d_depth_kv"] = grads[1]
+        ws.fill_(float("nan"))
+        call(got)
+        assert moda.moda_last_status() == 0
+        for k in ("dK", "dV", "d_depth_kv"):
+            assert torch.equal(got[k], want[k]), (k, repeat)
+        assert_same_gradients((got["dQ"],), (want["dQ"],), f"dQ, repeat {repeat}")
