@@ -1097,9 +1097,9 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 
     tc_fence_before_sync();
     __syncthreads();
-    grid_launch_dependents();                          // the finish kernel may come up
     abort_teardown(abort_flag, 256);
     __syncthreads();
+    grid_launch_dependents();                          // the finish kernel may come up
     if (warp == W_S) tmem_dealloc(tmem, kTmemCols);
     // what follows on the stream reads the accumulator and the depth gradients: this grid ends after the rows kernel has
     if (last_cta) grid_dependency_wait();
