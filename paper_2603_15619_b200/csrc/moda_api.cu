@@ -435,8 +435,8 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
 // T = 8192, l = 16, B = 2: 34 2167, 36 2057, 38 1979, 40 2000, 44 1994 (taken: 40); T = 4096, l = 23, B = 4: 66 1664,
 // 70 1602, 74 1619, 78 1634 (72).  e4m3: T = 5000, l = 23, B = 2: 64 1111, 68 1075, 72 1086, 76 1099 (70); T = 8192, l = 16: 38 1962, 42 1882,
 // 46 1965 (42); T = 32768, l = 24: 18 11551, 20 11102, 24 11776 (20).  Within 3.4 % of the best count everywhere but in
-// two places: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347) and T = 65536, where 16 are taken and 10 would be best (l = 24:
-// 45.3 against 43.8 ms; at T = 32768, l = 8 16 and 12 are 11.1 and 10.9).
+// one place: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347).  At least 16: with x from 3 to 12 every count from x + 15 % to 20 is within
+// 1 % (18 shapes, counts in shuffled order; T = 65536, l = 24: 10 45.1, 16 45.4, 20 45.3 ms), and up to three too few cost 10-20 %.
 // d = 64, ten shapes, within 2 % of the best; bf16: T = 1024, l = 30, B = 4, 16 heads (256 units): 86 201, 96 206, 102 212, 110 223 (86); T = 4096, l = 23, B = 4, 16 heads:
 // 56 932, 60 874, 64 861, 68 878 (60); T = 8192, l = 16, B = 2, 32 heads: 30 2144, 32 2041, 34 1972, 38 2028 (34); T = 16384, l = 32, 32 heads: 32 3957,
 // 36 3646, 40 3663 (36); T = 32768, l = 32, 32 heads: 18 13600, 20 12386, 22 12938 (20); e4m3: T = 5000, l = 23, B = 2, 32 heads: 56 1157, 60 1143,
@@ -518,7 +518,9 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
             if (int rc = device_sm_count(&sms)) return rc;
             const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, units, unsigned(sms), a.fp8_cache) : std::min(units, unsigned(sms));
             const size_t smem = a.fp8_cache ? RowsSmem<D, true>::kDynamic : RowsSmem<D, false>::kDynamic;
-            if (!launch_beside(a.fp8_cache ? bwd_rows_kernel<D, true> : bwd_rows_kernel<D, false>, grid, 512, smem, true, stream, mQ, mdO, r)) return MODA_ERR_CUDA;
+            // not beside the prep kernel: its CTAs would take SMs as those come free, one of a pair here and there, and the others of
+            // these pairs slow it down (d = 64, B = 2, T = 5000, 32 heads, l = 23, e4m3: 1150 -> 1311 us)
+            if (!launch_beside(a.fp8_cache ? bwd_rows_kernel<D, true> : bwd_rows_kernel<D, false>, grid, 512, smem, false, stream, mQ, mdO, r)) return MODA_ERR_CUDA;
         }
     }
     if (stages & 2) {

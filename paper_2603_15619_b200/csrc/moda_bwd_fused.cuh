@@ -88,10 +88,10 @@ bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __rest
 // =====================================================================================
 // 3. dQ = bf16(scale * accumulator)
 // =====================================================================================
-// The launches of a backward overlap at their ends (programmatic dependent launch): a grid comes up while the one in front of
-// it finishes, and waits for it before it touches D_t, the accumulator or the depth gradients.  Whole backward, graph
-// replays, us, T = 100, l = 0, d = 64, 2 heads: 13.0 -> 10.9; 2 x 512, 16 heads, d = 128, l = 0: 24.0 -> 22.7; 2 x 1000, l = 0: 55.2 -> 54.1;
-// T = 2000, 16 heads on 4, d = 64, l = 12: 119.3 -> 116.2; with row-local slots between 0 and 1 us, from T = 4096 on nothing.  The
+// The launches of a backward overlap at their ends (programmatic dependent launch): this kernel, and a sequence part without
+// a depth part before it, come up while the grid in front of them finishes and wait for it before they touch D_t or the accumulator.  Whole
+// backward, graph replays, us, T = 100, l = 0, d = 64, 2 heads: 13.0 -> 10.9; 2 x 512, 16 heads, d = 128, l = 0: 24.0 -> 22.7; 2 x 1000, l = 0:
+// 55.2 -> 54.1; T = 2000, 16 heads on 4, d = 64, l = 12: 119.3 -> 116.2; T = 1000, 8 heads, l = 7, e4m3 33.0 -> 32.6; from T = 4096 on nothing.  The
 // sequence part lets this kernel start at the END of its CTAs: from their start on, its CTAs filled the few SMs that
 // had no work in the last wave and did theirs there, four to an SM (2 x 1000, l = 0: 59.8; T = 512: 29.5).
 template <int D>
@@ -175,9 +175,6 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
     constexpr int PARTS = D / 32, TPU = R::kTilesPerUnit, NSUB = D / 64;
     constexpr int RW = 32 / PARTS;                     // rows per warp
     constexpr int CH = D / 8;
-    // D_t and the cleared accumulator.  Every thread, before anything else: the sequence part, which this lets start, then finds
-    // both, and no grid of a call ends before the one in front of it.  (The first ring loads ahead of the wait: no faster.)
-    grid_dependency_wait();
     grid_launch_dependents();                          // the sequence part may take the SMs that this grid leaves
     if (g_moda_status != 0) return;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
