@@ -437,10 +437,12 @@ inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
 // 46 1965 (42); T = 32768, l = 24: 18 11551, 20 11102, 24 11776 (20).  Within 3.4 % of the best count everywhere but in
 // one place: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347).  At least 16: with x from 3 to 12 every count from x + 15 % to 20 is within
 // 1 % (18 shapes, counts in shuffled order; T = 65536, l = 24: 10 45.1, 16 45.4, 20 45.3 ms), and up to three too few cost 10-20 %.
-// d = 64, ten shapes, within 2 % of the best; bf16: T = 1024, l = 30, B = 4, 16 heads (256 units): 86 201, 96 206, 102 212, 110 223 (86); T = 4096, l = 23, B = 4, 16 heads:
-// 56 932, 60 874, 64 861, 68 878 (60); T = 8192, l = 16, B = 2, 32 heads: 30 2144, 32 2041, 34 1972, 38 2028 (34); T = 16384, l = 32, 32 heads: 32 3957,
-// 36 3646, 40 3663 (36); T = 32768, l = 32, 32 heads: 18 13600, 20 12386, 22 12938 (20); e4m3: T = 5000, l = 23, B = 2, 32 heads: 56 1157, 60 1143,
-// 64 1183 (60); T = 32768, l = 32: 20 12828, 22 12598, 24 12922 (22).
+// d = 64 (counts in shuffled order, 9 to 11 rounds), bf16: T = 1024,
+// l = 30, B = 4, 16 heads (256 units): 84 236, 86 202, 96 203 (86); T = 4096, l = 23, B = 4, 16 heads: 56 965, 60 911, 64 881, 70 894 (70); T = 8192, l = 16, B = 2, 32
+// heads: 32 2271, 34 2186, 36 2227, 40 2236 (36); T = 16384, l = 32, 32 heads: 34 4299, 36 4186, 38 4212, 44 4183 (38); T = 32768, l = 32, 32 heads: 18 15691,
+// 20 14487, 22 13729, 24 13972, 28 13601 (22); T = 65536, l = 60, 16 heads: 18 27895, 20 27103, 22 26983 (20); e4m3: T = 5000, l = 23, B = 2, 32 heads: 58 1194, 62 1194,
+// 68 1207 (62); T = 32768, l = 32: 20 14715, 22 13607, 24 13220, 28 13456 (24).  Whole backward with 1.1 x + 2 for 1.06 x + 1: T = 32768, l = 32 14.11 ->
+// 13.81 ms, T = 65536, l = 60 28.87 -> 26.56, T = 3000, l = 12 473 -> 461 us, six more shapes within noise; at d = 128 no difference.
 inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms, bool fp8) {
     const double nq = num_tiles(T);
     const double depth = double(units) * (l + 1) * (fp8 ? 1.9 : 1.7);
@@ -448,7 +450,7 @@ inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, 
     const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.36 * n : 12.0 + (0.66 + 0.00035 * n) * n);
     const double x = sms * depth / (depth + seq);
     const auto even = [](double c) { return 2 * unsigned(std::ceil(c / 2)); };
-    unsigned share = std::max(16u, even(1.06 * x + 1.0));
+    unsigned share = std::max(16u, even(d == 128 ? 1.06 * x + 1.0 : 1.1 * x + 2.0));
     // few units for each SM: what counts is how many the busiest one has
     const unsigned rounds = (units + share - 1) / share;
     if (rounds > 1 && rounds <= 16) {
