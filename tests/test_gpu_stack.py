@@ -111,6 +111,9 @@ def test_backward_that_takes_up_a_slot_of_the_gradient_cache(B, T, H, Hk, d, l, 
     got = moda.moda_attn_bwd_gqa_slot(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, scale, grads, slot)
     assert moda.moda_last_status() == 0
     assert torch.equal(grads, other)                                         # slots < l alike, the others untouched
+    # the general form of the binding (a stream is named): the same kernels
+    more = moda.moda_attn_bwd_gqa_slot(x["Q"], x["K"], x["V"], cache, O, x["dO"], LSE, l, scale, grads, slot, stream=torch.cuda.current_stream())
+    assert torch.equal(more[1], got[1]) and torch.equal(more[2], got[2])
     assert_same_gradients(got[:1], (dQ,), "dQ with and without a slot")
     for new, plain, more in zip(got[1:], (dK, dV), add[2 * slot:]):
         want = plain.double() + more.double()
