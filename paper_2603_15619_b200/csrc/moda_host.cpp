@@ -216,17 +216,23 @@ PyObject* attn_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 // ---- the differentiable call ------------------------------------------------------------------------------------------
+constexpr const char* kBadShapes = "K and V must be bf16 [B, T, H_kv, d] tensors matching Q's B, T and d";
+void addressable(const Tensor& t) {
+    TORCH_CHECK_VALUE(t.defined() && t.is_cuda(), "device (CUDA) tensors required");
+    TORCH_CHECK_VALUE(t.is_contiguous(), "contiguous tensors required");
+}
 struct Attention : torch::autograd::Function<Attention> {
     static torch::autograd::variable_list forward(torch::autograd::AutogradContext* ctx, const Tensor& Q_, const Tensor& K_, const Tensor& V_,
                                                   const std::optional<Tensor>& depth_, int64_t l, double scale) {
         const Tensor Q = Q_.contiguous(), K = K_.contiguous(), V = V_.contiguous(), depth = l > 0 ? *depth_ : Tensor();
         Shape s;
-        shapes(Q, K, V, s);
+        TORCH_CHECK_VALUE(shapes(Q, K, V, s), kBadShapes);
         Tensor O, LSE;
         ::forward(s, Q, K, V, l > 0 ? &depth : nullptr, int(l), float(scale), nullptr, 0, O, LSE);
         ctx->save_for_backward({Q, K, V, depth, O, LSE});
         ctx->saved_data["l"] = l;
         ctx->saved_data["scale"] = scale;
+        if (l > 0) ctx->saved_data["type"] = int64_t(depth.scalar_type());
         ctx->mark_non_differentiable({LSE});
         ctx->set_materialize_grads(false);                     // nothing to fill for LSE
         return {O, LSE};
@@ -236,9 +242,19 @@ struct Attention : torch::autograd::Function<Attention> {
         const Tensor &Q = saved[0], &K = saved[1], &V = saved[2], &depth = saved[3], &O = saved[4], &LSE = saved[5];
         const int l = int(ctx->saved_data["l"].toInt());
         const float scale = float(ctx->saved_data["scale"].toDouble());
-        Shape s;
-        shapes(Q, K, V, s);
         const Tensor dO = grads[0].defined() ? grads[0].contiguous() : at::zeros_like(O);
+        // Saved-tensor hooks may hand back anything, and torch does not look at it: every tensor again, before a kernel gets its address.
+        Shape s;
+        for (const Tensor* t : {&Q, &K, &V, &O, &LSE, &dO}) addressable(*t);
+        TORCH_CHECK_VALUE(shapes(Q, K, V, s), kBadShapes);
+        TORCH_CHECK_VALUE(O.scalar_type() == at::kBFloat16 && O.numel() >= Q.numel() && dO.scalar_type() == at::kBFloat16 && dO.numel() >= Q.numel(),
+                          "O and its gradient must be bf16 tensors of Q's size");
+        TORCH_CHECK_VALUE(LSE.scalar_type() == at::kFloat && LSE.numel() >= int64_t(s.B) * s.H * s.T, "LSE must be an fp32 tensor of B H T elements");
+        if (l > 0) {
+            addressable(depth);
+            TORCH_CHECK_VALUE(int64_t(depth.scalar_type()) == ctx->saved_data["type"].toInt(), "depth_kv has changed its type");
+            TORCH_CHECK_VALUE(bytes_of(depth) >= lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l), "depth_kv holds fewer than l slots");
+        }
         Tensor dQ, dK, dV, dcache, ws;
         if (l > 0) {
             // the kernels write every element of slots < l; later slots of the caller's cache get no gradient

@@ -215,6 +215,27 @@ def test_differentiable_call_behaves_as_the_general_one(general, l):
     assert moda.moda_last_status() == 0
 
 
+UNPACKED = {"host memory": lambda t: t.cpu(), "strides": lambda t: t.repeat_interleave(2, -1)[..., ::2], "type": lambda t: t.double(),
+            "size": lambda t: t.flatten()[:t.numel() // 2], "shape": lambda t: t.flatten()[:64]}
+
+
+@gpu
+@pytest.mark.parametrize("how", UNPACKED)
+def test_what_a_saved_tensor_hook_hands_back_is_looked_at(how):
+    """Refused before anything is launched, whichever of the six saved tensors it is."""
+    for which in range(6):
+        x, cache = [t.requires_grad_() for t in _qkv(1, 130, 4, 2, 64)[:3]], _cache(1, 130, 2, 64, 2, 3)
+        seen = []
+        pack = lambda t: (seen.append(t), len(seen) - 1)[1]
+        unpack = lambda i: UNPACKED[how](seen[i].detach()) if i == which else seen[i]
+        with torch.autograd.graph.saved_tensors_hooks(pack, unpack):
+            O, _ = moda.moda_attention(*x, cache, 2)
+        assert len(seen) == 6
+        with pytest.raises(ValueError):
+            O.backward(torch.ones_like(O))
+    assert moda.moda_last_status() == 0
+
+
 @gpu
 def test_streams_and_threads():
     """A call follows the current stream, in threads of their own too, and outputs belong to it."""
