@@ -146,8 +146,7 @@ void backward(const Shape& s, const Tensor& Q, const Tensor& K, const Tensor& V,
     if (!dK.defined()) dK = like(K);
     if (!dV.defined()) dV = like(V);
     if (l > 0 && !dcache.defined()) {
-        const size_t n = lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l);
-        dcache = fresh({std::max<int64_t>(int64_t(n / 2), 8)}, at::kBFloat16, Q);
+        dcache = fresh({int64_t(lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l) / 2)}, at::kBFloat16, Q);
     }
     if (!ws.defined()) ws = fresh({int64_t(lib.moda_bwd_workspace_bytes_gqa(s.B, s.T, s.H, s.Hk, s.d, l))}, at::kByte, Q);
     const void* dep = l > 0 ? ptr(depth) : nullptr;
@@ -204,6 +203,8 @@ PyObject* attn_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!optional_dense(a[4], O) || !optional_dense(a[5], dO) || !optional_dense(a[6], LSE) || O == nullptr || dO == nullptr || LSE == nullptr) return none();
     for (int i = 0; i < 5; ++i)
         if (!optional_dense(a[9 + i], g[i])) return none();
+    // no gradient cache can be made for this width or so many slots: the Python form says so
+    if (l > 0 && g[3] == nullptr && lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l) == 0) return none();
     Tensor t[5];
     for (int i = 0; i < 5; ++i)
         if (g[i] != nullptr) t[i] = *g[i];

@@ -123,6 +123,16 @@ def test_wrong_arguments_are_refused_as_before(general):
            lambda: moda.moda_attn_fwd_gqa(Q.transpose(2, 3), K, V, None, 0, 0.1), lambda: moda.moda_attn_fwd_gqa(Q[..., :32], K[..., :32], V[..., :32], None, 0, 0.1),
            lambda: moda.moda_attention(Q, K, V, None, 2), lambda: moda.moda_attention(Q, K.float(), V), lambda: moda.moda_attn_fwd_gqa(Q, K, V, None, -1, 0.1),
            lambda: moda.moda_attn_fwd_append(Q, K, V, None, 0, 0.1, None, 0), lambda: moda.moda_attn_decode(Q[:, 0], K, V, None, 65, 0, 0.1)]
+    # backward: no gradient cache for 257 slots or 32 features, a scale, a stage mask, tensors that are missing or of another type or strides
+    LSE, cache = torch.zeros(1, 2, 64, device="cuda"), _cache(1, 64, 2, 64, 2, 3)
+    narrow = [t[..., :32].contiguous() for t in (Q, K, V)]
+    bwd = lambda q=Q, k=K, v=V, depth=cache, O=dO, g=dO, lse=LSE, l=1, scale=0.1, **kw: moda.moda_attn_bwd_gqa(q, k, v, depth, O, g, lse, l, scale, **kw)
+    slot = lambda g=dO, l=1, grads=cache, at=2, **kw: moda.moda_attn_bwd_gqa_slot(Q, K, V, cache, dO, g, LSE, l, 0.1, grads, at, **kw)
+    bad += [lambda: bwd(l=257), lambda: bwd(*narrow, O=narrow[0], g=narrow[0]), lambda: bwd(l=-1), lambda: bwd(scale=-1.0), lambda: bwd(stages=0),
+            lambda: bwd(stages=64), lambda: bwd(depth=None), lambda: bwd(O=None), lambda: bwd(g=dO.cpu()), lambda: bwd(g=dO.transpose(1, 2)),
+            lambda: bwd(q=Q.float()), lambda: bwd(k=K[:, :32]), lambda: bwd(l=257, d_depth_kv=cache), lambda: bwd(workspace=LSE),
+            lambda: slot(at=0), lambda: slot(at=-1), lambda: slot(at=256), lambda: slot(grads=None), lambda: slot(l=257), lambda: slot(g=dO.cpu()),
+            lambda: slot(workspace=LSE)]
     for i, f in enumerate(bad):
         want = general(_errors, f)
         assert want is not None and _errors(f) is want, (i, want, _errors(f))
