@@ -172,6 +172,31 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _sized(t, numel, dtype):
+    """Address of a tensor that a kernel reads or writes ``numel`` elements of type ``dtype`` of."""
+    if t is not None and (t.dtype != dtype or t.numel() < numel):
+        raise ValueError(f"{numel} elements of type {dtype} required, not {t.numel()} of type {t.dtype}")
+    return _ptr(t)
+
+
+def _bf16(t, numel):
+    return _sized(t, numel, torch.bfloat16)
+
+
+def _f32(t, numel):
+    return _sized(t, numel, torch.float32)
+
+
+def _slots(cache, n, *shape, e4m3=False):
+    """Address of a depth cache, or of its gradient, that holds at least ``n`` slots of ``shape`` = B, T, H_kv, d (a number of slots
+    that no cache has is the C call's to refuse)."""
+    if cache is not None:
+        need = (moda_depth_cache_e4m3_bytes if e4m3 else moda_depth_cache_bytes)(*shape, max(0, min(n, MODA_MAX_DEPTH + 1)))
+        if cache.numel() * cache.element_size() < need:
+            raise ValueError(f"{n} slots of this shape take {need} bytes, the depth cache has {cache.numel() * cache.element_size()}")
+    return _ptr(cache)
+
+
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
@@ -266,14 +291,16 @@ def depth_cache_window(cache, B, T, H, d, first_slot, n_slots=None):
 def moda_depth_cache_append(cache, slot, K_i, V_i, stream=None):
     B, T, H, d = _bthd(K_i, "K_i")
     assert _bthd(V_i, "V_i") == (B, T, H, d)
-    _check(load().moda_depth_cache_append(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+    _check(load().moda_depth_cache_append(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
+                                          _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
            "moda_depth_cache_append")
 
 
 def moda_depth_cache_unpack(cache, slot, K_i, V_i, stream=None):
     ref = K_i if K_i is not None else V_i
     B, T, H, d = _bthd(ref, "K_i/V_i")
-    _check(load().moda_depth_cache_unpack(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+    _check(load().moda_depth_cache_unpack(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
+                                          _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
            "moda_depth_cache_unpack")
 
 
@@ -281,7 +308,8 @@ def moda_depth_cache_unpack_add(cache, slot, K_i, V_i, stream=None):
     """K_i, V_i += slot ``slot`` of a (gradient) cache, each sum rounded to bf16 once."""
     ref = K_i if K_i is not None else V_i
     B, T, H, d = _bthd(ref, "K_i/V_i")
-    _check(load().moda_depth_cache_unpack_add(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+    _check(load().moda_depth_cache_unpack_add(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
+                                              _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
            "moda_depth_cache_unpack_add")
 
 
@@ -301,7 +329,8 @@ def moda_depth_cache_append_e4m3(cache, slot, K_i, V_i, stream=None):
     """Quantise K_i, V_i (bf16 [B,T,H,d]) into slot ``slot`` of an e4m3 depth cache (codes + one fp32 scale per row)."""
     B, T, H, d = _bthd(K_i, "K_i")
     assert _bthd(V_i, "V_i") == (B, T, H, d)
-    _check(load().moda_depth_cache_append_e4m3(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+    _check(load().moda_depth_cache_append_e4m3(_slots(cache, int(slot) + 1, B, T, H, d, e4m3=True), B, T, H, d, int(slot),
+                                               _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
            "moda_depth_cache_append_e4m3")
 
 
@@ -312,8 +341,8 @@ def moda_attn_fwd_e4m3(Q, K, V, depth_kv_e4m3, l, scale, O=None, LSE=None, strea
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd_e4m3(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv_e4m3) if l > 0 else None,
-                                     B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
+    _check(load().moda_attn_fwd_e4m3(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_e4m3, int(l), B, T, Hk, d, e4m3=True) if l > 0 else None,
+                                     B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
            "moda_attn_fwd_e4m3")
     return O, LSE
 
@@ -325,9 +354,9 @@ def moda_attn_fwd_append_e4m3(Q, K, V, depth_kv_e4m3, l, scale, append_cache_e4m
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd_append_e4m3(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv_e4m3) if l > 0 else None,
-                                            B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
-                                            _ptr(append_cache_e4m3), int(append_slot), _stream(stream)),
+    _check(load().moda_attn_fwd_append_e4m3(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_e4m3, int(l), B, T, Hk, d, e4m3=True) if l > 0 else None,
+                                            B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T),
+                                            _slots(append_cache_e4m3, int(append_slot) + 1, B, T, Hk, d, e4m3=True), int(append_slot), _stream(stream)),
            "moda_attn_fwd_append_e4m3")
     return O, LSE
 
@@ -343,9 +372,11 @@ def moda_attn_bwd_e4m3(Q, K, V, depth_kv_e4m3, O, dO, LSE, l, scale,
         d_depth_kv = alloc_depth_cache(B, T, H, d, l, Q.device, stream)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes(B, T, H, d, l),), torch.uint8, Q.device, stream)
-    _check(load().moda_attn_bwd_e4m3(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv_e4m3) if l > 0 else None,
-                                     _ptr(O), _ptr(dO), _ptr(LSE), B, T, H, d, int(l), float(scale),
-                                     _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv) if l > 0 else None,
+    _check(load().moda_attn_bwd_e4m3(_ptr(Q), _bf16(K, Q.numel()), _bf16(V, Q.numel()),
+                                     _slots(depth_kv_e4m3, int(l), B, T, H, d, e4m3=True) if l > 0 else None,
+                                     _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
+                                     _bf16(dQ, Q.numel()), _bf16(dK, Q.numel()), _bf16(dV, Q.numel()),
+                                     _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
                                      _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_bwd_e4m3")
     return dQ, dK, dV, d_depth_kv
@@ -355,14 +386,16 @@ def moda_depth_cache_append_pm(cache, slot, K_i, V_i, stream=None):
     """moda_depth_cache_append for the position-major layout (grouped-query calls through the *_pm entry points)."""
     B, T, H, d = _bthd(K_i, "K_i")
     assert _bthd(V_i, "V_i") == (B, T, H, d)
-    _check(load().moda_depth_cache_append_pm(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+    _check(load().moda_depth_cache_append_pm(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
+                                             _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
            "moda_depth_cache_append_pm")
 
 
 def moda_depth_cache_unpack_pm(cache, slot, K_i, V_i, stream=None):
     ref = K_i if K_i is not None else V_i
     B, T, H, d = _bthd(ref, "K_i/V_i")
-    _check(load().moda_depth_cache_unpack_pm(_ptr(cache), B, T, H, d, int(slot), _ptr(K_i), _ptr(V_i), _stream(stream)),
+    _check(load().moda_depth_cache_unpack_pm(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
+                                             _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
            "moda_depth_cache_unpack_pm")
 
 
@@ -373,8 +406,8 @@ def moda_attn_fwd_gqa_pm(Q, K, V, depth_kv_pm, l, scale, O=None, LSE=None, strea
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd_gqa_pm(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv_pm) if l > 0 else None,
-                                       B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
+    _check(load().moda_attn_fwd_gqa_pm(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_pm, int(l), B, T, Hk, d) if l > 0 else None,
+                                       B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
            "moda_attn_fwd_gqa_pm")
     return O, LSE
 
@@ -390,9 +423,10 @@ def moda_attn_bwd_gqa_pm(Q, K, V, depth_kv_pm, O, dO, LSE, l, scale,
         d_depth_kv_pm = alloc_depth_cache(B, T, Hk, d, l, Q.device, stream)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
-    _check(load().moda_attn_bwd_gqa_pm(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv_pm) if l > 0 else None,
-                                       _ptr(O), _ptr(dO), _ptr(LSE), B, T, H, Hk, d, int(l), float(scale),
-                                       _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv_pm) if l > 0 else None,
+    _check(load().moda_attn_bwd_gqa_pm(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_pm, int(l), B, T, Hk, d) if l > 0 else None,
+                                       _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, Hk, d, int(l), float(scale),
+                                       _bf16(dQ, Q.numel()), _bf16(dK, K.numel()), _bf16(dV, K.numel()),
+                                       _slots(d_depth_kv_pm, int(l), B, T, Hk, d) if l > 0 else None,
                                        _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_bwd_gqa_pm")
     return dQ, dK, dV, d_depth_kv_pm
@@ -416,8 +450,9 @@ def moda_kv_project_append(X, Wk, Wv, H_kv, cache=None, slot=0, store_kv=True, K
     else:
         K_out = V_out = None
     fn = load().moda_kv_project_append_e4m3 if e4m3 else load().moda_kv_project_append
-    _check(fn(_ptr(X), _ptr(Wk), _ptr(Wv), B, T, Dm, int(H_kv), d, _ptr(K_out), _ptr(V_out),
-              _ptr(cache), int(slot), _stream(stream)), "moda_kv_project_append_e4m3" if e4m3 else "moda_kv_project_append")
+    _check(fn(_ptr(X), _ptr(Wk), _ptr(Wv), B, T, Dm, int(H_kv), d, _bf16(K_out, B * T * n), _bf16(V_out, B * T * n),
+              _slots(cache, int(slot) + 1, B, T, int(H_kv), d, e4m3=e4m3), int(slot), _stream(stream)),
+           "moda_kv_project_append_e4m3" if e4m3 else "moda_kv_project_append")
     return K_out, V_out
 
 
@@ -436,8 +471,8 @@ def moda_depth_slot_mass(Q, depth_kv, LSE, l, scale, H_kv=None, mass=None, works
     need = int(load().moda_depth_slot_mass_workspace_bytes(B, T, H, int(l)))
     if workspace is None:
         workspace = _new((max(need, 16),), torch.uint8, Q.device, stream)
-    _check(load().moda_depth_slot_mass(_ptr(Q), _ptr(depth_kv) if l > 0 else None, _ptr(LSE), B, T, H, H_kv, d, int(l),
-                                       float(scale), _ptr(mass), _ptr(workspace), workspace.numel() * workspace.element_size(),
+    _check(load().moda_depth_slot_mass(_ptr(Q), _slots(depth_kv, int(l), B, T, H_kv, d) if l > 0 else None, _f32(LSE, B * H * T),
+                                       B, T, H, H_kv, d, int(l), float(scale), _f32(mass, B * H * int(l)), _ptr(workspace), workspace.numel() * workspace.element_size(),
                                        _stream(stream)), "moda_depth_slot_mass")
     return mass
 
@@ -450,8 +485,8 @@ def moda_attn_fwd(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=None):
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None,
-                                B, T, H, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
+    _check(load().moda_attn_fwd(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
+                                B, T, H, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
            "moda_attn_fwd")
     return O, LSE
 
@@ -474,9 +509,9 @@ def moda_attn_bwd(Q, K, V, depth_kv, O, dO, LSE, l, scale,
     need = moda_bwd_workspace_bytes(B, T, H, d, l)
     if workspace is None:
         workspace = _new((need,), torch.uint8, Q.device, stream)
-    args = [_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None,
-            _ptr(O), _ptr(dO), _ptr(LSE), B, T, H, d, int(l), float(scale),
-            _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv) if l > 0 else None,
+    args = [_ptr(Q), _bf16(K, Q.numel()), _bf16(V, Q.numel()), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
+            _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
+            _bf16(dQ, Q.numel()), _bf16(dK, Q.numel()), _bf16(dV, Q.numel()), _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
             _ptr(workspace), workspace.numel() * workspace.element_size()]
     if stages is None:
         _check(load().moda_attn_bwd(*args, _stream(stream)), "moda_attn_bwd")
@@ -502,8 +537,9 @@ def moda_attn_bwd_static_scratch(Q, K, V, depth_kv, O, dO, LSE, l, scale, dQ, dK
     if l > 0 and d_depth_kv is None:
         raise ValueError("d_depth_kv must be provided: this entry point allocates nothing")
     _check(load().moda_attn_bwd_static_scratch(
-        _ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None, _ptr(O), _ptr(dO), _ptr(LSE),
-        B, T, H, d, int(l), float(scale), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv) if l > 0 else None,
+        _ptr(Q), _bf16(K, Q.numel()), _bf16(V, Q.numel()), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
+        _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
+        _bf16(dQ, Q.numel()), _bf16(dK, Q.numel()), _bf16(dV, Q.numel()), _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
         _stream(stream)), "moda_attn_bwd_static_scratch")
     return dQ, dK, dV, d_depth_kv
 
@@ -531,8 +567,8 @@ def moda_attn_fwd_gqa(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=None
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd_gqa(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None,
-                                    B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
+    _check(load().moda_attn_fwd_gqa(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
+                                    B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
            "moda_attn_fwd_gqa")
     return O, LSE
 
@@ -549,9 +585,9 @@ def moda_attn_fwd_append(Q, K, V, depth_kv, l, scale, append_cache, append_slot,
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd_append(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None,
-                                       B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
-                                       _ptr(append_cache), int(append_slot), _stream(stream)),
+    _check(load().moda_attn_fwd_append(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
+                                       B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T),
+                                       _slots(append_cache, int(append_slot) + 1, B, T, Hk, d), int(append_slot), _stream(stream)),
            "moda_attn_fwd_append")
     return O, LSE
 
@@ -573,9 +609,9 @@ def moda_attn_bwd_gqa(Q, K, V, depth_kv, O, dO, LSE, l, scale,
         d_depth_kv = alloc_depth_cache(B, T, Hk, d, l, Q.device, stream)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
-    args = [_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None,
-            _ptr(O), _ptr(dO), _ptr(LSE), B, T, H, Hk, d, int(l), float(scale),
-            _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv) if l > 0 else None,
+    args = [_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
+            _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, Hk, d, int(l), float(scale),
+            _bf16(dQ, Q.numel()), _bf16(dK, K.numel()), _bf16(dV, K.numel()), _slots(d_depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
             _ptr(workspace), workspace.numel() * workspace.element_size()]
     if stages is None:
         _check(load().moda_attn_bwd_gqa(*args, _stream(stream)), "moda_attn_bwd_gqa")
@@ -607,8 +643,10 @@ def moda_attn_bwd_gqa_slot(Q, K, V, depth_kv, O, dO, LSE, l, scale, d_depth_kv, 
     dV = _new_like(V, stream) if dV is None else dV
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
-    _check(load().moda_attn_bwd_gqa_slot(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None, _ptr(O), _ptr(dO), _ptr(LSE),
-                                         B, T, H, Hk, d, int(l), float(scale), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(d_depth_kv),
+    _check(load().moda_attn_bwd_gqa_slot(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
+                                         _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T),
+                                         B, T, H, Hk, d, int(l), float(scale), _bf16(dQ, Q.numel()), _bf16(dK, K.numel()), _bf16(dV, K.numel()),
+                                         _slots(d_depth_kv, int(slot) + 1, B, T, Hk, d),
                                          _ptr(workspace), workspace.numel() * workspace.element_size(), int(slot), _stream(stream)),
            "moda_attn_bwd_gqa_slot")
     return dQ, dK, dV
@@ -639,7 +677,7 @@ def moda_attn_decode(q, K, V, depth_kv_token, T_kv, l, scale, O=None, LSE=None, 
     if workspace is None:
         workspace = _new((moda_decode_workspace_bytes(B, H, d),), torch.uint8, q.device, stream)
     _check(load().moda_attn_decode(_ptr(q), _ptr(K), _ptr(V), _ptr(depth_kv_token) if l > 0 else None,
-                                   B, int(T_kv), T_cap, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
+                                   B, int(T_kv), T_cap, H, Hk, d, int(l), float(scale), _bf16(O, B * H * d), _f32(LSE, B * H),
                                    _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_decode")
     return O, LSE
@@ -656,8 +694,8 @@ def moda_attn_fwd_prefill(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=
         O = _new_like(Q, stream)
     if LSE is None:
         LSE = _new((B, H, T_q), torch.float32, Q.device, stream)
-    _check(load().moda_attn_fwd_prefill(_ptr(Q), _ptr(K), _ptr(V), _ptr(depth_kv) if l > 0 else None,
-                                        B, T_q, T_kv, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
+    _check(load().moda_attn_fwd_prefill(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T_q, Hk, d) if l > 0 else None,
+                                        B, T_q, T_kv, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T_q),
                                         _stream(stream)), "moda_attn_fwd_prefill")
     return O, LSE
 
@@ -671,6 +709,10 @@ def _decode_outputs(q, O, LSE, workspace, stream):
     if workspace is None:
         workspace = _new((moda_decode_workspace_bytes(B, H, d),), torch.uint8, q.device, stream)
     return O, LSE, workspace
+
+
+def _token(depth_kv_token, l, B, Hk, d):
+    return _bf16(depth_kv_token, (l if l <= MODA_MAX_DEPTH else 0) * B * Hk * 2 * d) if l > 0 else None
 
 
 def _int32(t, name, shape):
@@ -688,8 +730,9 @@ def moda_attn_decode_varlen(q, K, V, seq_lens, depth_kv_token, max_seq_len, l, s
     _, T_cap, Hk, _ = _bthd(K, "K")
     _int32(seq_lens, "seq_lens", (B,))
     O, LSE, workspace = _decode_outputs(q, O, LSE, workspace, stream)
-    _check(load().moda_attn_decode_varlen(_ptr(q), _ptr(K), _ptr(V), _ptr(seq_lens), _ptr(depth_kv_token) if l > 0 else None,
-                                          B, int(max_seq_len), T_cap, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
+    _check(load().moda_attn_decode_varlen(_bf16(q, B * H * d), _bf16(K, B * T_cap * Hk * d), _bf16(V, B * T_cap * Hk * d), _ptr(seq_lens),
+                                          _token(depth_kv_token, l, B, Hk, d),
+                                          B, int(max_seq_len), T_cap, H, Hk, d, int(l), float(scale), _bf16(O, B * H * d), _f32(LSE, B * H),
                                           _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_decode_varlen")
     return O, LSE
@@ -708,10 +751,11 @@ def moda_attn_decode_paged(q, K_pages, V_pages, block_table, seq_lens, depth_kv_
     if block_table.dtype != torch.int32 or block_table.dim() != 2 or block_table.shape[0] != B:
         raise ValueError("block_table must be an int32 [B, max_blocks] tensor")
     O, LSE, workspace = _decode_outputs(q, O, LSE, workspace, stream)
-    _check(load().moda_attn_decode_paged(_ptr(q), _ptr(K_pages), _ptr(V_pages), _ptr(block_table), _ptr(seq_lens),
-                                         _ptr(depth_kv_token) if l > 0 else None,
+    _check(load().moda_attn_decode_paged(_bf16(q, B * H * d), _bf16(K_pages, num_pages * page_size * Hk * d),
+                                         _bf16(V_pages, num_pages * page_size * Hk * d), _ptr(block_table), _ptr(seq_lens),
+                                         _token(depth_kv_token, l, B, Hk, d),
                                          B, int(max_seq_len), page_size, num_pages, block_table.shape[1], H, Hk, d, int(l),
-                                         float(scale), _ptr(O), _ptr(LSE), _ptr(workspace),
+                                         float(scale), _bf16(O, B * H * d), _f32(LSE, B * H), _ptr(workspace),
                                          workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_decode_paged")
     return O, LSE

@@ -20,6 +20,7 @@
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <algorithm>
 #include <climits>
 #include <initializer_list>
 
@@ -115,6 +116,8 @@ Tensor like(const Tensor& t) { return at::empty(t.sizes(), t.options().requires_
 Tensor fresh(std::initializer_list<int64_t> shape, at::ScalarType type, const Tensor& on) {
     return at::empty(at::IntArrayRef(shape), on.options().dtype(type).requires_grad(false));
 }
+// A tensor that a kernel reads or writes n elements of, where it is given.
+bool holds(const Tensor* t, at::ScalarType type, int64_t n) { return t == nullptr || (t->scalar_type() == type && t->numel() >= n); }
 // A given tensor's own object, or the new tensor.
 PyObject* out(PyObject* given, const Tensor& made) { return given != Py_None ? Py_NewRef(given) : THPVariable_Wrap(made); }
 PyObject* none() { Py_RETURN_NONE; }
@@ -127,6 +130,10 @@ bool shapes(const Tensor& Q, const Tensor& K, const Tensor& V, Shape& s) {
     s = {int(Q.size(0)), int(Q.size(1)), int(Q.size(2)), int(K.size(2)), int(Q.size(3))};
     return K.size(0) == s.B && K.size(1) == s.T && K.size(3) == s.d && V.sizes() == K.sizes();
 }
+// Whether a depth cache, or its gradient, has n slots (a number that no cache has is the C call's to refuse).
+bool holds_slots(const Tensor* t, const Shape& s, int n) { return t == nullptr || bytes_of(*t) >= lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, n); }
+bool holds_slot(const Tensor* t, const Shape& s, int slot) { return holds_slots(t, s, std::min(slot, MODA_MAX_DEPTH) + 1); }
+int64_t rows(const Shape& s) { return int64_t(s.B) * s.H * s.T; }
 void forward(const Shape& s, const Tensor& Q, const Tensor& K, const Tensor& V, const Tensor* depth, int l, float scale,
              const Tensor* cache, int slot, Tensor& O, Tensor& LSE) {
     if (!O.defined()) O = like(Q);
@@ -178,6 +185,7 @@ PyObject* attn_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     Shape s;
     if (Q == nullptr || K == nullptr || V == nullptr || !shapes(*Q, *K, *V, s) || !optional_dense(a[3], depth) || !optional_dense(a[6], cache) ||
         !optional_dense(a[8], O) || !optional_dense(a[9], LSE)) return none();
+    if (!holds(O, at::kBFloat16, Q->numel()) || !holds(LSE, at::kFloat, rows(s)) || (l > 0 && !holds_slots(depth, s, l)) || !holds_slot(cache, s, slot)) return none();
     Tensor o = O != nullptr ? *O : Tensor(), lse = LSE != nullptr ? *LSE : Tensor();
     {
         NoGil nogil;
@@ -203,6 +211,10 @@ PyObject* attn_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!optional_dense(a[4], O) || !optional_dense(a[5], dO) || !optional_dense(a[6], LSE) || O == nullptr || dO == nullptr || LSE == nullptr) return none();
     for (int i = 0; i < 5; ++i)
         if (!optional_dense(a[9 + i], g[i])) return none();
+    const int64_t nq = Q->numel(), nk = K->numel();
+    if (!holds(O, at::kBFloat16, nq) || !holds(dO, at::kBFloat16, nq) || !holds(LSE, at::kFloat, rows(s)) || !holds(g[0], at::kBFloat16, nq) ||
+        !holds(g[1], at::kBFloat16, nk) || !holds(g[2], at::kBFloat16, nk)) return none();
+    if ((l > 0 && (!holds_slots(depth, s, l) || !holds_slots(g[3], s, l))) || (mode == kSlot && !holds_slot(g[3], s, arg))) return none();
     // no gradient cache can be made for this width or so many slots: the Python form says so
     if (l > 0 && g[3] == nullptr && lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l) == 0) return none();
     Tensor t[5];
@@ -248,13 +260,13 @@ struct Attention : torch::autograd::Function<Attention> {
         Shape s;
         for (const Tensor* t : {&Q, &K, &V, &O, &LSE, &dO}) addressable(*t);
         TORCH_CHECK_VALUE(shapes(Q, K, V, s), kBadShapes);
-        TORCH_CHECK_VALUE(O.scalar_type() == at::kBFloat16 && O.numel() >= Q.numel() && dO.scalar_type() == at::kBFloat16 && dO.numel() >= Q.numel(),
+        TORCH_CHECK_VALUE(holds(&O, at::kBFloat16, Q.numel()) && holds(&dO, at::kBFloat16, Q.numel()),
                           "O and its gradient must be bf16 tensors of Q's size");
-        TORCH_CHECK_VALUE(LSE.scalar_type() == at::kFloat && LSE.numel() >= int64_t(s.B) * s.H * s.T, "LSE must be an fp32 tensor of B H T elements");
+        TORCH_CHECK_VALUE(holds(&LSE, at::kFloat, rows(s)), "LSE must be an fp32 tensor of B H T elements");
         if (l > 0) {
             addressable(depth);
             TORCH_CHECK_VALUE(int64_t(depth.scalar_type()) == ctx->saved_data["type"].toInt(), "depth_kv has changed its type");
-            TORCH_CHECK_VALUE(bytes_of(depth) >= lib.moda_depth_cache_bytes(s.B, s.T, s.Hk, s.d, l), "depth_kv holds fewer than l slots");
+            TORCH_CHECK_VALUE(holds_slots(&depth, s, l), "depth_kv holds fewer than l slots");
         }
         Tensor dQ, dK, dV, dcache, ws;
         if (l > 0) {
@@ -278,7 +290,7 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (n != 6 || !plain_thread() || !int_arg(a[4], l) || l < 0 || !float_arg(a[5], scale)) return none();
     const Tensor *Q = plain(a[0]), *K = plain(a[1]), *V = plain(a[2]), *depth;
     Shape s;
-    if (Q == nullptr || K == nullptr || V == nullptr || !shapes(*Q, *K, *V, s) || !optional_dense(a[3], depth) || (l > 0 && depth == nullptr)) return none();
+    if (Q == nullptr || K == nullptr || V == nullptr || !shapes(*Q, *K, *V, s) || !optional_dense(a[3], depth) || (l > 0 && (depth == nullptr || !holds_slots(depth, s, l)))) return none();
     if (dual(*Q) || dual(*K) || dual(*V) || (depth != nullptr && dual(*depth))) return none();
     const Tensor q = *Q, k = *K, v = *V;
     const std::optional<Tensor> dep = depth != nullptr ? std::optional<Tensor>(*depth) : std::nullopt;
@@ -312,6 +324,7 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     }
     if (l > 0 && ((depth = dense(a[5], at::kBFloat16, 5)) == nullptr || !shape_is(*depth, {l, B, Hk, 2, d}))) return none();
     if (!optional_dense(a[9], O) || !optional_dense(a[10], LSE) || !optional_dense(a[11], ws)) return none();
+    if (!holds(O, at::kBFloat16, q->numel()) || !holds(LSE, at::kFloat, int64_t(B) * H)) return none();
     Tensor o = O != nullptr ? *O : Tensor(), lse = LSE != nullptr ? *LSE : Tensor(), w = ws != nullptr ? *ws : Tensor();
     {
         NoGil nogil;

@@ -138,6 +138,60 @@ def test_wrong_arguments_are_refused_as_before(general):
         assert want is not None and _errors(f) is want, (i, want, _errors(f))
 
 
+def _short(t):
+    return t.flatten()[:-1]
+
+
+def test_buffers_are_looked_at_before_their_address_is_taken():
+    """In host memory the check of the size and the type comes before the one of the device."""
+    x = torch.zeros(8, dtype=BF16)
+    for f, text in ((lambda: binding._bf16(x, 9), "9 elements"), (lambda: binding._bf16(x.float(), 8), "torch.bfloat16"), (lambda: binding._f32(x, 8), "torch.float32"),
+                    (lambda: binding._bf16(x, 8), "CUDA"), (lambda: binding._slots(x, 1, 1, 64, 2, 64), "65536 bytes"),
+                    (lambda: binding._slots(x, 257, 1, 64, 2, 64), "CUDA"), (lambda: binding._slots(x, -3, 1, 64, 2, 64), "CUDA"),
+                    (lambda: binding._slots(x, 1, 1, 64, 2, 64, e4m3=True), "bytes"), (lambda: binding._token(x, 2, 3, 2, 64), "1536 elements")):
+        with pytest.raises(ValueError, match=text):
+            f()
+    assert binding._bf16(None, 9) is None and binding._slots(None, 1, 1, 64, 2, 64) is None
+
+
+@gpu
+def test_buffers_that_are_too_small_or_of_another_type_are_refused(general):
+    Q, K, V, dO = _qkv(1, 64, 2, 2, 64)
+    O, LSE, cache = torch.empty_like(Q), torch.zeros(1, 2, 64, device="cuda"), _cache(1, 64, 2, 64, 2, 3)
+    cache8 = torch.zeros(moda.moda_depth_cache_e4m3_bytes(1, 64, 2, 64, 3), dtype=torch.uint8, device="cuda")
+    two = cache[:cache.numel() // 3 * 2]
+    q, tok, lens = Q[:, 0], torch.zeros(2, 1, 2, 2, 64, device="cuda", dtype=BF16), torch.tensor([9], dtype=torch.int32, device="cuda")
+    table = torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+    scale = 0.125
+    for wrong in (_short, lambda t: t.double()):
+        few = _short if wrong is _short else lambda t: t[:t.numel() // 4]     # caches: any type, enough bytes
+        calls = [lambda: moda.moda_attention(Q, K, V, few(two), 2),
+                 lambda: moda.moda_attn_decode(q, K, V, tok, 64, 2, scale, O=wrong(q)), lambda: moda.moda_attn_decode(q, K, V, tok, 64, 2, scale, LSE=wrong(LSE[:, :, 0])),
+                 lambda: moda.moda_attn_decode_varlen(q, K, V, lens, wrong(tok), 64, 2, scale), lambda: moda.moda_attn_decode_varlen(q, K, wrong(V), lens, tok, 64, 2, scale),
+                 lambda: moda.moda_attn_decode_paged(q, K, wrong(V), table, lens, tok, 64, 2, scale), lambda: moda.moda_attn_decode_paged(q, K, V, table, lens, wrong(tok), 64, 2, scale),
+                 lambda: moda.moda_depth_cache_append(few(two), 1, K, V), lambda: moda.moda_depth_cache_unpack(few(two), 1, O, O.clone()),
+                 lambda: moda.moda_depth_cache_unpack_add(cache, 1, O, wrong(V)), lambda: moda.moda_depth_cache_append_e4m3(few(cache8), 2, K, V),
+                 lambda: moda.moda_depth_slot_mass(Q, few(two), LSE, 2, scale), lambda: moda.moda_depth_slot_mass(Q, cache, wrong(LSE), 2, scale),
+                 lambda: moda.moda_kv_project_append(K.view(1, 64, 128), torch.zeros(128, 128, device="cuda", dtype=BF16), torch.zeros(128, 128, device="cuda", dtype=BF16), 2,
+                                                     cache=few(two), slot=1)]
+        for f, depth in ((moda.moda_attn_fwd_gqa, two), (moda.moda_attn_fwd, two), (moda.moda_attn_fwd_prefill, two), (moda.moda_attn_fwd_e4m3, cache8)):
+            l = 3 if depth is cache8 else 2
+            calls += [lambda f=f, depth=depth, l=l: f(Q, K, V, few(depth), l, scale), lambda f=f, depth=depth, l=l: f(Q, K, V, depth, l, scale, O=wrong(O)),
+                      lambda f=f, depth=depth, l=l: f(Q, K, V, depth, l, scale, LSE=wrong(LSE))]
+        calls += [lambda: moda.moda_attn_fwd_append(Q, K, V, None, 0, scale, few(two), 1), lambda: moda.moda_attn_fwd_append_e4m3(Q, K, V, None, 0, scale, few(cache8), 2)]
+        for f, depth in ((moda.moda_attn_bwd_gqa, two), (moda.moda_attn_bwd, two), (moda.moda_attn_bwd_e4m3, cache8)):
+            l = 3 if depth is cache8 else 2
+            calls += [lambda f=f, depth=depth, l=l: f(Q, K, V, few(depth), O, dO, LSE, l, scale), lambda f=f, depth=depth, l=l: f(Q, K, V, depth, wrong(O), dO, LSE, l, scale),
+                      lambda f=f, depth=depth, l=l: f(Q, K, V, depth, O, wrong(dO), LSE, l, scale), lambda f=f, depth=depth, l=l: f(Q, K, V, depth, O, dO, wrong(LSE), l, scale),
+                      lambda f=f, depth=depth, l=l: f(Q, K, V, depth, O, dO, LSE, l, scale, d_depth_kv=few(two))]
+            calls += [lambda f=f, depth=depth, l=l, n=n: f(Q, K, V, depth, O, dO, LSE, l, scale, **{n: wrong(O)}) for n in ("dQ", "dK", "dV")]
+        calls += [lambda: moda.moda_attn_bwd_gqa_slot(Q, K, V, two, O, dO, LSE, 1, scale, few(two), 1), lambda: moda.moda_attn_bwd_gqa_slot(Q, K, V, two, O, wrong(dO), LSE, 1, scale, two, 1)]
+        for i, f in enumerate(calls):
+            assert general(_errors, f) is ValueError and _errors(f) is ValueError, (wrong, i)
+    torch.cuda.synchronize()
+    assert moda.moda_last_status() == 0
+
+
 @gpu
 @pytest.mark.parametrize("l", [0, 2])
 def test_differentiable_call_behaves_as_the_general_one(general, l):
