@@ -1,15 +1,16 @@
-"""Builds the CUDA library (libmoda_b200.so, nvcc for sm_100a) and the host path of its hot calls (_host.so, g++) in-tree."""
+"""Builds the CUDA library (libmoda_b200.so, nvcc for sm_100a) and the host path of its hot calls (_host.<abi>.so, g++) in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
 
+from .binding import HOST_PATH as HOST
+
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmoda_b200.so")
 SOURCES = [os.path.join(CSRC, "moda_api.cu")]
-HOST = os.path.join(PKG, "_host.so")
 HOST_SOURCE = os.path.join(CSRC, "moda_host.cpp")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -47,7 +48,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 def build_host(force: bool = False, verbose: bool = False) -> str:
-    """The CPython extension that moves the hot calls' host work out of Python (csrc/moda_host.cpp). Returns the .so path."""
+    """The CPython extension that moves the hot calls' host work out of Python (csrc/moda_host.cpp). Returns the .so path,
+    which another Python or torch does not look for."""
     deps = (HOST_SOURCE, os.path.join(PKG, "..", "include", "moda.h"))
     if force or not os.path.exists(HOST) or any(os.path.getmtime(d) > os.path.getmtime(HOST) for d in deps):
         import sysconfig
@@ -65,7 +67,7 @@ def build_host(force: bool = False, verbose: bool = False) -> str:
         if verbose or res.returncode != 0:
             sys.stderr.write(res.stdout + res.stderr)
         if res.returncode != 0:
-            raise RuntimeError("g++ failed building _host.so")
+            raise RuntimeError(f"g++ failed building {HOST}")
         os.replace(tmp, HOST)
     return HOST
 

@@ -331,3 +331,34 @@ def test_streams_and_threads():
     for i in range(4):
         _same(out[i][:2], want)
         _same(out[i], out[0], loose=(2,))
+
+
+@pytest.fixture
+def other_host(monkeypatch, tmp_path):
+    """The binding as another Python or torch finds it: the extension's file has another name."""
+    monkeypatch.setattr(binding, "_host", None)
+    monkeypatch.setattr(binding, "HOST_PATH", str(tmp_path / "_host.so"))
+
+
+def test_without_the_extension_calls_take_the_python_form(other_host):
+    x = torch.zeros(1, 4, 2, 64, dtype=BF16)
+    for f in (lambda: moda.moda_attn_fwd_gqa(x, x, x, None, 0, 0.1), lambda: moda.moda_attention(x, x, x),
+              lambda: moda.moda_attn_bwd_gqa(x, x, x, None, x, x, x, 0, 0.1), lambda: moda.moda_attn_decode(x[:, 0], x, x, None, 4, 0, 0.1)):
+        with pytest.raises(ValueError, match="CUDA"):       # the Python form's own refusal
+            f()
+
+
+@gpu
+def test_results_without_the_extension(other_host):
+    Q, K, V, dO = _qkv(1, 130, 2, 2, 64)
+    O, LSE = moda.moda_attn_fwd_gqa(Q, K, V, None, 0, 0.125)
+    assert type(binding.host()).__name__ == "_NoHost"
+    x = [t.requires_grad_() for t in (Q, K, V)]
+    torch.autograd.grad(moda.moda_attention(*x, None, 0, 0.125)[0], x, dO)
+    _same((O, LSE), moda.moda_attention(*x, None, 0, 0.125))
+
+
+def test_a_build_is_for_one_python_and_one_torch():
+    import sysconfig
+    from paper_2603_15619_b200 import build
+    assert build.HOST == binding.HOST_PATH and torch.__version__ in build.HOST and sysconfig.get_config_var("SOABI") in build.HOST
