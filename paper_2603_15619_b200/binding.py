@@ -13,6 +13,7 @@ import os
 import sysconfig
 
 import torch
+from torch.utils._device import DeviceContext
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libmoda_b200.so")
@@ -165,7 +166,7 @@ def host():
         spec = importlib.util.spec_from_file_location(f"{__package__}._host", HOST_PATH)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)
-        module.bind(load()._handle, _check)
+        module.bind(load()._handle, _check, DeviceContext)
         _host = module
     return _host
 

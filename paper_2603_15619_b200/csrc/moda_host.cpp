@@ -14,9 +14,11 @@
 #include <dlfcn.h>
 
 #include <ATen/ATen.h>
+#include <ATen/PythonTorchFunctionTLS.h>
 #include <ATen/cuda/CUDAContext.h>
 #include <c10/core/DispatchKeySet.h>
 #include <torch/csrc/Exceptions.h>
+#include <torch/csrc/PyInterpreter.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -67,8 +69,19 @@ uint64_t plain_keys() {
                                   c10::DispatchKeySet(c10::DispatchKey::ADInplaceOrView)).raw_repr();
     return keys;
 }
-// No dispatch mode, functorch transform, functionalisation or tracer: their keys would be in the thread's included set.
+// A torch-function mode sees the torch calls of the Python form.  Not so the one of a default device (torch.set_default_device): it
+// fills in a device where none is given, and these calls give one.
+PyObject* device_mode = nullptr;                               // torch.utils._device.DeviceContext
+bool function_mode() {
+    using TLS = at::impl::PythonTorchFunctionTLS;
+    if (!at::impl::torch_function_mode_enabled()) return false;
+    for (int64_t i = 0; i < TLS::stack_len(); ++i)
+        if (reinterpret_cast<PyObject*>(Py_TYPE(TLS::get_stack_at(i)->ptr(getPyInterpreter()))) != device_mode) return true;
+    return false;
+}
+// No mode, functorch transform, functionalisation or tracer: but for torch-function modes their keys would be in the thread's included set.
 bool plain_thread() {
+    if (function_mode()) return false;
     static const uint64_t keys = (c10::DispatchKeySet(c10::DispatchKey::BackendSelect) | c10::DispatchKeySet(c10::DispatchKey::ADInplaceOrView)).raw_repr();
     return (c10::impl::tls_local_dispatch_key_set().included_.raw_repr() & ~keys) == 0;
 }
@@ -351,10 +364,10 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 // ---- module -----------------------------------------------------------------------------------------------------------
-// bind(handle of libmoda_b200.so, check): must come first
+// bind(handle of libmoda_b200.so, check, DeviceContext): must come first
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
-    if (n != 2) return PyErr_Format(PyExc_TypeError, "bind(handle, check)");
+    if (n != 3) return PyErr_Format(PyExc_TypeError, "bind(handle, check, device_mode)");
     void* handle = PyLong_AsVoidPtr(a[0]);
     if (PyErr_Occurred()) return nullptr;
 #define X(name)                                                                                            \
@@ -363,6 +376,7 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
     MODA_HOST_CALLS(X)
 #undef X
     Py_XSETREF(check_fn, Py_NewRef(a[1]));
+    Py_XSETREF(device_mode, Py_NewRef(a[2]));
     Py_RETURN_NONE;
     END_HANDLE_TH_ERRORS
 }

@@ -362,3 +362,42 @@ def test_a_build_is_for_one_python_and_one_torch():
     import sysconfig
     from paper_2603_15619_b200 import build
     assert build.HOST == binding.HOST_PATH and torch.__version__ in build.HOST and sysconfig.get_config_var("SOABI") in build.HOST
+
+
+class _Calls(torch.overrides.TorchFunctionMode):
+    """Names of the torch functions that pass a torch-function mode."""
+
+    def __init__(self):
+        super().__init__()
+        self.names = []
+
+    def __torch_function__(self, func, types, args=(), kwargs=None):
+        self.names.append(getattr(func, "__name__", str(func)))
+        return func(*args, **(kwargs or {}))
+
+
+@gpu
+def test_torch_function_modes_see_the_calls_they_saw(general):
+    Q, K, V, dO = _qkv(1, 64, 2, 2, 64)
+    O, LSE = moda.moda_attn_fwd_gqa(Q, K, V, None, 0, 0.125)
+
+    def seen(f):
+        with _Calls() as mode:
+            f()
+        return mode.names
+
+    for f in (lambda: moda.moda_attn_fwd_gqa(Q, K, V, None, 0, 0.125), lambda: moda.moda_attn_bwd_gqa(Q, K, V, None, O, dO, LSE, 0, 0.125),
+              lambda: moda.moda_attn_decode(Q[:, 0], K, V, None, 64, 0, 0.125), lambda: moda.moda_attention(Q, K, V)):
+        assert seen(f) == general(seen, f) and "empty_like" in seen(f)
+
+
+@gpu
+def test_a_default_device_does_not_cost_the_extension():
+    Q, K, V, _ = _qkv(1, 64, 2, 2, 64)
+    want = moda.moda_attn_fwd_gqa(Q, K, V, None, 0, 0.125)
+    with torch.device("cpu"):
+        got = binding.host().attn_fwd(Q, K, V, None, 0, 0.125, None, 0, None, None)
+        assert got is not None and got[0].is_cuda
+        with _Calls():
+            assert binding.host().attn_fwd(Q, K, V, None, 0, 0.125, None, 0, None, None) is None
+    _same(got, want)
