@@ -237,9 +237,9 @@ int moda_attn_bwd_stages(const void* Q, const void* K, const void* V, const void
  * The whole backward of a layer of a stack (H query heads on H_kv key/value heads, as in moda_attn_bwd_gqa): the depth
  * gradients are added to slots [0, l) of d_depth_kv (MODA_BWD_ACCUMULATE_DEPTH), and slot `slot` >= l of d_depth_kv, which
  * holds what the later layers left for this layer's own K, V, is added to dK, dV before they are rounded (the slot itself
- * stays as it is; MODA_ERR_BAD_SLOT for a slot below l).  d_depth_kv is needed with l == 0 too.  For the shapes where
- * moda_attn_bwd_takes_slot returns 1; elsewhere this call is MODA_ERR_BAD_GROUP, and moda_attn_bwd_gqa_stages with
- * moda_depth_cache_unpack_add behind it does the same.
+ * stays as it is; MODA_ERR_BAD_SLOT for a slot below l).  d_depth_kv is needed with l == 0 too.  It does what moda_attn_bwd_gqa_stages
+ * with moda_depth_cache_unpack_add behind it does, with dK, dV rounded once.  moda_attn_bwd_takes_slot returns 1 for every H, H_kv, d, l that
+ * the backward takes, 0 for others.
  */
 int moda_attn_bwd_gqa_slot(const void* Q, const void* K, const void* V, const void* depth_kv,
                            const void* O, const void* dO, const float* LSE,

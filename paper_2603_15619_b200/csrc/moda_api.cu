@@ -415,7 +415,7 @@ int launch_depth_bwd(DepthBwdParams m, cudaStream_t stream) {
 }
 
 // Which form of the backward a call takes: the fused form (moda_bwd_fused.cuh) unless the caller asks for
-// reproducible bits.  Grouped-query calls in the fused form run their depth part as the per-position kernel; in
+// reproducible bits (which a call with a slot of the gradient cache cannot).  Grouped-query calls in the fused form run their depth part as the per-position kernel; in
 // the split form they stay row-local: its dQ pass leaves the per-row factors that depth_grad_group_kernel sums
 // over the heads of a group.
 inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
@@ -883,7 +883,6 @@ int bwd_gqa(const void* Q, const void* K, const void* V, const void* depth_kv, c
         (l > 0 && !aligned16(depth_kv)) || ((l > 0 || slot >= 0) && !aligned16(d_depth_kv)))
         return MODA_ERR_MISALIGNED;
     const bool deterministic = (stages & MODA_BWD_DETERMINISTIC) != 0;
-    if (slot >= 0 && !bwd_uses_fused(d, H / H_kv, l, deterministic)) return MODA_ERR_BAD_GROUP;
     const size_t need = bwd_uses_fused(d, H / H_kv, l, deterministic) ? bwd_fused_workspace_bytes(B, T, H, d)
                                                                        : bwd_workspace_bytes_gqa(B, T, H, H_kv, l);
     if (!workspace || !aligned16(workspace) || workspace_bytes < need) return MODA_ERR_WORKSPACE;

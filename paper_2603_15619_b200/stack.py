@@ -15,8 +15,8 @@ C-ABI calls; it is plumbing: no arithmetic of the operator happens here.
 A token tensor chains the calls: the token behind slot l stands for the first l + 1 slots of the depth
 cache, and its gradient is a gradient cache of that many slots.  Backward runs the layers in reverse.
 The first layer of a pass writes its depth gradients into a new buffer, every layer below adds its own to
-slots < l of that buffer in place (the backward call's accumulate flag) and takes slot l, which by then
-holds the contributions of all later layers, as part of the gradient of its own K, V.  Because the buffer
+slots < l of that buffer in place and takes slot l, which by then holds the contributions of all later
+layers, as part of the gradient of its own K, V (moda_attn_bwd_gqa_slot does both).  Because the buffer
 travels as a gradient, passes over one stream do not see each other, also when one failed half way.
 """
 from __future__ import annotations
@@ -44,15 +44,11 @@ class _Attend(torch.autograd.Function):
         dO = torch.zeros_like(O) if dO is None else dO.contiguous()
         # slots < l of the gradient cache receive this layer's share
         grads, filled = slots.open(dtoken, l)
-        if filled and binding.moda_attn_bwd_takes_slot(Q.shape[2], K.shape[2], Q.shape[3], l):
-            # the fused backward adds slot l, which later layers attended to, where it stores dK, dV
-            dQ, dK, dV = binding.moda_attn_bwd_gqa_slot(Q, K, V, slots.cache if l > 0 else None, O, dO, LSE, l, ctx.scale, grads, l)
-            return dQ, dK, dV, slots.close(grads, filled, l), None, None, None
-        dQ, dK, dV, _ = binding.moda_attn_bwd_gqa(
-            Q, K, V, slots.cache if l > 0 else None, O, dO, LSE, l, ctx.scale, d_depth_kv=grads if l > 0 else None,
-            stages=binding.MODA_BWD_ALL_STAGES | (binding.MODA_BWD_ACCUMULATE_DEPTH if filled else 0))
-        if filled:                                             # later layers attended to slot l
-            binding.moda_depth_cache_unpack_add(grads, l, dK, dV)
+        args = (Q, K, V, slots.cache if l > 0 else None, O, dO, LSE, l, ctx.scale)
+        if filled:                                             # later layers attended to slot l: added where dK, dV are stored
+            dQ, dK, dV = binding.moda_attn_bwd_gqa_slot(*args, grads, l)
+        else:
+            dQ, dK, dV, _ = binding.moda_attn_bwd_gqa(*args, d_depth_kv=grads if l > 0 else None)
         return dQ, dK, dV, slots.close(grads, filled, l), None, None, None
 
 

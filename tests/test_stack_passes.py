@@ -23,13 +23,13 @@ class Operator:
     """The calls that stack.py makes.  ``fail_at``: number of the backward call that raises before it writes anything."""
 
     def __init__(self, monkeypatch):
-        self.calls, self.fail_at = 0, None
+        self.calls, self.fail_at, self.names = 0, None, []
         nan = lambda t, **kw: torch.full(t.shape, float("nan"), dtype=t.dtype)
         monkeypatch.setattr(torch, "empty_like", nan)
         monkeypatch.setattr(binding, "moda_depth_cache_bytes", lambda *a: 2 * SLOT * a[-1])
         monkeypatch.setattr(binding, "alloc_depth_cache", lambda *a: torch.full((SLOT * a[4],), float("nan"), dtype=torch.bfloat16))
-        for name in ("moda_attn_fwd_append", "moda_attn_bwd_gqa", "moda_depth_cache_append", "moda_depth_cache_unpack",
-                     "moda_depth_cache_unpack_add", "moda_kv_project_append"):
+        for name in ("moda_attn_fwd_append", "moda_attn_bwd_gqa", "moda_attn_bwd_gqa_slot", "moda_depth_cache_append", "moda_depth_cache_unpack",
+                     "moda_kv_project_append"):
             monkeypatch.setattr(binding, name, getattr(self, name))
 
     def moda_attn_fwd_append(self, Q, K, V, depth, l, scale, cache, slot):
@@ -39,17 +39,25 @@ class Operator:
         self.moda_depth_cache_append(cache, slot, K, V)
         return O, torch.zeros(B, H, T)
 
-    def moda_attn_bwd_gqa(self, Q, K, V, depth, O, dO, LSE, l, scale, d_depth_kv=None, stages=None):
+    def backward_call(self, name):
         self.calls += 1
+        self.names.append(name)
         if self.calls == self.fail_at:
-            raise moda.ModaError(-2, "moda_attn_bwd_gqa")
+            raise moda.ModaError(-2, name)
+
+    def moda_attn_bwd_gqa(self, Q, K, V, depth, O, dO, LSE, l, scale, d_depth_kv=None):
+        self.backward_call("moda_attn_bwd_gqa")
         for i in range(l):
-            g = torch.stack([coef(l, i) * dO, 2 * coef(l, i) * dO])
-            if stages & binding.MODA_BWD_ACCUMULATE_DEPTH:
-                slots_of(d_depth_kv)[i].add_(g)
-            else:
-                slots_of(d_depth_kv)[i].copy_(g)
+            slots_of(d_depth_kv)[i].copy_(torch.stack([coef(l, i) * dO, 2 * coef(l, i) * dO]))
         return dO.clone(), dO.clone(), dO.clone(), d_depth_kv
+
+    def moda_attn_bwd_gqa_slot(self, Q, K, V, depth, O, dO, LSE, l, scale, d_depth_kv, slot):
+        self.backward_call("moda_attn_bwd_gqa_slot")
+        assert slot >= l
+        for i in range(l):
+            slots_of(d_depth_kv)[i].add_(torch.stack([coef(l, i) * dO, 2 * coef(l, i) * dO]))
+        left = slots_of(d_depth_kv)[slot]
+        return dO.clone(), dO + left[0], dO + left[1]
 
     def moda_depth_cache_append(self, cache, slot, K, V):
         slots_of(cache)[slot] = torch.stack([K, V]).detach()
@@ -57,10 +65,6 @@ class Operator:
     def moda_depth_cache_unpack(self, cache, slot, K, V):
         K.copy_(slots_of(cache[:SLOT * (slot + 1)])[slot, 0])
         V.copy_(slots_of(cache[:SLOT * (slot + 1)])[slot, 1])
-
-    def moda_depth_cache_unpack_add(self, cache, slot, K, V):
-        K.add_(slots_of(cache[:SLOT * (slot + 1)])[slot, 0])
-        V.add_(slots_of(cache[:SLOT * (slot + 1)])[slot, 1])
 
     def moda_kv_project_append(self, X, Wk, Wv, H_kv, cache, slot, store_kv):
         self.moda_depth_cache_append(cache, slot, (X @ Wk.t()).view(B, T, H, D), (X @ Wv.t()).view(B, T, H, D))
@@ -138,6 +142,13 @@ def test_passes_over_one_stream_do_not_see_each_other(op, order):
         want = [torch.zeros(x.shape) if w is None else w for x, w in zip(stack.leaves, stack.grads(which))]
         got = [torch.zeros(x.shape) if g is None else g for x, g in zip(stack.leaves, run_pass(stack, outs, which, retain_graph=True))]
         check(got, want)
+
+
+def test_layers_below_the_first_take_up_their_slot_in_their_backward_call(op):
+    stack = Stack()
+    _, outs = stack.run()
+    run_pass(stack, outs, (0, 1, 2))
+    assert op.names == ["moda_attn_bwd_gqa", "moda_attn_bwd_gqa_slot", "moda_attn_bwd_gqa_slot"]
 
 
 @pytest.mark.parametrize("fail_at", [1, 2, 3])
