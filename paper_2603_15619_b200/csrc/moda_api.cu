@@ -6,6 +6,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "launch_rules.h"
 #include "moda_bwd.cuh"
 #include "moda_bwd_fused.cuh"
 #include "moda_cache.cuh"
@@ -421,43 +422,6 @@ int launch_depth_bwd(DepthBwdParams m, cudaStream_t stream) {
 inline bool bwd_uses_fused(int d, int G, int l, bool deterministic) {
     if (deterministic) return false;
     return G == 1 || l == 0 || gqa_depth_split_bwd(d, G, l);
-}
-
-// How many SMs the depth part of a fused backward gets beside the sequence part.  Measured SM time: an entry of the row
-// ring 1.75 us (16 SMs at it) to 2.0 us (50), e4m3 a tenth more; an iteration of the sequence part at d = 128 2.7 us
-// and 5 us per key tile around them; at d = 64 12 us per key tile and 1.33 us an iteration, rising to 1.5 us for the longest (their runs
-// last long enough for the clocks to come down, which the depth part, bound by HBM, does not feel).  With the share
-// x = depth / (depth + sequence) of all SMs both
-// parts end together; a few SMs more than that cost less than a few too few, because SMs that the depth part leaves go on
-// with the sequence part.  The number is even: with an odd one a CTA shares its pair of SMs with a CTA of the sequence part,
-// and the whole depth part waits for that one.
-// Whole backward, us, by SMs (rounds of one count differ by 4-8 %).  d = 128, 26 shapes, bf16:
-// T = 8192, l = 16, B = 2: 34 2167, 36 2057, 38 1979, 40 2000, 44 1994 (taken: 40); T = 4096, l = 23, B = 4: 66 1664,
-// 70 1602, 74 1619, 78 1634 (72).  e4m3: T = 5000, l = 23, B = 2: 64 1111, 68 1075, 72 1086, 76 1099 (70); T = 8192, l = 16: 38 1962, 42 1882,
-// 46 1965 (42); T = 32768, l = 24: 18 11551, 20 11102, 24 11776 (20).  Within 3.4 % of the best count everywhere but in
-// one place: e4m3 at T = 1024 (124 taken, 130 best: 363 against 347).  At least 16: with x from 3 to 12 every count from x + 15 % to 20 is within
-// 1 % (18 shapes, counts in shuffled order; T = 65536, l = 24: 10 45.1, 16 45.4, 20 45.3 ms), and up to three too few cost 10-20 %.
-// d = 64 (counts in shuffled order, 9 to 11 rounds), bf16: T = 1024,
-// l = 30, B = 4, 16 heads (256 units): 84 236, 86 202, 96 203 (86); T = 4096, l = 23, B = 4, 16 heads: 56 965, 60 911, 64 881, 70 894 (70); T = 8192, l = 16, B = 2, 32
-// heads: 32 2271, 34 2186, 36 2227, 40 2236 (36); T = 16384, l = 32, 32 heads: 34 4299, 36 4186, 38 4212, 44 4183 (38); T = 32768, l = 32, 32 heads: 18 15691,
-// 20 14487, 22 13729, 24 13972, 28 13601 (22); T = 65536, l = 60, 16 heads: 18 27895, 20 27103, 22 26983 (20); e4m3: T = 5000, l = 23, B = 2, 32 heads: 58 1194, 62 1194,
-// 68 1207 (62); T = 32768, l = 32: 20 14715, 22 13607, 24 13220, 28 13456 (24).  Whole backward with 1.1 x + 2 for 1.06 x + 1: T = 32768, l = 32 14.11 ->
-// 13.81 ms, T = 65536, l = 60 28.87 -> 26.56, T = 3000, l = 12 473 -> 461 us, six more shapes within noise; at d = 128 no difference.
-inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, unsigned sms, bool fp8) {
-    const double nq = num_tiles(T);
-    const double depth = double(units) * (l + 1) * (fp8 ? 1.9 : 1.7);
-    const double n = nq + 1;
-    const double seq = double(bh) * nq * (d == 128 ? 5.0 + 1.36 * n : 12.0 + (0.66 + 0.00035 * n) * n);
-    const double x = sms * depth / (depth + seq);
-    const auto even = [](double c) { return 2 * unsigned(std::ceil(c / 2)); };
-    unsigned share = std::max(16u, even(d == 128 ? 1.06 * x + 1.0 : 1.1 * x + 2.0));
-    // few units for each SM: what counts is how many the busiest one has
-    const unsigned rounds = (units + share - 1) / share;
-    if (rounds > 1 && rounds <= 16) {
-        const unsigned fewer = even(std::ceil(double(units) / (rounds - 1)));
-        share = (100 * fewer <= 112 * share && fewer <= sms) ? fewer : even(std::ceil(double(units) / rounds));
-    }
-    return std::min(units, std::min(share, sms));
 }
 
 // A launch that may start before the grid in front of it has ended (that grid lets it, and it waits itself before it reads
