@@ -464,7 +464,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     const bool split_depth = G > 1 && a.l > 0;             // depth part by the per-position kernel after the finish kernel
     const unsigned tiles = unsigned(B) * H * num_tiles(T);
     constexpr int kRowThreads = kTileRows * (D / 32);
-    bool beside_rows = false;
+    bool beside_rows = false, finish_behind_rows = false;
     if (stages & 1) {
         bwd_prep_kernel<D><<<tiles, kRowThreads, 0, stream>>>(static_cast<const __nv_bfloat16*>(a.O), static_cast<const __nv_bfloat16*>(a.dO),
                                                              delta, dq_acc, B, T, H);
@@ -483,6 +483,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
             int sms = 0;
             if (int rc = device_sm_count(&sms)) return rc;
             const unsigned grid = beside_rows ? bwd_row_ctas(D, (long long)B * H, T, a.l, units, unsigned(sms), a.fp8_cache) : std::min(units, unsigned(sms));
+            finish_behind_rows = grid + tiles > unsigned(sms);
             const size_t smem = a.fp8_cache ? RowsSmem<D, true>::kDynamic : RowsSmem<D, false>::kDynamic;
             // not beside the prep kernel: its CTAs would take SMs as those come free, one of a pair here and there, and the others of
             // these pairs slow it down (d = 64, B = 2, T = 5000, 32 heads, l = 23, e4m3: 1150 -> 1311 us)
@@ -496,6 +497,7 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
         f.scale = a.scale; f.scale_log2 = a.scale * kLog2e;
         f.slot_grad = static_cast<const uint4*>(a.slot_grad);
         f.beside_rows = beside_rows ? 1 : 0;
+        f.finish_behind_rows = beside_rows && finish_behind_rows ? 1 : 0;
         if (!launch_beside(a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true> : moda_bwd_fused_kernel<D, false>, unsigned(B) * Hk * num_tiles(T),
                            L::kThreads, L::kDynamic, (stages & 1) != 0, stream, mK, mV, mQ, mdO, mdK, mdV, f)) return MODA_ERR_CUDA;
     }

@@ -93,7 +93,9 @@ bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __rest
 // backward, graph replays, us, T = 100, l = 0, d = 64, 2 heads: 13.0 -> 10.9; 2 x 512, 16 heads, d = 128, l = 0: 24.0 -> 22.7; 2 x 1000, l = 0:
 // 55.2 -> 54.1; T = 2000, 16 heads on 4, d = 64, l = 12: 119.3 -> 116.2; T = 1000, 8 heads, l = 7, e4m3 33.0 -> 32.6; from T = 4096 on nothing.  The
 // sequence part lets this kernel start at the END of its CTAs: from their start on, its CTAs filled the few SMs that
-// had no work in the last wave and did theirs there, four to an SM (2 x 1000, l = 0: 59.8; T = 512: 29.5).
+// had no work in the last wave and did theirs there, four to an SM (2 x 1000, l = 0: 59.8; T = 512: 29.5).  So it is with the few SMs that the
+// depth part leaves where that one ends last: with more CTAs here than such SMs they are let go behind it (B = 4, 32 heads, d = 128: T = 100, l = 64
+// 189.3 -> 184.3, T = 128, l = 48 152.6 -> 148.2, T = 100, l = 6 35.8 -> 35.3); with fewer, beside it (2 x 100, 16 heads, d = 64, l = 3: 14.2, behind it 14.5).
 template <int D>
 __global__ void __launch_bounds__(kTileRows * (D / 32))
 bwd_dq_finish_kernel(const float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dQ, int B, int T, int H, float scale) {
@@ -524,6 +526,7 @@ struct FusedParams {
     float scale, scale_log2;
     const uint4* slot_grad;     // SLOT: the slot of a gradient cache that dK, dV take up
     int beside_rows;    // launched beside bwd_rows_kernel (which has not finished): the grid must not end before it
+    int finish_behind_rows;     // the finish kernel is let go behind that kernel as well
 };
 
 template <int D, bool SLOT = false>
@@ -1096,7 +1099,9 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     __syncthreads();
     abort_teardown(abort_flag, 256);
     __syncthreads();
-    grid_launch_dependents();                          // the finish kernel may come up
+    // the finish kernel may come up: beside the end of the rows kernel if there is room for it on the SMs that one leaves
+    if (last_cta && p.finish_behind_rows) grid_dependency_wait();
+    grid_launch_dependents();
     if (warp == W_S) tmem_dealloc(tmem, kTmemCols);
     // what follows on the stream reads the accumulator and the depth gradients: this grid ends after the rows kernel has
     if (last_cta) grid_dependency_wait();

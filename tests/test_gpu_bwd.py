@@ -262,7 +262,8 @@ def test_forward_and_backward_replayed_from_a_graph(B, T, H, d, l, e4m3):
 
 
 @pytest.mark.parametrize("B,T,H,Hk,d,l", [(1, 1, 1, 1, 64, 0), (1, 100, 2, 2, 64, 0), (1, 129, 2, 2, 128, 0), (2, 512, 16, 16, 128, 0),
-                                          (2, 513, 8, 8, 128, 5), (4, 300, 16, 16, 64, 3), (1, 640, 8, 1, 64, 12), (2, 400, 4, 2, 128, 0)])
+                                          (2, 513, 8, 8, 128, 5), (4, 300, 16, 16, 64, 3), (1, 640, 8, 1, 64, 12), (2, 400, 4, 2, 128, 0),
+                                          (4, 128, 32, 32, 128, 24), (4, 100, 32, 32, 64, 9)])
 def test_overlapping_launches_find_what_the_ones_in_front_of_them_write(B, T, H, Hk, d, l):
     """The launches of a backward overlap at their ends; the stages called one by one do not.  The scratch holds NaN before each call."""
     x = synthetic.make_gqa(B, T, H, Hk, d, l, seed=91, device="cuda")
