@@ -48,4 +48,12 @@ inline unsigned bwd_row_ctas(int d, long long bh, int T, int l, unsigned units, 
     return std::min(units, std::min(share, sms));
 }
 
+// Whether the two row warpgroups of the fused backward's sequence part (d = 64) take alternate iterations, or share each (moda_bwd_fused.cuh).
+// A CTA has G (tiles + 1) / 2 iterations in the mean; with few of them the one or two that do not come in pairs weigh more than what the
+// pairs win.  Whole backward, l = 0, us, shared / alternate, by batch x heads: T = 100: 1 x 2 10.5 / 11.3, 8 x 32 19.8 / 21.4; T = 256: 12.2 / 12.8, 41.9 / 45.0; T = 512:
+// 15.1 / 15.4, 93.0 / 96.7; T = 640: 16.5 / 16.5, 124 / 128; T = 768 (twice the mean = 7): 18.0 / 17.7, 2 x 16 27.7 / 28.2, 156 / 160; T = 900 (9): 20.7 / 20.0,
+// 36.3 / 35.7, 218 / 220; T = 1200: 23.6 / 22.4, 45.9 / 45.0, 303 / 303; T = 2000: 31.8 / 29.6, 88.3 / 85.3, 4 x 32 331 / 322.  G = 4: T = 100 (8) 15.8 / 16.0,
+// T = 300 (16) 27.2 / 26.4; G = 8: T = 100 (16) 21.3 / 20.9, T = 256 (24) 38.1 / 36.1.
+inline bool bwd_alternates(int d, int T, int G) { return d == 64 && G * ((T + 127) / 128 + 1) > 7; }
+
 }  // namespace moda

@@ -444,7 +444,10 @@ bool launch_beside(void (*kernel)(P...), unsigned grid, unsigned threads, size_t
 template <int D>
 int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     const int B = a.B, T = a.T, H = a.H, Hk = a.Hk, G = a.H / a.Hk;
-    using L = FusedSmem<D>;
+    const bool alternate = bwd_alternates(D, T, G);
+    const int seq_smem = alternate ? FusedSmem<D>::kDynamic : FusedSmem<D, false>::kDynamic;
+    const auto seq_kernel = alternate ? a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true> : moda_bwd_fused_kernel<D, false>
+                                      : a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true, false> : moda_bwd_fused_kernel<D, false, false>;
     CUtensorMap mK, mV, mQ, mdO, mdK, mdV;
     if (!make_bthd_map(&mK, a.K, B, T, Hk, D) || !make_bthd_map(&mV, a.V, B, T, Hk, D) ||
         !make_bthd_map(&mQ, a.Q, B, T, H, D) || !make_bthd_map(&mdO, a.dO, B, T, H, D) ||
@@ -454,7 +457,10 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
     int dev = 0;
     if (!cuda_ok(cudaGetDevice(&dev))) return MODA_ERR_CUDA;
     if (configured_dev != dev) {
-        if (!set_smem_limit(moda_bwd_fused_kernel<D>, L::kDynamic) || !set_smem_limit(moda_bwd_fused_kernel<D, true>, L::kDynamic) || !set_smem_limit(bwd_rows_kernel<D>, RowsSmem<D, false>::kDynamic) ||
+        if (!set_smem_limit(moda_bwd_fused_kernel<D>, FusedSmem<D>::kDynamic) || !set_smem_limit(moda_bwd_fused_kernel<D, true>, FusedSmem<D>::kDynamic) ||
+            !set_smem_limit(moda_bwd_fused_kernel<D, false, false>, FusedSmem<D, false>::kDynamic) ||
+            !set_smem_limit(moda_bwd_fused_kernel<D, true, false>, FusedSmem<D, false>::kDynamic) ||
+            !set_smem_limit(bwd_rows_kernel<D>, RowsSmem<D, false>::kDynamic) ||
             !set_smem_limit(bwd_rows_kernel<D, true>, RowsSmem<D, true>::kDynamic))
             return MODA_ERR_CUDA;
         configured_dev = dev;
@@ -498,8 +504,8 @@ int launch_bwd_fused(const BwdArgs& a, int stages, cudaStream_t stream) {
         f.slot_grad = static_cast<const uint4*>(a.slot_grad);
         f.beside_rows = beside_rows ? 1 : 0;
         f.finish_behind_rows = beside_rows && finish_behind_rows ? 1 : 0;
-        if (!launch_beside(a.slot_grad != nullptr ? moda_bwd_fused_kernel<D, true> : moda_bwd_fused_kernel<D, false>, unsigned(B) * Hk * num_tiles(T),
-                           L::kThreads, L::kDynamic, (stages & 1) != 0, stream, mK, mV, mQ, mdO, mdK, mdV, f)) return MODA_ERR_CUDA;
+        if (!launch_beside(seq_kernel, unsigned(B) * Hk * num_tiles(T), FusedSmem<D>::kThreads, seq_smem, (stages & 1) != 0, stream,
+                           mK, mV, mQ, mdO, mdK, mdV, f)) return MODA_ERR_CUDA;
     }
     if (stages & 4) {
         if (!launch_beside(bwd_dq_finish_kernel<D>, tiles, kRowThreads, 0, (stages & 2) != 0, stream, static_cast<const float*>(dq_acc),

@@ -412,22 +412,22 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 // 2b. Sequence part: dK, dV and the dQ tiles
 // =====================================================================================
 // 512 threads (in warp order):
-//   row warps    two warpgroups.  d = 128: both work on the same iteration, a thread owns one key row (= tensor-memory
-//                lane) and 64 of its 128 query columns.  d = 64: they take alternate iterations, a thread owns one key row
-//                and all 128 query columns.  Either way P^T, then dS^T.
+//   row warps    two warpgroups.  "Shared" (d = 128; d = 64 with few iterations a CTA): both work on the same iteration, a thread owns
+//                one key row (= tensor-memory lane) and 64 of its 128 query columns.  "Alternate" (d = 64): they take alternate
+//                iterations, a thread owns one key row and all 128 query columns.  Either way P^T, then dS^T.
 //   drain warps  one warpgroup: a thread owns one query row of the dQ tile; it copies the row out of tensor memory
 //                (which frees the region at once) and hands it, 8 KiB at a time through a staging ring in shared
 //                memory, to bulk reductions into the fp32 accumulator, at whatever pace L2 takes them, without
 //                holding up the row warps.
 //   then         a loader warp (TMA tiles; the per-query terms as bf16 parts for the extra k-step) and three warps
-//                that issue the contractions: S; dP (d = 64: and dV); dV, dQ, dK (d = 64: dK, dQ).  MMAs of
+//                that issue the contractions: S; dP (alternate: and dV); dV, dQ, dK (alternate: dK, dQ).  MMAs of
 //                different warps are ordered by mbarriers only.  (One warp for all five, in the order in which they become
 //                ready, took 1.5 times as long at d = 64: its waits and commits come one after the other.)
 //
 // Tensor memory (fp32 columns): X, 128 columns per buffer, S^T overlaid by P^T (bf16) -- one buffer at d = 128,
 // two at d = 64 (where dK and dV leave room);  Y, 128 columns, dP^T;  dK, D columns;  dV, D columns.  512 columns at either head
-// width.  The dQ tile takes Y behind dP^T of the same iteration (d = 128), or the half of an X buffer that P^T has left
-// (d = 64: dQ_i behind P_{i+1}, so that neither dP_{i+1} nor S_{i+1} waits for the copy).
+// width.  The dQ tile takes Y behind dP^T of the same iteration (shared), or the half of an X buffer that P^T has left
+// (alternate: dQ_i behind P_{i+1}, so that neither dP_{i+1} nor S_{i+1} waits for the copy).
 //
 // What bounds it (cycle stamps per warp role, T = 8192): the rate at which a dQ tile's additions are taken by L2 (64 KiB
 // of fp32 per iteration per SM at d = 128; all SMs together sustain about 5.9 TB/s in a kernel that does nothing else,
@@ -436,7 +436,7 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 // dQ staging 64 KiB in and out, against 128 bytes per clock) is at two thirds of its peak since the row warps no
 // longer load the per-query terms.
 //
-// Two dependency chains per iteration i at d = 128, which overlap each other and the next iteration:
+// Two dependency chains per shared iteration i, which overlap each other and the next iteration:
 //   X:  S'_i = S_i - LSE / scale -> P_i^T = exp2(S' c) (row warps) -> dV_i -> X free -> S_{i+1}
 //   Y:  dP'_i = dP_i - D -> dS_i^T = P o dP' to shared memory (row warps) -> dQ_i -> copied out (drain warps) -> Y free -> dP_{i+1}
 // and dK_i, issued behind dQ_i, fills the tensor pipe while the row warps exponentiate tile i+1.
@@ -447,26 +447,26 @@ bwd_rows_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant_
 // one's exponentials overlap the other's dS.  What that needs: P^T in registers for a whole row (160 registers),
 // dP_{i+1} as soon as dP_i is in registers, a second dS buffer, a fourth Q stage (a tile is in use for two and a half iterations
 // and takes some 1200 cycles to arrive) -- paid for with two of the four staging chunks.  Cycles per iteration about 2300 now; T = 32768,
-// 32 heads, whole backward 13.1 -> 11.3 ms (1.15-1.18), T = 16384, 64 heads on 8 6.8 -> 5.8, T = 8192, 16 heads 474 -> 425 us, T = 1000 37.9 -> 37.3,
-// T = 300 16.4 -> 16.8 (two or three iterations: one warpgroup has the longer pass of the last).  Measured on the way, T = 32768, gain over
+// 32 heads, whole backward 13.1 -> 11.3 ms (1.15-1.18), T = 16384, 64 heads on 8 6.8 -> 5.8, T = 8192, 16 heads 474 -> 425 us.
+// With few iterations a CTA it loses (one warpgroup has the whole pass of an odd last one): bwd_alternates in launch_rules.h.  Measured on the way, T = 32768, gain over
 // the shared iteration: scores in four loads of 32 columns, each waited for, 1.02 (all 128 requested at once: 1.15); dQ in its own tile's X
 // buffer 1.07; dQ before dK 1.06; three Q stages and four chunks 1.04; chunks of 4 KiB 0.93, or of one warp's 32 rows (no barrier among
 // the drain warps) 0.93; one X buffer with P^T and dQ in columns of their own 1.15.  dS^T in tensor memory as well, as dK's A operand,
 // with the shared iteration: 1.01 (d = 128: 0.97).
 
-template <int D>
+// ALT: the two row warpgroups take alternate iterations; else both work on each, half of the query columns a warpgroup.
+template <int D, bool ALT = (D == 64)>
 struct FusedSmem {
+    static_assert(!ALT || D == 64, "tensor memory has room for two S^T buffers at d = 64 only");
     static constexpr int kRowWGs = 2;                          // row warpgroups
-    static constexpr bool kAlternate = (D == 64);              // they take alternate iterations; else half of the query columns each
-    static constexpr int kCols = kAlternate ? kTileRows : kTileRows / kRowWGs;     // query columns per row-warp thread
     static constexpr int kThreads = (kRowWGs * 4 + 8) * 32;    // row warps, 4 drain warps, loader + 3 issuers
     static constexpr int kTileBytes = kTileRows * D * 2;       // 128 x D bf16
     static constexpr int kSubBytes = kTileRows * 128;          // 128 x 64 sub-tile (128-byte rows)
     // Stages of Q_i.  Q_i is read by S_i early and by dK_i late in its iteration, and a tile takes 1200 to 1600
     // cycles from the TMA issue to the first MMA that uses it, so with two stages the chain "dK_{i-2} completes ->
-    // load Q_i -> S_i -> P_i -> dS_i -> dK_i" spans two iterations and sets the pace; d = 64, where an iteration is in flight for longer,
-    // takes four.
-    static constexpr int kStages = (D == 64) ? 4 : 2;
+    // load Q_i -> S_i -> P_i -> dS_i -> dK_i" spans two iterations and sets the pace; alternate iterations, which are in flight for longer,
+    // take four.
+    static constexpr int kStages = (D == 128) ? 2 : ALT ? 4 : 3;
     // dO_i is read by dP_i and dV_i, both of which complete before dP_{i+1} can be issued; at d = 128 one
     // stage leaves the 32 KiB that the dQ staging buffer needs
     static constexpr int kdOStages = (D == 128) ? 1 : 2;
@@ -476,9 +476,9 @@ struct FusedSmem {
     static constexpr int kdO = kQ + kStages * kTileBytes;      // stages of dO_i
     static constexpr int kdS = kdO + kdOStages * kTileBytes;   // dS^T: 128 keys x 128 queries bf16, one buffer per warpgroup that fills one
     static constexpr int kdSBytes = kTileRows * kTileRows * 2;
-    static constexpr int kdSBufs = kAlternate ? 2 : 1;
+    static constexpr int kdSBufs = ALT ? 2 : 1;
     static constexpr int kStg = kdS + kdSBufs * kdSBytes;   // ring of 8 KiB chunks (16 feature columns of a dQ tile, fp32, accumulator layout)
-    static constexpr int kStgSlots = (D == 128) ? 3 : 2;       // d = 128: three as fast as four, two cost 3-4 %
+    static constexpr int kStgSlots = (D == 128) ? 3 : ALT ? 2 : 4;       // d = 128: three as fast as four, two cost 3-4 %
     static constexpr int kStgBytes = kStgSlots * 16 * kTileRows * 4;
     // Operands of the extra k-step that adds the per-query terms to the two score contractions (see the kernel):
     // 2 KiB chunks of [128 rows][8 bf16] (unswizzled core matrices, 16 bytes per row): one per Q stage with the
@@ -502,16 +502,16 @@ struct FusedSmem {
 enum FusedBar : int {
     kFBarKV = 0,
     kFBarQFull = 1,     // +stage (<= 4), count 32: Q_i and the per-query terms of the stage have landed
-    kFBarQEmpty = 5,    // +stage (<= 4): dK_i complete (Q_i, the row terms and, d = 128, the dS buffer are free)
+    kFBarQEmpty = 5,    // +stage (<= 4): dK_i complete (Q_i, the row terms and, shared iterations, the dS buffer are free)
     kFBardOFull = 9,    // +stage (<= 2)
     kFBardOEmpty = 11,  // +stage (<= 2), count 2: dP_i and dV_i complete
     kFBarSFull = 13,    // +X buffer: S_i complete
     kFBarPFull = 15,    // +X buffer, count kRowArrivals: P_i^T written
-    kFBardPFull = 17,   // +X buffer: dP_i complete
+    kFBardPFull = 17,   // +dS buffer: dP_i complete
     kFBardSFull = 19,   // +dS buffer, count kRowArrivals: dS_i^T written to shared memory, dP_i consumed
     kFBardSFree = 21,   // +dS buffer: dQ_i and dK_i complete (alternating warpgroups)
     kFBarXFree = 23,    // +X buffer: dV_i complete (alternating warpgroups: and dQ_i copied out): the buffer may take S_{i + buffers}
-    kFBardQFull = 25,   // +X buffer: dQ_i complete
+    kFBardQFull = 25,   // +dS buffer: dQ_i complete
     kFBarYFree = 27,    // count 128: dQ_i copied out (alternating warpgroups: dP_i in registers): Y may take dP_{i+1}
     kFBarFinal = 28,    // last dV and dK complete, count = warps that issue them
     kFBarDrain = 29,    // +issuer (3): abort path only
@@ -529,23 +529,23 @@ struct FusedParams {
     int finish_behind_rows;     // the finish kernel is let go behind that kernel as well
 };
 
-template <int D, bool SLOT = false>
-__global__ void __launch_bounds__(FusedSmem<D>::kThreads, 1)
+template <int D, bool SLOT = false, bool ALT = (D == 64)>
+__global__ void __launch_bounds__(FusedSmem<D, ALT>::kThreads, 1)
 moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
                       const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapdO,
                       const __grid_constant__ CUtensorMap mapdK, const __grid_constant__ CUtensorMap mapdV,
                       const FusedParams p) {
-    using L = FusedSmem<D>;
+    using L = FusedSmem<D, ALT>;
     constexpr int NSUB = D / 64;
-    constexpr int NRW = L::kRowWGs, COLS = L::kCols, NROW = 128 * NRW;      // row warpgroups, columns per thread, row threads
-    constexpr bool ALT = L::kAlternate;
+    constexpr int NRW = L::kRowWGs, NROW = 128 * NRW;             // row warpgroups, row threads
     constexpr int kRowArrivals = ALT ? 128 : NROW;
     constexpr int W_DRAIN = 4 * NRW, W_LOAD = W_DRAIN + 4, W_S = W_LOAD + 1, W_DP = W_LOAD + 2;
     constexpr int W_ACC = W_LOAD + 3;                             // issues the three accumulating contractions
     constexpr int NOTHER = (L::kThreads / 32 - W_LOAD) * 32;      // threads of the loader / issuer warps
     constexpr uint32_t kTmemCols = 512;
-    // d = 64 leaves room for a second S^T / P^T buffer: one per row warpgroup
-    constexpr int XB = (D == 64) ? 2 : 1;
+    // d = 64 leaves room for a second S^T / P^T buffer: one per row warpgroup, or S_{i+1} while they work on tile i (B = 8, 32 heads, l = 0: T = 640
+    // 128 us with one buffer, 124 with two; T = 256 42.5, 41.9)
+    constexpr int XB = (D == 64) ? 2 : 1, WB = ALT ? 2 : 1;       // S^T / P^T buffers; dP, dS and dQ barriers
     constexpr uint32_t kColX = 0, kColY = 128 * XB, kColdK = kColY + 128, kColdV = kColdK + D;
     static_assert(kColdV + D <= kTmemCols, "tensor-memory plan too large");
 
@@ -637,23 +637,19 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     constexpr int kRegsLaunch = 128;
     static_assert(L::kThreads == 512, "the register shares below assume 512 threads");
     // Shares measured (T = 8192 .. 65536): the issuing warps need about 100 registers to keep their descriptors and
-    // barrier addresses without spills; d = 128: 128 / 160 / 96 (42.1 ms at T = 65536 against 44.1 with 136 / 160 / 80).  d = 64: 128
-    // scores and what becomes of them in a row thread, a dQ row of 64 in a drain thread.
-    constexpr int kRegsRow = (D == 128) ? 128 : 160, kRegsDrain = (D == 128) ? 160 : 96, kRegsOther = 96;
+    // barrier addresses without spills; d = 128: 128 / 160 / 96 (42.1 ms at T = 65536 against 44.1 with 136 / 160 / 80).  Alternate iterations:
+    // 128 scores and what becomes of them in a row thread, a dQ row of 64 in a drain thread; d = 64, shared: 28.5 ms with 152 / 152 / 56, 27.6 with
+    // 136 / 136 / 104 (T = 32768, H = 32).
+    constexpr int kRegsRow = (D == 128) ? 128 : ALT ? 160 : 136, kRegsDrain = (D == 128) ? 160 : ALT ? 96 : 136, kRegsOther = (D == 128 || ALT) ? 96 : 104;
     static_assert(NROW * kRegsRow + 128 * kRegsDrain + NOTHER * kRegsOther <= L::kThreads * kRegsLaunch, "register shares exceed the CTA's pool");
     // setmaxnreg.inc to less than the current count (or .dec to more) is an illegal instruction
     static_assert(kRegsRow >= kRegsLaunch && kRegsOther <= kRegsLaunch, "setmaxnreg direction");
     if (warp < W_DRAIN) {
         // =========================== row warps: P^T, dS^T, dK / dV epilogue ===========================
         setmaxnreg_inc<kRegsRow>();
-        const int hc = warp >> 2;                            // which COLS query columns of every iteration
+        const int hc = warp >> 2;                            // which row warpgroup
         const int r = tid & 127;                             // key row inside the tile = TMEM lane
         const uint32_t lane_addr = uint32_t((warp & 3) * 32) << 16;
-        const uint32_t tX0 = tmem + lane_addr + kColX + hc * COLS;
-        const uint32_t tY = tmem + lane_addr + kColY + hc * COLS;
-        // this thread's row of dS^T: sub-tile of its 64-column half, 128-byte rows, its first 16-byte chunk
-        uint8_t* ds_row = smem + L::kdS + ((hc * COLS) >> 6) * L::kSubBytes + r * 128;
-        const int ds_chunk0 = ((hc * COLS) & 63) >> 3;
         if constexpr (ALT) {
             // this warpgroup's iterations: hc, hc + 2, ...  One key row and all 128 query columns of each.
             const uint32_t tXw = tmem + lane_addr + kColX + hc * 128, tYw = tmem + lane_addr + kColY;
@@ -732,6 +728,10 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 mbar_arrive(bar(kFBardSFull + hc));
             }
         } else {
+        constexpr int COLS = kTileRows / NRW;                // query columns per thread, of every iteration
+        static_assert(COLS == 64, "a 64-column sub-tile of dS^T per warpgroup");
+        const uint32_t tX0 = tmem + lane_addr + kColX + hc * COLS, tY = tmem + lane_addr + kColY + hc * COLS;
+        uint8_t* ds_row = smem + L::kdS + hc * L::kSubBytes + r * 128;
 #pragma unroll 1
         for (int it = 0, qi = kt; it < n_it; ++it, qi = (qi + 1 < nk) ? qi + 1 : kt) {
             uint32_t pk[COLS / 2];                           // P_i^T of this thread: COLS values, bf16 pairs
@@ -771,8 +771,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 }
             }
             // P^T (bf16, two per column) overlays the first half of the columns this thread has read
-            if constexpr (COLS == 64) tmem_st32(tX, *reinterpret_cast<uint32_t(*)[32]>(pk));
-            else tmem_st16(tX, *reinterpret_cast<uint32_t(*)[16]>(pk));
+            tmem_st32(tX, pk);
             tmem_wait_st();
             tc_fence_before_sync();
             mbar_arrive(bar(kFBarPFull + xb));
@@ -798,7 +797,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                         w[k] = pack_bf16x2(x0, x1);
                     }
                     const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-                    *reinterpret_cast<uint4*>(ds_row + (((ds_chunk0 + g) ^ (r & 7)) << 4)) = v;
+                    *reinterpret_cast<uint4*>(ds_row + ((g ^ (r & 7)) << 4)) = v;
                 }
             }
             fence_proxy_async_smem();                        // generic-proxy stores -> read by the MMAs (async proxy)
@@ -808,7 +807,6 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 
         }
         // ---- epilogue: dK (scaled) by the first warpgroup, dV by the second ----
-        if (hc < 2) {
         // In a stack the later layers' gradient of this layer's K, V lies in a slot of the gradient cache, whose K or V block
         // of this tile is laid out as the threads read it here (chunk, then row: 512 contiguous bytes per warp).  A copy kernel
         // behind the backward would read and write dK, dV once more: 12.5 us a layer at 2 x 1000 positions of 16 heads, and the pass
@@ -862,7 +860,6 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             tma_store_commit();
             tma_store_wait_read();
         }
-        }
     } else if (warp < W_LOAD) {
         // =========================== drain warps: dQ tile -> fp32 accumulator ===========================
         // The tile leaves the SM as bulk reductions (cp.reduce.async.bulk, fp32 add in L2) from a staging buffer
@@ -879,8 +876,8 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         int slot = 0;
 #pragma unroll 1
         for (int it = 0, qi = kt; it < n_it; ++it) {
-            const int xb = it % XB;
-            mbar_wait(bar(kFBardQFull + xb), (it / XB) & 1, abort_flag, 120);
+            const int xb = it % WB;
+            mbar_wait(bar(kFBardQFull + xb), (it / WB) & 1, abort_flag, 120);
             tc_fence_after_sync();
             uint32_t o[D];
 #pragma unroll
@@ -925,7 +922,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
           // 16 queries per k-step: 8 columns; with half the columns per row warpgroup, in the block of the one that owns them
 #pragma unroll 4
           for (int kk = 0; kk < kTileRows / 16; ++kk)
-              umma_ts(tmem + kColdV, tmem + kColX + xb * 128 + (ALT ? kk * 8 : (kk / (COLS / 16)) * COLS + (kk % (COLS / 16)) * 8), dvb + uint64_t(kk * 128),
+              umma_ts(tmem + kColdV, tmem + kColX + xb * 128 + (ALT ? kk * 8 : (kk >> 2) * 64 + (kk & 3) * 8), dvb + uint64_t(kk * 128),
                       idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
           umma_commit(bar(kFBarXFree + xb));
           umma_commit(bar(kFBardOEmpty + dst));
@@ -1016,7 +1013,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
                 const int xb = it % nb;
                 const uint32_t col = is_s ? kColX + xb * 128 : kColY;
                 const uint32_t free_bar = is_s ? bar(kFBarXFree + xb) : bar(kFBarYFree);
-                const int ob = it % XB;
+                const int ob = it % WB;
                 if (it >= nb) mbar_wait2(bar(full0 + st), (it / nst) & 1, free_bar, ((it - nb) / nb) & 1, abort_flag, 141, is_s ? 142 : 143);
                 else mbar_wait(bar(full0 + st), (it / nst) & 1, abort_flag, 141);
                 // dP also needs the Q stage's per-query terms (they arrive with Q_i)
@@ -1044,11 +1041,11 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             drain_on_abort(is_s ? 0 : 1);
         }
       } else if (warp == W_ACC) {
-        // ============ MMA issuer of the accumulating contractions.  d = 128: dV_i += P^T dO (P^T from tensor memory, dO MN-major),
+        // ============ MMA issuer of the accumulating contractions.  Shared iterations: dV_i += P^T dO (P^T from tensor memory, dO MN-major),
         // ============ then, once dS_i^T is in shared memory, dQ_tile = dS K into Y (dS^T and K both MN-major) and
         // ============ dK += dS^T Q (dS^T K-major, Q MN-major).  P_i, dS_i, P_{i+1} are produced in this order, so one
         // ============ warp can take the three in turn.  dQ before dK: its tile has to be copied out before dP of the next
-        // ============ iteration can land, dK only has to finish before dS_{i+1} is written.  d = 64: dK_i, then dQ_i, whose columns
+        // ============ iteration can land, dK only has to finish before dS_{i+1} is written.  Alternate: dK_i, then dQ_i, whose columns
         // ============ P_{i+1} has to leave first.
         {
             constexpr uint32_t idesc_dq = make_idesc_bf16(128, D, true, true);
@@ -1058,14 +1055,14 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
             const uint64_t dkb0 = desc_mnmajor_sw128(sbase + L::kQ, 0, L::kSubBytes);
 #pragma unroll 1
             for (int it = 0; it < n_it; ++it) {
-                const int st = it % L::kStages, dst = it % L::kdOStages, xb = it % XB;
+                const int st = it % L::kStages, dst = it % L::kdOStages, xb = it % XB, wb = it % WB;
                 if constexpr (!ALT) {
                     mbar_wait2(bar(kFBarPFull + xb), (it / XB) & 1, bar(kFBardOFull + dst), (it / L::kdOStages) & 1, abort_flag, 144, 145);
                     tc_fence_after_sync();
                     issue_dV(it, dst, xb);
                 }
-                const uint64_t dsb = uint64_t((ALT ? xb * L::kdSBytes : 0) >> 4);
-                mbar_wait(bar(kFBardSFull + xb), (it / XB) & 1, abort_flag, 146);
+                const uint64_t dsb = uint64_t((wb * L::kdSBytes) >> 4);
+                mbar_wait(bar(kFBardSFull + wb), (it / WB) & 1, abort_flag, 146);
                 tc_fence_after_sync();
                 const uint64_t dkb = dkb0 + uint64_t((st * L::kTileBytes) >> 4);
                 auto issue_dK = [&]() {
@@ -1085,7 +1082,7 @@ moda_bwd_fused_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 #pragma unroll 4
                 for (int kk = 0; kk < kTileRows / 16; ++kk)
                     umma_ss(tmem + (ALT ? kColX + (xb ^ 1) * 128 + 64 : kColY), dqa0 + dsb + uint64_t(kk * 128), dqb0 + uint64_t(kk * 128), idesc_dq, kk > 0);
-                umma_commit(bar(kFBardQFull + xb));
+                umma_commit(bar(kFBardQFull + wb));
                 if constexpr (ALT) umma_commit(bar(kFBardSFree + xb));
                 else issue_dK();
             }

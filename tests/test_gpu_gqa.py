@@ -167,7 +167,7 @@ def test_autograd_wrapper_gives_the_oracle_gradients():
 # d = 64: the fused backward's two row warpgroups take alternate (query head, query tile) pairs of a key tile: one pair in all, an odd
 # and an even number, a last tile with one row, and pairs that run on from one head of a group to the next.
 @pytest.mark.parametrize("H,Hk", [(1, 1), (6, 2)])
-@pytest.mark.parametrize("T", [1, 128, 129, 256, 385, 513, 1153])
+@pytest.mark.parametrize("T", [1, 128, 129, 256, 385, 513, 768, 769, 1000, 1153])
 def test_narrow_backward_with_alternating_warpgroups(T, H, Hk):
     x = synthetic.make_gqa(1, T, H, Hk, 64, 0, seed=5, device="cuda")
     scale = 64 ** -0.5

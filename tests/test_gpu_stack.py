@@ -89,7 +89,7 @@ def test_accumulate_flag_adds_the_depth_gradients_to_what_the_cache_holds(B, T, 
     assert rel_l2(acc.double().cpu().numpy(), want2.cpu().numpy()) < 1e-2
 
 
-@pytest.mark.parametrize("B,T,H,Hk,d,l,slot", [(1, 1, 1, 1, 64, 0, 0), (1, 127, 2, 2, 128, 0, 2), (2, 129, 3, 3, 128, 3, 3), (2, 257, 3, 3, 64, 2, 4),
+@pytest.mark.parametrize("B,T,H,Hk,d,l,slot", [(1, 1, 1, 1, 64, 0, 0), (1, 127, 2, 2, 128, 0, 2), (2, 129, 3, 3, 128, 3, 3), (2, 257, 3, 3, 64, 2, 4), (1, 900, 2, 2, 64, 2, 3), (1, 385, 4, 2, 64, 1, 1),
                                                (1, 1000, 2, 2, 128, 5, 6), (1, 700, 4, 4, 64, 9, 9), (1, 300, 8, 2, 128, 0, 1),
                                                (1, 200, 8, 1, 64, 12, 12), (2, 130, 16, 1, 64, 9, 10)])
 def test_backward_that_takes_up_a_slot_of_the_gradient_cache(B, T, H, Hk, d, l, slot):

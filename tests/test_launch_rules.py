@@ -10,6 +10,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 SOURCE = r"""
 #include "launch_rules.h"
+extern "C" int alternates(int d, int T, int G) { return moda::bwd_alternates(d, T, G); }
 extern "C" unsigned row_ctas(int d, int bh, int T, int l, unsigned units, unsigned sms, int fp8) { return moda::bwd_row_ctas(d, bh, T, l, units, sms, fp8 != 0); }
 """
 
@@ -49,3 +50,11 @@ def test_sms_of_the_depth_part_over_all_shapes(rules):
         assert 1 <= n <= min(units, sms), case
         assert n % 2 == 0 or n == units, case
         assert n >= min(16, units) or -(-units // n) == -(-units // 16), case
+
+
+def test_alternate_iterations_where_they_were_measured_to_win(rules):
+    assert not any(rules.alternates(128, T, G) for T in (1, 65536) for G in (1, 8))
+    for T, G in ((1, 1), (512, 1), (768, 1), (128, 3), (256, 2)):
+        assert not rules.alternates(64, T, G)
+    for T, G in ((769, 1), (65536, 1), (129, 3), (257, 2), (300, 4), (100, 8)):
+        assert rules.alternates(64, T, G)
