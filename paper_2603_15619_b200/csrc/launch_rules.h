@@ -6,6 +6,19 @@
 
 namespace moda {
 
+// Whether a d = 128 forward takes the kernel with two softmax warpgroups (moda_fwd_wide128.cuh).  It is the faster one where the key tiles
+// set the pace; where the depth slots do, its ring of three units against five and the smaller register share of its depth warps
+// cost it up to a fifth.  us, one warpgroup -> two (B = 2, 16 heads): l = 0: T = 128 7.2 -> 7.2, T = 1000 23.9 -> 22.2, T = 2048 57.7 -> 51.9,
+// T = 8192 552 -> 481, T = 16384 2339 -> 1964.  l = 4: T = 1000 27.1 -> 25.8, T = 512 11.4 -> 11.8.  l = 8: T = 4096 238 -> 223, T = 2048 84.0 -> 84.3,
+// T = 1000 33.1 -> 37.9.  l = 16: T = 8192 716 -> 714 and 719 -> 650, T = 4096 268 -> 291.  l = 24: T = 16384 2545 -> 2420, T = 8192 802 -> 842.  e4m3,
+// l = 8: T = 2048 73.6 -> 73.4, T = 1000 30.2 -> 33.8; l = 16: T = 8192 714 -> 631, T = 4096 235 -> 260.  2000 over 15000, l = 24, B = 4: 1192 -> 985.
+// With a key tile or two there is little to alternate: T = 100, 2 heads: l = 1 7.26 -> 7.35, l = 2 7.81 -> 8.08 (e4m3 7.77 -> 8.39); T = 129: l = 1 7.68 -> 7.53, l = 2
+// 8.08 -> 8.28; T = 256, B = 4, 32 heads: l = 1 16.4 -> 16.2, l = 2 17.4 -> 17.7; T = 300: l = 2 26.2 -> 26.0 (e4m3 26.1 -> 26.2).
+inline bool fwd_two_softmax(int T_q, int T_kv, int l) {
+    const long long keys = 2ll * T_kv - T_q;                 // twice the mean number of keys of a query: T when T_q = T_kv = T
+    return keys > 128 && 128ll * l < keys && 560ll * l <= keys + 1120;
+}
+
 // How many SMs the depth part of a fused backward gets beside the sequence part.  Measured SM time: an entry of the row
 // ring 1.75 us (16 SMs at it) to 2.0 us (50), e4m3 a tenth more; an iteration of the sequence part at d = 128 2.7 us
 // and 5 us per key tile around them; at d = 64 11 us per key tile and 1.33 us an iteration, rising to 1.5 us for the longest (their runs

@@ -207,17 +207,6 @@ inline bool fwd_depth_heavy(int T_q, int T_kv, int l, int d) {
     return d == 128 && l > 0 && 2ll * l * d >= 2ll * T_kv - T_q;
 }
 
-// Whether a d = 128 forward takes the kernel with two softmax warpgroups (moda_fwd_wide128.cuh).  It is the faster one where the key tiles
-// set the pace; where the depth slots do, its ring of three units against five and the smaller register share of its depth warps
-// cost it up to a fifth.  us, one warpgroup -> two (B = 2, 16 heads): l = 0: T = 128 7.2 -> 7.2, T = 1000 23.9 -> 22.2, T = 2048 57.7 -> 51.9,
-// T = 8192 552 -> 481, T = 16384 2339 -> 1964.  l = 4: T = 1000 27.1 -> 25.8, T = 512 11.4 -> 11.8.  l = 8: T = 4096 238 -> 223, T = 2048 84.0 -> 84.3,
-// T = 1000 33.1 -> 37.9.  l = 16: T = 8192 716 -> 714 and 719 -> 650, T = 4096 268 -> 291.  l = 24: T = 16384 2545 -> 2420, T = 8192 802 -> 842.  e4m3,
-// l = 8: T = 2048 73.6 -> 73.4, T = 1000 30.2 -> 33.8; l = 16: T = 8192 714 -> 631, T = 4096 235 -> 260.  2000 over 15000, l = 24, B = 4: 1192 -> 985.
-inline bool fwd_two_softmax(int T_q, int T_kv, int l) {
-    // against twice the mean number of keys of a query: 2 T_kv - T_q, T when T_q = T_kv = T
-    return 560ll * l <= 2ll * T_kv - T_q + 1120;
-}
-
 // Whether a grouped-query forward runs its depth part as the separate per-position kernel.  Measured at
 // d = 64 (T = 16384, 8 key/value heads): the fused row-local path costs about 2.3 us per (query head per
 // group, slot), the separate kernel about 200 us plus 11.7 us per slot whatever the group size, so the

@@ -10,6 +10,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 SOURCE = r"""
 #include "launch_rules.h"
+extern "C" int two_softmax(int T_q, int T_kv, int l) { return moda::fwd_two_softmax(T_q, T_kv, l); }
 extern "C" int alternates(int d, int T, int G) { return moda::bwd_alternates(d, T, G); }
 extern "C" unsigned row_ctas(int d, int bh, int T, int l, unsigned units, unsigned sms, int fp8) { return moda::bwd_row_ctas(d, bh, T, l, units, sms, fp8 != 0); }
 """
@@ -58,3 +59,11 @@ def test_alternate_iterations_where_they_were_measured_to_win(rules):
         assert not rules.alternates(64, T, G)
     for T, G in ((769, 1), (65536, 1), (129, 3), (257, 2), (300, 4), (100, 8)):
         assert rules.alternates(64, T, G)
+
+
+def test_two_softmax_warpgroups_where_they_were_measured_to_win(rules):
+    for T, l in ((129, 0), (129, 1), (256, 1), (257, 2), (512, 2), (2048, 4), (4096, 8), (8192, 16), (16384, 24)):
+        assert rules.two_softmax(T, T, l), (T, l)
+    for T, l in ((1, 0), (128, 0), (128, 1), (129, 2), (256, 2), (512, 4), (1000, 8), (4096, 16), (8192, 24)):
+        assert not rules.two_softmax(T, T, l), (T, l)
+    assert rules.two_softmax(2000, 15000, 24) and rules.two_softmax(1, 100, 0) and rules.two_softmax(1, 65536, 24) and not rules.two_softmax(64, 96, 1)
