@@ -252,3 +252,28 @@ def test_quantiser_is_bit_exact_over_a_wide_range_of_rows_and_on_ties():
         assert np.array_equal(scales[:, kv], ref_scale), "row scales differ"
         bad = np.argwhere(codes[:, kv] != ref_codes)
         assert bad.size == 0, f"{len(bad)} codes differ, first at {bad[0]}: got {codes[:, kv][tuple(bad[0])]}, want {ref_codes[tuple(bad[0])]}"
+
+
+@pytest.mark.parametrize("B,T,H,Hk,l", [(3, 2190, 16, 16, 3), (4, 1100, 22, 22, 2), (2, 2400, 22, 11, 3), (2, 4500, 16, 16, 8)])
+def test_forward_on_pairs_of_query_tiles_against_the_oracle(B, T, H, Hk, l):
+    """d = 128 with enough CTAs for a pair of query tiles each (an odd number of tiles leaves one alone): the depth ring and its stages run on
+    from the first tile of a CTA to the second.  Three heads against the oracle, through an e4m3 and a bf16 cache."""
+    d, scale = 128, 128 ** -0.5
+    tiles = -(-T // 128)
+    pairs = B * H * ((tiles + 1) // 2)
+    assert pairs >= 296 and 100 * pairs >= 93 * 148 * -(-pairs // 148)       # the kernel takes pairs (launch_fwd in moda_api.cu)
+    x = synthetic.make_gqa(B, T, H, Hk, d, l, seed=83, device="cuda")
+    cache8, cache = build_cache8(x["Kd"], x["Vd"]), moda.alloc_depth_cache(B, T, Hk, d, l)
+    for i in range(l):
+        moda.moda_depth_cache_append(cache, i, x["Kd"][i].contiguous(), x["Vd"][i].contiguous())
+    got8 = moda.moda_attn_fwd_e4m3(x["Q"], x["K"], x["V"], cache8, l, scale)
+    got = moda.moda_attn_fwd_gqa(x["Q"], x["K"], x["V"], cache, l, scale)
+    assert moda.moda_last_status() == 0
+    for b, h in ((0, 0), (B - 1, H // 2), (B - 1, H - 1)):
+        hk = h // (H // Hk)
+        one = lambda t, i: f64(t[..., b:b + 1, :, i:i + 1, :])
+        Kd, Vd = one(x["Kd"], hk), one(x["Vd"], hk)
+        hat = [orc.dequantize_e4m3_rows(*orc.quantize_e4m3_rows(t)) for t in (Kd, Vd)]
+        for (O, LSE), slots in ((got8, hat), (got, (Kd, Vd))):
+            ref = orc.forward(one(x["Q"], h), one(x["K"], hk), one(x["V"], hk), *slots, scale)
+            assert_forward_close(O[b:b + 1, :, h:h + 1], LSE[b:b + 1, h:h + 1], *ref, f"{(b, h)}")
