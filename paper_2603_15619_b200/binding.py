@@ -181,28 +181,34 @@ def _ptr(t):
     return t.data_ptr()
 
 
-def _sized(t, numel, dtype):
-    """Address of a tensor that a kernel reads or writes ``numel`` elements of type ``dtype`` of."""
-    if t is not None and (t.dtype != dtype or t.numel() < numel):
+def _given(t, numel, dtype):
+    """A tensor of the caller's that a kernel reads or writes ``numel`` elements of."""
+    if t.dtype != dtype or t.numel() < numel:
         raise ValueError(f"{numel} elements of type {dtype} required, not {t.numel()} of type {t.dtype}")
-    return _ptr(t)
+    return t
 
 
-def _bf16(t, numel):
-    return _sized(t, numel, torch.bfloat16)
+def _bf16(t, numel, dtype=torch.bfloat16):
+    """Its address."""
+    if t is None:
+        return None
+    if t.dtype is dtype and t.numel() >= numel and t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
+    return _ptr(_given(t, numel, dtype))                       # says what is wrong
 
 
 def _f32(t, numel):
-    return _sized(t, numel, torch.float32)
+    return _bf16(t, numel, torch.float32)
 
 
-def _slots(cache, n, *shape, e4m3=False):
-    """Address of a depth cache, or of its gradient, that holds at least ``n`` slots of ``shape`` = B, T, H_kv, d (a number of slots
-    that no cache has is the C call's to refuse)."""
-    if cache is not None:
-        need = (moda_depth_cache_e4m3_bytes if e4m3 else moda_depth_cache_bytes)(*shape, max(0, min(n, MODA_MAX_DEPTH + 1)))
-        if cache.numel() * cache.element_size() < need:
-            raise ValueError(f"{n} slots of this shape take {need} bytes, the depth cache has {cache.numel() * cache.element_size()}")
+def _slots(cache, n, B, T, H, d, e4m3=False):
+    """Address of a depth cache, or of its gradient, that holds at least ``n`` slots (a number of slots or a width that no cache has is the
+    C call's to refuse).  The size as moda_depth_cache_bytes and moda_depth_cache_e4m3_bytes give it, without the calls' 2 us: K and V rows of
+    2 d bytes, or of d codes and an fp32 scale, in whole tiles of 128 positions."""
+    if cache is not None and 0 < n <= MODA_MAX_DEPTH and (d == 64 or d == 128):
+        need = n * B * H * ((T + 127) >> 7) * 256 * (d + 4 if e4m3 else 2 * d)
+        if cache.nbytes < need:
+            raise ValueError(f"{n} slots of this shape take {need} bytes, the depth cache has {cache.nbytes}")
     return _ptr(cache)
 
 
@@ -299,17 +305,19 @@ def depth_cache_window(cache, B, T, H, d, first_slot, n_slots=None):
 
 def moda_depth_cache_append(cache, slot, K_i, V_i, stream=None):
     B, T, H, d = _bthd(K_i, "K_i")
+    n = B * T * H * d
     assert _bthd(V_i, "V_i") == (B, T, H, d)
     _check(load().moda_depth_cache_append(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
-                                          _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
+                                          _bf16(K_i, n), _bf16(V_i, n), _stream(stream)),
            "moda_depth_cache_append")
 
 
 def moda_depth_cache_unpack(cache, slot, K_i, V_i, stream=None):
     ref = K_i if K_i is not None else V_i
     B, T, H, d = _bthd(ref, "K_i/V_i")
+    n = B * T * H * d
     _check(load().moda_depth_cache_unpack(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
-                                          _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
+                                          _bf16(K_i, n), _bf16(V_i, n), _stream(stream)),
            "moda_depth_cache_unpack")
 
 
@@ -317,8 +325,9 @@ def moda_depth_cache_unpack_add(cache, slot, K_i, V_i, stream=None):
     """K_i, V_i += slot ``slot`` of a (gradient) cache, each sum rounded to bf16 once."""
     ref = K_i if K_i is not None else V_i
     B, T, H, d = _bthd(ref, "K_i/V_i")
+    n = B * T * H * d
     _check(load().moda_depth_cache_unpack_add(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
-                                              _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
+                                              _bf16(K_i, n), _bf16(V_i, n), _stream(stream)),
            "moda_depth_cache_unpack_add")
 
 
@@ -337,21 +346,20 @@ def alloc_depth_cache_e4m3(B, T, H, d, l_max, device="cuda", stream=None) -> tor
 def moda_depth_cache_append_e4m3(cache, slot, K_i, V_i, stream=None):
     """Quantise K_i, V_i (bf16 [B,T,H,d]) into slot ``slot`` of an e4m3 depth cache (codes + one fp32 scale per row)."""
     B, T, H, d = _bthd(K_i, "K_i")
+    n = B * T * H * d
     assert _bthd(V_i, "V_i") == (B, T, H, d)
     _check(load().moda_depth_cache_append_e4m3(_slots(cache, int(slot) + 1, B, T, H, d, e4m3=True), B, T, H, d, int(slot),
-                                               _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
+                                               _bf16(K_i, n), _bf16(V_i, n), _stream(stream)),
            "moda_depth_cache_append_e4m3")
 
 
 def moda_attn_fwd_e4m3(Q, K, V, depth_kv_e4m3, l, scale, O=None, LSE=None, stream=None):
     """moda_attn_fwd_gqa with the depth slots read from an e4m3 cache."""
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T, torch.float32)
     _check(load().moda_attn_fwd_e4m3(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_e4m3, int(l), B, T, Hk, d, e4m3=True) if l > 0 else None,
-                                     B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
+                                     B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
            "moda_attn_fwd_e4m3")
     return O, LSE
 
@@ -359,12 +367,10 @@ def moda_attn_fwd_e4m3(Q, K, V, depth_kv_e4m3, l, scale, O=None, LSE=None, strea
 def moda_attn_fwd_append_e4m3(Q, K, V, depth_kv_e4m3, l, scale, append_cache_e4m3, append_slot, O=None, LSE=None, stream=None):
     """moda_attn_fwd_e4m3 that also quantises K, V into slot ``append_slot`` of an e4m3 cache (a second launch behind it)."""
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T, torch.float32)
     _check(load().moda_attn_fwd_append_e4m3(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_e4m3, int(l), B, T, Hk, d, e4m3=True) if l > 0 else None,
-                                            B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T),
+                                            B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
                                             _slots(append_cache_e4m3, int(append_slot) + 1, B, T, Hk, d, e4m3=True), int(append_slot), _stream(stream)),
            "moda_attn_fwd_append_e4m3")
     return O, LSE
@@ -374,17 +380,18 @@ def moda_attn_bwd_e4m3(Q, K, V, depth_kv_e4m3, O, dO, LSE, l, scale,
                        dQ=None, dK=None, dV=None, d_depth_kv=None, workspace=None, stream=None):
     """moda_attn_bwd with the depth slots read from an e4m3 cache; the depth gradients come back in the bf16 cache layout."""
     B, T, H, d = _bthd(Q, "Q")
-    dQ = _new_like(Q, stream) if dQ is None else dQ
-    dK = _new_like(K, stream) if dK is None else dK
-    dV = _new_like(V, stream) if dV is None else dV
+    n = Q.numel()
+    dQ = _new_like(Q, stream) if dQ is None else _given(dQ, n, torch.bfloat16)
+    dK = _new_like(K, stream) if dK is None else _given(dK, K.numel(), torch.bfloat16)
+    dV = _new_like(V, stream) if dV is None else _given(dV, V.numel(), torch.bfloat16)
     if l > 0 and d_depth_kv is None:
         d_depth_kv = alloc_depth_cache(B, T, H, d, l, Q.device, stream)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes(B, T, H, d, l),), torch.uint8, Q.device, stream)
-    _check(load().moda_attn_bwd_e4m3(_ptr(Q), _bf16(K, Q.numel()), _bf16(V, Q.numel()),
+    _check(load().moda_attn_bwd_e4m3(_ptr(Q), _bf16(K, n), _bf16(V, n),
                                      _slots(depth_kv_e4m3, int(l), B, T, H, d, e4m3=True) if l > 0 else None,
-                                     _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
-                                     _bf16(dQ, Q.numel()), _bf16(dK, Q.numel()), _bf16(dV, Q.numel()),
+                                     _bf16(O, n), _bf16(dO, n), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
+                                     _ptr(dQ), _ptr(dK), _ptr(dV),
                                      _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
                                      _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_bwd_e4m3")
@@ -394,29 +401,29 @@ def moda_attn_bwd_e4m3(Q, K, V, depth_kv_e4m3, O, dO, LSE, l, scale,
 def moda_depth_cache_append_pm(cache, slot, K_i, V_i, stream=None):
     """moda_depth_cache_append for the position-major layout (grouped-query calls through the *_pm entry points)."""
     B, T, H, d = _bthd(K_i, "K_i")
+    n = B * T * H * d
     assert _bthd(V_i, "V_i") == (B, T, H, d)
     _check(load().moda_depth_cache_append_pm(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
-                                             _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
+                                             _bf16(K_i, n), _bf16(V_i, n), _stream(stream)),
            "moda_depth_cache_append_pm")
 
 
 def moda_depth_cache_unpack_pm(cache, slot, K_i, V_i, stream=None):
     ref = K_i if K_i is not None else V_i
     B, T, H, d = _bthd(ref, "K_i/V_i")
+    n = B * T * H * d
     _check(load().moda_depth_cache_unpack_pm(_slots(cache, int(slot) + 1, B, T, H, d), B, T, H, d, int(slot),
-                                             _bf16(K_i, B * T * H * d), _bf16(V_i, B * T * H * d), _stream(stream)),
+                                             _bf16(K_i, n), _bf16(V_i, n), _stream(stream)),
            "moda_depth_cache_unpack_pm")
 
 
 def moda_attn_fwd_gqa_pm(Q, K, V, depth_kv_pm, l, scale, O=None, LSE=None, stream=None):
     """moda_attn_fwd_gqa with the depth slots in the position-major layout (H_kv < H)."""
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T, torch.float32)
     _check(load().moda_attn_fwd_gqa_pm(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_pm, int(l), B, T, Hk, d) if l > 0 else None,
-                                       B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
+                                       B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
            "moda_attn_fwd_gqa_pm")
     return O, LSE
 
@@ -425,16 +432,17 @@ def moda_attn_bwd_gqa_pm(Q, K, V, depth_kv_pm, O, dO, LSE, l, scale,
                          dQ=None, dK=None, dV=None, d_depth_kv_pm=None, workspace=None, stream=None):
     """moda_attn_bwd_gqa with the depth slots and the depth gradients in the position-major layout."""
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    dQ = _new_like(Q, stream) if dQ is None else dQ
-    dK = _new_like(K, stream) if dK is None else dK
-    dV = _new_like(V, stream) if dV is None else dV
+    n = Q.numel()
+    dQ = _new_like(Q, stream) if dQ is None else _given(dQ, n, torch.bfloat16)
+    dK = _new_like(K, stream) if dK is None else _given(dK, K.numel(), torch.bfloat16)
+    dV = _new_like(V, stream) if dV is None else _given(dV, V.numel(), torch.bfloat16)
     if l > 0 and d_depth_kv_pm is None:
         d_depth_kv_pm = alloc_depth_cache(B, T, Hk, d, l, Q.device, stream)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
     _check(load().moda_attn_bwd_gqa_pm(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv_pm, int(l), B, T, Hk, d) if l > 0 else None,
-                                       _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, Hk, d, int(l), float(scale),
-                                       _bf16(dQ, Q.numel()), _bf16(dK, K.numel()), _bf16(dV, K.numel()),
+                                       _bf16(O, n), _bf16(dO, n), _f32(LSE, B * H * T), B, T, H, Hk, d, int(l), float(scale),
+                                       _ptr(dQ), _ptr(dK), _ptr(dV),
                                        _slots(d_depth_kv_pm, int(l), B, T, Hk, d) if l > 0 else None,
                                        _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_bwd_gqa_pm")
@@ -454,12 +462,12 @@ def moda_kv_project_append(X, Wk, Wv, H_kv, cache=None, slot=0, store_kv=True, K
         raise ValueError("Wk, Wv must be bf16 [H_kv d, D_model] tensors matching X")
     d = n // H_kv
     if store_kv:
-        K_out = _new((B, T, H_kv, d), torch.bfloat16, X.device, stream) if K_out is None else K_out
-        V_out = _new((B, T, H_kv, d), torch.bfloat16, X.device, stream) if V_out is None else V_out
+        K_out = _new((B, T, H_kv, d), torch.bfloat16, X.device, stream) if K_out is None else _given(K_out, B * T * n, torch.bfloat16)
+        V_out = _new((B, T, H_kv, d), torch.bfloat16, X.device, stream) if V_out is None else _given(V_out, B * T * n, torch.bfloat16)
     else:
         K_out = V_out = None
     fn = load().moda_kv_project_append_e4m3 if e4m3 else load().moda_kv_project_append
-    _check(fn(_ptr(X), _ptr(Wk), _ptr(Wv), B, T, Dm, int(H_kv), d, _bf16(K_out, B * T * n), _bf16(V_out, B * T * n),
+    _check(fn(_ptr(X), _ptr(Wk), _ptr(Wv), B, T, Dm, int(H_kv), d, _ptr(K_out), _ptr(V_out),
               _slots(cache, int(slot) + 1, B, T, int(H_kv), d, e4m3=e4m3), int(slot), _stream(stream)),
            "moda_kv_project_append_e4m3" if e4m3 else "moda_kv_project_append")
     return K_out, V_out
@@ -475,13 +483,12 @@ def moda_depth_slot_mass(Q, depth_kv, LSE, l, scale, H_kv=None, mass=None, works
     positions (Q and LSE of the forward call; the bf16 row-interleaved cache it read)."""
     B, T, H, d = _bthd(Q, "Q")
     H_kv = H if H_kv is None else int(H_kv)
-    if mass is None:
-        mass = _new((B, H, int(l)), torch.float32, Q.device, stream)
+    mass = _new((B, H, int(l)), torch.float32, Q.device, stream) if mass is None else _given(mass, B * H * int(l), torch.float32)
     need = int(load().moda_depth_slot_mass_workspace_bytes(B, T, H, int(l)))
     if workspace is None:
         workspace = _new((max(need, 16),), torch.uint8, Q.device, stream)
     _check(load().moda_depth_slot_mass(_ptr(Q), _slots(depth_kv, int(l), B, T, H_kv, d) if l > 0 else None, _f32(LSE, B * H * T),
-                                       B, T, H, H_kv, d, int(l), float(scale), _f32(mass, B * H * int(l)), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                       B, T, H, H_kv, d, int(l), float(scale), _ptr(mass), _ptr(workspace), workspace.numel() * workspace.element_size(),
                                        _stream(stream)), "moda_depth_slot_mass")
     return mass
 
@@ -490,12 +497,10 @@ def moda_attn_fwd(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=None):
     """O [B,T,H,d] bf16 and LSE [B,H,T] fp32 of the MoDA operator (outputs allocated if not given)."""
     B, T, H, d = _bthd(Q, "Q")
     assert _bthd(K, "K") == (B, T, H, d) and _bthd(V, "V") == (B, T, H, d)
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T, torch.float32)
     _check(load().moda_attn_fwd(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
-                                B, T, H, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
+                                B, T, H, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
            "moda_attn_fwd")
     return O, LSE
 
@@ -510,17 +515,18 @@ def moda_attn_bwd(Q, K, V, depth_kv, O, dO, LSE, l, scale,
 
     With ``stages`` (a MODA_BWD_STAGE_* mask) the call goes through moda_attn_bwd_stages."""
     B, T, H, d = _bthd(Q, "Q")
-    dQ = _new_like(Q, stream) if dQ is None else dQ
-    dK = _new_like(Q, stream) if dK is None else dK
-    dV = _new_like(Q, stream) if dV is None else dV
+    n = Q.numel()
+    dQ = _new_like(Q, stream) if dQ is None else _given(dQ, n, torch.bfloat16)
+    dK = _new_like(Q, stream) if dK is None else _given(dK, Q.numel(), torch.bfloat16)
+    dV = _new_like(Q, stream) if dV is None else _given(dV, Q.numel(), torch.bfloat16)
     if l > 0 and d_depth_kv is None:
         d_depth_kv = alloc_depth_cache(B, T, H, d, l, Q.device, stream)
     need = moda_bwd_workspace_bytes(B, T, H, d, l)
     if workspace is None:
         workspace = _new((need,), torch.uint8, Q.device, stream)
-    args = [_ptr(Q), _bf16(K, Q.numel()), _bf16(V, Q.numel()), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
-            _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
-            _bf16(dQ, Q.numel()), _bf16(dK, Q.numel()), _bf16(dV, Q.numel()), _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
+    args = [_ptr(Q), _bf16(K, n), _bf16(V, n), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
+            _bf16(O, n), _bf16(dO, n), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
+            _ptr(dQ), _ptr(dK), _ptr(dV), _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
             _ptr(workspace), workspace.numel() * workspace.element_size()]
     if stages is None:
         _check(load().moda_attn_bwd(*args, _stream(stream)), "moda_attn_bwd")
@@ -543,12 +549,13 @@ def moda_attn_bwd_static_scratch(Q, K, V, depth_kv, O, dO, LSE, l, scale, dQ, dK
     Limit: B*H*T <= MODA_STATIC_SCRATCH_ROWS (error -11 beyond it).  Calls on one device share that
     array: do not let two of them overlap on the GPU."""
     B, T, H, d = _bthd(Q, "Q")
+    n = Q.numel()
     if l > 0 and d_depth_kv is None:
         raise ValueError("d_depth_kv must be provided: this entry point allocates nothing")
     _check(load().moda_attn_bwd_static_scratch(
-        _ptr(Q), _bf16(K, Q.numel()), _bf16(V, Q.numel()), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
-        _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
-        _bf16(dQ, Q.numel()), _bf16(dK, Q.numel()), _bf16(dV, Q.numel()), _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
+        _ptr(Q), _bf16(K, n), _bf16(V, n), _slots(depth_kv, int(l), B, T, H, d) if l > 0 else None,
+        _bf16(O, n), _bf16(dO, n), _f32(LSE, B * H * T), B, T, H, d, int(l), float(scale),
+        _bf16(dQ, n), _bf16(dK, n), _bf16(dV, n), _slots(d_depth_kv, int(l), B, T, H, d) if l > 0 else None,
         _stream(stream)), "moda_attn_bwd_static_scratch")
     return dQ, dK, dV, d_depth_kv
 
@@ -572,12 +579,10 @@ def moda_attn_fwd_gqa(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=None
     if stream is None and (out := host().attn_fwd(Q, K, V, depth_kv, l, scale, None, 0, O, LSE)) is not None:
         return out
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T, torch.float32)
     _check(load().moda_attn_fwd_gqa(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
-                                    B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T), _stream(stream)),
+                                    B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE), _stream(stream)),
            "moda_attn_fwd_gqa")
     return O, LSE
 
@@ -590,12 +595,10 @@ def moda_attn_fwd_append(Q, K, V, depth_kv, l, scale, append_cache, append_slot,
         if out is not None:
             return out
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T, torch.float32)
     _check(load().moda_attn_fwd_append(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
-                                       B, T, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T),
+                                       B, T, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
                                        _slots(append_cache, int(append_slot) + 1, B, T, Hk, d), int(append_slot), _stream(stream)),
            "moda_attn_fwd_append")
     return O, LSE
@@ -611,16 +614,17 @@ def moda_attn_bwd_gqa(Q, K, V, depth_kv, O, dO, LSE, l, scale,
         if out is not None:
             return out
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    dQ = _new_like(Q, stream) if dQ is None else dQ
-    dK = _new_like(K, stream) if dK is None else dK
-    dV = _new_like(V, stream) if dV is None else dV
+    n = Q.numel()
+    dQ = _new_like(Q, stream) if dQ is None else _given(dQ, n, torch.bfloat16)
+    dK = _new_like(K, stream) if dK is None else _given(dK, K.numel(), torch.bfloat16)
+    dV = _new_like(V, stream) if dV is None else _given(dV, V.numel(), torch.bfloat16)
     if l > 0 and d_depth_kv is None:
         d_depth_kv = alloc_depth_cache(B, T, Hk, d, l, Q.device, stream)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
     args = [_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
-            _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T), B, T, H, Hk, d, int(l), float(scale),
-            _bf16(dQ, Q.numel()), _bf16(dK, K.numel()), _bf16(dV, K.numel()), _slots(d_depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
+            _bf16(O, n), _bf16(dO, n), _f32(LSE, B * H * T), B, T, H, Hk, d, int(l), float(scale),
+            _ptr(dQ), _ptr(dK), _ptr(dV), _slots(d_depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
             _ptr(workspace), workspace.numel() * workspace.element_size()]
     if stages is None:
         _check(load().moda_attn_bwd_gqa(*args, _stream(stream)), "moda_attn_bwd_gqa")
@@ -647,14 +651,15 @@ def moda_attn_bwd_gqa_slot(Q, K, V, depth_kv, O, dO, LSE, l, scale, d_depth_kv, 
         if out is not None:
             return out[:3]
     B, T, H, Hk, d = _gqa_shapes(Q, K, V)
-    dQ = _new_like(Q, stream) if dQ is None else dQ
-    dK = _new_like(K, stream) if dK is None else dK
-    dV = _new_like(V, stream) if dV is None else dV
+    n = Q.numel()
+    dQ = _new_like(Q, stream) if dQ is None else _given(dQ, n, torch.bfloat16)
+    dK = _new_like(K, stream) if dK is None else _given(dK, K.numel(), torch.bfloat16)
+    dV = _new_like(V, stream) if dV is None else _given(dV, V.numel(), torch.bfloat16)
     if workspace is None:
         workspace = _new((moda_bwd_workspace_bytes_gqa(B, T, H, Hk, d, l),), torch.uint8, Q.device, stream)
     _check(load().moda_attn_bwd_gqa_slot(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T, Hk, d) if l > 0 else None,
-                                         _bf16(O, Q.numel()), _bf16(dO, Q.numel()), _f32(LSE, B * H * T),
-                                         B, T, H, Hk, d, int(l), float(scale), _bf16(dQ, Q.numel()), _bf16(dK, K.numel()), _bf16(dV, K.numel()),
+                                         _bf16(O, n), _bf16(dO, n), _f32(LSE, B * H * T),
+                                         B, T, H, Hk, d, int(l), float(scale), _ptr(dQ), _ptr(dK), _ptr(dV),
                                          _slots(d_depth_kv, int(slot) + 1, B, T, Hk, d),
                                          _ptr(workspace), workspace.numel() * workspace.element_size(), int(slot), _stream(stream)),
            "moda_attn_bwd_gqa_slot")
@@ -679,14 +684,12 @@ def moda_attn_decode(q, K, V, depth_kv_token, T_kv, l, scale, O=None, LSE=None, 
     if l > 0 and (depth_kv_token is None or tuple(depth_kv_token.shape) != (l, B, Hk, 2, d)
                   or depth_kv_token.dtype != torch.bfloat16):
         raise ValueError("depth_kv_token must be a bf16 [l, B, H_kv, 2, d] tensor")
-    if O is None:
-        O = _new_like(q, stream)
-    if LSE is None:
-        LSE = _new((B, H), torch.float32, q.device, stream)
+    O = _new_like(q, stream) if O is None else _given(O, B * H * d, torch.bfloat16)
+    LSE = _new((B, H), torch.float32, q.device, stream) if LSE is None else _given(LSE, B * H, torch.float32)
     if workspace is None:
         workspace = _new((moda_decode_workspace_bytes(B, H, d),), torch.uint8, q.device, stream)
     _check(load().moda_attn_decode(_ptr(q), _ptr(K), _ptr(V), _ptr(depth_kv_token) if l > 0 else None,
-                                   B, int(T_kv), T_cap, H, Hk, d, int(l), float(scale), _bf16(O, B * H * d), _f32(LSE, B * H),
+                                   B, int(T_kv), T_cap, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
                                    _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_decode")
     return O, LSE
@@ -699,22 +702,18 @@ def moda_attn_fwd_prefill(Q, K, V, depth_kv, l, scale, O=None, LSE=None, stream=
     Bk, T_kv, Hk, dk = _bthd(K, "K")
     if (Bk, dk) != (B, d) or _bthd(V, "V") != (B, T_kv, Hk, d):
         raise ValueError("K and V must be bf16 [B, T_kv, H_kv, d] tensors matching Q's B and d")
-    if O is None:
-        O = _new_like(Q, stream)
-    if LSE is None:
-        LSE = _new((B, H, T_q), torch.float32, Q.device, stream)
+    O = _new_like(Q, stream) if O is None else _given(O, Q.numel(), torch.bfloat16)
+    LSE = _new((B, H, T_q), torch.float32, Q.device, stream) if LSE is None else _given(LSE, B * H * T_q, torch.float32)
     _check(load().moda_attn_fwd_prefill(_ptr(Q), _ptr(K), _ptr(V), _slots(depth_kv, int(l), B, T_q, Hk, d) if l > 0 else None,
-                                        B, T_q, T_kv, H, Hk, d, int(l), float(scale), _bf16(O, Q.numel()), _f32(LSE, B * H * T_q),
+                                        B, T_q, T_kv, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
                                         _stream(stream)), "moda_attn_fwd_prefill")
     return O, LSE
 
 
 def _decode_outputs(q, O, LSE, workspace, stream):
     B, H, d = q.shape
-    if O is None:
-        O = _new_like(q, stream)
-    if LSE is None:
-        LSE = _new((B, H), torch.float32, q.device, stream)
+    O = _new_like(q, stream) if O is None else _given(O, B * H * d, torch.bfloat16)
+    LSE = _new((B, H), torch.float32, q.device, stream) if LSE is None else _given(LSE, B * H, torch.float32)
     if workspace is None:
         workspace = _new((moda_decode_workspace_bytes(B, H, d),), torch.uint8, q.device, stream)
     return O, LSE, workspace
@@ -741,7 +740,7 @@ def moda_attn_decode_varlen(q, K, V, seq_lens, depth_kv_token, max_seq_len, l, s
     O, LSE, workspace = _decode_outputs(q, O, LSE, workspace, stream)
     _check(load().moda_attn_decode_varlen(_bf16(q, B * H * d), _bf16(K, B * T_cap * Hk * d), _bf16(V, B * T_cap * Hk * d), _ptr(seq_lens),
                                           _token(depth_kv_token, l, B, Hk, d),
-                                          B, int(max_seq_len), T_cap, H, Hk, d, int(l), float(scale), _bf16(O, B * H * d), _f32(LSE, B * H),
+                                          B, int(max_seq_len), T_cap, H, Hk, d, int(l), float(scale), _ptr(O), _ptr(LSE),
                                           _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_decode_varlen")
     return O, LSE
@@ -764,7 +763,7 @@ def moda_attn_decode_paged(q, K_pages, V_pages, block_table, seq_lens, depth_kv_
                                          _bf16(V_pages, num_pages * page_size * Hk * d), _ptr(block_table), _ptr(seq_lens),
                                          _token(depth_kv_token, l, B, Hk, d),
                                          B, int(max_seq_len), page_size, num_pages, block_table.shape[1], H, Hk, d, int(l),
-                                         float(scale), _bf16(O, B * H * d), _f32(LSE, B * H), _ptr(workspace),
+                                         float(scale), _ptr(O), _ptr(LSE), _ptr(workspace),
                                          workspace.numel() * workspace.element_size(), _stream(stream)),
            "moda_attn_decode_paged")
     return O, LSE

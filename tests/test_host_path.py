@@ -152,6 +152,11 @@ def test_buffers_are_looked_at_before_their_address_is_taken():
         with pytest.raises(ValueError, match=text):
             f()
     assert binding._bf16(None, 9) is None and binding._slots(None, 1, 1, 64, 2, 64) is None
+    for B, T, H, d, n in ((1, 1, 1, 64, 1), (2, 128, 3, 128, 4), (3, 129, 2, 64, 256), (1, 1000, 16, 128, 7)):
+        for e4m3, size in ((False, moda.moda_depth_cache_bytes(B, T, H, d, n)), (True, moda.moda_depth_cache_e4m3_bytes(B, T, H, d, n))):
+            for short, text in ((1, "take"), (0, "CUDA")):
+                with pytest.raises(ValueError, match=text):
+                    binding._slots(torch.empty(size - short, dtype=torch.uint8, device="meta"), n, B, T, H, d, e4m3=e4m3)
 
 
 @gpu
