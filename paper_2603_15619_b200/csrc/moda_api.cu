@@ -259,11 +259,11 @@ int launch_depth_merge(DepthMergeParams m, cudaStream_t stream) {
 // position-major bf16 (moda_cache.cuh).
 enum CacheKind { kCacheRows = 0, kCacheE4m3 = 1, kCachePm = 2 };
 
-// Dynamic shared memory of the forward kernel that reads an e4m3 depth cache (only the variant each head size runs exists).
-template <int D>
-constexpr int fwd_smem_e4m3() {
-    if constexpr (D == 64) return Fwd2Smem<64, true>::kDynamic;
-    else return FwdSmem<128, 2, true>::kDynamic;
+// Dynamic shared memory of the forward kernels (only the variant that each head size runs exists).
+template <int D, bool FP8>
+constexpr int fwd_smem() {
+    if constexpr (D == 64) return Fwd2Smem<64, FP8>::kDynamic;
+    else return FwdSmem<128, 2, FP8>::kDynamic;
 }
 
 template <int D>
@@ -271,8 +271,7 @@ int launch_fwd(const void* Q, const void* K, const void* V, const void* depth_kv
                float scale, void* O, float* LSE, void* append_slot, cudaStream_t stream, CacheKind kind = kCacheRows) {
     const bool fp8 = kind == kCacheE4m3, pm = kind == kCachePm;
     constexpr bool kWide = (D == 64);
-    constexpr int kSmem = kWide ? Fwd2Smem<D>::kDynamic : FwdSmem<D, 2>::kDynamic;
-    constexpr int kSmem8 = fwd_smem_e4m3<D>();
+    constexpr int kSmem = fwd_smem<D, false>(), kSmem8 = fwd_smem<D, true>();
     constexpr int kSmemDeep = FwdSmem<128, 1>::kDynamic;
     constexpr int kThreads = kWide ? kFwd2Threads : kFwdThreads;
     CUtensorMap mQ, mK, mV, mO;

@@ -1,8 +1,7 @@
-// MoDA forward kernel, wide variant: two softmax warpgroups and (for d = 64) three score buffers.
-// Same operator, boundary and data layout as moda_fwd_kernel (see moda_fwd.cuh); used where the
-// exponentials, not the tensor pipe, set the pace (d = 64: a 128x128 score tile costs 1024 SFU cycles
-// but only 512 tensor cycles), and where TMEM has room for a third score buffer (O and o_d take
-// 64 columns each at d = 64).
+// MoDA forward kernel at d = 64: two softmax warpgroups and three score buffers (the d = 128 form with two is in moda_fwd_wide128.cuh).
+// Same operator, boundary and data layout as moda_fwd_kernel (see moda_fwd.cuh).  The exponentials, not the tensor pipe, set the
+// pace (a 128x128 score tile costs 1024 SFU cycles but only 512 tensor cycles), and TMEM has room for a third score buffer (O
+// and o_d take 64 columns each).
 //
 // One CTA owns one (b, h, 128-query-row tile).  512 threads, four warpgroups:
 //
@@ -22,9 +21,7 @@
 //   warp 14          depth-cache producer (bulk copies).
 //   warp 15          MMA issuer for O += P_j V_j.
 //
-// TMEM columns (fp32): S/P buffer b = j mod stages at [128 b, 128 b + 128); then O (D columns) and
-// o_d (D columns): d = 64: 3 buffers, O at 384, o_d at 448 (d = 128 would get 2 buffers, O at 256,
-// o_d at 384).
+// TMEM columns (fp32): S/P buffer b = j mod 3 at [128 b, 128 b + 128), O at 384, o_d at 448.
 #pragma once
 
 #include "moda_cache.cuh"
@@ -39,11 +36,12 @@ constexpr int kFwdBN = 128;                 // keys per inner tile
 
 template <int D, bool FP8 = false>
 struct Fwd2Smem {
+    static_assert(D == 64, "tensor memory holds three score buffers at d = 64 only");
     static constexpr int kTileBytes = kTileRows * D * 2;          // one 128 x D bf16 tile
     static constexpr int kSubBytes = kTileRows * 128;             // one 128 x 64 sub-tile
-    // K / V ring stages = score buffers in TMEM.  d = 64 leaves TMEM room for a third buffer, which
-    // is what lets the two softmax warpgroups run without waiting for each other's P to be consumed.
-    static constexpr int kStages = (D == 64) ? 3 : 2;
+    // K / V ring stages = score buffers in TMEM.  The third is what lets the two softmax warpgroups run without waiting for each
+    // other's P to be consumed.
+    static constexpr int kStages = 3;
     static constexpr int kKeyTileBytes = kFwdBN * D * 2;          // one BN x D bf16 key / value tile
     static constexpr int kKeySubBytes = kFwdBN * 128;             // one BN x 64 sub-tile
     static constexpr int kQ = 0;
@@ -58,7 +56,7 @@ struct Fwd2Smem {
     // with the 128 row scales beside them (moda_cache.cuh)
     static constexpr int kUnitBytes = FP8 ? kTileRows * D : 8 * kTileRows * 16;
     static constexpr int kScaleBytes = FP8 ? kTileRows * 4 : 0;
-    static constexpr int kRingStages = (D == 128) ? 3 : 5;
+    static constexpr int kRingStages = 5;
     static constexpr int kScale = kRing + kRingStages * kUnitBytes;   // [ring stage][128] fp32 (e4m3 only)
     static constexpr int kBars = kScale + kRingStages * kScaleBytes;
     static constexpr int kNumBars = 48;
@@ -96,7 +94,7 @@ moda_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     using L = Fwd2Smem<D, FP8>;
     constexpr int NSUB = D / 64;
     constexpr uint32_t kTmemCols = 512;
-    constexpr uint32_t kColO = L::kStages * 128, kColOd = kColO + ((D == 128) ? 128 : 64);
+    constexpr uint32_t kColO = L::kStages * 128, kColOd = kColO + D;
 
     if (g_moda_status != 0) return;   // an earlier kernel gave up a wait: do not pile up more timeouts
 

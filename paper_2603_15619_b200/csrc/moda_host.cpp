@@ -2,9 +2,9 @@
 // C entry points of libmoda_b200.so, and the autograd node of moda_attention.
 //
 // It serves the plain case alone: torch.Tensor (or Parameter) objects on the device, contiguous, of the documented types and
-// shapes, on the current stream, with no dispatch mode, transform or tracer active.  For anything else a function
-// returns None and the caller goes on with its own code (binding.py, autograd.py), which knows every check and says what
-// is wrong.  A call through here makes the same C call with the same arguments.
+// sizes, on the current stream, with no mode, transform or tracer active.  For anything else a function returns None and the
+// caller goes on with its own code (binding.py, autograd.py), which has the same checks and says what is wrong.  A call through here
+// makes the same C call with the same arguments.
 //
 // Why: at the sizes of a decode step or of a small layer the device waits for the host.  Microseconds a call in a loop, through
 // Python and ctypes -> through here: decode of one sequence over 8192 keys 15.9 -> 12.3 (10 on the device); T = 256, 2 heads, l = 4:
