@@ -189,7 +189,7 @@ def _given(t, numel, dtype):
 
 
 def _bf16(t, numel, dtype=torch.bfloat16):
-    """Its address."""
+    """Address of such a tensor, None for None."""
     if t is None:
         return None
     if t.dtype is dtype and t.numel() >= numel and t.is_cuda and t.is_contiguous():

@@ -5,6 +5,7 @@ import os
 import subprocess
 import sys
 
+from . import binding
 from .binding import HOST_PATH as HOST
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -69,6 +70,8 @@ def build_host(force: bool = False, verbose: bool = False) -> str:
         if res.returncode != 0:
             raise RuntimeError(f"g++ failed building {HOST}")
         os.replace(tmp, HOST)
+    if isinstance(binding._host, binding._NoHost):            # calls of this process that came before the build
+        binding._host = None
     return HOST
 
 

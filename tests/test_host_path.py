@@ -369,6 +369,13 @@ def test_a_build_is_for_one_python_and_one_torch():
     assert build.HOST == binding.HOST_PATH and torch.__version__ in build.HOST and sysconfig.get_config_var("SOABI") in build.HOST
 
 
+def test_a_build_is_taken_up_by_the_process_that_makes_it(monkeypatch):
+    from paper_2603_15619_b200 import build
+    monkeypatch.setattr(binding, "_host", binding._NoHost())
+    build.build_host()
+    assert binding.host().__spec__.origin == binding.HOST_PATH
+
+
 class _Calls(torch.overrides.TorchFunctionMode):
     """Names of the torch functions that pass a torch-function mode."""
 
